@@ -68,8 +68,14 @@ enum {
  * work is cut into equal ranges of (128-row block, K step), one per resident
  * CTA, and shared blocks are reduced from fp32 partials in a fixed order) --
  * on mma.sync with the codes dequantised in registers, except, with 16-byte
- * aligned x and codes: int4 with 17 <= M <= 64 (K a multiple of 128), and
- * int8 with 33 <= M <= 64 or K >= 16384, which run on tcgen05 with each
+ * aligned x and codes: int4 and a bf16 result with M <= 16 and at least 2^24
+ * weights, or SwiGLU with M <= 32 and at least 2^28 (scales and zeros 16-byte
+ * aligned too), which runs on tcgen05 with 8-bit operands (the codes as they
+ * are; x split by a first kernel into two e4m3 pieces an element, which carry
+ * it exactly down to 2^-13 of its row's largest value and to 2^-23 of that
+ * value below; scales and zero points applied in fp32; a row of x that holds an
+ * infinity or a NaN gives NaN); int4 with 17 <= M <= 64 otherwise, and int8
+ * with 33 <= M <= 64 or K >= 16384, which run on tcgen05 with each
  * weight expanded in TMEM (int4 to bf16((q - z) s) as the prefill GEMM does,
  * int8 to the integer code, its row scale applied to the fp32 sums); bf16
  * with 17 <= M <= 64 on matrices that give every SM at least 48 items of 32
@@ -96,7 +102,8 @@ size_t fp_op_linear_workspace_bytes(int wquant, int M, int N, int K);
 /* The weight-only linear of fp_op_linear for FP_W_GPTQ4 weights (codes,
  * scales, zeros as fp_op_quantize_gptq4 writes them; perm the act order).
  * y = x W^T with W in channel order.  M <= 64: x is gathered into the act
- * order in the workspace (one kernel) and the int4 decode linear runs on it;
+ * order in the workspace (one kernel, which also splits it where the linear
+ * takes 8-bit operands) and the int4 decode linear runs on it;
  * M > 64: the weights are expanded back into channel order (the inverse act
  * order is computed into the workspace) and the prefill GEMM multiplies x as
  * it is.  workspace: 256-byte aligned, at least

@@ -102,6 +102,19 @@ inline cudaError_t launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t 
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// As launch, always with the programmatic-serialisation attribute: the kernel
+// may start while the one before it in the stream runs, and waits for it
+// (pdl_wait) before it touches anything that kernel writes.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                Args... args) {
+  const bool was = g_pdl;
+  g_pdl = true;
+  const cudaError_t e = launch(kern, grid, block, smem, s, args...);
+  g_pdl = was;
+  return e;
+}
+
 // Lifts a kernel's dynamic shared-memory limit to `bytes` once per device:
 // function attributes belong to each device's context, so a process that
 // drives several GPUs sets it on each.  `done` (one per call site) holds a

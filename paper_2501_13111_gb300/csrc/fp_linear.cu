@@ -793,7 +793,7 @@ static cudaError_t launch_mma(int epi, const uint16_t* x, int M, int N, int K, c
 // Workspace of one linear launch: the ticket area, then either split-K
 // partials (decode GEMV) or the bf16 expansion of quantised weights (prefill
 // GEMM).  The ticket area is never written by the prefill path.
-size_t linear_ws_bytes(int wquant, int M, int N, int K) {
+size_t linear_ws_need(int wquant, int M, int N, int K) {
   if (M > 64 && gemm_tc_ok(M, N, K)) {
     const size_t w = gemm_tc_ws_bytes(wquant, N, K);
     return w ? counter_bytes(0) + w : 0;
@@ -808,6 +808,22 @@ size_t linear_ws_bytes(int wquant, int M, int N, int K) {
   return w;
 }
 
+size_t linear_ws_bytes(int wquant, int M, int N, int K) {
+  size_t w = linear_ws_need(wquant, M, N, K);
+  for (int epi : {FP_EPI_STORE, FP_EPI_SWIGLU})
+    if (f8_ok(wquant, epi, M, N, K)) w = std::max(w, f8_ws_bytes(epi, M, N, K));
+  return w;
+}
+
+// The int4 decode linear with 8-bit operands, wherever its workspace fits
+// (TMA needs 16-byte aligned codes; x, scales and zeros are read in 16-byte pieces).
+static bool take_f8(int wquant, int epi, const uint16_t* x, int M, int N, int K, const void* codes,
+                    const uint16_t* scales, const uint16_t* zeros, const void* ws, size_t ws_bytes) {
+  return f8_ok(wquant, epi, M, N, K) && ws &&
+         (((uintptr_t)x | (uintptr_t)codes | (uintptr_t)scales | (uintptr_t)zeros | (uintptr_t)ws) & 15) == 0 &&
+         ws_bytes >= f8_ws_bytes(epi, M, N, K);
+}
+
 size_t linear_ws_bytes_upto(int wquant, int max_m, int N, int K) {
   size_t w = 0;
   for (int m = 1; m <= std::min(max_m, 64); ++m) w = std::max(w, linear_ws_bytes(wquant, m, N, K));
@@ -820,7 +836,7 @@ cudaError_t launch_linear(int wquant, int epi, const uint16_t* x, int M, int N, 
                           void* ws, size_t ws_bytes, cudaStream_t s, int32_t* err) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (M > 64 && gemm_tc_ok(M, N, K)) {
-    const size_t need = linear_ws_bytes(wquant, M, N, K);
+    const size_t need = linear_ws_need(wquant, M, N, K);
     // int8 / int4 without room for the bf16 expansion: dequantise inside the GEMM
     if (need > 0 && (!ws || ws_bytes < need) && gemm_wq_ok(wquant, epi, M, N, K, x, codes))
       return launch_gemm_wq(wquant, epi, x, M, N, K, codes, scales, zeros, residual, y, err, s);
@@ -829,6 +845,8 @@ cudaError_t launch_linear(int wquant, int epi, const uint16_t* x, int M, int N, 
     return launch_gemm_tc(wquant, epi, x, M, N, K, codes, scales, zeros, residual, y, scratch,
                           need ? ws_bytes - counter_bytes(0) : 0, err, s);
   }
+  if (take_f8(wquant, epi, x, M, N, K, codes, scales, zeros, ws, ws_bytes))
+    return launch_f8(epi, x, nullptr, M, N, K, codes, scales, zeros, residual, y, ws, ws_bytes, err, s);
   // bf16 weights at 17-64 tokens: the TMA-fed tcgen05 GEMV where every SM gets
   // enough 32 KB items to hide their per-item cost (16-byte aligned x and weights)
   if (btc_ok(wquant, epi, M, N, K) && btc_preferred(epi, N, K) && ((uintptr_t)x & 15) == 0 &&
@@ -858,24 +876,32 @@ cudaError_t launch_linear(int wquant, int epi, const uint16_t* x, int M, int N, 
 namespace fpk {
 
 // ---- GPTQ4 (int4 over an act order)
-// Decode (M <= 64): the workspace holds the int4 linear's own workspace
-// (ticket area first, kept at offset 0 whatever the shape) and then x in act
-// order, xp[m][j] = x[m][perm[j]]; the stored matrix is a plain int4 g128
-// matrix of the act-order channels, so y = xp W_stored^T.  Prefill: the
+// Decode (M <= 64): the stored matrix is a plain int4 g128 matrix of the
+// act-order channels, so y = xp W_stored^T with xp[m][j] = x[m][perm[j]].  The
+// int4 linear with 8-bit operands reads x through perm while it splits it;
+// otherwise the workspace holds the int4 linear's own workspace (ticket area
+// first, kept at offset 0 whatever the shape) and then xp.  Prefill: the
 // bf16 expansion puts each weight back in channel order (inv, the inverse
 // act order; computed into the workspace when the caller passes none) and
 // the GEMM multiplies x as it is.
 static size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 static size_t gptq4_xp_offset(int M, int N, int K) {
-  return align256(std::max(linear_ws_bytes(FP_W_INT4_G128, M, N, K), counter_bytes(0)));
+  return align256(std::max(linear_ws_need(FP_W_INT4_G128, M, N, K), counter_bytes(0)));
+}
+
+size_t linear_gptq4_ws_need(int M, int N, int K, bool with_inv) {
+  if (M <= 0 || N <= 0 || K <= 0) return 0;
+  if (M > 64) return align256(std::max(linear_ws_need(FP_W_INT4_G128, M, N, K), counter_bytes(0))) +
+                     (with_inv ? align256((size_t)K * 4) : 0);
+  return gptq4_xp_offset(M, N, K) + align256((size_t)M * K * 2);
 }
 
 size_t linear_gptq4_ws_bytes(int M, int N, int K, bool with_inv) {
-  if (M <= 0 || N <= 0 || K <= 0) return 0;
-  if (M > 64) return align256(std::max(linear_ws_bytes(FP_W_INT4_G128, M, N, K), counter_bytes(0))) +
-                     (with_inv ? align256((size_t)K * 4) : 0);
-  return gptq4_xp_offset(M, N, K) + align256((size_t)M * K * 2);
+  size_t w = linear_gptq4_ws_need(M, N, K, with_inv);
+  for (int epi : {FP_EPI_STORE, FP_EPI_SWIGLU})
+    if (f8_ok(FP_W_INT4_G128, epi, M, N, K)) w = std::max(w, align256(f8_ws_bytes(epi, M, N, K)));
+  return w;
 }
 
 size_t linear_gptq4_ws_bytes_upto(int max_m, int N, int K, bool with_inv) {
@@ -890,10 +916,10 @@ cudaError_t launch_linear_gptq4(int epi, const uint16_t* x, int M, int N, int K,
                                 const uint16_t* zeros, const uint16_t* residual, void* y, void* ws, size_t ws_bytes,
                                 cudaStream_t s, int32_t* err) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  if (!ws || ws_bytes < linear_gptq4_ws_bytes(M, N, K, inv == nullptr)) return cudaErrorInvalidValue;
+  if (!ws || ws_bytes < linear_gptq4_ws_need(M, N, K, inv == nullptr)) return cudaErrorInvalidValue;
   if (M > 64) {
     if (!gemm_tc_ok(M, N, K)) return cudaErrorInvalidValue;
-    const size_t lin = align256(std::max(linear_ws_bytes(FP_W_INT4_G128, M, N, K), counter_bytes(0)));
+    const size_t lin = align256(std::max(linear_ws_need(FP_W_INT4_G128, M, N, K), counter_bytes(0)));
     if (!inv) {
       int32_t* tmp = (int32_t*)((char*)ws + lin);
       FP_CUDA_TRY(launch_invert_perm(perm, K, tmp, err, s));
@@ -902,6 +928,8 @@ cudaError_t launch_linear_gptq4(int epi, const uint16_t* x, int M, int N, int K,
     return launch_gemm_tc(FP_W_GPTQ4, epi, x, M, N, K, codes, scales, zeros, residual, y,
                           (char*)ws + counter_bytes(0), lin - counter_bytes(0), err, s, inv);
   }
+  if (take_f8(FP_W_INT4_G128, epi, x, M, N, K, codes, scales, zeros, ws, ws_bytes))
+    return launch_f8(epi, x, perm, M, N, K, codes, scales, zeros, residual, y, ws, ws_bytes, err, s);
   uint16_t* xp = (uint16_t*)((char*)ws + gptq4_xp_offset(M, N, K));
   FP_CUDA_TRY(launch_gather_cols(x, M, K, perm, xp, err, s));
   return launch_linear(FP_W_INT4_G128, epi, xp, M, N, K, codes, scales, zeros, residual, y, ws,

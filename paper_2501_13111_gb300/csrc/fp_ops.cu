@@ -59,7 +59,7 @@ int fp_op_linear_gptq4(int epilogue, const uint16_t* x, int M, int N, int K, con
   if (epilogue == FP_EPI_SWIGLU && N % 2 != 0) return FP_ERR_INVALID_ARG;
   if (K % 128 != 0) return FP_ERR_UNSUPPORTED;
   if (M == 0) return FP_OK;
-  if (!workspace || workspace_bytes < linear_gptq4_ws_bytes(M, N, K, true) || ((uintptr_t)workspace & 255))
+  if (!workspace || workspace_bytes < linear_gptq4_ws_need(M, N, K, true) || ((uintptr_t)workspace & 255))
     return FP_ERR_INVALID_ARG;
   return cuda_status(launch_linear_gptq4(epilogue, x, M, N, K, perm, nullptr, codes, scales, zeros, residual, y,
                                          workspace, workspace_bytes, (cudaStream_t)stream, err));
@@ -87,7 +87,7 @@ int fp_op_linear(int wquant, int epilogue, const uint16_t* x, int M, int N, int 
   if (epilogue == FP_EPI_SWIGLU && N % 2 != 0) return FP_ERR_INVALID_ARG;
   if (K % k_align(wquant) != 0) return FP_ERR_UNSUPPORTED;
   if (M == 0) return FP_OK;
-  size_t need = linear_ws_bytes(wquant, M, N, K);
+  size_t need = linear_ws_need(wquant, M, N, K);
   // quantised prefill without room for the bf16 expansion: the GEMM that
   // dequantises in the kernel needs no workspace
   const bool no_scratch = !workspace || workspace_bytes < need;

@@ -296,14 +296,16 @@ bool bad_shape(const fp_arch* a, int wq, std::string& why) {
     h->tr.after(cls);                                          \
   } while (0)
 
-// One block linear: the GPTQ4 path (its decode gather counts as a launch of
-// its own) or the weight-only linear of the handle's format.
+// One block linear: the GPTQ4 path or the weight-only linear of the handle's
+// format.  At decode both int4 formats take a second kernel (x split into its
+// pieces, or gathered into the act order), counted here.
 cudaError_t block_linear(fp_handle* h, int epi, const uint16_t* x, int M, const Mat& W, const uint16_t* R, void* y) {
   if (h->wq == FP_W_GPTQ4) {
     if (M <= 64) h->launches += 1;
     return launch_linear_gptq4(epi, x, M, W.N, W.K, W.perm, W.inv, W.codes, W.scales, W.zeros, R, y, h->lin_ws,
                                h->lin_ws_bytes, h->stream, h->err);
   }
+  if (f8_ok(h->wq, epi, M, W.N, W.K)) h->launches += 1;
   return launch_linear(h->wq, epi, x, M, W.N, W.K, W.codes, W.scales, W.zeros, R, y, h->lin_ws, h->lin_ws_bytes,
                        h->stream, h->err);
 }

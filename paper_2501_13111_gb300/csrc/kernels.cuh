@@ -55,7 +55,9 @@ cudaError_t launch_attention_prefill(const uint16_t* q, int q_stride, int B, int
 // ---- weight-only linear (fp_linear.cu)
 // Split-K ticket counters at the head of a linear's workspace (zero at rest).
 constexpr int kLinTicketSlots = 4096;
-// Workspace of one launch with exactly these M, N, K (any epilogue); 0 if none.
+// Workspace of one launch with exactly these M, N, K (any epilogue); 0 if none:
+// what a call must bring (need), and what it brings for the fastest path (bytes).
+size_t linear_ws_need(int wquant, int M, int N, int K);
 size_t linear_ws_bytes(int wquant, int M, int N, int K);
 // Largest workspace over every M in [1, max_m].
 size_t linear_ws_bytes_upto(int wquant, int max_m, int N, int K);
@@ -66,12 +68,21 @@ cudaError_t launch_linear(int wquant, int epi, const uint16_t* x, int M, int N, 
 // GPTQ4 linear (fp_linear.cu): decode gathers x into the act order, prefill
 // expands the weights back into channel order.  inv may be NULL (computed
 // into the workspace, which is then K * 4 bytes larger for M > 64).
+size_t linear_gptq4_ws_need(int M, int N, int K, bool with_inv);
 size_t linear_gptq4_ws_bytes(int M, int N, int K, bool with_inv);
 size_t linear_gptq4_ws_bytes_upto(int max_m, int N, int K, bool with_inv);
 cudaError_t launch_linear_gptq4(int epi, const uint16_t* x, int M, int N, int K, const int32_t* perm,
                                 const int32_t* inv, const void* codes, const uint16_t* scales,
                                 const uint16_t* zeros, const uint16_t* residual, void* y, void* ws, size_t ws_bytes,
                                 cudaStream_t s, int32_t* err);
+
+// ---- int4 decode linear on tcgen05 with 8-bit operands (fp_gemv_f8.cu)
+bool f8_ok(int wquant, int epi, int M, int N, int K);
+size_t f8_ws_bytes(int epi, int M, int N, int K);
+// perm: the act order of a GPTQ4 matrix, else NULL.  Two kernels.
+cudaError_t launch_f8(int epi, const uint16_t* x, const int32_t* perm, int M, int N, int K, const void* codes,
+                      const uint16_t* scales, const uint16_t* zeros, const uint16_t* residual, void* y, void* ws,
+                      size_t ws_bytes, int32_t* err, cudaStream_t s);
 
 // ---- int4 / int8 decode linear at 17-64 tokens on tcgen05 (fp_gemv_tc.cu)
 bool q4tc_ok(int wquant, int epi, int M, int N, int K);

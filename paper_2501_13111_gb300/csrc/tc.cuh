@@ -80,6 +80,14 @@ FP_DEV void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_
       : "memory");
 }
 
+// 1-D bulk copy: bytes a multiple of 16, both addresses 16-byte aligned.
+FP_DEV void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups
 // 1024 bytes apart (stride byte offset), fixed field 0b001 at bit 46.
 FP_DEV uint64_t sdesc(uint32_t saddr) {
@@ -115,6 +123,19 @@ FP_DEV void tc_mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t
       "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// As tc_mma_ts for 8-bit operands (kind::f8f6f4, K 32 per instruction): A
+// four K elements per 32-bit TMEM column.
+FP_DEV void tc_mma_ts_f8(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Instruction descriptor, kind::f8f6f4: fp32 accumulator, e4m3 A and B, both K-major.
+constexpr uint32_t tc_idesc_e4m3(int m, int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
 FP_DEV void tc_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
@@ -127,6 +148,8 @@ FP_DEV void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;
 
 #define FP_R8(b) "=r"(r[b]), "=r"(r[b + 1]), "=r"(r[b + 2]), "=r"(r[b + 3]), "=r"(r[b + 4]), "=r"(r[b + 5]), \
                  "=r"(r[b + 6]), "=r"(r[b + 7])
+#define FP_Q8(b) "=r"(q[b]), "=r"(q[b + 1]), "=r"(q[b + 2]), "=r"(q[b + 3]), "=r"(q[b + 4]), "=r"(q[b + 5]), \
+                 "=r"(q[b + 6]), "=r"(q[b + 7])
 #define FP_W8(b) "r"(r[b]), "r"(r[b + 1]), "r"(r[b + 2]), "r"(r[b + 3]), "r"(r[b + 4]), "r"(r[b + 5]), \
                  "r"(r[b + 6]), "r"(r[b + 7])
 
@@ -179,6 +202,38 @@ FP_DEV void tc_ld(uint32_t taddr, uint32_t* r) {
   }
 }
 
+// tc_ld of N columns from two places with one wait (N = 4, 8 or 16).
+template <int N>
+FP_DEV void tc_ld_pair(uint32_t ta, uint32_t tb, uint32_t* r, uint32_t* q) {
+  if constexpr (N == 4) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3])
+        : "r"(ta), "r"(tb)
+        : "memory");
+  } else if constexpr (N == 8) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : FP_R8(0), FP_Q8(0)
+        : "r"(ta), "r"(tb)
+        : "memory");
+  } else {
+    static_assert(N == 16, "tc_ld_pair: 4, 8 or 16 columns");
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, "
+        "[%33];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : FP_R8(0), FP_R8(8), FP_Q8(0), FP_Q8(8)
+        : "r"(ta), "r"(tb)
+        : "memory");
+  }
+}
+
 FP_DEV void tc_ld32(uint32_t taddr, float* v) {
   uint32_t r[32];
   tc_ld<32>(taddr, r);
@@ -206,6 +261,7 @@ FP_DEV void tc_st16(uint32_t taddr, const uint32_t* r) {
 FP_DEV void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 #undef FP_R8
+#undef FP_Q8
 #undef FP_W8
 
 // ---- host: tensor maps (fp_gemm_tc.cu)

@@ -1,0 +1,138 @@
+"""The int4 decode linear with 8-bit operands (large matrices at up to 16
+tokens, the largest SwiGLU at up to 32) against the oracle's dequantisation, on
+sampled output columns; and against the general decode path."""
+import numpy as np
+import pytest
+
+import synth
+from oracle import model as M
+from oracle import quant
+from tests.gpu_helpers import dev, empty, host, ptr, rel_err, torch_mod
+
+pytestmark = pytest.mark.gpu
+
+# One rounding of the result to bf16 (8 significant bits: half a unit of 1 is
+# 2^-8); the sums are fp32 and x is carried to 2^-23 of its row's largest value,
+# both far below.
+TOL = 1.05 * 2.0 ** -8
+
+
+@pytest.fixture(scope="module")
+def fp():
+    torch_mod()
+    import paper_2501_13111_gb300 as fp
+
+    return fp
+
+
+def _weights(fp, n, k, seed, perm=None):
+    w = empty(n * k, np.uint16)
+    fp.fp_op_init_weights(ptr(w), n * k, seed, 3)
+    codes, scales, zeros = empty(n * k // 2), empty(n * k // 128, np.uint16), empty(n * k // 128, np.uint16)
+    if perm is None:
+        fp.fp_op_quantize(2, ptr(w), n, k, ptr(codes), ptr(scales), ptr(zeros))
+    else:
+        fp.fp_op_quantize_gptq4(ptr(w), n, k, ptr(perm), ptr(codes), ptr(scales), ptr(zeros))
+    return codes, scales, zeros
+
+
+def _rows(n, k, seed, rows):
+    """The oracle's dequantised weights of some rows of that matrix."""
+    w = np.stack([synth.normal_bf16(seed, 3, int(r) * k, k) for r in rows])
+    return quant.quantize_weight(w, 2)[1]
+
+
+def _x(m, k, seed):
+    """Rows with small elements, one large one in the last row, a zero row where there are several."""
+    x = quant.bf16_to_f32(synth.uniform_bf16(seed, m, (m, k), -2.0, 2.0))
+    x[:, 1::7] *= 2.0 ** -11
+    x[-1, 5] = 300.0
+    if m > 2:
+        x[1] = 0.0
+    return synth.f32_to_bf16_bits(x)
+
+
+# ragged row tiles, an odd number of groups (a half item at each row's end), CTAs
+# that cover whole tiles and tiles shared by several, every token tile
+@pytest.mark.parametrize("m,n,k,epi", [
+    (1, 4104, 4096, 0), (8, 12008, 1408, 1), (9, 4104, 4096, 1), (16, 8240, 2176, 2), (7, 140000, 128, 0),
+    (16, 1200, 14080, 1), (5, 65664, 256, 2), (32, 65600, 4096, 2), (17, 67096, 4096, 2)])
+def test_matches_oracle(fp, m, n, k, epi):
+    codes, scales, zeros = _weights(fp, n, k, 9)
+    x, nout = _x(m, k, 8), n // 2 if epi == 2 else n
+    r = synth.uniform_bf16(7, m, (m, nout), -1.0, 1.0)
+    rd = dev(r)
+    ws_b = fp.fp_op_linear_workspace_bytes(2, m, n, k)
+    ws = empty(ws_b)
+    out = dev(r) if epi == 1 else empty(m * nout, np.uint16)  # the residual may be the output
+    for _ in range(2 if epi != 1 else 1):  # the workspace serves a second call
+        fp.fp_op_linear(2, epi, ptr(dev(x)), m, n, k, ptr(codes), ptr(scales), ptr(zeros),
+                        ptr(out if epi == 1 else rd), ptr(out), ptr(ws), ws_b)
+    got = quant.bf16_to_f32(host(out, np.uint16)).reshape(m, nout).astype(np.float64)
+    assert not host(ws, np.uint8)[:16384].any()  # the tickets are zero again
+    cols = np.unique(np.concatenate([[0, 1, nout - 1], np.random.default_rng(m).integers(0, nout, 60)]))
+    xf = quant.bf16_to_f32(x).astype(np.float64)
+    ref = xf @ _rows(n, k, 9, cols).T
+    if epi == 1:
+        ref = ref + quant.bf16_to_f32(r).astype(np.float64)[:, cols]
+    elif epi == 2:
+        ref = M.silu(ref) * (xf @ _rows(n, k, 9, cols + nout).T)
+    for i in range(m):  # row by row: the row with the large element must not hide the others
+        assert rel_err(got[i:i + 1][:, cols], ref[i:i + 1]) <= TOL, (i, rel_err(got[i:i + 1][:, cols], ref[i:i + 1]))
+
+
+@pytest.mark.parametrize("m,epi", [(1, 0), (8, 1), (13, 2)])
+def test_agrees_with_the_general_path(fp, m, epi):
+    """Scales at an address that is not a multiple of 16 keep the mma.sync path."""
+    n, k = 8200, 4096
+    codes, scales, zeros = _weights(fp, n, k, 11)
+    nout = n // 2 if epi == 2 else n
+    x, r = dev(_x(m, k, 3)), dev(synth.uniform_bf16(4, m, (m, nout), -1.0, 1.0))
+    shifted = dev(np.concatenate([np.zeros(1, np.uint16), host(scales, np.uint16)]))
+    ws_b = fp.fp_op_linear_workspace_bytes(2, m, n, k)
+    ws, res = empty(ws_b), []
+    for sc in (ptr(scales), ptr(shifted) + 2):
+        out = empty(m * nout, np.uint16)
+        fp.fp_op_linear(2, epi, ptr(x), m, n, k, ptr(codes), sc, ptr(zeros), ptr(r), ptr(out), ptr(ws), ws_b)
+        res.append(quant.bf16_to_f32(host(out, np.uint16)).reshape(m, nout).astype(np.float64))
+    for a, b in zip(*res):
+        assert rel_err(a[None], b[None]) <= 2 * TOL
+
+
+def test_gptq4_reads_x_through_the_act_order(fp):
+    m, n, k = 6, 4608, 4096
+    order = np.random.default_rng(5).permutation(k).astype(np.int32)
+    perm = dev(order)
+    codes, scales, zeros = _weights(fp, n, k, 12, perm)
+    x = _x(m, k, 6)
+    ws_b = max(fp.fp_op_linear_gptq4_workspace_bytes(m, n, k), fp.fp_op_linear_workspace_bytes(2, m, n, k))
+    ws, err, a, b = empty(ws_b), empty(1, np.int32), empty(m * n, np.uint16), empty(m * n, np.uint16)
+    fp.fp_op_linear_gptq4(0, ptr(dev(x)), m, n, k, ptr(perm), ptr(codes), ptr(scales), ptr(zeros), None, ptr(a),
+                          ptr(ws), ws_b, ptr(err))
+    fp.fp_op_linear(2, 0, ptr(dev(np.ascontiguousarray(x[:, order]))), m, n, k, ptr(codes), ptr(scales), ptr(zeros),
+                    None, ptr(b), ptr(ws), ws_b)
+    assert np.array_equal(host(a, np.uint16), host(b, np.uint16)) and host(err, np.int32)[0] == 0
+    # an entry outside [0, K) reads as zero and is reported
+    order[7] = k
+    x0 = x.copy()
+    lost = int(np.setdiff1d(np.arange(k), order)[0])
+    x0[:, lost] = 0
+    fp.fp_op_linear_gptq4(0, ptr(dev(x)), m, n, k, ptr(dev(order)), ptr(codes), ptr(scales), ptr(zeros), None, ptr(a),
+                          ptr(ws), ws_b, ptr(err))
+    order[7] = lost
+    fp.fp_op_linear(2, 0, ptr(dev(np.ascontiguousarray(x0[:, order]))), m, n, k, ptr(codes), ptr(scales), ptr(zeros),
+                    None, ptr(b), ptr(ws), ws_b)
+    assert np.array_equal(host(a, np.uint16), host(b, np.uint16)) and host(err, np.int32)[0] == 1
+
+
+def test_beyond_fp16_is_reported_as_on_the_general_path(fp):
+    m, n, k = 4, 4608, 4096
+    perm = dev(np.arange(k, dtype=np.int32))
+    codes, scales, zeros = _weights(fp, n, k, 12)
+    x = _x(m, k, 6)
+    x[2, 100] = synth.f32_to_bf16_bits(np.array([7e4], np.float32))[0]
+    ws_b = fp.fp_op_linear_gptq4_workspace_bytes(m, n, k)
+    ws, err, out = empty(ws_b), empty(1, np.int32), empty(m * n, np.uint16)
+    fp.fp_op_linear_gptq4(0, ptr(dev(x)), m, n, k, ptr(perm), ptr(codes), ptr(scales), ptr(zeros), None, ptr(out),
+                          ptr(ws), ws_b, ptr(err))
+    assert host(err, np.int32)[0] == 3

@@ -1,140 +1,182 @@
 // Prefill attention on the tcgen05 tensor cores: paged cache of bf16 or int8
 // codes with per-(token, KV head) fp32 scales, head_dim 128.
 //
-// o = softmax(q K^T / sqrt(hd) + causal mask) V for the S query rows of one
+// o = softmax(q K^T / sqrt(hd) + causal mask) V for the S query rows of every
 // (sequence, head) against cache positions 0..S-1 (Sec. 5.1: the block's
-// attention).  CTA = 128 query rows of one (b, h), key tiles of 128; two
-// CTAs per SM (256 TMEM columns and 97 KiB of shared memory each), so one
-// CTA's softmax overlaps the other's MMAs and loads:
-//   warp 0      TMA: the Q tile once (two 64-column boxes of the q rows), then
-//               (bf16 cache) per key tile its K rows and its V rows page by
-//               page (a [16][64] box per 16-token page and half of head_dim,
-//               128-byte swizzle, one box per lane); K(t + 1) loads once S(t)
-//               has read K(t), V(t + 1) once P(t) V(t) has read V(t);
-//   warp 1      allocates the TMEM and issues the MMAs: S = Q K^T (M 128
-//               queries, N 128 keys, K 16 over head_dim; K-major operands),
-//               then O += P V (A = P from TMEM, B = V read MN-major);
-//   warps 2-5   softmax, one query row (TMEM lane) per thread, over 32-column
-//               chunks: a first pass for the row maximum (log2 domain), a
-//               second for P = 2^(s - m) written as bf16 over the scores
-//               already read.  The reference maximum m only moves when a tile
-//               raises it by more than 2^8 (O and the row sum are rescaled
-//               then); P never exceeds 256, and o / l is exact either way.
-//   int8 cache: both products run on fp16 operands.  Warps 0, 6 and 7
-//               (after warp 0 has issued the Q copy) convert the Q tile to
-//               fp16 in place once, then widen the codes: each loads its
-//               rows' 16-byte code chunks and turns each pair into the fp16
-//               pair (1024 + q + 128) by one byte permute, minus 1152 --
-//               exact -- in the same swizzled layout the TMA writes, and
-//               stages the tile's K scales and its V scales times 2^sigma;
-//               the softmax multiplies each score column by its K scale and
-//               each P column by its scaled V scale in fp32 (the row sum
-//               takes the unscaled P) and packs P as fp16.  sigma, one per
-//               CTA, is the largest power of two keeping 256 * (largest V
-//               scale of the sequence) * 2^sigma within 65280, so P stays in
-//               the fp16 normal range; the output divides it out.  A q beyond
-//               the fp16 range sets status 3.
-// TMEM columns: scores S [0, 128) with P over [0, 64), O [128, 256).  Every
-// mbarrier wait is bounded (error 2 past the limit); a page id out of range
-// reads zeros and sets error 1.
+// attention), for prompts of more than 128 tokens (fp_attn_short.cu takes the
+// shorter ones).  One persistent CTA per SM walks work items of two query tiles
+// of 128 rows that read the same keys and values: two heads of one KV head's
+// group where groups are even, else 256 consecutive rows of a head (single tiles
+// where pairs would leave SMs idle).  Key tiles of 128.
+// Tensor memory holds, for each of the two tiles, its scores (128 columns, P
+// written over them as 16-bit pairs) and its output accumulator (128 columns):
+//   warps 0-3   softmax of tile 0, warps 4-7 of tile 1: one query row (TMEM
+//               lane) per thread, the tile's 128 scores held in registers
+//               between the row maximum and P = 2^(s - m).  The reference
+//               maximum m only moves when a tile raises it by more than 2^8 (O
+//               and the row sum are rescaled then); P never exceeds 256, and
+//               o / l is exact either way.  At the end of an item they write
+//               their rows of O;
+//   warp 8      TMA: the item's Q tiles (two 64-column boxes each), then (bf16
+//               cache) per key tile its K rows and its V rows page by page (a
+//               [16][64] box per 16-token page and half of head_dim, 128-byte
+//               swizzle, one box per lane) into rings of two tiles each;
+//   warp 9      owns the TMEM and issues the MMAs.  For each key tile and query
+//               tile in turn: O += P(t) V(t) (A = P from TMEM, V read MN-major),
+//               then S(t + 1) = Q K(t + 1)^T over the scores that P(t) V(t) has
+//               read (one thread's MMAs execute in order), so one tile's softmax
+//               runs while the other tile's two products do.
+//   int8 cache: both products run on fp16 operands.  Warps 10-15 convert the
+//               item's Q tiles to fp16 in place once, then widen the codes: each
+//               loads its rows' 16-byte code chunks and turns each pair into the
+//               fp16 pair (1024 + q + 128) by one byte permute, minus 1152 --
+//               exact -- in the same swizzled layout the TMA writes, and stages
+//               the tile's K scales and its V scales times 2^sigma; the softmax
+//               multiplies each score column by its K scale and each P column by
+//               its scaled V scale in fp32 (the row sum takes the unscaled P)
+//               and packs P as fp16.  sigma, one per item, is the largest power
+//               of two keeping 256 * (largest V scale of the item's keys) *
+//               2^sigma within 65280, so P stays in the fp16 normal range; the
+//               output divides it out.  A q beyond the fp16 range sets status 3.
+// What bounds it: a key tile's products take 2 x 16 MMAs of 65 cycles for the two
+// query tiles, 2080 cycles, which also fill shared memory's bandwidth; a step
+// takes 4100 (the softmax of a tile about 1600, its P V and next scores 1040, and
+// the hand-offs between the roles), with the int8 cache 8700 (the scales of the
+// keys are read by every row, and the widening shares the issue slots).
+// Measured, whole launches, bf16 cache, 4 x 2048 tokens, 64 / 8 heads | 8 x 1024,
+// 40 heads | int8 cache, the first shape:
+//   one 128-row tile per CTA, two CTAs per SM (before)       338 | 151 | 982 us
+//   two tiles per CTA                                        333 | 161 | 725
+//   every lane runs the MMA loop (one lane's issue took 144
+//     cycles for an MMA that runs 65)                        297 | 138 | 641
+//   output rows through shared memory, shorter first rounds  283 | 126 | 608
+// Key tiles in halves of 64, so that a tile's own two products overlap its
+// softmax, took 360 us: the waits cost more than they hid.
+// Every mbarrier wait is bounded (error 2 past the limit); a page id out of
+// range reads zeros and sets error 1.
 #include <algorithm>
 #include <type_traits>
 
+#include "attn_tc.cuh"
 #include "common.cuh"
-#include "kernels.cuh"
-#include "tc.cuh"
 
 namespace fpk {
 
-constexpr int kPaB = 128;  // query rows per CTA = keys per tile
-constexpr int kPaHD = 128;
-constexpr int kPaWiden = 3;                                 // int8 cache: warps widening codes (0, 6, 7)
+constexpr int kPaWarpTma = 8, kPaWarpMma = 9, kPaWarpWiden = 10;
+constexpr int kPaWiden = 6;                                 // int8 cache: warps widening codes
 constexpr int kPaWRows = (kPaB + 4 * kPaWiden - 1) / (4 * kPaWiden);  // tile rows per widening thread
 template <bool KV8>
-constexpr int pa_threads() { return KV8 ? 256 : 192; }
-constexpr uint32_t kPaTmemCols = 256;
-constexpr uint32_t kPaS = 0, kPaO = 128;
-constexpr int kPaHalf = kPaB * 128;          // bytes of one [128 rows][64 bf16] swizzled half
-constexpr int kPaTile = 2 * kPaHalf;         // one [128][128] bf16 operand
-constexpr int kPaSmem = 3 * kPaTile + 1024;  // Q, K, V, alignment
-constexpr float kPaLog2e = 1.4426950408889634f;
-// score columns per TMEM load in the softmax (64-column loads measured
-// slower: 201 / 319 against 211 / 356 TFLOP/s at the 7B / 13B shapes)
-constexpr int kPaCW = 32;
+constexpr int pa_threads() { return KV8 ? (kPaWarpWiden + kPaWiden) * 32 : 384; }
+// Registers a thread, moved to the softmax, which holds a row of scores: bf16
+// cache 168 at launch (384 threads), 2 x 208 + 88 = 3 x 168; int8 cache 128 (512
+// threads), 2 x 160 + 2 x 96 = 4 x 128
+template <bool KV8>
+constexpr int pa_reg_soft() { return KV8 ? 160 : 208; }
+template <bool KV8>
+constexpr int pa_reg_other() { return KV8 ? 96 : 88; }
+constexpr uint32_t kPaTmemCols = 512;
+constexpr uint32_t kPaO = 256;               // O of tile j at kPaO + 128 j, its scores at 128 j
+constexpr int kPaRing = 2;                   // K tiles, V tiles in shared memory
+constexpr int kPaScl = 4;                    // tiles of int8 scales
+constexpr int kPaSmem = (2 + 2 * kPaRing) * kPaTile + 8 * kPaStage + 1024;  // Q, K, V, output, alignment
 constexpr float kPaSlack = 8.f;  // log2 of the largest P allowed before the reference maximum moves
 
-// Shared-memory descriptor of an MN-major operand with 128-byte swizzle:
-// 64-element atoms along MN `lbo` bytes apart, 8-row groups along K 1024
-// bytes apart.
-FP_DEV uint64_t sdesc_mn(uint32_t saddr, uint32_t lbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
+// Two fp32 lanes at once: a b + c, a b, a + b.
+FP_DEV float2 pa_fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n .reg .b64 a, b, c, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mov.b64 c, {%6, %7};\n"
+      " fma.rn.f32x2 d, a, b, c;\n mov.b64 {%0, %1}, d;\n}\n"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+FP_DEV float2 pa_mul2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
+      " mul.rn.f32x2 d, a, b;\n mov.b64 {%0, %1}, d;\n}\n"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+FP_DEV float2 pa_add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
+      " add.rn.f32x2 d, a, b;\n mov.b64 {%0, %1}, d;\n}\n"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return d;
 }
 
-// 16 consecutive 32-bit columns into this thread's TMEM lane.
-FP_DEV void pa_st16(uint32_t taddr, const uint32_t* r) { tc_st16(taddr, r); }
+// How the query tiles are put together into work items (chosen by the host).
+struct PaPlan {
+  int pair;       // 0: one tile an item; 1: the same rows of two heads; 2: 256 rows of a head
+  int units;      // items of one (sequence, head or pair of heads)
+  int items;
+  bool longest_first;
+};
 
-// 2^x by the hardware approximation (subnormal results flush to zero: P
-// values below 2^-126 carry no weight next to the row's maximum of 1 .. 256).
-FP_DEV float pa_ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
+// Item `i` of CTA round n.  Few rounds: the items in order of length, every other
+// round backwards.  Many: the items of one (sequence, head) are consecutive, so
+// the CTAs that run together share keys and values in L2, and which of its query
+// tiles an item takes is rotated from one round to the next, so that no CTA keeps
+// drawing the long ones.
+FP_DEV int pa_item(const PaPlan& p, int n) {
+  const int c = blockIdx.x, g = gridDim.x;
+  return n * g + (p.longest_first && (n & 1) ? g - 1 - c : c);
 }
 
-// (lo, hi) -> bf16x2, round to nearest even.
-FP_DEV uint32_t pa_pack(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-
-// (lo, hi) -> fp16x2, round to nearest even.
-FP_DEV uint32_t pa_pack_h(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-
-// Signed bytes a and b of w as the fp16 pair (q_a, q_b), exact: the byte
-// permute places q + 128 under the fp16 exponent of 1024 (0x64nn = 1024 + nn),
-// one fp16x2 subtraction of 1152 leaves q.
-FP_DEV uint32_t pa_i8h2(uint32_t u, uint32_t sel) {
-  uint32_t h = __byte_perm(u, 0x64646464u, sel);
-  asm("sub.rn.f16x2 %0, %0, %1;" : "+r"(h) : "r"(0x64806480u));
-  return h;
-}
+// A work item: up to two query tiles of sequence b that share KV head kvh.
+struct PaItem {
+  int b, h[2], q0[2], nt[2], kvh;  // nt: key tiles up to the diagonal (0: no rows in this tile)
+  FP_DEV PaItem(int i, int S, int H, int Hkv, const PaPlan& p) {
+    const unsigned heads = p.pair == 1 ? H / 2 : H, all = (unsigned)p.items / (unsigned)p.units;
+    unsigned hb, r;
+    if (p.longest_first) {
+      r = (unsigned)i / all, hb = (unsigned)i % all;
+    } else {
+      hb = (unsigned)i / (unsigned)p.units;
+      r = ((unsigned)i % (unsigned)p.units + hb * p.units / gridDim.x) % (unsigned)p.units;
+    }
+    const int u = p.units - 1 - (int)r;
+    b = hb / heads;
+    const int hh = hb % heads;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      h[j] = p.pair == 1 ? 2 * hh + j : hh;
+      q0[j] = p.pair == 2 ? (2 * u + j) * kPaB : u * kPaB;
+      nt[j] = q0[j] < S && (j == 0 || p.pair) ? (min(q0[j] + kPaB, S) - 1) / kPaB + 1 : 0;
+    }
+    kvh = (unsigned)h[0] / ((unsigned)H / (unsigned)Hkv);
+  }
+  FP_DEV int tiles() const { return max(nt[0], nt[1]); }
+  // of tile j (a runtime index into the arrays would put them in local memory)
+  FP_DEV int head(int j) const { return j ? h[1] : h[0]; }
+  FP_DEV int row0(int j) const { return j ? q0[1] : q0[0]; }
+  FP_DEV int key_tiles(int j) const { return j ? nt[1] : nt[0]; }
+};
 
 template <bool KV8>
-__global__ void __launch_bounds__(pa_threads<KV8>(), 2)
+__global__ void __launch_bounds__(pa_threads<KV8>(), 1)
     attn_prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                            const __grid_constant__ CUtensorMap map_v, const int8_t* __restrict__ k8,
                            const int8_t* __restrict__ v8, const float* __restrict__ k_scale,
                            const float* __restrict__ v_scale, int S, int H, int Hkv, int page_size,
-                           const int32_t* __restrict__ page_table, int pages_per_seq, int n_pages,
+                           const int32_t* __restrict__ page_table, int pages_per_seq, int n_pages, PaPlan plan,
                            uint16_t* __restrict__ out, int32_t* err) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ uint64_t qfull, qconv, kfull, kempty, vfull, vempty, sfull, pfull, ofull, mma_done;
-  __shared__ float s_vmax[KV8 ? 3 : 1];  // int8: the widening warps' largest V scales
-  __shared__ float s_unscale;             // int8: 2^-sigma, removed from the output
+  __shared__ uint64_t qfull, qconv, qempty, kfull[kPaRing], kempty[kPaRing], vfull[kPaRing], vempty[kPaRing], sfull[2],
+      pfull[2], ofull[2], oempty[2], vmet, mma_done;
+  __shared__ float s_vmax[2][kPaWiden];  // int8: the widening warps' largest V scales, by item parity
+  __shared__ float s_unscale[4];          // int8: 2^-sigma, removed from the output; by item % 4
   __shared__ uint32_t tmem_base;
   __shared__ int abort_word;
-  __shared__ __align__(16) float s_scl[KV8 ? 4 * kPaB : 4];  // int8: [K, V][tile parity][key] scales
+  __shared__ __align__(16) float s_scl[KV8 ? 2 * kPaScl * kPaB : 4];  // int8: [K, V][tile % 4][key] scales
   volatile int* abort_flag = &abort_word;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sQ = smem;
-  uint8_t* sK = smem + kPaTile;
-  uint8_t* sV = smem + 2 * kPaTile;
+  uint8_t* sK = smem + 2 * kPaTile;
+  uint8_t* sV = sK + kPaRing * kPaTile;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qt = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int kvh = h / (H / Hkv);
-  const int q0 = qt * kPaB;
-  const int nt = (min(q0 + kPaB, S) - 1) / kPaB + 1;  // key tiles up to the diagonal
   auto fail = [&]() {
     *abort_flag = 1;
     if (err) atomicExch(err, 2);
@@ -144,18 +186,25 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 2)
   if (threadIdx.x == 0) {
     mbar_init(&qfull, 1);
     mbar_init(&qconv, kPaWiden);  // int8: the widening warps converted Q to fp16
-    mbar_init(&kfull, KV8 ? kPaWiden : 1);
-    mbar_init(&kempty, 1);
-    mbar_init(&vfull, KV8 ? kPaWiden : 1);
-    mbar_init(&vempty, 1);
-    mbar_init(&sfull, 1);
-    mbar_init(&pfull, 4);
-    mbar_init(&ofull, 1);
+    mbar_init(&qempty, 1);
+    mbar_init(&vmet, kPaWiden);
+    for (int i = 0; i < kPaRing; ++i) {
+      mbar_init(&kfull[i], KV8 ? kPaWiden : 1);
+      mbar_init(&kempty[i], 1);
+      mbar_init(&vfull[i], KV8 ? kPaWiden : 1);
+      mbar_init(&vempty[i], 1);
+    }
+    for (int j = 0; j < 2; ++j) {
+      mbar_init(&sfull[j], 1);
+      mbar_init(&pfull[j], 4);
+      mbar_init(&ofull[j], 1);
+      mbar_init(&oempty[j], 4);
+    }
     mbar_init(&mma_done, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {
+  if (warp == kPaWarpMma) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
                  "r"(kPaTmemCols)
                  : "memory");
@@ -167,355 +216,399 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 2)
   const uint32_t tmem = tmem_base;
   pdl_wait();
 
-  if (KV8 && (warp == 0 || warp >= 6)) {
-    // ---------------- int8 cache: the Q copy, then widening of the key tiles
-    if (warp == 0 && lane == 0) {
-      mbar_expect_tx(&qfull, kPaTile);
-      tma_load_2d(sQ, &map_q, h * kPaHD, b * S + q0, &qfull);
-      tma_load_2d(sQ + kPaHalf, &map_q, h * kPaHD + 64, b * S + q0, &qfull);
-    }
-    const int wi = (warp == 0 ? 0 : warp - 5) * 32 + lane;  // 0 .. 95
-    const int c = wi & 7;                                     // code chunk: head_dim 16c .. 16c + 15
-    const int rbase = wi >> 3;                                // tile rows rbase + 12i (< 128)
-    const int32_t* ptv = page_table + (long long)b * pages_per_seq;
-    // sigma: from the largest V scale over the keys this CTA reads
-    float vmax = 0.f;
-    const int nkeys = min(q0 + kPaB, S);
-    for (int key = wi; key < nkeys; key += 32 * kPaWiden) {
-      const int pg = __ldg(ptv + key / page_size);
-      if (pg >= 0 && pg < n_pages) vmax = fmaxf(vmax, __ldg(v_scale + (pg * Hkv + kvh) * page_size + key % page_size));
-    }
-    vmax = warp_max(vmax);
-    if (lane == 0) s_vmax[warp == 0 ? 0 : warp - 5] = vmax;
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * kPaWiden) : "memory");
-    vmax = fmaxf(fmaxf(s_vmax[0], s_vmax[1]), s_vmax[2]);
-    // 2^sigma with 256 * vmax * 2^sigma <= 65280 (vmax = 0: no V weight at all)
-    const int sigma = vmax > 0.f ? min(60, max(-60, (int)floorf(log2f(255.f / vmax)))) : 0;
-    const float vmul = exp2f((float)sigma);
-    // published before the first code tile, which every softmax wait follows
-    if (wi == 0) s_unscale = exp2f((float)-sigma);
-    // Q to fp16 in place (the element order of the swizzled tile is kept)
-    bool ok = __all_sync(0xffffffffu, mbar_wait(&qfull, 0));
-    if (ok) {
-      bool over = false;
-      for (int i = wi; i < kPaTile / 16; i += 32 * kPaWiden) {
-        uint4* p = reinterpret_cast<uint4*>(sQ) + i;
-        const uint4 v = *p;
-        const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-        uint32_t o[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float2 f = bf2x2f(w4[j]);
-          over |= fabsf(f.x) > 65504.f || fabsf(f.y) > 65504.f;
-          o[j] = pa_pack_h(f.x, f.y);
-        }
-        *p = make_uint4(o[0], o[1], o[2], o[3]);
-      }
-      if (over && err) atomicExch(err, 3);  // q outside the fp16 range: the output is invalid
-      fence_proxy_async();
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&qconv);
-    // its bf16 form is chunks cb, cb + 1 of half c / 4 of the swizzled row;
-    // the lanes of the upper half store the odd chunk first, so the eight
-    // lanes of one row write eight distinct 16-byte bank groups
-    const int cb = 2 * (c & 3), half_off = (c >> 2) * kPaHalf;
-    const int32_t* pt = ptv;
-    for (int t = 0; t < nt && ok; ++t) {
-      int rowi[kPaWRows];  // pool row of each of the thread's keys (< 2^31); -1 reads zeros
-#pragma unroll
-      for (int i = 0; i < kPaWRows; ++i) {
-        const int row = rbase + 4 * kPaWiden * i, key = t * kPaB + row;
-        rowi[i] = -1;
-        if (row < kPaB && key < S) {
-          const int pg = __ldg(pt + key / page_size);
-          if (pg >= 0 && pg < n_pages) rowi[i] = (pg * Hkv + kvh) * page_size + key % page_size;
-          else if (err && c == 0) atomicExch(err, 1);
-        }
-      }
-      // the tile's K and V scales go out with its K codes: the softmax reads
-      // both once S(t) is complete, which only the K tile's barrier precedes
-      float sck[kPaWRows], scv[kPaWRows];
-#pragma unroll
-      for (int i = 0; i < kPaWRows; ++i) {
-        sck[i] = (c == 0 && rowi[i] >= 0) ? __ldg(k_scale + rowi[i]) : 0.f;
-        scv[i] = (c == 0 && rowi[i] >= 0) ? __ldg(v_scale + rowi[i]) * vmul : 0.f;
-      }
-#pragma unroll 1
-      for (int which = 0; which < 2; ++which) {
-        const int8_t* pool = which ? v8 : k8;
-        uint4 w[kPaWRows];
-        // the codes are read before the wait for the buffer
-#pragma unroll
-        for (int i = 0; i < kPaWRows; ++i)
-          w[i] = rowi[i] >= 0 ? ld_nc16(pool + (long long)rowi[i] * kPaHD + c * 16) : make_uint4(0, 0, 0, 0);
-        ok = t == 0 || mbar_wait(which ? &vempty : &kempty, (t - 1) & 1);
-        if (!__all_sync(0xffffffffu, ok) || __any_sync(0xffffffffu, *abort_flag != 0)) {
-          ok = false;
-          break;
-        }
-        uint8_t* dst = (which ? sV : sK) + half_off;
-#pragma unroll
-        for (int i = 0; i < kPaWRows; ++i) {
-          const int row = rbase + 4 * kPaWiden * i, sw = row & 7;
-          if (row >= kPaB) break;
-          const uint32_t ww[4] = {w[i].x ^ 0x80808080u, w[i].y ^ 0x80808080u, w[i].z ^ 0x80808080u,
-                                  w[i].w ^ 0x80808080u};
-          uint32_t o[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) o[j] = pa_i8h2(ww[j >> 1], (j & 1) ? 0x4342 : 0x4140);
-          const uint4 e = make_uint4(o[0], o[1], o[2], o[3]), f = make_uint4(o[4], o[5], o[6], o[7]);
-          uint8_t* rp = dst + row * 128;
-          if (c < 4) {
-            *reinterpret_cast<uint4*>(rp + ((cb ^ sw) << 4)) = e;
-            *reinterpret_cast<uint4*>(rp + (((cb + 1) ^ sw) << 4)) = f;
-          } else {
-            *reinterpret_cast<uint4*>(rp + (((cb + 1) ^ sw) << 4)) = f;
-            *reinterpret_cast<uint4*>(rp + ((cb ^ sw) << 4)) = e;
-          }
-          if (which == 0 && c == 0) {
-            // buffer t & 1 was last read by the softmax of tile t - 2, which
-            // completed before S(t - 1) was issued and so before this K tile's wait
-            s_scl[(t & 1) * kPaB + row] = sck[i];
-            s_scl[(2 + (t & 1)) * kPaB + row] = scv[i];
-          }
-        }
-        fence_proxy_async();  // the MMAs read the tile through the async proxy
-        __syncwarp();
-        if (lane == 0) mbar_arrive(which ? &vfull : &kfull);
-      }
-    }
-    if (!ok && lane == 0) fail();
-  } else if (warp == 0) {
-    // ---------------- TMA producer: lanes 0-15 each copy one [16][64] box of
-    // a key tile (page lane & 7, head_dim half lane >> 3); lane 0 arms the
-    // barriers.  The next tile's page ids are read while this one is in flight.
-    const int32_t* pt = page_table + (long long)b * pages_per_seq;
-    const int pg = lane & 7, half = (lane >> 3) & 1;
-    auto page_row = [&](int t) {  // pool row of this lane's page of tile t; -16 reads zeros
-      const int key0 = t * kPaB + pg * 16;
-      if (lane >= 16 || key0 >= S) return -16;
-      const int id = __ldg(pt + key0 / page_size);
-      if (id >= 0 && id < n_pages) return (id * Hkv + kvh) * page_size;
-      if (err && half == 0) atomicExch(err, 1);
-      return -16;
-    };
-    if (lane == 0) {
+  if (warp >= kPaWarpTma) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(pa_reg_other<KV8>()));
+  if (warp == kPaWarpTma) {
+    // ---------------- TMA producer: lane 0 copies Q; lanes 0-15 each copy one
+    // [16][64] box of a key tile (page lane & 7, head_dim half lane >> 3).  The
+    // next tile's page ids are read while this one is in flight.
+    if (lane == 0 && !KV8) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
-      mbar_expect_tx(&qfull, kPaTile);
-      tma_load_2d(sQ, &map_q, h * kPaHD, b * S + q0, &qfull);
-      tma_load_2d(sQ + kPaHalf, &map_q, h * kPaHD + 64, b * S + q0, &qfull);
     }
-    int row = page_row(0);
-    int kiss = 0, viss = 0;
+    const int pg = lane & 7, half = (lane >> 3) & 1;
+    int n = 0, kn = 0, iss[3] = {0, 0, 0};  // items, key tiles; copies issued of Q, K, V
     bool ok = true;
-    for (int t = 0; t < nt; ++t) {
-      if (t > 0) {
-        ok = mbar_wait(&kempty, (t - 1) & 1);
-        if (!__all_sync(0xffffffffu, ok) || __any_sync(0xffffffffu, *abort_flag != 0)) {
-          ok = false;
-          break;
+    for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
+      const PaItem w(i, S, H, Hkv, plan);
+      if (n > 0) ok = __all_sync(0xffffffffu, mbar_wait(&qempty, (n - 1) & 1)) && !*abort_flag;
+      if (!__all_sync(0xffffffffu, ok)) break;
+      iss[0] = n + 1;
+      if (lane == 0) {
+        mbar_expect_tx(&qfull, (w.nt[1] > 0 ? 2 : 1) * kPaTile);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          if (w.nt[j] > 0) {
+            tma_load_2d(sQ + j * kPaTile, &map_q, w.h[j] * kPaHD, w.b * S + w.q0[j], &qfull);
+            tma_load_2d(sQ + j * kPaTile + kPaHalf, &map_q, w.h[j] * kPaHD + 64, w.b * S + w.q0[j], &qfull);
+          }
+      }
+      if constexpr (!KV8) {
+        const int32_t* pt = page_table + (long long)w.b * pages_per_seq;
+        auto page_row = [&](int t) {  // pool row of this lane's page of tile t; -16 reads zeros
+          const int key0 = t * kPaB + pg * 16;
+          if (lane >= 16 || key0 >= S) return -16;
+          const int id = __ldg(pt + key0 / page_size);
+          if (id >= 0 && id < n_pages) return (id * Hkv + w.kvh) * page_size;
+          if (err && half == 0) atomicExch(err, 1);
+          return -16;
+        };
+        const int nt = w.tiles();
+        int row = page_row(0);
+        for (int t = 0; t < nt && ok; ++t, ++kn) {
+          const int s = kn % kPaRing, ph = ((kn / kPaRing) & 1) ^ 1;
+#pragma unroll
+          for (int v = 0; v < 2 && ok; ++v) {
+            uint64_t* full = v ? &vfull[s] : &kfull[s];
+            if (kn >= kPaRing) ok = mbar_wait(v ? &vempty[s] : &kempty[s], ph);
+            ok = __all_sync(0xffffffffu, ok && !*abort_flag);
+            if (!ok) break;
+            if (lane == 0) mbar_expect_tx(full, kPaTile);
+            __syncwarp();
+            if (lane < 16)
+              tma_load_2d((v ? sV : sK) + s * kPaTile + half * kPaHalf + pg * 2048, v ? &map_v : &map_k, half * 64, row,
+                          full);
+            iss[1 + v] = kn + 1;
+          }
+          if (t + 1 < nt) row = page_row(t + 1);
         }
       }
-      if (lane == 0) mbar_expect_tx(&kfull, kPaTile);
-      __syncwarp();
-      if (lane < 16) tma_load_2d(sK + half * kPaHalf + pg * 2048, &map_k, half * 64, row, &kfull);
-      kiss = t + 1;
-      if (t > 0) {
-        ok = mbar_wait(&vempty, (t - 1) & 1);
-        if (!__all_sync(0xffffffffu, ok) || __any_sync(0xffffffffu, *abort_flag != 0)) {
-          ok = false;
-          break;
-        }
-      }
-      if (lane == 0) mbar_expect_tx(&vfull, kPaTile);
-      __syncwarp();
-      if (lane < 16) tma_load_2d(sV + half * kPaHalf + pg * 2048, &map_v, half * 64, row, &vfull);
-      viss = t + 1;
-      if (t + 1 < nt) row = page_row(t + 1);
     }
     if (lane == 0) {
       if (!ok) fail();
       // copies still in flight land before the CTA leaves
-      mbar_wait(&qfull, 0);
-      if (kiss > 0) mbar_wait(&kfull, (kiss - 1) & 1);
-      if (viss > 0) mbar_wait(&vfull, (viss - 1) & 1);
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer
-    if (lane == 0) {
-      // Q, K both K-major; V MN-major.  int8 cache: fp16 operands (A and B
-      // of one MMA always share their type), bf16 cache: bf16
-      constexpr uint32_t f16 = KV8 ? ((1u << 7) | (1u << 10)) : 0u;
-      constexpr uint32_t idesc_s = tc_idesc(kPaB, kPaB) & ~f16;
-      constexpr uint32_t idesc_o = (tc_idesc(kPaB, kPaHD) | (1u << 16)) & ~f16;
-      bool ok = KV8 ? mbar_wait(&qconv, 0) : mbar_wait(&qfull, 0);
-      const uint32_t q = smem_u32(sQ), k = smem_u32(sK), v = smem_u32(sV);
-      for (int t = 0; t < nt && ok; ++t) {
-        // S(t) overwrites P(t - 1): its P V has completed (in order with this thread's MMAs)
-        ok = mbar_wait(&kfull, t & 1) && (t == 0 || mbar_wait(&ofull, (t - 1) & 1)) && !*abort_flag;
-        if (!ok) break;
-        tc_fence_after();
+      if (iss[0] > 0) mbar_wait(&qfull, (iss[0] - 1) & 1);
 #pragma unroll
-        for (int kk = 0; kk < kPaHD / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * kPaHalf + (kk & 3) * 32;
-          tc_mma(tmem + kPaS, sdesc(q + off), sdesc(k + off), idesc_s, kk > 0 ? 1u : 0u);
-        }
-        tc_commit(&sfull);
-        tc_commit(&kempty);
-        ok = mbar_wait(&pfull, t & 1) && mbar_wait(&vfull, t & 1) && !*abort_flag;
-        if (!ok) break;
-        tc_fence_after();
-#pragma unroll
-        for (int kk = 0; kk < kPaB / 16; ++kk)  // 16 keys: two 8-row groups of the V tile
-          tc_mma_ts(tmem + kPaO, tmem + kPaS + kk * 8, sdesc_mn(v + kk * 2048, kPaHalf), idesc_o,
-                    (t > 0 || kk > 0) ? 1u : 0u);
-        tc_commit(&ofull);
-        tc_commit(&vempty);
-      }
-      if (!ok) fail();
-      tc_commit(&mma_done);
-      mbar_wait(&mma_done, 0);
+      for (int v = 0; v < 2; ++v)
+        for (int t = max(0, iss[1 + v] - kPaRing); t < iss[1 + v]; ++t)
+          mbar_wait(v ? &vfull[t % kPaRing] : &kfull[t % kPaRing], (t / kPaRing) & 1);
     }
-  } else {
-    // ---------------- softmax: thread = query row (TMEM lane 32 (warp % 4) + lane)
-    const int quad = warp & 3, row = quad * 32 + lane;
-    const int qrow = q0 + row;  // position in the sequence
-    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
-    const float scale = kPaLog2e * rsqrtf((float)kPaHD);
-    float m = -INFINITY, l = 0.f;  // reference maximum (log2 domain) and row sum
+  } else if (warp == kPaWarpMma) {
+    // ---------------- MMA issuer: every lane runs the loop, one issues.
+    // Q, K both K-major; V MN-major.  int8 cache: fp16 operands (A and B
+    // of one MMA always share their type), bf16 cache: bf16
+    constexpr uint32_t f16 = KV8 ? ((1u << 7) | (1u << 10)) : 0u;
+    constexpr uint32_t idesc_s = tc_idesc(kPaB, kPaB) & ~f16;
+    constexpr uint32_t idesc_o = (tc_idesc(kPaB, kPaHD) | (1u << 16)) & ~f16;
+    const uint64_t qd = sdesc(smem_u32(sQ)), kd = sdesc(smem_u32(sK)), vd = sdesc_mn(smem_u32(sV), kPaHalf);
+    int n = 0, kn = 0, pn[2] = {0, 0}, on[2] = {0, 0};
     bool ok = true;
-    for (int t = 0; t < nt; ++t) {
-      ok = mbar_wait(&sfull, t & 1);
-      if (!__all_sync(0xffffffffu, ok) || __any_sync(0xffffffffu, *abort_flag != 0)) {
-        ok = false;
-        break;
+    // descriptor start addresses count 16-byte units
+    auto scores = [&](int j, int s) {  // S_j = Q_j K^T of ring tile s (issuing lane only)
+      const uint64_t qj = qd + j * (kPaTile >> 4), ks = kd + s * (kPaTile >> 4);
+#pragma unroll
+      for (int kk = 0; kk < kPaHD / 16; ++kk) {
+        const int off = ((kk >> 2) * kPaHalf + (kk & 3) * 32) >> 4;
+        tc_mma(tmem + j * kPaB, qj + off, ks + off, idesc_s, kk > 0 ? 1u : 0u);
       }
+      tc_commit(&sfull[j]);
+    };
+    for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
+      const PaItem w(i, S, H, Hkv, plan);
+      const int nt = w.tiles();
+      ok = mbar_wait(KV8 ? &qconv : &qfull, n & 1) && mbar_wait(&kfull[kn % kPaRing], (kn / kPaRing) & 1) && !*abort_flag;
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
       tc_fence_after();
-      const int key0 = t * kPaB;
-      // keys past this row or past S only occur in the diagonal tile
-      const bool masked = key0 + kPaB - 1 > q0 || key0 + kPaB > S;
-      // raw scores of chunk c (kPaCW columns); masked keys read -inf
-      auto load_raw = [&](auto mask, int c, float* v) {
-        uint32_t r[kPaCW];
-        tc_ld<kPaCW>(lane_base + kPaS + c * kPaCW, r);
-        if constexpr (KV8) {
-          // K scale of each key column (masked columns are overwritten below)
-          const float4* k4 = reinterpret_cast<const float4*>(s_scl + (t & 1) * kPaB + c * kPaCW);
+      if (elect_one()) {
 #pragma unroll
-          for (int i = 0; i < kPaCW / 4; ++i) {
-            const float4 f = k4[i];
-            r[4 * i] = __float_as_uint(__uint_as_float(r[4 * i]) * f.x);
-            r[4 * i + 1] = __float_as_uint(__uint_as_float(r[4 * i + 1]) * f.y);
-            r[4 * i + 2] = __float_as_uint(__uint_as_float(r[4 * i + 2]) * f.z);
-            r[4 * i + 3] = __float_as_uint(__uint_as_float(r[4 * i + 3]) * f.w);
+        for (int j = 0; j < 2; ++j)
+          if (w.nt[j] > 0) scores(j, kn % kPaRing);
+        tc_commit(&kempty[kn % kPaRing]);
+        if (nt == 1) tc_commit(&qempty);
+      }
+      __syncwarp();
+      for (int t = 0; t < nt && ok; ++t, ++kn) {
+        const int s = kn % kPaRing, s1 = (kn + 1) % kPaRing;
+        ok = mbar_wait(&vfull[s], (kn / kPaRing) & 1);
+        if (t + 1 < nt) ok = ok && mbar_wait(&kfull[s1], ((kn + 1) / kPaRing) & 1);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          if (t >= w.nt[j] || !ok) continue;
+          // P_j(t) is written, and (first tile) the last item's output has been read
+          ok = mbar_wait(&pfull[j], pn[j] & 1) && (t > 0 || on[j] == 0 || mbar_wait(&oempty[j], (on[j] - 1) & 1)) &&
+               !*abort_flag;
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) continue;
+          ++pn[j];
+          tc_fence_after();
+          if (elect_one()) {
+            const uint64_t vs = vd + s * (kPaTile >> 4);
+#pragma unroll
+            for (int kk = 0; kk < kPaB / 16; ++kk)  // 16 keys: two 8-row groups of the V tile
+              tc_mma_ts(tmem + kPaO + j * kPaHD, tmem + j * kPaB + kk * 8, vs + kk * (2048 >> 4), idesc_o,
+                        (t > 0 || kk > 0) ? 1u : 0u);
+            if (t + 1 < w.nt[j]) scores(j, s1);
+            else tc_commit(&ofull[j]);
+          }
+          __syncwarp();
+          if (t + 1 >= w.nt[j]) ++on[j];
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (elect_one()) {
+          tc_commit(&vempty[s]);
+          if (t + 1 < nt) tc_commit(&kempty[s1]);
+          if (t + 2 == nt) tc_commit(&qempty);  // the item's last scores: Q may be overwritten
+        }
+        __syncwarp();
+      }
+    }
+    if (!ok && lane == 0) fail();
+    if (elect_one()) tc_commit(&mma_done);
+    __syncwarp();
+    mbar_wait(&mma_done, 0);
+  } else if (KV8 && warp >= kPaWarpWiden) {
+    // ---------------- int8 cache: Q to fp16, then widening of the key tiles
+    const int wi = (warp - kPaWarpWiden) * 32 + lane;  // 0 .. 191
+    constexpr int WT = 32 * kPaWiden;
+    const int c = wi & 7;                                     // code chunk: head_dim 16c .. 16c + 15
+    const int rbase = wi >> 3;                                // tile rows rbase + 24i (< 128)
+    // its bf16 form is chunks cb, cb + 1 of half c / 4 of the swizzled row;
+    // the lanes of the upper half store the odd chunk first, so the eight
+    // lanes of one row write eight distinct 16-byte bank groups
+    const int cb = 2 * (c & 3), half_off = (c >> 2) * kPaHalf;
+    int n = 0, kn = 0;
+    bool ok = true;
+    for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
+      const PaItem w(i, S, H, Hkv, plan);
+      const int nt = w.tiles();
+      const int32_t* pt = page_table + (long long)w.b * pages_per_seq;
+      // sigma: from the largest V scale over the keys the item reads
+      float vmax = 0.f;
+      const int nkeys = min(nt * kPaB, S);
+#pragma unroll 4
+      for (int key = wi; key < nkeys; key += WT) {
+        const int pg = __ldg(pt + key / page_size);
+        if (pg >= 0 && pg < n_pages) vmax = fmaxf(vmax, __ldg(v_scale + (pg * Hkv + w.kvh) * page_size + key % page_size));
+      }
+      vmax = warp_max(vmax);
+      // (a warp that reaches the next item's meeting has read this item's values)
+      if (lane == 0) {
+        s_vmax[n & 1][warp - kPaWarpWiden] = vmax;
+        mbar_arrive(&vmet);
+      }
+      ok = __all_sync(0xffffffffu, mbar_wait(&vmet, n & 1));
+#pragma unroll
+      for (int x = 0; x < kPaWiden; ++x) vmax = fmaxf(vmax, s_vmax[n & 1][x]);
+      // 2^sigma with 256 * vmax * 2^sigma <= 65280 (vmax = 0: no V weight at all)
+      const int sigma = vmax > 0.f ? min(60, max(-60, (int)floorf(log2f(255.f / vmax)))) : 0;
+      const float vmul = exp2f((float)sigma);
+      // Q to fp16 in place (the element order of the swizzled tiles is kept)
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(&qfull, n & 1));
+      if (ok) {
+        bool over = false;
+        const int q16 = (w.nt[1] > 0 ? 2 : 1) * (kPaTile / 16);
+#pragma unroll 4
+        for (int x = wi; x < q16; x += WT) {
+          uint4* p = reinterpret_cast<uint4*>(sQ) + x;
+          const uint4 v = *p;
+          const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+          uint32_t o[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 f = bf2x2f(w4[j]);
+            over |= fabsf(f.x) > 65504.f || fabsf(f.y) > 65504.f;
+            o[j] = pa_pack_h(f.x, f.y);
+          }
+          *p = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+        if (over && err) atomicExch(err, 3);  // q outside the fp16 range: the output is invalid
+        // published with Q, which every score of the item follows; this slot's
+        // last reader was the epilogue of item n - 4: the scores of item n - 1,
+        // whose last use of Q preceded this item's Q, follow P of item n - 2 and
+        // so that tile's epilogue of item n - 3
+        if (wi == 0) s_unscale[n & 3] = exp2f((float)-sigma);
+        fence_proxy_async();
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&qconv);
+      for (int t = 0; t < nt && ok; ++t, ++kn) {
+        const int s = kn % kPaRing, ph = ((kn / kPaRing) & 1) ^ 1;
+        int rowi[kPaWRows];  // pool row of each of the thread's keys (< 2^31); -1 reads zeros
+#pragma unroll
+        for (int r = 0; r < kPaWRows; ++r) {
+          const int row = rbase + 4 * kPaWiden * r, key = t * kPaB + row;
+          rowi[r] = -1;
+          if (row < kPaB && key < S) {
+            const int pg = __ldg(pt + key / page_size);
+            if (pg >= 0 && pg < n_pages) rowi[r] = (pg * Hkv + w.kvh) * page_size + key % page_size;
+            else if (err && c == 0) atomicExch(err, 1);
           }
         }
+        // the tile's K and V scales go out with its K codes: the softmax reads
+        // both once S(t) is complete, which only the K tile's barrier precedes
+        float sck[kPaWRows], scv[kPaWRows];
 #pragma unroll
-        for (int i = 0; i < kPaCW; ++i) {
-          v[i] = __uint_as_float(r[i]);
-          if constexpr (decltype(mask)::value) {
-            const int key = key0 + c * kPaCW + i;
-            if (key > qrow || key >= S) v[i] = -INFINITY;
+        for (int r = 0; r < kPaWRows; ++r) {
+          sck[r] = (c == 0 && rowi[r] >= 0) ? __ldg(k_scale + rowi[r]) : 0.f;
+          scv[r] = (c == 0 && rowi[r] >= 0) ? __ldg(v_scale + rowi[r]) * vmul : 0.f;
+        }
+#pragma unroll 1
+        for (int which = 0; which < 2; ++which) {
+          const int8_t* pool = which ? v8 : k8;
+          uint4 cw[kPaWRows];
+          // the codes are read before the wait for the buffer
+#pragma unroll
+          for (int r = 0; r < kPaWRows; ++r)
+            cw[r] = rowi[r] >= 0 ? ld_nc16(pool + (long long)rowi[r] * kPaHD + c * 16) : make_uint4(0, 0, 0, 0);
+          if (kn >= kPaRing) ok = mbar_wait(which ? &vempty[s] : &kempty[s], ph);
+          if (!__all_sync(0xffffffffu, ok) || __any_sync(0xffffffffu, *abort_flag != 0)) {
+            ok = false;
+            break;
           }
-        }
-      };
-      // pass 1: the row maximum of the raw scores (scale > 0 keeps the order)
-      auto row_max = [&](auto mask) {
-        float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll 1
-        for (int c = 0; c < kPaB / kPaCW; ++c) {
-          float v[kPaCW];
-          load_raw(mask, c, v);
+          uint8_t* dst = (which ? sV : sK) + s * kPaTile + half_off;
 #pragma unroll
-          for (int i = 0; i < kPaCW; ++i) m4[i & 3] = fmaxf(m4[i & 3], v[i]);
-        }
-        return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-      };
-      const float mraw = masked ? row_max(std::true_type{}) : row_max(std::false_type{});
-      const float mx = mraw * scale;
-      // move the reference when the tile would exceed it by more than 2^kPaSlack
-      float corr = 1.f;
-      if (mx > m + kPaSlack) {
-        corr = exp2f(m - mx);  // 0 on the first tile
-        m = mx;
-        l *= corr;
-      }
-      if (t > 0 && __any_sync(0xffffffffu, corr != 1.f)) {
-        // O holds P V of the earlier tiles (complete: S(t) was issued after it)
-#pragma unroll 1
-        for (int c = 0; c < kPaHD / 32; ++c) {
-          uint32_t r[32];
-          tc_ld<32>(lane_base + kPaO + c * 32, r);
+          for (int r = 0; r < kPaWRows; ++r) {
+            const int row = rbase + 4 * kPaWiden * r, sw = row & 7;
+            if (row >= kPaB) break;
+            const uint32_t ww[4] = {cw[r].x ^ 0x80808080u, cw[r].y ^ 0x80808080u, cw[r].z ^ 0x80808080u,
+                                    cw[r].w ^ 0x80808080u};
+            uint32_t o[8];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * corr);
-          tc_st32(lane_base + kPaO + c * 32, r);
-        }
-      }
-      // pass 2: P = 2^(s scale - m) as bf16 pairs over the score columns already read
-      const float mref = m == -INFINITY ? 0.f : m;
-      auto write_p = [&](auto mask) {
-        float p4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-        for (int c = 0; c < kPaB / kPaCW; ++c) {
-          float v[kPaCW];
-          load_raw(mask, c, v);
-          uint32_t pw[kPaCW / 2];
-#pragma unroll
-          for (int i = 0; i < kPaCW; i += 2) {
-            const float p0 = pa_ex2(fmaf(v[i], scale, -mref)), p1 = pa_ex2(fmaf(v[i + 1], scale, -mref));
-            p4[i & 3] += p0;
-            p4[(i + 1) & 3] += p1;
-            if constexpr (KV8) {
-              // V scale of each key column: P V then takes the codes as they are
-              const float2 vs = *reinterpret_cast<const float2*>(s_scl + (2 + (t & 1)) * kPaB + c * kPaCW + i);
-              pw[i / 2] = pa_pack_h(p0 * vs.x, p1 * vs.y);
+            for (int j = 0; j < 8; ++j) o[j] = pa_i8h2(ww[j >> 1], (j & 1) ? 0x4342 : 0x4140);
+            const uint4 e = make_uint4(o[0], o[1], o[2], o[3]), f = make_uint4(o[4], o[5], o[6], o[7]);
+            uint8_t* rp = dst + row * 128;
+            if (c < 4) {
+              *reinterpret_cast<uint4*>(rp + ((cb ^ sw) << 4)) = e;
+              *reinterpret_cast<uint4*>(rp + (((cb + 1) ^ sw) << 4)) = f;
             } else {
-              pw[i / 2] = pa_pack(p0, p1);
+              *reinterpret_cast<uint4*>(rp + (((cb + 1) ^ sw) << 4)) = f;
+              *reinterpret_cast<uint4*>(rp + ((cb ^ sw) << 4)) = e;
+            }
+            if (which == 0 && c == 0) {
+              // slot kn % 4 was last read by the softmax of tile kn - 4; K tile
+              // kn - 2 has been multiplied, which its P V (of tile kn - 3) preceded
+              s_scl[(kn % kPaScl) * kPaB + row] = sck[r];
+              s_scl[(kPaScl + kn % kPaScl) * kPaB + row] = scv[r];
             }
           }
-          pa_st16(lane_base + kPaS + c * (kPaCW / 2), pw);
-        }
-        return (p4[0] + p4[1]) + (p4[2] + p4[3]);
-      };
-      const float ps = masked ? write_p(std::true_type{}) : write_p(std::false_type{});
-      l += ps;
-      tc_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&pfull);
-    }
-    if (ok) {
-      ok = mbar_wait(&ofull, (nt - 1) & 1);
-      ok = __all_sync(0xffffffffu, ok);
-    }
-    if (ok) {
-      tc_fence_after();
-      // int8 cache: P carried the V scales times 2^sigma
-      const float inv = (KV8 ? s_unscale : 1.f) / l;
-      uint16_t* dst = out + ((long long)b * S + qrow) * ((long long)H * kPaHD) + (long long)h * kPaHD;
-#pragma unroll 1
-      for (int c = 0; c < kPaHD / 32; ++c) {
-        uint32_t r[32];
-        tc_ld<32>(lane_base + kPaO + c * 32, r);
-        if (qrow < S) {
-#pragma unroll
-          for (int i = 0; i < 32; i += 8)
-            *reinterpret_cast<uint4*>(dst + c * 32 + i) =
-                make_uint4(pack_bf2(__uint_as_float(r[i]) * inv, __uint_as_float(r[i + 1]) * inv),
-                           pack_bf2(__uint_as_float(r[i + 2]) * inv, __uint_as_float(r[i + 3]) * inv),
-                           pack_bf2(__uint_as_float(r[i + 4]) * inv, __uint_as_float(r[i + 5]) * inv),
-                           pack_bf2(__uint_as_float(r[i + 6]) * inv, __uint_as_float(r[i + 7]) * inv));
+          fence_proxy_async();  // the MMAs read the tile through the async proxy
+          __syncwarp();
+          if (lane == 0) mbar_arrive(which ? &vfull[s] : &kfull[s]);
         }
       }
-    } else if (lane == 0) {
-      fail();
     }
+    if (!ok && lane == 0) fail();
+  } else if (warp < kPaWarpTma) {
+    // ---------------- softmax: thread = query row (TMEM lane 32 (warp % 4) + lane) of tile j
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(pa_reg_soft<KV8>()));
+    const int j = warp >> 2, quad = warp & 3, row = quad * 32 + lane;
+    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
+    const uint32_t ts = lane_base + j * kPaB, to = lane_base + kPaO + j * kPaHD;
+    const float scale = kPaLog2e * rsqrtf((float)kPaHD);
+    int n = 0, kn = 0, sn = 0, on = 0;  // items, key tiles, this tile's scores and outputs
+    bool ok = true;
+    for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
+      const PaItem w(i, S, H, Hkv, plan);
+      const int nt = w.key_tiles(j), qrow = w.row0(j) + row;  // position in the sequence
+      float m = -INFINITY;                            // reference maximum (log2 domain)
+      float2 l2[4];                                   // row sum
+#pragma unroll
+      for (int y = 0; y < 4; ++y) l2[y] = make_float2(0.f, 0.f);
+      for (int t = 0; t < nt; ++t, ++sn) {
+        ok = mbar_wait(&sfull[j], sn & 1);
+        if (!__all_sync(0xffffffffu, ok)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        uint32_t r[kPaB];
+        tc_ld<64>(ts, r);
+        tc_ld<64>(ts + 64, r + 64);
+        float* v = reinterpret_cast<float*>(r);
+        const int key0 = t * kPaB;
+        const float* ks = s_scl + ((kn + t) % kPaScl) * kPaB;
+        if constexpr (KV8) {
+#pragma unroll
+          for (int x = 0; x < kPaB; x += 4) {  // K scale of each key column
+            const float4 f = *reinterpret_cast<const float4*>(ks + x);
+            const float2 a = pa_mul2(make_float2(v[x], v[x + 1]), make_float2(f.x, f.y));
+            const float2 b = pa_mul2(make_float2(v[x + 2], v[x + 3]), make_float2(f.z, f.w));
+            v[x] = a.x, v[x + 1] = a.y, v[x + 2] = b.x, v[x + 3] = b.y;
+          }
+        }
+        if (t == nt - 1) {  // the diagonal tile: keys after this row (and so past S) are masked
+#pragma unroll
+          for (int x = 0; x < kPaB; ++x)
+            if (key0 + x > qrow) v[x] = -INFINITY;
+        }
+        float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int x = 0; x < kPaB; x += 8)
+#pragma unroll
+          for (int y = 0; y < 4; ++y) m4[y] = fmaxf(m4[y], fmaxf(v[x + 2 * y], v[x + 2 * y + 1]));
+        const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * scale;
+        // move the reference when the tile would exceed it by more than 2^kPaSlack
+        float corr = 1.f;
+        if (mx > m + kPaSlack) {
+          corr = exp2f(m - mx);  // 0 on the first tile
+          m = mx;
+#pragma unroll
+          for (int y = 0; y < 4; ++y) l2[y] = pa_mul2(l2[y], make_float2(corr, corr));
+        }
+        if (t > 0 && __any_sync(0xffffffffu, corr != 1.f)) {
+          // O holds P V of the earlier tiles (complete: S(t) was issued after it)
+#pragma unroll 1
+          for (int x = 0; x < kPaHD / 16; ++x) {
+            uint32_t o[16];
+            tc_ld<16>(to + x * 16, o);
+#pragma unroll
+            for (int y = 0; y < 16; ++y) o[y] = __float_as_uint(__uint_as_float(o[y]) * corr);
+            tc_st16(to + x * 16, o);
+          }
+        }
+        // P = 2^(s scale - m) as 16-bit pairs over the score columns
+        const float mref = m == -INFINITY ? 0.f : m;
+        const float2 sc2 = make_float2(scale, scale), nm2 = make_float2(-mref, -mref);
+        const float* vs = s_scl + (kPaScl + (kn + t) % kPaScl) * kPaB;
+#pragma unroll
+        for (int x0 = 0; x0 < kPaB; x0 += 32) {
+          uint32_t pw[16];
+#pragma unroll
+          for (int x = 0; x < 32; x += 2) {
+            const float2 e = pa_fma2(make_float2(v[x0 + x], v[x0 + x + 1]), sc2, nm2);
+            float2 p = make_float2(pa_ex2(e.x), pa_ex2(e.y));
+            l2[(x >> 1) & 3] = pa_add2(l2[(x >> 1) & 3], p);
+            if constexpr (KV8) {
+              // V scale of each key column: P V then takes the codes as they are
+              p = pa_mul2(p, *reinterpret_cast<const float2*>(vs + x0 + x));
+              pw[x / 2] = pa_pack_h(p.x, p.y);
+            } else {
+              pw[x / 2] = pa_pack(p.x, p.y);
+            }
+          }
+          tc_st16(ts + x0 / 2, pw);
+        }
+        tc_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&pfull[j]);
+      }
+      kn += w.tiles();
+      if (!ok) break;
+      if (nt == 0) continue;
+      const float l = ((l2[0].x + l2[0].y) + (l2[1].x + l2[1].y)) + ((l2[2].x + l2[2].y) + (l2[3].x + l2[3].y));
+      // ---- the item's output
+      ok = __all_sync(0xffffffffu, mbar_wait(&ofull[j], on & 1));
+      if (!ok) break;
+      ++on;
+      tc_fence_after();
+      // int8 cache: P carried the V scales times 2^sigma
+      const float inv = (KV8 ? s_unscale[n & 3] : 1.f) / l;
+      const int pos = w.row0(j) + quad * 32;
+      pa_write_rows(to, inv, sV + kPaRing * kPaTile + warp * kPaStage,
+                    out + ((long long)w.b * S + pos) * ((long long)H * kPaHD) + (long long)w.head(j) * kPaHD,
+                    (long long)H * kPaHD, pos, S, [&]() {
+                      tc_fence_before();
+                      __syncwarp();
+                      if (lane == 0) mbar_arrive(&oempty[j]);
+                    });
+    }
+    if (!ok && lane == 0) fail();
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) {
+  if (warp == kPaWarpMma) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kPaTmemCols) : "memory");
   }
@@ -526,7 +619,35 @@ bool attention_prefill_tc_ok(int B, int S, int n_heads, const fp_kv_view& kv, co
   return (kv.kvquant == FP_KV_BF16 || (kv8 && kv.k_scale && kv.v_scale)) && kv.head_dim == kPaHD &&
          kv.page_size == 16 && B >= 1 && S >= 1 && n_heads % kv.n_kv_heads == 0 && q_stride % 8 == 0 &&
          ((uintptr_t)q & 15) == 0 && ((uintptr_t)kv.k_pool & 15) == 0 && ((uintptr_t)kv.v_pool & 15) == 0 &&
-         (long long)kv.n_pages * kv.n_kv_heads * kv.page_size < (1LL << 31) && tensor_maps_available();
+         (long long)kv.n_pages * kv.n_kv_heads * kv.page_size < (1LL << 31) &&
+         (long long)B * n_heads * ((S + kPaB - 1) / kPaB) < (1LL << 26) && tensor_maps_available();
+}
+
+// Pairs of tiles where they keep the SMs busy, single tiles where pairs would
+// leave SMs idle or make one CTA's share too long: the smaller of the two
+// makespans (the mean share of an SM, or the longest item), with a key tile at
+// 4100 cycles for a pair and 3000 for one tile, and 3500 cycles an item
+// (measured, bf16 cache).
+static PaPlan pa_plan(int B, int S, int H, int G, int sms) {
+  const long long tiles = (S + kPaB - 1) / kPaB;
+  const int pair = G % 2 == 0 ? 1 : 2;
+  auto make = [&](int pr) {
+    PaPlan p{};
+    p.pair = pr;
+    p.units = (int)(pr == 2 ? (tiles + 1) / 2 : tiles);
+    p.items = (int)((long long)B * (pr == 1 ? H / 2 : H) * p.units);
+    p.longest_first = p.items <= 4LL * sms;
+    return p;
+  };
+  auto span = [&](const PaPlan& p) {
+    const double step = p.pair ? 4100 : 3000, longest = tiles * step + 3500;
+    double sum = 0;  // key tiles of a head's items
+    for (long long u = 0; u < p.units; ++u) sum += (double)std::min(tiles, p.pair == 2 ? 2 * u + 2 : u + 1);
+    const double heads = (double)p.items / p.units;
+    return std::max((sum * step + 3500.0 * p.units) * heads / sms, longest);
+  };
+  const PaPlan two = make(pair), one = make(0);
+  return span(one) < span(two) ? one : two;
 }
 
 template <bool KV8>
@@ -534,11 +655,18 @@ static cudaError_t launch_pa_tc(const CUtensorMap& mq, const CUtensorMap& mk, co
                                 int n_heads, const fp_kv_view& kv, uint16_t* out, int32_t* err, cudaStream_t s) {
   static std::atomic<unsigned long long> attr{0};
   FP_CUDA_TRY(smem_limit_once(attn_prefill_tc_kernel<KV8>, kPaSmem, &attr));
-  const dim3 grid((S + kPaB - 1) / kPaB, n_heads, B);
-  return launch(attn_prefill_tc_kernel<KV8>, grid, dim3(pa_threads<KV8>()), (size_t)kPaSmem, s, mq, mk, mv,
-                (const int8_t*)kv.k_pool, (const int8_t*)kv.v_pool, (const float*)kv.k_scale,
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        sms <= 0)
+      sms = 152;
+  }
+  const PaPlan plan = pa_plan(B, S, n_heads, n_heads / kv.n_kv_heads, sms);
+  return launch(attn_prefill_tc_kernel<KV8>, dim3(std::min(plan.items, sms)), dim3(pa_threads<KV8>()), (size_t)kPaSmem,
+                s, mq, mk, mv, (const int8_t*)kv.k_pool, (const int8_t*)kv.v_pool, (const float*)kv.k_scale,
                 (const float*)kv.v_scale, S, n_heads, kv.n_kv_heads, kv.page_size, kv.page_table, kv.pages_per_seq,
-                kv.n_pages, out, err);
+                kv.n_pages, plan, out, err);
 }
 
 cudaError_t launch_attention_prefill_tc(const uint16_t* q, int q_stride, int B, int S, int n_heads,
@@ -547,12 +675,16 @@ cudaError_t launch_attention_prefill_tc(const uint16_t* q, int q_stride, int B, 
   const long long pool_rows = (long long)kv.n_pages * kv.n_kv_heads * kv.page_size;
   // q [B S][q_stride] bf16, box [128 rows][64]
   if (!make_tensor_map(&mq, q, (long long)B * S, q_stride, 2, kPaB, 64, 128)) return cudaErrorInvalidValue;
-  if (kv.kvquant == FP_KV_INT8) return launch_pa_tc<true>(mq, mq, mq, B, S, n_heads, kv, out, err, s);
+  const bool one_tile = S <= kPaB && B <= 65535;  // B: the grid's y extent
+  if (kv.kvquant == FP_KV_INT8)
+    return one_tile ? launch_attention_prefill_short(mq, mq, mq, B, S, n_heads, kv, out, err, s)
+                    : launch_pa_tc<true>(mq, mq, mq, B, S, n_heads, kv, out, err, s);
   // bf16 pools [pages Hkv 16][128], box [16 rows][64]
   if (!make_tensor_map(&mk, kv.k_pool, pool_rows, kPaHD, 2, 16, 64, 128) ||
       !make_tensor_map(&mv, kv.v_pool, pool_rows, kPaHD, 2, 16, 64, 128))
     return cudaErrorInvalidValue;
-  return launch_pa_tc<false>(mq, mk, mv, B, S, n_heads, kv, out, err, s);
+  return one_tile ? launch_attention_prefill_short(mq, mk, mv, B, S, n_heads, kv, out, err, s)
+                  : launch_pa_tc<false>(mq, mk, mv, B, S, n_heads, kv, out, err, s);
 }
 
 }  // namespace fpk

@@ -80,6 +80,16 @@ FP_DEV void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_
       : "memory");
 }
 
+// One lane of a converged warp (always the same one).  A warp whose lanes all
+// run the issuing loop, with only the MMAs and commits behind this, keeps their
+// descriptors in uniform registers; a loop that one lane runs alone moves every
+// operand of every MMA there first, which took longer than the MMA.
+FP_DEV bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
 // 1-D bulk copy: bytes a multiple of 16, both addresses 16-byte aligned.
 FP_DEV void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(

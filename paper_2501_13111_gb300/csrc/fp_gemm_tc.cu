@@ -1,11 +1,13 @@
 // Prefill weight-only linear on the 5th-generation tensor cores.
 //
 // y[M][N] = x[M][K] W[N][K]^T for M > 64 (prefill), the dense contraction of
-// the block's linear layers.  One persistent CTA per SM walks 128 x 256
-// output tiles, each over the whole K:
+// the block's linear layers.  Persistent: a pair of CTAs (on two SMs) walks
+// 256 x 256 output tiles, each over the whole K, or, where that needs more rounds,
+// one CTA 128 x 256 tiles:
 //   warp 0      TMA producer: x tile [128][64] and W tile [256][64] (bf16,
-//               128-byte swizzled, K-major) into a 4-stage shared ring,
-//               completion counted in bytes on mbarrier full[s];
+//               128-byte swizzled, K-major; half of the W tile in each CTA of a
+//               pair) into a 4-stage (6-stage) shared ring, completion counted
+//               in bytes on mbarrier full[s] (of the even CTA);
 //   warp 1      allocates 512 TMEM columns (two fp32 accumulators) and, from
 //               one thread, issues tcgen05.mma (M 128, N 256, K 16);
 //               tcgen05.commit frees each stage (empty[s]) and signals a full
@@ -37,9 +39,17 @@ static __device__ long long g_stage_wait_limit = fpk::kTcSpinLimit;
 
 namespace fpk {
 
-constexpr int kTcBM = 128, kTcBN = 256, kTcBK = 64, kTcStages = 4;
+constexpr int kTcBM = 128, kTcBN = 256, kTcBK = 64;
 constexpr int kTcThreads = 192;
-constexpr uint32_t kTcStageBytes = (kTcBM + kTcBN) * kTcBK * 2;  // 48 KiB
+// Shared memory of a stage and the ring's depth, one CTA / each CTA of a pair
+// (which holds its own 128 rows of x and half of the 256 weight rows).
+template <bool PAIR>
+struct TcGeom {
+  static constexpr int kBRows = PAIR ? kTcBN / 2 : kTcBN;
+  static constexpr uint32_t kStageBytes = (kTcBM + kBRows) * kTcBK * 2;  // 48 / 32 KiB
+  static constexpr int kStages = PAIR ? 6 : 4;
+  static constexpr int kSmem = kStages * kStageBytes + 1024;
+};
 constexpr uint32_t kTcTmemCols = 512;  // two 256-column fp32 accumulators
 
 // ------------------------------------------------------------------ kernel
@@ -51,57 +61,83 @@ constexpr uint32_t kTcTmemCols = 512;  // two 256-column fp32 accumulators
 // SCALE: multiply output column n by bf16 scales[n] (int8 weights; SwiGLU:
 // the up column by scales[up_off + n]).  Output (and residual) rows are ldy
 // elements apart, so a launch can fill a band of columns of a wider output.
-template <int EPI, bool SCALE>
+// PAIR: clusters of two CTAs on a 256 x 256 tile (cta_group::2): CTA r of a pair
+// keeps rows 128 r .. of x and of the output, and loads half of the weight rows,
+// which both read; the even CTA issues the MMAs.
+template <int EPI, bool SCALE, bool PAIR>
 __global__ void __launch_bounds__(kTcThreads, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, int M, int N,
                    int K, const uint16_t* __restrict__ scales, long long up_off, const uint16_t* R, void* Y,
                    int ldy, int32_t* err) {
+  using G = TcGeom<PAIR>;
+  constexpr int ST = G::kStages, CG = PAIR ? 2 : 1;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ uint64_t full[kTcStages], empty[kTcStages], tfull[2], tempty[2], mma_done;
+  __shared__ uint64_t full[ST], empty[ST], tfull[2], tempty[2], mma_done, never;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_word;
   volatile int* abort_flag = &abort_word;  // set by a role that gave up waiting
   // stage buffers must be 1024-byte aligned for the 128-byte swizzle
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = PAIR ? (int)cluster_rank() : 0;
   constexpr int NR = EPI == FP_EPI_SWIGLU ? 2 : 1;
   const int Nout = NR == 2 ? N / 2 : N;
   constexpr int BNout = kTcBN / NR;
-  const int tiles_m = (M + kTcBM - 1) / kTcBM, tiles_n = (Nout + BNout - 1) / BNout;
+  const int tiles_m = (M + CG * kTcBM - 1) / (CG * kTcBM), tiles_n = (Nout + BNout - 1) / BNout;
   const int ntiles = tiles_m * tiles_n;
   const int kblocks = (K + kTcBK - 1) / kTcBK;
+  const int first_tile = blockIdx.x / CG, tile_step = gridDim.x / CG;
   auto tile_origin = [&](int t, int& m0, int& n0) {
-    constexpr int GM = 16;
+    constexpr int GM = 16 / CG;
     const int span = GM * tiles_n;
     const int first = (t / span) * GM;
     const int gs = min(GM, tiles_m - first);
     const int r = t % span;
-    m0 = (first + r % gs) * kTcBM;
+    m0 = (first + r % gs) * (CG * kTcBM) + rank * kTcBM;
     n0 = (r / gs) * BNout;
+  };
+  auto fail = [&]() {
+    if constexpr (PAIR) {  // both CTAs stop
+      for (uint32_t r = 0; r < 2; ++r)
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(&abort_word, r)), "r"(1) : "memory");
+    } else {
+      *abort_flag = 1;
+    }
+    if (err) atomicExch(err, 2);
   };
 
   pdl_trigger();
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kTcStages; ++s) {
+    for (int s = 0; s < ST; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
-      mbar_init(&tfull[b], 1);   // tcgen05.commit of the tile's last MMAs
-      mbar_init(&tempty[b], 4);  // one arrival per epilogue warp
+      mbar_init(&tfull[b], 1);        // tcgen05.commit of the tile's last MMAs
+      mbar_init(&tempty[b], 4 * CG);  // one arrival per epilogue warp (of both CTAs)
     }
     mbar_init(&mma_done, 1);
+    mbar_init(&never, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if constexpr (PAIR) cluster_sync();  // the peer's barriers are up before anything signals them
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                 "r"(kTcTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                   "r"(kTcTmemCols)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                   "r"(kTcTmemCols)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync();  // both tensor memories are allocated
   tc_fence_after();
   const uint32_t tmem = tmem_base;
   pdl_wait();
@@ -110,85 +146,97 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // ---------------- TMA producer
     if (lane == 0) {
       int it = 0;  // k-blocks issued, across tiles
-      for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+      for (int t = first_tile; t < ntiles && !*abort_flag; t += tile_step) {
         int m0, n0;
         tile_origin(t, m0, n0);
         for (int kb = 0; kb < kblocks; ++kb, ++it) {
-          const int s = it % kTcStages;
-          if (!mbar_wait(&empty[s], ((it / kTcStages) & 1) ^ 1) || *abort_flag) {
-            *abort_flag = 1;
-            if (err) atomicExch(err, 2);
+          const int s = it % ST;
+          if (!mbar_wait(&empty[s], ((it / ST) & 1) ^ 1) || *abort_flag) {
+            fail();
             break;
           }
-          uint8_t* a = smem + s * kTcStageBytes;
+          uint8_t* a = smem + s * G::kStageBytes;
           uint8_t* b = a + kTcBM * kTcBK * 2;
-          mbar_expect_tx(&full[s], kTcStageBytes);
-          tma_load_2d(a, &map_x, kb * kTcBK, m0, &full[s]);
-          if (NR == 1) {
-            tma_load_2d(b, &map_w, kb * kTcBK, n0, &full[s]);
+          if constexpr (PAIR) {
+            // the bytes of both CTAs count on the even CTA's barrier
+            if (rank == 0) mbar_expect_tx(&full[s], 2 * G::kStageBytes);
+            const uint32_t bar = cluster_addr(&full[s], 0);
+            const int wrow = NR == 2 ? (rank ? Nout + n0 : n0) : n0 + rank * G::kBRows;  // SwiGLU: gate rows | up rows
+            tma_load_2d_pair(a, &map_x, kb * kTcBK, m0, bar);
+            tma_load_2d_pair(b, &map_w, kb * kTcBK, wrow, bar);
           } else {
-            tma_load_2d(b, &map_w, kb * kTcBK, n0, &full[s]);                              // gate rows
-            tma_load_2d(b + 128 * kTcBK * 2, &map_w, kb * kTcBK, Nout + n0, &full[s]);  // up rows
+            mbar_expect_tx(&full[s], G::kStageBytes);
+            tma_load_2d(a, &map_x, kb * kTcBK, m0, &full[s]);
+            tma_load_2d(b, &map_w, kb * kTcBK, n0, &full[s]);  // SwiGLU: gate rows
+            if (NR == 2) tma_load_2d(b + 128 * kTcBK * 2, &map_w, kb * kTcBK, Nout + n0, &full[s]);  // up rows
           }
         }
       }
-      // copies still in flight land before the CTA leaves (their stages are its shared memory)
-      for (int j = max(0, it - kTcStages); j < it; ++j) mbar_wait(&full[j % kTcStages], (j / kTcStages) & 1);
+      // copies still in flight land before the CTA leaves (their stages are its
+      // shared memory); a pair leaves together, after the even CTA has seen both's.
+      // After an abort the two may have issued different numbers of copies: a
+      // bounded wait for what never comes outlasts them
+      if (rank == 0)
+        for (int j = max(0, it - ST); j < it; ++j) mbar_wait(&full[j % ST], (j / ST) & 1);
+      if (PAIR && *abort_flag) mbar_wait(&never, 0);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = tc_idesc(kTcBM, kTcBN);
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t idesc = tc_idesc(CG * kTcBM, kTcBN);
       const long long stage_limit = g_stage_wait_limit;
+      auto commit = [&](uint64_t* bar) {
+        if constexpr (PAIR) tc_commit_pair(bar);
+        else tc_commit(bar);
+      };
       int it = 0, lt = 0;
-      for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x, ++lt) {
+      for (int t = first_tile; t < ntiles && !*abort_flag; t += tile_step, ++lt) {
         const int acc = lt & 1;
         // the epilogue has drained this accumulator (local tile lt - 2)
         if (!mbar_wait(&tempty[acc], ((lt >> 1) & 1) ^ 1) || *abort_flag) {
-          *abort_flag = 1;
-          if (err) atomicExch(err, 2);
+          fail();
           break;
         }
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)acc * kTcBN;
         bool ok = true;
         for (int kb = 0; kb < kblocks; ++kb, ++it) {
-          const int s = it % kTcStages;
-          if (!mbar_wait_n(&full[s], (it / kTcStages) & 1, stage_limit) || *abort_flag) {
+          const int s = it % ST;
+          if (!mbar_wait_n(&full[s], (it / ST) & 1, stage_limit) || *abort_flag) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a = smem_u32(smem + s * kTcStageBytes);
+          const uint32_t a = smem_u32(smem + s * G::kStageBytes);
           const uint32_t b = a + kTcBM * kTcBK * 2;
 #pragma unroll
-          for (int kk = 0; kk < kTcBK / 16; ++kk)
-            tc_mma(d, sdesc(a + kk * 32), sdesc(b + kk * 32), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-          tc_commit(&empty[s]);  // stage s is free once these MMAs have read it
+          for (int kk = 0; kk < kTcBK / 16; ++kk) {
+            if constexpr (PAIR) tc_mma_pair(d, sdesc(a + kk * 32), sdesc(b + kk * 32), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+            else tc_mma(d, sdesc(a + kk * 32), sdesc(b + kk * 32), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+          }
+          commit(&empty[s]);  // stage s is free once these MMAs have read it
         }
         if (!ok) {
-          *abort_flag = 1;
-          if (err) atomicExch(err, 2);
+          fail();
           break;
         }
-        tc_commit(&tfull[acc]);  // the tile's accumulator is complete
+        commit(&tfull[acc]);  // the tile's accumulator is complete
       }
       // every MMA issued has completed before TMEM is released
-      tc_commit(&mma_done);
+      commit(&mma_done);
       mbar_wait(&mma_done, 0);
     }
   } else {
     // ---------------- epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31
     const int q = warp & 3;
     int lt = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
+    for (int t = first_tile; t < ntiles; t += tile_step, ++lt) {
       const int acc = lt & 1;
       int m0, n0;
       tile_origin(t, m0, n0);
       const bool ok = mbar_wait(&tfull[acc], (lt >> 1) & 1);
       if (!ok || *abort_flag) {
-        if (!ok && err) atomicExch(err, 2);
-        *abort_flag = 1;
+        fail();
         break;
       }
       tc_fence_after();
@@ -246,62 +294,112 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       // this warp's reads of the accumulator are done: hand the buffer back to the MMA thread
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[acc])) : "memory");
+      if (lane == 0) {
+        if constexpr (PAIR) mbar_arrive_cluster(cluster_addr(&tempty[acc], 0));
+        else mbar_arrive(&tempty[acc]);
+      }
     }
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync();  // neither CTA leaves while the other's MMAs, copies or arrivals may touch it
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
+    if constexpr (PAIR)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
   }
 }
 
 // ------------------------------------------------------------------ dequant to bf16
 // int8: w = q (exact; the row scale is applied by the GEMM epilogue).
-// int4: w = bf16((q - z) * s), 8 elements (one packed word) per thread.
+// int4: w = bf16((q - z) * s), 8 elements (one packed word) at a time.
 // GPTQ4: the same expansion back into channel order: output channel k is
 // act-order column j = inv[k] (inv the inverse of the act order), with the
-// scale and zero of group j / 128; 8 consecutive channels per thread.
-__global__ void dequant_kernel(int wquant, const void* __restrict__ codes, const uint16_t* __restrict__ scales,
-                               const uint16_t* __restrict__ zeros, int N, int K, uint16_t* __restrict__ out,
-                               const int32_t* __restrict__ inv) {
+// scale and zero of group j / 128; 8 consecutive channels at a time.
+// Output row r is row r0 + r of the matrix for r < cols, row up0 + r - cols
+// after (SwiGLU: the band's gate rows, then its up rows).  A thread takes four
+// words a block's width apart, so that its loads are in flight together and
+// every access of a warp is contiguous (one word a thread at a time, its row found
+// by a division, took 35 us more on 22016 x 4096 int4).  Bound by memory, the
+// codes read and the bf16 written.  Running the expansion of one band beside the
+// GEMM of the band before, in more and smaller bands, lost more to the GEMMs'
+// starts and last rounds than it hid (22016 x 4096 int8, 4096 rows: 518-548 us
+// against 507).
+constexpr int kDqThreads = 128, kDqWords = 4;
+
+template <int WQ>
+__global__ void __launch_bounds__(kDqThreads)
+    dequant_kernel(const void* __restrict__ codes, const uint16_t* __restrict__ scales,
+                   const uint16_t* __restrict__ zeros, long long r0, long long up0, int cols, int rows, int K,
+                   uint16_t* __restrict__ out, const int32_t* __restrict__ inv) {
   pdl_trigger();
   pdl_wait();
-  const long long words = (long long)N * K / 8;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (long long)gridDim.x * blockDim.x) {
-    const long long e0 = i * 8;
-    const long long row = e0 / K;
-    const int k0 = (int)(e0 % K);
-    float f[8];
-    if (wquant == FP_W_GPTQ4) {
-      const uint32_t* cw = (const uint32_t*)codes + row * (K / 8);
-      const long long g0 = row * (K / 128);
+  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+    const long long row = r < cols ? r0 + r : up0 + (r - cols);
+    const int w0 = blockIdx.x * (kDqThreads * kDqWords) + threadIdx.x, words = K / 8;
+    uint16_t* o = out + (long long)r * K;
+    if constexpr (WQ == FP_W_GPTQ4) {
+      const uint32_t* cw = (const uint32_t*)codes + row * words;
+      const uint16_t *sr = scales + row * (K / 128), *zr = zeros + row * (K / 128);
+      for (int i = 0; i < kDqWords; ++i) {
+        const int w = w0 + i * kDqThreads;
+        if (w >= words) break;
+        float f[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int a = min(max(inv[k0 + j], 0), K - 1);  // the inverse comes from the act order, in range
-        const int e = a & 7, nib = (e >> 1) + 4 * (e & 1);  // element e of a word sits in this nibble
-        const float q = (float)((cw[a >> 3] >> (4 * nib)) & 0xF);
-        f[j] = (q - bf2f(zeros[g0 + (a >> 7)])) * bf2f(scales[g0 + (a >> 7)]);
+        for (int j = 0; j < 8; ++j) {
+          const int a = min(max(inv[w * 8 + j], 0), K - 1);  // the inverse comes from the act order, in range
+          const int e = a & 7, nib = (e >> 1) + 4 * (e & 1);  // element e of a word sits in this nibble
+          const float q = (float)((cw[a >> 3] >> (4 * nib)) & 0xF);
+          f[j] = (q - bf2f(zr[a >> 7])) * bf2f(sr[a >> 7]);
+        }
+        *reinterpret_cast<uint4*>(o + (long long)w * 8) =
+            make_uint4(pack_bf2(f[0], f[1]), pack_bf2(f[2], f[3]), pack_bf2(f[4], f[5]), pack_bf2(f[6], f[7]));
       }
-    } else if (wquant == FP_W_INT8) {
-      const uint2 c = *reinterpret_cast<const uint2*>((const int8_t*)codes + e0);
-      const uint32_t w[2] = {c.x, c.y};
+    } else if constexpr (WQ == FP_W_INT8) {
+      const uint2* cr = (const uint2*)codes + row * words;
+      uint2 c[kDqWords];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) f[j] = (float)(int8_t)((w[j >> 2] >> (8 * (j & 3))) & 0xFF);
+      for (int i = 0; i < kDqWords; ++i)
+        c[i] = w0 + i * kDqThreads < words ? __ldg(cr + w0 + i * kDqThreads) : make_uint2(0u, 0u);
+#pragma unroll
+      for (int i = 0; i < kDqWords; ++i) {
+        const uint32_t w[2] = {c[i].x, c[i].y};
+        float f[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) f[j] = (float)(int8_t)((w[j >> 2] >> (8 * (j & 3))) & 0xFF);
+        if (w0 + i * kDqThreads < words)
+          *reinterpret_cast<uint4*>(o + (long long)(w0 + i * kDqThreads) * 8) =
+              make_uint4(pack_bf2(f[0], f[1]), pack_bf2(f[2], f[3]), pack_bf2(f[4], f[5]), pack_bf2(f[6], f[7]));
+      }
     } else {
-      const uint32_t w = *reinterpret_cast<const uint32_t*>((const uint8_t*)codes + e0 / 2);
-      const long long gi = row * (K / 128) + k0 / 128;
-      const float s = bf2f(scales[gi]), z = bf2f(zeros[gi]);
-      // nibbles i and i + 4 hold elements 2i and 2i + 1
+      const uint32_t* cr = (const uint32_t*)codes + row * words;
+      const uint16_t *sr = scales + row * (K / 128), *zr = zeros + row * (K / 128);
+      uint32_t c[kDqWords];
+      float s[kDqWords], z[kDqWords];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        f[2 * j] = ((float)((w >> (4 * j)) & 0xF) - z) * s;
-        f[2 * j + 1] = ((float)((w >> (4 * j + 16)) & 0xF) - z) * s;
+      for (int i = 0; i < kDqWords; ++i) {
+        const int w = w0 + i * kDqThreads;
+        const bool in = w < words;
+        c[i] = in ? __ldg(cr + w) : 0u;
+        s[i] = in ? bf2f(__ldg(sr + w / 16)) : 0.f;  // 16 words per group
+        z[i] = in ? bf2f(__ldg(zr + w / 16)) : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < kDqWords; ++i) {
+        float f[8];
+        // nibbles i and i + 4 hold elements 2i and 2i + 1
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          f[2 * j] = ((float)((c[i] >> (4 * j)) & 0xF) - z[i]) * s[i];
+          f[2 * j + 1] = ((float)((c[i] >> (4 * j + 16)) & 0xF) - z[i]) * s[i];
+        }
+        if (w0 + i * kDqThreads < words)
+          *reinterpret_cast<uint4*>(o + (long long)(w0 + i * kDqThreads) * 8) =
+              make_uint4(pack_bf2(f[0], f[1]), pack_bf2(f[2], f[3]), pack_bf2(f[4], f[5]), pack_bf2(f[6], f[7]));
       }
     }
-    *reinterpret_cast<uint4*>(out + e0) =
-        make_uint4(pack_bf2(f[0], f[1]), pack_bf2(f[2], f[3]), pack_bf2(f[4], f[5]), pack_bf2(f[6], f[7]));
   }
 }
 
@@ -370,17 +468,7 @@ size_t gemm_tc_ws_bytes(int wquant, int N, int K) {
 
 bool gemm_tc_ok(int M, int N, int K) { return M > 64 && K % 8 == 0 && N >= 1 && encode_fn() != nullptr; }
 
-template <int EPI, bool SCALE>
-static cudaError_t launch_tc_t(const CUtensorMap& mx, const CUtensorMap& mw, int M, int N, int K,
-                               const uint16_t* scales, long long up_off, const uint16_t* R, void* Y, int ldy,
-                               int32_t* err, cudaStream_t s) {
-  auto kern = gemm_tc_kernel<EPI, SCALE>;
-  const size_t smem = (size_t)kTcStages * kTcStageBytes + 1024;
-  static std::atomic<unsigned long long> attr{0};
-  FP_CUDA_TRY(smem_limit_once(kern, (int)smem, &attr));
-  const int Nout = EPI == FP_EPI_SWIGLU ? N / 2 : N;
-  const int bn = kTcBN / (EPI == FP_EPI_SWIGLU ? 2 : 1);
-  const long long tiles = (long long)((Nout + bn - 1) / bn) * ((M + kTcBM - 1) / kTcBM);
+static int tc_sms() {
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -388,9 +476,52 @@ static cudaError_t launch_tc_t(const CUtensorMap& mx, const CUtensorMap& mw, int
         sms <= 0)
       sms = 152;
   }
+  return sms;
+}
+
+static long long tc_tiles(int epi, int M, int N, int cg) {
+  const int nout = epi == FP_EPI_SWIGLU ? N / 2 : N, bn = kTcBN / (epi == FP_EPI_SWIGLU ? 2 : 1);
+  return (long long)((nout + bn - 1) / bn) * ((M + cg * kTcBM - 1) / (cg * kTcBM));
+}
+
+// A pair works through its 256 x 256 tile in 0.92 of the time that a CTA takes for
+// its 128 x 256 (8192^3: 669 against 727 us; half of the weight rows' copies and
+// reads leave shared memory, whose bandwidth bounds the single CTA), so it is taken
+// unless its coarser tiles cost more rounds than that saves.
+static bool tc_pair(int epi, int M, int N) {
+  const long long sms = tc_sms(), t1 = tc_tiles(epi, M, N, 1), t2 = tc_tiles(epi, M, N, 2);
+  return (t2 + sms / 2 - 1) / (sms / 2) * 92 <= (t1 + sms - 1) / sms * 100;
+}
+
+template <int EPI, bool SCALE>
+static cudaError_t launch_tc_t(const CUtensorMap& mx, const CUtensorMap& mw, int M, int N, int K,
+                               const uint16_t* scales, long long up_off, const uint16_t* R, void* Y, int ldy,
+                               int32_t* err, cudaStream_t s) {
   // persistent: one CTA per SM (its shared ring and 512 TMEM columns fill the SM)
-  const dim3 grid((unsigned)std::min<long long>(tiles, sms));
-  return launch(kern, grid, dim3(kTcThreads), smem, s, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err);
+  if (tc_pair(EPI, M, N)) {
+    auto kern = gemm_tc_kernel<EPI, SCALE, true>;
+    static std::atomic<unsigned long long> attr{0};
+    FP_CUDA_TRY(smem_limit_once(kern, TcGeom<true>::kSmem, &attr));
+    const long long pairs = std::min<long long>(tc_tiles(EPI, M, N, 2), tc_sms() / 2);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * pairs));
+    cfg.blockDim = dim3(kTcThreads);
+    cfg.dynamicSmemBytes = TcGeom<true>::kSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = g_pdl ? 1 : 0;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 2, at[1].val.clusterDim.y = 1, at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err);
+  }
+  auto kern = gemm_tc_kernel<EPI, SCALE, false>;
+  static std::atomic<unsigned long long> attr{0};
+  FP_CUDA_TRY(smem_limit_once(kern, TcGeom<false>::kSmem, &attr));
+  return launch(kern, dim3((unsigned)std::min<long long>(tc_tiles(EPI, M, N, 1), tc_sms())), dim3(kTcThreads),
+                (size_t)TcGeom<false>::kSmem, s, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err);
 }
 
 template <int EPI>
@@ -412,16 +543,14 @@ static cudaError_t launch_tc_any(int epi, bool sc, const CUtensorMap& mx, const 
   }
 }
 
-// Expand rows [r0, r0 + rows) of a quantised matrix into out [rows][K] bf16.
-static cudaError_t dequant_rows(int wquant, const void* codes, const uint16_t* scales, const uint16_t* zeros, long long r0,
-                                int rows, int K, uint16_t* out, const int32_t* inv, cudaStream_t s) {
-  const bool grouped = wquant == FP_W_INT4_G128 || wquant == FP_W_GPTQ4;
-  const uint8_t* c = (const uint8_t*)codes + (wquant == FP_W_INT8 ? r0 * K : r0 * (K / 2));
-  const uint16_t* sc = grouped ? scales + r0 * (K / 128) : scales;
-  const uint16_t* ze = grouped ? zeros + r0 * (K / 128) : zeros;
-  const long long words = (long long)rows * K / 8;
-  const int blocks = (int)std::min<long long>((words + 255) / 256, 152 * 16);
-  return launch(dequant_kernel, dim3(blocks), dim3(256), 0, s, wquant, (const void*)c, sc, ze, rows, K, out, inv);
+// Expands a band into out [nr * cols][K] bf16: rows c0 .. of the matrix and, with
+// SwiGLU (nr 2), rows Nout + c0 .. behind them.
+template <int WQ>
+static cudaError_t dequant_band(const void* codes, const uint16_t* scales, const uint16_t* zeros, int nr, int Nout, int c0,
+                                int cols, int K, uint16_t* out, const int32_t* inv, cudaStream_t s) {
+  const int per = kDqThreads * kDqWords * 8;  // elements of a row per block
+  return launch(dequant_kernel<WQ>, dim3((K + per - 1) / per, std::min(nr * cols, 65535)), dim3(kDqThreads), 0, s, codes,
+                scales, zeros, (long long)c0, (long long)Nout + c0, cols, nr * cols, K, out, inv);
 }
 
 cudaError_t launch_gemm_tc(int wquant, int epi, const uint16_t* x, int M, int N, int K, const void* codes,
@@ -429,12 +558,13 @@ cudaError_t launch_gemm_tc(int wquant, int epi, const uint16_t* x, int M, int N,
                            void* ws, size_t ws_bytes, int32_t* err, cudaStream_t s, const int32_t* inv) {
   const int nr = epi == FP_EPI_SWIGLU ? 2 : 1;
   const int Nout = nr == 2 ? N / 2 : N;
-  const int wbox = epi == FP_EPI_SWIGLU ? 128 : 256;
+  // rows of a weight box, per band: half a tile where a pair shares it or the gate and the up rows do
+  auto wbox = [&](int n) { return epi == FP_EPI_SWIGLU || tc_pair(epi, M, n) ? 128 : 256; };
   const bool sc = wquant == FP_W_INT8;
   CUtensorMap mx, mw;
   if (!make_map(&mx, x, M, K, kTcBM)) return cudaErrorInvalidValue;
   if (wquant == FP_W_BF16) {
-    if (!make_map(&mw, codes, N, K, wbox)) return cudaErrorInvalidValue;
+    if (!make_map(&mw, codes, N, K, wbox(N))) return cudaErrorInvalidValue;
     return launch_tc_any(epi, sc, mx, mw, M, N, K, scales, Nout, residual, y, Nout, err, s);
   }
   if (!ws || ws_bytes < gemm_tc_ws_bytes(wquant, N, K)) return cudaErrorInvalidValue;
@@ -444,13 +574,25 @@ cudaError_t launch_gemm_tc(int wquant, int epi, const uint16_t* x, int M, int N,
   const int band = band_cols(epi, N, K);
   for (int c0 = 0; c0 < Nout; c0 += band) {
     const int cols = std::min(band, Nout - c0);
-    FP_CUDA_TRY(dequant_rows(wquant, codes, scales, zeros, c0, cols, K, w, inv, s));
-    if (nr == 2)
-      FP_CUDA_TRY(dequant_rows(wquant, codes, scales, zeros, (long long)Nout + c0, cols, K, w + (size_t)cols * K, inv, s));
-    if (!make_map(&mw, w, (long long)nr * cols, K, wbox)) return cudaErrorInvalidValue;
+    switch (wquant) {
+      case FP_W_INT8:
+        FP_CUDA_TRY(dequant_band<FP_W_INT8>(codes, scales, zeros, nr, Nout, c0, cols, K, w, inv, s));
+        break;
+      case FP_W_GPTQ4:
+        FP_CUDA_TRY(dequant_band<FP_W_GPTQ4>(codes, scales, zeros, nr, Nout, c0, cols, K, w, inv, s));
+        break;
+      default:
+        FP_CUDA_TRY(dequant_band<FP_W_INT4_G128>(codes, scales, zeros, nr, Nout, c0, cols, K, w, inv, s));
+    }
+    if (!make_map(&mw, w, (long long)nr * cols, K, wbox(nr * cols))) return cudaErrorInvalidValue;
     const uint16_t* r = residual ? residual + c0 : nullptr;
     void* yb = epi == FP_EPI_F32 ? (void*)((float*)y + c0) : (void*)((uint16_t*)y + c0);
-    FP_CUDA_TRY(launch_tc_any(epi, sc, mx, mw, M, nr * cols, K, sc ? scales + c0 : scales, Nout, r, yb, Nout, err, s));
+    const bool was = g_pdl;
+    g_pdl = true;  // the GEMM's set-up overlaps the expansion
+    const cudaError_t e =
+        launch_tc_any(epi, sc, mx, mw, M, nr * cols, K, sc ? scales + c0 : scales, Nout, r, yb, Nout, err, s);
+    g_pdl = was;
+    FP_CUDA_TRY(e);
   }
   return cudaSuccess;
 }

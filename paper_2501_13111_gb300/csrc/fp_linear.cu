@@ -13,7 +13,9 @@
 //    per 128-group, s (acc - (1024 + z) sum x)), so the weights enter exactly.
 //    The (row block, K step) work is cut into equal contiguous ranges, one
 //    per resident CTA; a row block shared by several CTAs is finished by the
-//    last of them from fp32 partials (no spinning).
+//    last of them from fp32 partials (no spinning).  Smaller matrices give a
+//    cluster of CTAs to each row block instead, summed through distributed
+//    shared memory.
 //  * gemv_kernel (fallback: larger M or a K that is not a multiple of the
 //    MMA super-step): CUDA cores, one warp per output row.
 #include <algorithm>
@@ -214,6 +216,7 @@ struct MmaFmt<FP_W_INT8> { static constexpr int KT = 16; };
 template <>
 struct MmaFmt<FP_W_INT4_G128> { static constexpr int KT = 32; };
 
+constexpr int kGemvMaxCluster = 8;  // CTAs that share a row block through distributed shared memory
 constexpr int kGemvWarps = 8;  // warps per CTA; each owns one 16-row tile (two for SwiGLU: gate and up)
 
 // 16-byte asynchronous global -> shared copy (L2 only), and its group fences.
@@ -313,7 +316,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32) gemv_mma_kernel(const uint16_
                                                        const void* __restrict__ codes,
                                                        const uint16_t* __restrict__ scales,
                                                        const uint16_t* __restrict__ zeros, const uint16_t* R,
-                                                       void* Y, long long total, int S, int W,
+                                                       void* Y, long long total, int S, int W, int cl,
                                                        float* __restrict__ ws, unsigned* __restrict__ counters,
                                                        int32_t* err) {
   constexpr int KT = MmaFmt<WQ>::KT, SUP = 4 * KT, KS = KT / 4, CH = KT / 8;
@@ -328,7 +331,10 @@ __global__ void __launch_bounds__(kGemvWarps * 32) gemv_mma_kernel(const uint16_
   const int Nout = NR == 2 ? N / 2 : N;
   const int groups = K / 128;
   const long long C = gridDim.x, c = blockIdx.x;
-  const long long begin = c * total / C, end = (c + 1) * total / C;
+  // cl > 0: a cluster of cl CTAs per row block, each with a share of its steps
+  const int own = cl ? blockIdx.x / cl : 0, rank = cl ? blockIdx.x % cl : 0;
+  const long long begin = cl ? (long long)own * S + rank * S / cl : c * total / C;
+  const long long end = cl ? (long long)own * S + (rank + 1) * S / cl : (c + 1) * total / C;
   const int L = (int)(end - begin);
 
   uint4* ring = smem;
@@ -526,6 +532,62 @@ __global__ void __launch_bounds__(kGemvWarps * 32) gemv_mma_kernel(const uint16_
     if (cur < seg_end) continue;
 
     // ---- row block b is done for this CTA
+    if (cl) {
+      // sums through distributed shared memory: every CTA leaves its own in its
+      // shared memory (the ring is free), and each finishes a share of the
+      // outputs, adding the CTAs' sums in rank order
+      cp_async_wait<0>();
+      __syncthreads();
+      float* part = reinterpret_cast<float*>(smem);
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int m = nt * 8 + 2 * t + (i & 1);
+            if (m < M) part[(m * NR + r) * ROWS + warp * 16 + g + 8 * (i >> 1)] = acc[r][nt][i];
+          }
+      asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+      const uint32_t p0 = (uint32_t)__cvta_generic_to_shared(part);
+      for (int idx = rank + cl * (int)threadIdx.x; idx < M * (ROWS / 4); idx += cl * (int)blockDim.x) {
+        const int m = idx / (ROWS / 4), lr = (idx % (ROWS / 4)) * 4;
+        float v[NR][4];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) v[r][0] = v[r][1] = v[r][2] = v[r][3] = 0.f;
+        for (int k0 = 0; k0 < cl; k0 += 4) {  // four CTAs' loads in flight
+          float4 a[NR][4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+              a[r][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (k0 + k < cl) {
+                uint32_t p;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                             : "=r"(p)
+                             : "r"(p0 + ((m * NR + r) * ROWS + lr) * 4), "r"(k0 + k));
+                asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                             : "=f"(a[r][k].x), "=f"(a[r][k].y), "=f"(a[r][k].z), "=f"(a[r][k].w)
+                             : "r"(p)
+                             : "memory");
+              }
+            }
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int r = 0; r < NR; ++r) v[r][0] += a[r][k].x, v[r][1] += a[r][k].y, v[r][2] += a[r][k].z, v[r][3] += a[r][k].w;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int row = b * ROWS + lr + e;
+          if (row < Nout) finish(m, row, v[0][e], v[NR - 1][e]);
+        }
+      }
+      // nobody leaves while its sums are being read
+      asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+      return;
+    }
     const long long c0 = gemv_cta_of((long long)b * S, C, total);
     const long long c1 = gemv_cta_of((long long)(b + 1) * S - 1, C, total);
     if (c0 == c1) {
@@ -589,7 +651,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32) gemv_mma_kernel(const uint16_
 
 // ---------------------------------------------------------------- planning
 struct GemvPlan {
-  int NT, ctas, S, W, blocks;
+  int NT, ctas, S, W, blocks, cl;
   long long total;
   size_t smem, ws;
 };
@@ -626,6 +688,29 @@ struct SmemLimits {
   int per_sm;       // usable by CTAs on one SM
   int static_bytes;
 };
+
+// CTAs per row block where a cluster of them sums through distributed shared
+// memory, 0 where the ranges are cut evenly over all CTAs and sums go through
+// global memory and a ticket.  The cluster spares the fence, the ticket and two
+// round trips to L2 (2-3 us), but uses only whole multiples of the row blocks, at
+// most eight CTAs each.  Measured in a graph, us, cluster / even ranges:
+//   int8, 8 tokens   1024 x 512 4.7 / 5.4     4096 x 4096 10.8 / 12.7   12288 x 4096 16.6 / 18.1
+//                    22016 x 4096 (SwiGLU) 23.4 / 26.4   4096 x 11008 18.5 / 19.2 (22 steps a CTA)
+//                    5120 x 13824 24.9 / 23.3 (27)       8192 x 28672 75.5 / 53.5 (56)
+//   bf16, 8 tokens   4096 x 11008 22.7 / 25.7 (43)       8192 x 28672 121 / 93 (112)
+//   two CTAs a block 57344 x 8192 int8 100 / 98
+//   int8, 32 tokens  4096 x 4096 17.1 / 23.1             5120 x 5120 30.3 / 25.1
+// In the forward pass (g_pdl) the next kernel's CTAs start while this one drains,
+// and a cluster has to wait for room for all its CTAs at once, so only matrices
+// below 16 MB take it there: two layers of the 7B shape in int8, 100 steps, 32.5 ms without
+// clusters, 34.2 ms with them everywhere; 2048 x 5504 in int8 (matrices of 4 to
+// 22 MB), 50 steps, 10.5 without / 9.2 ms with; 1024 x 2816 in bf16 8.9 / 6.6 ms.
+static int gemv_cluster(int wq, int blocks, int S, int M, int nr, int ctas, int ring_bytes) {
+  if (M * nr * kGemvWarps * 16 * 4 > ring_bytes) return 0;  // the sums lie where the ring was
+  if (M > 16 && (long long)blocks * S * mma_kt(wq) > (1LL << 24) / (4 * kGemvWarps * 16)) return 0;
+  const int cl = std::min({ctas / blocks, kGemvMaxCluster, S});
+  return cl >= 3 && (S + cl - 1) / cl * nr <= (wq == FP_W_BF16 ? 44 : 24) ? cl : 0;
+}
 
 // occ_max = CTAs per SM the kernel's registers allow.  The plan takes the
 // most CTAs per SM whose shared memory (ring + an x window of at least a
@@ -665,6 +750,7 @@ static GemvPlan plan_gemv(int wq, int epi, int M, int N, int K, int occ_max, con
   }
   if (best_occ == 0) return p;  // ctas == 0: no plan
   p.ctas = (int)std::min<long long>(p.total, (long long)best_occ * sms);
+  p.cl = gemv_cluster(wq, p.blocks, p.S, M, nr, p.ctas, ring);
   p.W = std::min(best_w, p.S);
   p.smem = (size_t)ring + (size_t)p.W * NT * SUP * 16 +
            (size_t)(wq == FP_W_INT4_G128 ? p.W : (wq == FP_W_INT8 ? 1 : 0)) * NT * 8 * 4;
@@ -762,8 +848,25 @@ static cudaError_t launch_mma_t(const uint16_t* x, int M, int N, int K, const vo
   if (!ws || ws_bytes < p.ws || ((uintptr_t)ws & 15)) return cudaErrorInvalidValue;
   unsigned* counters = (unsigned*)ws;
   float* part = (float*)((char*)ws + counter_bytes(p.blocks));
+  constexpr long long kStepBytes = 4 * kGemvWarps * 16 * (EPI == FP_EPI_SWIGLU ? 2 : 1) * 16;  // weights of a step
+  if (p.cl && (!g_pdl || p.total * kStepBytes < (1LL << 24))) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.blocks * p.cl);
+    cfg.blockDim = dim3(kGemvWarps * 32);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = g_pdl ? 1 : 0;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = p.cl, at[1].val.clusterDim.y = 1, at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, gemv_mma_kernel<WQ, NT, EPI>, x, M, N, K, codes, scales, zeros, R, y, p.total, p.S,
+                              p.W, p.cl, part, counters, err);
+  }
   return launch(gemv_mma_kernel<WQ, NT, EPI>, dim3(p.ctas), dim3(kGemvWarps * 32), p.smem, s, x, M, N, K, codes,
-                scales, zeros, R, y, p.total, p.S, p.W, part, counters, err);
+                scales, zeros, R, y, p.total, p.S, p.W, 0, part, counters, err);
 }
 
 template <int WQ, int EPI>

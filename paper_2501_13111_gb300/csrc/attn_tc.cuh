@@ -58,25 +58,24 @@ FP_DEV uint32_t pa_i8h2(uint32_t u, uint32_t sel) {
   return h;
 }
 
-// 32 rows of an output tile (this warp's TMEM lanes, 128 columns from `to` on),
-// times inv, to out (rows from `pos` on, those below S; `ld` elements apart).
-// Through shared memory, four lanes to a row's 64 bytes (16 bytes of 32 rows a
-// store took 5 us a tile); chunk c of row r is staged at c ^ (r / 2 % 4).
-// `read` runs once the last columns have been read.
-template <typename F>
-FP_DEV void pa_write_rows(uint32_t to, float inv, uint8_t* stage, uint16_t* out, long long ld, int pos, int S, F read) {
+// 32 rows of an output tile (this warp's TMEM lanes), COLS columns from x0 on, to out
+// (rows from `pos` on, those below S; `ld` elements apart).  load(x, r) gives
+// columns x .. x + 31 of the thread's row.  Through shared memory, four lanes to a
+// row's 64 bytes (16 bytes of 32 rows a store took 5 us a tile); chunk c of row r
+// is staged at c ^ (r / 2 % 4).
+template <int COLS, typename F>
+FP_DEV void pa_write_rows(F load, int x0, uint8_t* stage, uint16_t* out, long long ld, int pos, int S) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int x0 = 0; x0 < kPaHD; x0 += 32) {
-    uint32_t r[32];
-    tc_ld<32>(to + x0, r);
-    if (x0 + 32 == kPaHD) read();
+  for (int x1 = 0; x1 < COLS; x1 += 32, x0 += 32) {
+    float r[32];
+    load(x0, r);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       uint32_t o[4];
 #pragma unroll
       for (int y = 0; y < 4; ++y)
-        o[y] = pa_pack(__uint_as_float(r[8 * c + 2 * y]) * inv, __uint_as_float(r[8 * c + 2 * y + 1]) * inv);
+        o[y] = pa_pack(r[8 * c + 2 * y], r[8 * c + 2 * y + 1]);
       *reinterpret_cast<uint4*>(stage + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
     }
     __syncwarp();
@@ -88,6 +87,13 @@ FP_DEV void pa_write_rows(uint32_t to, float inv, uint8_t* stage, uint16_t* out,
     }
     __syncwarp();
   }
+}
+
+// 32 columns of an output accumulator in TMEM, times inv.
+FP_DEV void pa_load_out(uint32_t to, float inv, float* r) {
+  tc_ld<32>(to, reinterpret_cast<uint32_t*>(r));
+#pragma unroll
+  for (int y = 0; y < 32; ++y) r[y] *= inv;
 }
 
 // Prompts of at most kPaB tokens (fp_attn_short.cu), from launch_attention_prefill_tc.

@@ -307,9 +307,9 @@ __global__ void __launch_bounds__(KV8 ? 256 : 192, 2)
       // tile serves as the staging buffer
       const float inv = (KV8 ? s_unscale : 1.f) / l;
       const int pos = quad * 32;
-      pa_write_rows(lane_base + kPsO, inv, sQ + quad * kPaStage,
-                    out + ((long long)b * S + pos) * ((long long)H * kPaHD) + (long long)h * kPaHD,
-                    (long long)H * kPaHD, pos, S, [] {});
+      pa_write_rows<kPaHD>([&](int x, float* r) { pa_load_out(lane_base + kPsO + x, inv, r); }, 0, sQ + quad * kPaStage,
+                           out + ((long long)b * S + pos) * ((long long)H * kPaHD) + (long long)h * kPaHD,
+                           (long long)H * kPaHD, pos, S);
     } else if (lane == 0) {
       fail();
     }

@@ -6,8 +6,11 @@
 // attention), for prompts of more than 128 tokens (fp_attn_short.cu takes the
 // shorter ones).  One persistent CTA per SM walks work items of two query tiles
 // of 128 rows that read the same keys and values: two heads of one KV head's
-// group where groups are even, else 256 consecutive rows of a head (single tiles
-// where pairs would leave SMs idle).  Key tiles of 128.
+// group where groups are even, else 256 consecutive rows of a head.  Key tiles of
+// 128.  Where pairs would leave SMs idle or one CTA's share too long, an item is
+// one query tile whose key tiles the two softmax groups take in turn (`split`),
+// each with its own maximum, row sum and accumulator; they are added at the end,
+// half of the columns by each group.
 // Tensor memory holds, for each of the two tiles, its scores (128 columns, P
 // written over them as 16-bit pairs) and its output accumulator (128 columns):
 //   warps 0-3   softmax of tile 0, warps 4-7 of tile 1: one query row (TMEM
@@ -49,7 +52,11 @@
 //   two tiles per CTA                                        333 | 161 | 725
 //   every lane runs the MMA loop (one lane's issue took 144
 //     cycles for an MMA that runs 65)                        297 | 138 | 641
-//   output rows through shared memory, shorter first rounds  283 | 126 | 608
+//   output rows through shared memory, shorter first rounds  284 | 126 | 616
+// A query tile's keys in turn by the two groups, bf16 | int8 cache: 8 heads, 1 x 1024
+// tokens 19.7 | 39.5 us, 1 x 4096 61 | 133, 40 heads, 1 x 1024 27.1 | 52 (one 128-row
+// tile per CTA 20.4 | 49.5, 70 | 211, 31.5 | 71; with two V tiles in the ring, as for
+// pairs, 23.7, 82 and 31.2 with the bf16 cache: V held up the copies of K).
 // Key tiles in halves of 64, so that a tile's own two products overlap its
 // softmax, took 360 us: the waits cost more than they hid.
 // Every mbarrier wait is bounded (error 2 past the limit); a page id out of
@@ -76,7 +83,8 @@ template <bool KV8>
 constexpr int pa_reg_other() { return KV8 ? 96 : 88; }
 constexpr uint32_t kPaTmemCols = 512;
 constexpr uint32_t kPaO = 256;               // O of tile j at kPaO + 128 j, its scores at 128 j
-constexpr int kPaRing = 2;                   // K tiles, V tiles in shared memory
+constexpr int kPaRing = 2;                   // K tiles in shared memory, and V tiles; a shared query
+                                             // tile leaves room for a third V tile
 constexpr int kPaScl = 4;                    // tiles of int8 scales
 constexpr int kPaSmem = (2 + 2 * kPaRing) * kPaTile + 8 * kPaStage + 1024;  // Q, K, V, output, alignment
 constexpr float kPaSlack = 8.f;  // log2 of the largest P allowed before the reference maximum moves
@@ -109,7 +117,8 @@ FP_DEV float2 pa_add2(float2 a, float2 b) {
 
 // How the query tiles are put together into work items (chosen by the host).
 struct PaPlan {
-  int pair;       // 0: one tile an item; 1: the same rows of two heads; 2: 256 rows of a head
+  int pair;       // 0: one query tile an item, its key tiles taken in turn by the two
+                  // softmax groups; 1: the same rows of two heads; 2: 256 rows of a head
   int units;      // items of one (sequence, head or pair of heads)
   int items;
   bool longest_first;
@@ -155,7 +164,8 @@ struct PaItem {
   FP_DEV int key_tiles(int j) const { return j ? nt[1] : nt[0]; }
 };
 
-template <bool KV8>
+// split: the two softmax groups share a query tile (plan.pair == 0)
+template <bool KV8, bool split>
 __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
     attn_prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                            const __grid_constant__ CUtensorMap map_v, const int8_t* __restrict__ k8,
@@ -163,18 +173,20 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
                            const float* __restrict__ v_scale, int S, int H, int Hkv, int page_size,
                            const int32_t* __restrict__ page_table, int pages_per_seq, int n_pages, PaPlan plan,
                            uint16_t* __restrict__ out, int32_t* err) {
+  constexpr int RV = split ? kPaRing + 1 : kPaRing;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ uint64_t qfull, qconv, qempty, kfull[kPaRing], kempty[kPaRing], vfull[kPaRing], vempty[kPaRing], sfull[2],
-      pfull[2], ofull[2], oempty[2], vmet, mma_done;
+  __shared__ uint64_t qfull, qconv, qempty, kfull[kPaRing], kempty[kPaRing], vfull[RV], vempty[RV], sfull[2],
+      pfull[2], ofull[2], oempty[2], vmet, met, mma_done;
   __shared__ float s_vmax[2][kPaWiden];  // int8: the widening warps' largest V scales, by item parity
   __shared__ float s_unscale[4];          // int8: 2^-sigma, removed from the output; by item % 4
+  __shared__ float2 s_ml[2][2][split ? kPaB : 1];  // reference maximum and row sum; by item parity, group
   __shared__ uint32_t tmem_base;
   __shared__ int abort_word;
   __shared__ __align__(16) float s_scl[KV8 ? 2 * kPaScl * kPaB : 4];  // int8: [K, V][tile % 4][key] scales
   volatile int* abort_flag = &abort_word;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sQ = smem;
-  uint8_t* sK = smem + 2 * kPaTile;
+  uint8_t* sK = smem + (split ? 1 : 2) * kPaTile;
   uint8_t* sV = sK + kPaRing * kPaTile;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   auto fail = [&]() {
@@ -191,6 +203,8 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
     for (int i = 0; i < kPaRing; ++i) {
       mbar_init(&kfull[i], KV8 ? kPaWiden : 1);
       mbar_init(&kempty[i], 1);
+    }
+    for (int i = 0; i < RV; ++i) {
       mbar_init(&vfull[i], KV8 ? kPaWiden : 1);
       mbar_init(&vempty[i], 1);
     }
@@ -198,8 +212,9 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
       mbar_init(&sfull[j], 1);
       mbar_init(&pfull[j], 4);
       mbar_init(&ofull[j], 1);
-      mbar_init(&oempty[j], 4);
+      mbar_init(&oempty[j], split ? 8 : 4);
     }
+    mbar_init(&met, 8);
     mbar_init(&mma_done, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -255,11 +270,11 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
         const int nt = w.tiles();
         int row = page_row(0);
         for (int t = 0; t < nt && ok; ++t, ++kn) {
-          const int s = kn % kPaRing, ph = ((kn / kPaRing) & 1) ^ 1;
 #pragma unroll
           for (int v = 0; v < 2 && ok; ++v) {
+            const int ring = v ? RV : kPaRing, s = kn % ring, ph = ((kn / ring) & 1) ^ 1;
             uint64_t* full = v ? &vfull[s] : &kfull[s];
-            if (kn >= kPaRing) ok = mbar_wait(v ? &vempty[s] : &kempty[s], ph);
+            if (kn >= ring) ok = mbar_wait(v ? &vempty[s] : &kempty[s], ph);
             ok = __all_sync(0xffffffffu, ok && !*abort_flag);
             if (!ok) break;
             if (lane == 0) mbar_expect_tx(full, kPaTile);
@@ -279,8 +294,8 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
       if (iss[0] > 0) mbar_wait(&qfull, (iss[0] - 1) & 1);
 #pragma unroll
       for (int v = 0; v < 2; ++v)
-        for (int t = max(0, iss[1 + v] - kPaRing); t < iss[1 + v]; ++t)
-          mbar_wait(v ? &vfull[t % kPaRing] : &kfull[t % kPaRing], (t / kPaRing) & 1);
+        for (int t = max(0, iss[1 + v] - (v ? RV : kPaRing)); t < iss[1 + v]; ++t)
+          mbar_wait(v ? &vfull[t % RV] : &kfull[t % kPaRing], (t / (v ? RV : kPaRing)) & 1);
     }
   } else if (warp == kPaWarpMma) {
     // ---------------- MMA issuer: every lane runs the loop, one issues.
@@ -294,13 +309,20 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
     bool ok = true;
     // descriptor start addresses count 16-byte units
     auto scores = [&](int j, int s) {  // S_j = Q_j K^T of ring tile s (issuing lane only)
-      const uint64_t qj = qd + j * (kPaTile >> 4), ks = kd + s * (kPaTile >> 4);
+      const uint64_t qj = qd + (split ? 0 : j) * (kPaTile >> 4), ks = kd + s * (kPaTile >> 4);
 #pragma unroll
       for (int kk = 0; kk < kPaHD / 16; ++kk) {
         const int off = ((kk >> 2) * kPaHalf + (kk & 3) * 32) >> 4;
         tc_mma(tmem + j * kPaB, qj + off, ks + off, idesc_s, kk > 0 ? 1u : 0u);
       }
       tc_commit(&sfull[j]);
+    };
+    auto values = [&](int j, int s, bool first) {  // O_j (+)= P_j V of ring tile s (issuing lane only)
+      const uint64_t vs = vd + s * (kPaTile >> 4);
+#pragma unroll
+      for (int kk = 0; kk < kPaB / 16; ++kk)  // 16 keys: two 8-row groups of the V tile
+        tc_mma_ts(tmem + kPaO + j * kPaHD, tmem + j * kPaB + kk * 8, vs + kk * (2048 >> 4), idesc_o,
+                  (!first || kk > 0) ? 1u : 0u);
     };
     for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
       const PaItem w(i, S, H, Hkv, plan);
@@ -309,6 +331,50 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
+      if constexpr (split) {
+        // one query tile: key tile t is group t % 2's, scores two tiles ahead
+        if (elect_one()) {
+          scores(0, kn % kPaRing);
+          tc_commit(&kempty[kn % kPaRing]);
+          if (nt == 1) tc_commit(&qempty);
+        }
+        __syncwarp();
+        if (nt > 1) {
+          ok = __all_sync(0xffffffffu, mbar_wait(&kfull[(kn + 1) % kPaRing], ((kn + 1) / kPaRing) & 1));
+          if (!ok) break;
+          if (elect_one()) {
+            scores(1, (kn + 1) % kPaRing);
+            tc_commit(&kempty[(kn + 1) % kPaRing]);
+            if (nt == 2) tc_commit(&qempty);
+          }
+          __syncwarp();
+        }
+        for (int t = 0; t < nt && ok; ++t, ++kn) {
+          const int s = kn % kPaRing, sv = kn % RV, j = t & 1;  // s: of key tiles t and t + 2
+          const int p = j ? pn[1] : pn[0], o = j ? on[1] : on[0];
+          ok = mbar_wait(&vfull[sv], (kn / RV) & 1) &&
+               (t + 2 >= nt || mbar_wait(&kfull[s], ((kn + kPaRing) / kPaRing) & 1)) && mbar_wait(&pfull[j], p & 1) &&
+               (t > 1 || o == 0 || mbar_wait(&oempty[j], (o - 1) & 1)) && !*abort_flag;
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          tc_fence_after();
+          if (elect_one()) {
+            values(j, sv, t < 2);
+            tc_commit(&vempty[sv]);
+            if (t + 2 < nt) {
+              scores(j, s);
+              tc_commit(&kempty[s]);
+            } else {
+              tc_commit(&ofull[j]);
+            }
+            if (t + 3 == nt) tc_commit(&qempty);
+          }
+          __syncwarp();
+          if (j) ++pn[1], on[1] += t + 2 >= nt;
+          else ++pn[0], on[0] += t + 2 >= nt;
+        }
+        continue;
+      }
       if (elect_one()) {
 #pragma unroll
         for (int j = 0; j < 2; ++j)
@@ -332,11 +398,7 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
           ++pn[j];
           tc_fence_after();
           if (elect_one()) {
-            const uint64_t vs = vd + s * (kPaTile >> 4);
-#pragma unroll
-            for (int kk = 0; kk < kPaB / 16; ++kk)  // 16 keys: two 8-row groups of the V tile
-              tc_mma_ts(tmem + kPaO + j * kPaHD, tmem + j * kPaB + kk * 8, vs + kk * (2048 >> 4), idesc_o,
-                        (t > 0 || kk > 0) ? 1u : 0u);
+            values(j, s, t == 0);
             if (t + 1 < w.nt[j]) scores(j, s1);
             else tc_commit(&ofull[j]);
           }
@@ -423,7 +485,6 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&qconv);
       for (int t = 0; t < nt && ok; ++t, ++kn) {
-        const int s = kn % kPaRing, ph = ((kn / kPaRing) & 1) ^ 1;
         int rowi[kPaWRows];  // pool row of each of the thread's keys (< 2^31); -1 reads zeros
 #pragma unroll
         for (int r = 0; r < kPaWRows; ++r) {
@@ -446,12 +507,13 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
 #pragma unroll 1
         for (int which = 0; which < 2; ++which) {
           const int8_t* pool = which ? v8 : k8;
+          const int ring = which ? RV : kPaRing, s = kn % ring, ph = ((kn / ring) & 1) ^ 1;
           uint4 cw[kPaWRows];
           // the codes are read before the wait for the buffer
 #pragma unroll
           for (int r = 0; r < kPaWRows; ++r)
             cw[r] = rowi[r] >= 0 ? ld_nc16(pool + (long long)rowi[r] * kPaHD + c * 16) : make_uint4(0, 0, 0, 0);
-          if (kn >= kPaRing) ok = mbar_wait(which ? &vempty[s] : &kempty[s], ph);
+          if (kn >= ring) ok = mbar_wait(which ? &vempty[s] : &kempty[s], ph);
           if (!__all_sync(0xffffffffu, ok) || __any_sync(0xffffffffu, *abort_flag != 0)) {
             ok = false;
             break;
@@ -496,16 +558,17 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
     const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
     const uint32_t ts = lane_base + j * kPaB, to = lane_base + kPaO + j * kPaHD;
     const float scale = kPaLog2e * rsqrtf((float)kPaHD);
-    int n = 0, kn = 0, sn = 0, on = 0;  // items, key tiles, this tile's scores and outputs
+    const int jq = split ? 0 : j, first = split ? j : 0, stride = split ? 2 : 1;  // query tile; this group's key tiles
+    int n = 0, kn = 0, sn = 0, on = 0;  // items, key tiles, this group's scores and outputs
     bool ok = true;
     for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
       const PaItem w(i, S, H, Hkv, plan);
-      const int nt = w.key_tiles(j), qrow = w.row0(j) + row;  // position in the sequence
+      const int nt = w.key_tiles(jq), qrow = w.row0(jq) + row;  // position in the sequence
       float m = -INFINITY;                            // reference maximum (log2 domain)
       float2 l2[4];                                   // row sum
 #pragma unroll
       for (int y = 0; y < 4; ++y) l2[y] = make_float2(0.f, 0.f);
-      for (int t = 0; t < nt; ++t, ++sn) {
+      for (int t = first; t < nt; t += stride, ++sn) {
         ok = mbar_wait(&sfull[j], sn & 1);
         if (!__all_sync(0xffffffffu, ok)) {
           ok = false;
@@ -546,7 +609,7 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
 #pragma unroll
           for (int y = 0; y < 4; ++y) l2[y] = pa_mul2(l2[y], make_float2(corr, corr));
         }
-        if (t > 0 && __any_sync(0xffffffffu, corr != 1.f)) {
+        if (t > first && __any_sync(0xffffffffu, corr != 1.f)) {
           // O holds P V of the earlier tiles (complete: S(t) was issued after it)
 #pragma unroll 1
           for (int x = 0; x < kPaHD / 16; ++x) {
@@ -589,20 +652,66 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
       if (nt == 0) continue;
       const float l = ((l2[0].x + l2[0].y) + (l2[1].x + l2[1].y)) + ((l2[2].x + l2[2].y) + (l2[3].x + l2[3].y));
       // ---- the item's output
+      const int pos = w.row0(jq) + quad * 32;
+      uint8_t* stage = sV + RV * kPaTile + warp * kPaStage;
+      uint16_t* dst = out + ((long long)w.b * S + pos) * ((long long)H * kPaHD) + (long long)w.head(jq) * kPaHD;
+      const long long ld = (long long)H * kPaHD;
+      // int8 cache: P carried the V scales times 2^sigma
+      if constexpr (split) {
+        // the groups' sums over their key tiles, each with its own reference
+        // maximum, added; each group finishes half of the columns
+        const bool both = nt > 1;
+        s_ml[n & 1][j][row] = make_float2(m, l);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&met);
+        ok = __all_sync(0xffffffffu, mbar_wait(&met, n & 1) && mbar_wait(&ofull[0], n & 1) &&
+                                         (!both || mbar_wait(&ofull[1], on & 1)));
+        if (!ok) break;
+        on += both;
+        tc_fence_after();
+        const float2 ml0 = s_ml[n & 1][0][row], ml1 = s_ml[n & 1][1][row];
+        const float mm = fmaxf(ml0.x, ml1.x);
+        float a0 = 1.f, a1 = 0.f, ls = ml0.y;
+        if (both) {
+          a0 = exp2f(ml0.x - mm), a1 = exp2f(ml1.x - mm);
+          ls = a0 * ml0.y + a1 * ml1.y;
+        }
+        const float inv = (KV8 ? s_unscale[n & 3] : 1.f) / ls;
+        a0 *= inv, a1 *= inv;
+        pa_write_rows<kPaHD / 2>(
+            [&](int x, float* r) {
+              pa_load_out(lane_base + kPaO + x, a0, r);
+              if (both) {
+                uint32_t u[32];
+                tc_ld<32>(lane_base + kPaO + kPaHD + x, u);
+#pragma unroll
+                for (int y = 0; y < 32; ++y) r[y] = fmaf(a1, __uint_as_float(u[y]), r[y]);
+              }
+            },
+            j * (kPaHD / 2), stage, dst, ld, pos, S);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(&oempty[0]);
+          if (both) mbar_arrive(&oempty[1]);
+        }
+        continue;
+      }
       ok = __all_sync(0xffffffffu, mbar_wait(&ofull[j], on & 1));
       if (!ok) break;
       ++on;
       tc_fence_after();
-      // int8 cache: P carried the V scales times 2^sigma
       const float inv = (KV8 ? s_unscale[n & 3] : 1.f) / l;
-      const int pos = w.row0(j) + quad * 32;
-      pa_write_rows(to, inv, sV + kPaRing * kPaTile + warp * kPaStage,
-                    out + ((long long)w.b * S + pos) * ((long long)H * kPaHD) + (long long)w.head(j) * kPaHD,
-                    (long long)H * kPaHD, pos, S, [&]() {
-                      tc_fence_before();
-                      __syncwarp();
-                      if (lane == 0) mbar_arrive(&oempty[j]);
-                    });
+      pa_write_rows<kPaHD>(
+          [&](int x, float* r) {
+            pa_load_out(to + x, inv, r);
+            if (x + 32 == kPaHD) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&oempty[j]);
+            }
+          },
+          0, stage, dst, ld, pos, S);
     }
     if (!ok && lane == 0) fail();
   }
@@ -623,11 +732,10 @@ bool attention_prefill_tc_ok(int B, int S, int n_heads, const fp_kv_view& kv, co
          (long long)B * n_heads * ((S + kPaB - 1) / kPaB) < (1LL << 26) && tensor_maps_available();
 }
 
-// Pairs of tiles where they keep the SMs busy, single tiles where pairs would
-// leave SMs idle or make one CTA's share too long: the smaller of the two
-// makespans (the mean share of an SM, or the longest item), with a key tile at
-// 4100 cycles for a pair and 3000 for one tile, and 3500 cycles an item
-// (measured, bf16 cache).
+// Pairs of tiles where they keep the SMs busy, else single tiles with their keys cut
+// in two: the smaller of the two makespans (the mean share of an SM, or the longest
+// item), with 4100 cycles for a step of two tiles' products and 3500 an item, 4000
+// with the two groups' sums added (measured, bf16 cache).
 static PaPlan pa_plan(int B, int S, int H, int G, int sms) {
   const long long tiles = (S + kPaB - 1) / kPaB;
   const int pair = G % 2 == 0 ? 1 : 2;
@@ -640,21 +748,31 @@ static PaPlan pa_plan(int B, int S, int H, int G, int sms) {
     return p;
   };
   auto span = [&](const PaPlan& p) {
-    const double step = p.pair ? 4100 : 3000, longest = tiles * step + 3500;
-    double sum = 0;  // key tiles of a head's items
-    for (long long u = 0; u < p.units; ++u) sum += (double)std::min(tiles, p.pair == 2 ? 2 * u + 2 : u + 1);
-    const double heads = (double)p.items / p.units;
-    return std::max((sum * step + 3500.0 * p.units) * heads / sms, longest);
+    const double step = 4100, item = p.pair ? 3500 : 4000;
+    double sum = 0;  // steps of a head's items
+    for (long long u = 0; u < p.units; ++u)
+      sum += (double)(p.pair == 2 ? std::min(tiles, 2 * u + 2) : p.pair == 1 ? u + 1 : u / 2 + 1);
+    const double heads = (double)p.items / p.units, longest = (double)(p.pair ? tiles : (tiles + 1) / 2) * step + item;
+    return std::max((sum * step + item * p.units) * heads / sms, longest);
   };
   const PaPlan two = make(pair), one = make(0);
   return span(one) < span(two) ? one : two;
 }
 
+template <bool KV8, bool SPLIT>
+static cudaError_t launch_pa_plan(const PaPlan& plan, int ctas, const CUtensorMap& mq, const CUtensorMap& mk,
+                                  const CUtensorMap& mv, int S, int n_heads, const fp_kv_view& kv, uint16_t* out,
+                                  int32_t* err, cudaStream_t s) {
+  static std::atomic<unsigned long long> attr{0};
+  FP_CUDA_TRY(smem_limit_once(attn_prefill_tc_kernel<KV8, SPLIT>, kPaSmem, &attr));
+  return launch(attn_prefill_tc_kernel<KV8, SPLIT>, dim3(ctas), dim3(pa_threads<KV8>()), (size_t)kPaSmem, s, mq, mk, mv,
+                (const int8_t*)kv.k_pool, (const int8_t*)kv.v_pool, (const float*)kv.k_scale, (const float*)kv.v_scale,
+                S, n_heads, kv.n_kv_heads, kv.page_size, kv.page_table, kv.pages_per_seq, kv.n_pages, plan, out, err);
+}
+
 template <bool KV8>
 static cudaError_t launch_pa_tc(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, int B, int S,
                                 int n_heads, const fp_kv_view& kv, uint16_t* out, int32_t* err, cudaStream_t s) {
-  static std::atomic<unsigned long long> attr{0};
-  FP_CUDA_TRY(smem_limit_once(attn_prefill_tc_kernel<KV8>, kPaSmem, &attr));
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -663,10 +781,9 @@ static cudaError_t launch_pa_tc(const CUtensorMap& mq, const CUtensorMap& mk, co
       sms = 152;
   }
   const PaPlan plan = pa_plan(B, S, n_heads, n_heads / kv.n_kv_heads, sms);
-  return launch(attn_prefill_tc_kernel<KV8>, dim3(std::min(plan.items, sms)), dim3(pa_threads<KV8>()), (size_t)kPaSmem,
-                s, mq, mk, mv, (const int8_t*)kv.k_pool, (const int8_t*)kv.v_pool, (const float*)kv.k_scale,
-                (const float*)kv.v_scale, S, n_heads, kv.n_kv_heads, kv.page_size, kv.page_table, kv.pages_per_seq,
-                kv.n_pages, plan, out, err);
+  const int ctas = std::min(plan.items, sms);
+  return plan.pair ? launch_pa_plan<KV8, false>(plan, ctas, mq, mk, mv, S, n_heads, kv, out, err, s)
+                   : launch_pa_plan<KV8, true>(plan, ctas, mq, mk, mv, S, n_heads, kv, out, err, s);
 }
 
 cudaError_t launch_attention_prefill_tc(const uint16_t* q, int q_stride, int B, int S, int n_heads,

@@ -1,6 +1,6 @@
 """Prefill attention where its work items can go wrong: prompts around one and two
 tiles of 128 rows, KV groups of even and odd size (pairs of heads, pairs of row
-tiles, single tiles), few items and many (the two orders), both caches."""
+tiles, single tiles with their keys cut in two), few items and many (the two orders), both caches."""
 import numpy as np
 import pytest
 
@@ -25,7 +25,8 @@ def fp():
 @pytest.mark.parametrize("B,H,Hkv,S", [
     (2, 3, 3, 128), (2, 3, 3, 129), (1, 3, 1, 256), (2, 3, 1, 257), (1, 6, 6, 385),  # odd groups, ragged second tiles
     (2, 4, 2, 128), (3, 4, 2, 255), (1, 8, 2, 641),                                   # pairs of heads
-    (20, 16, 16, 300), (41, 32, 4, 129)])                                             # more items than four rounds of SMs
+    (20, 16, 16, 300), (41, 32, 4, 129),                                              # more items than four rounds of SMs
+    (1, 8, 2, 300), (1, 2, 2, 1153), (1, 40, 40, 520), (3, 8, 8, 1024)])              # a query tile's keys cut in two
 def test_work_items(fp, kvq, B, H, Hkv, S):
     hd = 128
     c = Cache(fp, kvq, B, S + 7, Hkv, hd, seed=S + H + kvq)

@@ -311,7 +311,10 @@ __host__ __device__ constexpr int gemv_stages(int tiles) { return tiles >= 2 ? 3
 // (deterministic) and runs the epilogue.
 FP_DEV long long gemv_cta_of(long long i, long long C, long long total) { return ((i + 1) * C - 1) / total; }
 
-template <int WQ, int NT, int EPI>
+// CL: a cluster of cl CTAs per row block, each with a share of its steps.  (An
+// instance of its own: the code beside the even ranges changed their registers and
+// cost 4096 x 11008 in bf16 at 17 tokens 2 us.)
+template <int WQ, int NT, int EPI, bool CL>
 __global__ void __launch_bounds__(kGemvWarps * 32) gemv_mma_kernel(const uint16_t* __restrict__ X, int M, int N, int K,
                                                        const void* __restrict__ codes,
                                                        const uint16_t* __restrict__ scales,
@@ -331,10 +334,9 @@ __global__ void __launch_bounds__(kGemvWarps * 32) gemv_mma_kernel(const uint16_
   const int Nout = NR == 2 ? N / 2 : N;
   const int groups = K / 128;
   const long long C = gridDim.x, c = blockIdx.x;
-  // cl > 0: a cluster of cl CTAs per row block, each with a share of its steps
-  const int own = cl ? blockIdx.x / cl : 0, rank = cl ? blockIdx.x % cl : 0;
-  const long long begin = cl ? (long long)own * S + rank * S / cl : c * total / C;
-  const long long end = cl ? (long long)own * S + (rank + 1) * S / cl : (c + 1) * total / C;
+  const int own = CL ? blockIdx.x / cl : 0, rank = CL ? blockIdx.x % cl : 0;
+  const long long begin = CL ? (long long)own * S + rank * S / cl : c * total / C;
+  const long long end = CL ? (long long)own * S + (rank + 1) * S / cl : (c + 1) * total / C;
   const int L = (int)(end - begin);
 
   uint4* ring = smem;
@@ -532,7 +534,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32) gemv_mma_kernel(const uint16_
     if (cur < seg_end) continue;
 
     // ---- row block b is done for this CTA
-    if (cl) {
+    if constexpr (CL) {
       // sums through distributed shared memory: every CTA leaves its own in its
       // shared memory (the ring is free), and each finishes a share of the
       // outputs, adding the CTAs' sums in rank order
@@ -787,13 +789,14 @@ static int gemv_occupancy(SmemLimits* lim) {
   static int occ = 0;
   static SmemLimits l{};
   if (!occ) {
-    auto kern = gemv_mma_kernel<WQ, NT, EPI>;
+    auto kern = gemv_mma_kernel<WQ, NT, EPI, false>;
     cudaFuncAttributes fa{};
     int st = cudaFuncGetAttributes(&fa, kern) == cudaSuccess ? (int)fa.sharedSizeBytes : 64;
     l.static_bytes = st;
     l.per_cta_dyn = max_smem_optin() - st;
     l.per_sm = smem_per_sm();
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, l.per_cta_dyn);
+    cudaFuncSetAttribute(gemv_mma_kernel<WQ, NT, EPI, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, l.per_cta_dyn);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kGemvWarps * 32, 0) != cudaSuccess || occ <= 0)
       occ = 2;
     (void)cudaGetLastError();
@@ -862,10 +865,10 @@ static cudaError_t launch_mma_t(const uint16_t* x, int M, int N, int K, const vo
     at[1].val.clusterDim.x = p.cl, at[1].val.clusterDim.y = 1, at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemv_mma_kernel<WQ, NT, EPI>, x, M, N, K, codes, scales, zeros, R, y, p.total, p.S,
-                              p.W, p.cl, part, counters, err);
+    return cudaLaunchKernelEx(&cfg, gemv_mma_kernel<WQ, NT, EPI, true>, x, M, N, K, codes, scales, zeros, R, y, p.total,
+                              p.S, p.W, p.cl, part, counters, err);
   }
-  return launch(gemv_mma_kernel<WQ, NT, EPI>, dim3(p.ctas), dim3(kGemvWarps * 32), p.smem, s, x, M, N, K, codes,
+  return launch(gemv_mma_kernel<WQ, NT, EPI, false>, dim3(p.ctas), dim3(kGemvWarps * 32), p.smem, s, x, M, N, K, codes,
                 scales, zeros, R, y, p.total, p.S, p.W, 0, part, counters, err);
 }
 

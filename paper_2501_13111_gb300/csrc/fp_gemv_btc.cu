@@ -242,30 +242,17 @@ __global__ void __launch_bounds__(kBtThreads, 1)
       t = __shfl_sync(0xffffffffu, t, 0);
       if (t != (unsigned)(c1 - c0)) continue;
       __threadfence();
-      // the sum over the CTAs in CTA order (deterministic), eight tokens' loads
-      // in flight per CTA rather than one
       const int cnt = (int)(c1 - c0) + 1;
       const float* p0 = ws + (size_t)(b + c0) * slot + lr;
+      constexpr int TB = NR == 2 ? 8 : 16;  // tokens summed together
+#pragma unroll 1
+      for (int i0 = 0; i0 < M; i0 += TB) {
+        float v[TB], u[TB], rv[TB];
 #pragma unroll
-      for (int i0 = 0; i0 < MT; i0 += 8) {
-        if (i0 >= M) break;
-        float v[8], u[8], rv[8];
+        for (int i = 0; i < TB; ++i) v[i] = u[i] = 0.f, rv[i] = resid(i0 + i);
+        sum_partials<TB, NR, kBtRows, 4>(p0 + (size_t)i0 * NR * kBtRows, slot, cnt, M - i0, v, u);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = u[i] = 0.f, rv[i] = resid(i0 + i);
-        for (int cc = 0; cc < cnt; ++cc) {
-          const float* pc = p0 + (size_t)cc * slot;
-          float t[8], t2[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const bool in = i0 + i < M;
-            t[i] = in ? __ldcg(pc + (size_t)(i0 + i) * NR * kBtRows) : 0.f;
-            t2[i] = (NR == 2 && in) ? __ldcg(pc + (size_t)(i0 + i) * NR * kBtRows + kBtRows) : 0.f;
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) v[i] += t[i], u[i] += t2[i];
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < TB; ++i)
           if (i0 + i < M && row < Nout) finish(i0 + i, v[i], u[i], rv[i]);
       }
       if (lane == 0) counters[b * 4 + ew] = 0u;

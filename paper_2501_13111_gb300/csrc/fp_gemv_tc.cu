@@ -493,27 +493,14 @@ __global__ void __launch_bounds__(kQ4Threads, 1)
       t = __shfl_sync(0xffffffffu, t, 0);
       if (t != (unsigned)(c1 - c0)) continue;
       __threadfence();
-      // the sum over the CTAs in CTA order (deterministic), eight tokens' loads
-      // in flight per CTA rather than one
       const int cnt = (int)(c1 - c0) + 1;
       const float* p0 = ws + (size_t)(b + c0) * slot + (size_t)m0 * NR * kQ4Rows + lr;
-#pragma unroll
+#pragma unroll 1
       for (int i0 = 0; i0 < MQ; i0 += 8) {
         float v[8], u[8], rv[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = u[i] = 0.f, rv[i] = resid(m0 + i0 + i);
-        for (int cc = 0; cc < cnt; ++cc) {
-          const float* pc = p0 + (size_t)cc * slot;
-          float t[8], t2[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const bool in = m0 + i0 + i < M;
-            t[i] = in ? __ldcg(pc + (size_t)(i0 + i) * NR * kQ4Rows) : 0.f;
-            t2[i] = (NR == 2 && in) ? __ldcg(pc + (size_t)(i0 + i) * NR * kQ4Rows + kQ4Rows) : 0.f;
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) v[i] += t[i], u[i] += t2[i];
-        }
+        sum_partials<8, NR, kQ4Rows, NR == 2 ? 1 : 2>(p0 + (size_t)i0 * NR * kQ4Rows, slot, cnt, M - m0 - i0, v, u);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
           if (m0 + i0 + i < M && row < Nout) finish(m0 + i0 + i, v[i], u[i], rv[i]);

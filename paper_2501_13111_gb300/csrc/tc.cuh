@@ -326,4 +326,31 @@ bool make_tensor_map(CUtensorMap* map, const void* base, long long rows, long lo
                      int box_rows, int box_cols, int swizzle_bytes);
 bool tensor_maps_available();
 
+// The sums of a row tile that several CTAs share: v[i] += sum over CTAs of the
+// partials of token i at p0 + CTA * slot + i * NR * ROWS (u: the second row set of
+// SwiGLU), in CTA order, for the first `m` of TB tokens.  The loads of UC CTAs are in
+// flight together: one CTA after another, a tile shared by five waited out an L2
+// latency five times per eight tokens.
+template <int TB, int NR, int ROWS, int UC>
+FP_DEV void sum_partials(const float* p0, size_t slot, int cnt, int m, float* v, float* u) {
+#pragma unroll 1
+  for (int cc = 0; cc < cnt; cc += UC) {
+    float t[NR][UC][TB];
+#pragma unroll
+    for (int k = 0; k < UC; ++k)
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+#pragma unroll
+        for (int i = 0; i < TB; ++i)
+          t[r][k][i] = cc + k < cnt && i < m ? __ldcg(p0 + (size_t)(cc + k) * slot + (size_t)(i * NR + r) * ROWS) : 0.f;
+#pragma unroll
+    for (int k = 0; k < UC; ++k)
+#pragma unroll
+      for (int i = 0; i < TB; ++i) {
+        v[i] += t[0][k][i];
+        if (NR == 2) u[i] += t[NR - 1][k][i];
+      }
+  }
+}
+
 }  // namespace fpk

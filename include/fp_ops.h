@@ -160,7 +160,8 @@ int fp_op_rope_kv(uint16_t* qkv, int B, int S, int row_stride, int n_heads, cons
  * at h*head_dim), attends over positions 0 .. len[b]-1 of the cache
  * (softmax(q K^T / sqrt(hd)) V, query head j reads KV head j / (H/Hkv));
  * out bf16 [B][n_heads*head_dim].  Split over the context in chunks; the
- * partial results go to `workspace` (fp_op_attention_decode_workspace_bytes
+ * partial results stay in the shared memory of a cluster of CTAs or, past
+ * eight splits, go to `workspace` (fp_op_attention_decode_workspace_bytes
  * for at most max_len cached positions) and a second kernel combines them.
  * len[b] in [1, max_len]; a larger len[b] is clipped to max_len and sets
  * *err = 1 (err may be NULL). */
@@ -173,8 +174,8 @@ size_t fp_op_attention_decode_workspace_bytes(int B, int n_heads, int head_dim, 
  * heads of head_dim, a kvquant cache of 16-token pages with 16-byte aligned
  * pools, and max_len cached positions (0 for a non-positive argument).  With
  * 1 split the kernel normalises in place and never touches the workspace;
- * with more, the partials go to the workspace and a second kernel merges
- * them. */
+ * with more, the CTAs of a cluster merge their partials or the partials go to
+ * the workspace and a second kernel merges them. */
 int fp_op_attention_decode_splits(int B, int n_kv_heads, int head_dim, int kvquant, int max_len);
 
 /* Decode attention without a caller workspace, for callers that cannot

@@ -30,9 +30,11 @@ static constexpr float kLog2e = 1.4426950408889634f;
 // score fragments.  bf16 caches enter as they are (P in bf16); int8 codes
 // are widened exactly to fp16 in shared memory (P in fp16) and their
 // per-token scales applied in fp32 to the scores (K) and to P (V).  The 4
-// warps are merged at the end; a second kernel merges the context splits.
+// warps are merged at the end; the context splits by the cluster that their CTAs
+// form (dec_cluster), or by a second kernel.
 // =====================================================================
 constexpr int kDecTT = 64;  // tokens per tile
+constexpr int kDecMaxCluster = 8;  // CTAs that share a (sequence, KV head) through distributed shared memory
 
 // Ring depth: 3 tiles (two in flight, 2 CTAs per SM with the bf16 cache) when
 // the (sequence, KV head) pairs leave SMs with room, else 2 tiles (one in
@@ -42,6 +44,7 @@ struct DecodeGeom {
   int chunk;   // positions per split (multiple of kDecTT)
   int splits;  // ceil(max_len / chunk)
   int nb;      // ring depth
+  int cl;      // CTAs of a cluster that shares a (sequence, KV head); 0: no clusters
 };
 
 static int dec_sm_count() {
@@ -77,16 +80,35 @@ static int dec_max_splits(long long pairs, int tiles) {
   return (int)std::max<long long>(std::max<long long>(s, 1), dec_min_splits(tiles));
 }
 
-// occ > 0: CTAs per SM of the kernel the geometry is for (the int8 page-streaming
-// kernel: 4); occ 0: the mma.sync tile kernel, whose ring depth sets it.
-static DecodeGeom decode_geom(int B, int n_kv_heads, int max_len, int occ = 0) {
+// CTAs of the cluster that shares a (sequence, KV head), 0 for splits through the
+// workspace.  Eight CTAs take the place of more splits while that leaves each few
+// tiles: 8 with the int8 page-streaming kernel, 5 with the tile kernel.  That kernel's
+// splits fill the SMs, and clusters of other than two or four CTAs pack badly into
+// the SMs that share a cluster, so they need a quarter of the slots to spare.
+// Cold cache, us, cluster / splits and combine:
+//   int8   1 x 4000, 8 KV heads 17.5 / 21.6   5 x 1500, 2 KV heads 14.8 / 19.7
+//          3 x 228, 8 KV heads 13.3 / 15.5    8 x 3000, 8 KV heads 21.4 / 23.7
+//   bf16   1 x 612, 32 KV heads 13.5 / 15.5   3 x 2000, 24 KV heads 25.1 / 28.3
+//          1 x 4000, 8 KV heads (8 tiles each) 23.7 / 21.8
+//          12 x 700, 4 KV heads (clusters of six, 288 of 304 slots) 25.3 / 19.6
+static int dec_cluster(long long pairs, int splits, int tiles, long long slots, bool i8) {
+  const int cl = std::min(splits, kDecMaxCluster);
+  if (splits < 2 || (splits > cl && tiles > cl * (i8 ? 8 : 5))) return 0;
+  if (!i8 && cl != 2 && cl != 4 && pairs * cl > slots * 3 / 4) return 0;
+  return cl;
+}
+
+// Splits of up to eight CTAs are a cluster, whose CTAs add their sums through
+// distributed shared memory instead of the workspace and a second kernel, and which
+// cuts each sequence's own length evenly (dec_cluster).
+static DecodeGeom decode_geom(int B, int n_kv_heads, int max_len, bool i8 = false) {
   const long long pairs = (long long)B * n_kv_heads;
   const int nb = dec_ring_depth(pairs);
-  const long long slots = (long long)dec_sm_count() * (occ > 0 ? occ : dec_occ(nb));
+  const long long slots = (long long)dec_sm_count() * dec_occ(nb);
   const int tiles = std::max(1, (max_len + kDecTT - 1) / kDecTT);
   const int smax = std::min(dec_max_splits(pairs, tiles),
                             (int)std::max<long long>(std::min<long long>(tiles, 4), 2 * slots / std::max(1LL, pairs)));
-  DecodeGeom best{tiles * kDecTT, 1, nb};
+  DecodeGeom best{tiles * kDecTT, 1, nb, 0};
   double best_t = 1e30;
   for (int s = std::max(1, dec_min_splits(tiles)); s <= smax; ++s) {
     const int per = (tiles + s - 1) / s;
@@ -99,24 +121,26 @@ static DecodeGeom decode_geom(int B, int n_kv_heads, int max_len, int occ = 0) {
       best.splits = (max_len + best.chunk - 1) / best.chunk;
     }
   }
+  best.cl = dec_cluster(pairs, best.splits, tiles, slots, i8);
+  if (best.cl) best.chunk = (tiles + best.cl - 1) / best.cl * kDecTT;
   return best;
 }
 
 // The int8 cache with head_dim 128 (16-byte aligned pools, 16-token pages)
 // runs the page-streaming kernel.  It shares the tile kernel's split
-// geometry: scoring its 4 CTAs per SM split the 70B-shaped context in two,
+// counts: scoring its 4 CTAs per SM split the 70B-shaped context in two,
 // which measured slower (42 us against 36 us; each warp's ring fill and the
 // merge weigh more on half the pages, and the combine pass is added).
 static bool dec_i8_shape(int kvquant, int head_dim, int page_size) {
   return kvquant == FP_KV_INT8 && head_dim == 128 && page_size == 16;
 }
 static DecodeGeom decode_geom_for(int B, int n_kv_heads, int head_dim, int kvquant, int page_size, int max_len) {
-  (void)head_dim, (void)kvquant, (void)page_size;
-  return decode_geom(B, n_kv_heads, max_len);
+  return decode_geom(B, n_kv_heads, max_len, dec_i8_shape(kvquant, head_dim, page_size));
 }
 
 int attention_decode_launches(int B, int n_kv_heads, int head_dim, int kvquant, int max_len) {
-  return decode_geom_for(B, n_kv_heads, head_dim, kvquant, 16, max_len).splits == 1 ? 1 : 2;
+  const DecodeGeom g = decode_geom_for(B, n_kv_heads, head_dim, kvquant, 16, max_len);
+  return g.splits == 1 || g.cl ? 1 : 2;
 }
 
 int attention_decode_splits(int B, int n_kv_heads, int head_dim, int kvquant, int max_len) {
@@ -197,11 +221,62 @@ constexpr size_t dec_smem_bytes() {
          (size_t)kDecTT * ld * 2 * 2;
 }
 
-// The ring, which also holds the 4-warp merge buffer after the loop; the
+// The ring, which also holds the merge buffers (4 warps, and the CTA's sums for
+// its cluster) after the loop; the
 // chunk's page ids follow it.
 template <int HD, int KVQ, int G, int NB>
 constexpr size_t dec_stage_bytes() {
-  return std::max(dec_smem_bytes<HD, KVQ, NB>(), (size_t)4 * G * (HD + 2) * sizeof(float));
+  return std::max(dec_smem_bytes<HD, KVQ, NB>(), (size_t)5 * G * (HD + 2) * sizeof(float));
+}
+
+// Where a cluster of `cl` CTAs (ranks along the grid's y) shares a (sequence, KV
+// head), the ranges of whole `unit`-token blocks of its T positions; t0 == t1: none.
+FP_DEV void dec_cluster_range(int T, int cl, int rank, int unit, int* t0, int* t1) {
+  const long long n = (T + unit - 1) / unit;
+  *t0 = (int)(n * rank / cl) * unit;
+  *t1 = min(T, (int)(n * (rank + 1) / cl) * unit);
+  if (*t1 < *t0) *t1 = *t0;
+}
+
+// The cluster's sums: each CTA has left its un-normalised output, maximum (log2
+// domain) and row sum of the G heads in `part` [G][HD + 2] of its shared memory; each
+// finishes a share of the outputs, adding the CTAs' sums in rank order.
+template <int HD, int G>
+FP_DEV void dec_cluster_finish(const float* part, int cl, int rank, uint16_t* __restrict__ out) {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+  const uint32_t p0 = (uint32_t)__cvta_generic_to_shared(part);
+  auto remote = [&](int k, int i) {
+    uint32_t p;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(p0 + i * 4), "r"(k));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(p) : "memory");
+    return v;
+  };
+  for (int i = rank * blockDim.x + threadIdx.x; i < G * HD; i += cl * blockDim.x) {
+    const int g = i / HD, e = i % HD;
+    float o[kDecMaxCluster], m[kDecMaxCluster], l[kDecMaxCluster], M = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < kDecMaxCluster; ++k) {
+      if (k >= cl) break;
+      o[k] = remote(k, g * (HD + 2) + e);
+      m[k] = remote(k, g * (HD + 2) + HD);
+      l[k] = remote(k, g * (HD + 2) + HD + 1);
+    }
+#pragma unroll
+    for (int k = 0; k < kDecMaxCluster; ++k)
+      if (k < cl) M = fmaxf(M, m[k]);
+    float ov = 0.f, L = 0.f;
+#pragma unroll
+    for (int k = 0; k < kDecMaxCluster; ++k) {
+      if (k >= cl) break;
+      const float f = m[k] == -INFINITY ? 0.f : exp2f(m[k] - M);
+      ov += o[k] * f;
+      L += l[k] * f;
+    }
+    out[i] = f2bf(ov / L);
+  }
+  // nobody leaves while its sums are being read
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // Workspace layout for (b, h, split): o [HD] fp32 (un-normalised, relative to
@@ -210,7 +285,7 @@ template <int HD, int KVQ, int G, int NB>
 __global__ void __launch_bounds__(128) attn_decode_kernel(const uint16_t* __restrict__ q, int q_stride, int H,
                                                           fp_kv_view kv, const int32_t* __restrict__ len,
                                                           int len_add, int max_len, int chunk, int splits,
-                                                          float* __restrict__ ws, uint16_t* __restrict__ out,
+                                                          int cl, float* __restrict__ ws, uint16_t* __restrict__ out,
                                                           int32_t* err) {
   constexpr int TT = kDecTT, LD = HD + 8;
   constexpr bool I8 = KVQ == FP_KV_INT8;
@@ -236,20 +311,21 @@ __global__ void __launch_bounds__(128) attn_decode_kernel(const uint16_t* __rest
     if (err && split == 0 && threadIdx.x == 0) atomicExch(err, 1);
     T = max_len;
   }
-  const int t0 = split * chunk;
-  if (t0 >= T) {
-    if (splits == 1)  // empty context: zero output
+  int t0 = split * chunk, t1 = min(T, t0 + chunk);
+  if (cl && T > 0) {
+    dec_cluster_range(T, cl, split, TT, &t0, &t1);
+  } else if (t0 >= T) {
+    if (split == 0 && (splits == 1 || cl))  // empty context: zero output
       for (int i = threadIdx.x; i < G * HD; i += 128) out[((long long)b * H + kvh * G) * HD + i] = 0;
     return;
   }
-  const int t1 = min(T, t0 + chunk);
   const int ntile = (t1 - t0 + TT - 1) / TT;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // ---- the page ids of positions t0 .. t1-1, staged once (past the table: -1)
   int* spt = reinterpret_cast<int*>(smem + dec_stage_bytes<HD, KVQ, G, NB>());
   {
     const int32_t* pt = kv.page_table + (long long)b * kv.pages_per_seq;
-    const int lp0 = t0 / kv.page_size, n = (t1 - 1) / kv.page_size - lp0 + 1;
+    const int lp0 = t0 / kv.page_size, n = t1 > t0 ? (t1 - 1) / kv.page_size - lp0 + 1 : 0;
     for (int i = tid; i < n; i += 128) spt[i] = lp0 + i < kv.pages_per_seq ? pt[lp0 + i] : -1;
     __syncthreads();
   }
@@ -460,6 +536,12 @@ __global__ void __launch_bounds__(128) attn_decode_kernel(const uint16_t* __rest
       out[((long long)b * H + kvh * G + g) * HD + e] = f2bf(ov / L);
       continue;
     }
+    if (cl) {
+      float* p = red + (4 * G + g) * (HD + 2);
+      p[e] = ov;
+      if (e == 0) p[HD] = M, p[HD + 1] = L;
+      continue;
+    }
     const long long row = ((long long)b * H + kvh * G + g) * splits + split;
     float* w = ws + row * (HD + 2);
     w[e] = ov;
@@ -468,6 +550,7 @@ __global__ void __launch_bounds__(128) attn_decode_kernel(const uint16_t* __rest
       w[HD + 1] = L;
     }
   }
+  if (cl) dec_cluster_finish<HD, G>(red + 4 * G * (HD + 2), cl, split, out + ((long long)b * H + kvh * G) * HD);
 }
 
 // Combine the splits of one (b, h): o = sum_s o_s 2^(m_s - M) / sum_s l_s 2^(m_s - M).
@@ -521,7 +604,8 @@ __global__ void attn_combine_kernel(int H, const int32_t* __restrict__ len, int 
 // 1152 sum_d Q[h][d], outputs 1152 sum_t P'[t][h].  Online softmax in the
 // log2 domain per head, the K scales multiplying the score columns.  The
 // warps are merged in shared memory at the end; the result is normalised in
-// place (one split) or written as (o, m, l) for attn_combine_kernel.
+// place (one split), added to those of the cluster, or written as (o, m, l) for
+// attn_combine_kernel.
 // =====================================================================
 constexpr int kD8Warps = 4, kD8Stages = 3;
 constexpr int kD8PageBytes = 2 * 16 * 128 + 2 * 16 * 4;  // K and V codes, then K and V scales
@@ -541,7 +625,7 @@ constexpr size_t d8_smem_bytes(int chunk) {
 template <int G>
 __global__ void __launch_bounds__(kD8Warps * 32) attn_decode_i8_kernel(
     const uint16_t* __restrict__ q, int q_stride, int H, fp_kv_view kv, const int32_t* __restrict__ len,
-    int len_add, int max_len, int chunk, int splits, float* __restrict__ ws, uint16_t* __restrict__ out,
+    int len_add, int max_len, int chunk, int splits, int cl, float* __restrict__ ws, uint16_t* __restrict__ out,
     int32_t* err) {
   constexpr int HD = 128;
   extern __shared__ __align__(16) uint8_t smem[];
@@ -557,13 +641,14 @@ __global__ void __launch_bounds__(kD8Warps * 32) attn_decode_i8_kernel(
     if (err && split == 0 && threadIdx.x == 0) atomicExch(err, 1);
     T = max_len;
   }
-  const int t0 = split * chunk;
-  if (t0 >= T) {
-    if (splits == 1)  // empty context: zero output
+  int t0 = split * chunk, t1 = min(T, t0 + chunk);
+  if (cl && T > 0) {
+    dec_cluster_range(T, cl, split, 16, &t0, &t1);
+  } else if (t0 >= T) {
+    if (split == 0 && (splits == 1 || cl))  // empty context: zero output
       for (int i = threadIdx.x; i < G * HD; i += blockDim.x) out[((long long)b * H + kvh * G) * HD + i] = 0;
     return;
   }
-  const int t1 = min(T, t0 + chunk);
   const int np = (t1 - t0 + 15) / 16;  // pages of the split (t0 is a multiple of 64)
   // ---- the split's page ids, staged once (past the table: -1)
   int* spt = reinterpret_cast<int*>(smem + kD8Warps * kD8Stages * kD8PageBytes);
@@ -778,6 +863,12 @@ __global__ void __launch_bounds__(kD8Warps * 32) attn_decode_i8_kernel(
       out[((long long)b * H + kvh * G + hh) * HD + e] = f2bf(ov / L);
       continue;
     }
+    if (cl) {
+      float* p = red + (kD8Warps * 8 + hh) * (HD + 2);
+      p[e] = ov;
+      if (e == 0) p[HD] = M, p[HD + 1] = L;
+      continue;
+    }
     const long long row = ((long long)b * H + kvh * G + hh) * splits + split;
     float* w = ws + row * (HD + 2);
     w[e] = ov;
@@ -786,6 +877,26 @@ __global__ void __launch_bounds__(kD8Warps * 32) attn_decode_i8_kernel(
       w[HD + 1] = L;
     }
   }
+  if (cl) dec_cluster_finish<HD, G>(red + kD8Warps * 8 * (HD + 2), cl, split, out + ((long long)b * H + kvh * G) * HD);
+}
+
+// Launch with clusters of cl CTAs along y, one per (sequence, KV head).
+template <typename... KArgs, typename... Args>
+static cudaError_t dec_launch_cluster(void (*kern)(KArgs...), int pairs, int cl, int threads, size_t smem,
+                                      cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pairs, cl);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = g_pdl ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 1, at[1].val.clusterDim.y = cl, at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 template <int G>
@@ -796,9 +907,12 @@ static cudaError_t launch_decode_i8(const uint16_t* q, int q_stride, int B, int 
   auto kern = attn_decode_i8_kernel<G>;
   static std::atomic<unsigned long long> attr{0};
   FP_CUDA_TRY(smem_limit_once(kern, (int)d8_smem_bytes(kDecMaxChunkTiles * kDecTT), &attr));
+  if (g.cl)
+    return dec_launch_cluster(kern, B * kv.n_kv_heads, g.cl, kD8Warps * 32, smem, s, q, q_stride, H, kv, len, len_add,
+                              max_len, g.chunk, g.splits, g.cl, ws, out, err);
   dim3 grid(B * kv.n_kv_heads, g.splits);
   cudaError_t e = launch(kern, grid, dim3(kD8Warps * 32), smem, s, q, q_stride, H, kv, len, len_add, max_len,
-                         g.chunk, g.splits, ws, out, err);
+                         g.chunk, g.splits, 0, ws, out, err);
   if (e != cudaSuccess || g.splits == 1) return e;
   e = launch(attn_combine_kernel<128>, dim3(B * H), dim3(128), 0, s, H, len, len_add, max_len, g.chunk, g.splits,
              (const float*)ws, out);
@@ -814,9 +928,12 @@ static cudaError_t launch_decode_nb(const uint16_t* q, int q_stride, int B, int 
   const size_t smem = dec_stage_bytes<HD, KVQ, G, NB>() + ((size_t)g.chunk / kv.page_size + 2) * sizeof(int);
   auto kern = attn_decode_kernel<HD, KVQ, G, NB>;
   if (smem > 48 * 1024) FP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (g.cl)
+    return dec_launch_cluster(kern, B * kv.n_kv_heads, g.cl, 128, smem, s, q, q_stride, H, kv, len, len_add, max_len,
+                              g.chunk, g.splits, g.cl, ws, out, err);
   dim3 grid(B * kv.n_kv_heads, g.splits);
   cudaError_t e = launch(kern, grid, dim3(128), smem, s, q, q_stride, H, kv, len, len_add, max_len, g.chunk,
-                         g.splits, ws, out, err);
+                         g.splits, 0, ws, out, err);
   if (e != cudaSuccess || g.splits == 1) return e;
   e = launch(attn_combine_kernel<HD>, dim3(B * H), dim3(HD), 0, s, H, len, len_add, max_len, g.chunk, g.splits,
              (const float*)ws, out);

@@ -38,7 +38,7 @@ cudaError_t launch_rope_kv(uint16_t* qkv, int B, int S, int row_stride, int n_he
 
 // ---- attention (fp_attention.cu)
 size_t attention_decode_ws_bytes(int B, int n_heads, int head_dim, int max_len);
-// Kernels one decode-attention launch runs: 1 (one split, normalised in place) or 2 (splits + combine).
+// Kernels one decode-attention launch runs: 1 (one split, or a cluster of them) or 2 (splits + combine).
 int attention_decode_launches(int B, int n_kv_heads, int head_dim, int kvquant, int max_len);
 // Context splits of one decode-attention launch (1: the partials workspace is not touched).
 int attention_decode_splits(int B, int n_kv_heads, int head_dim, int kvquant, int max_len);

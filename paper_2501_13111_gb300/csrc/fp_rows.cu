@@ -160,7 +160,8 @@ FP_DEV void better(float& bv, int& bi, float v, int i) {
 }
 
 __global__ void __cluster_dims__(kArgmaxCTAs, 1, 1) __launch_bounds__(256)
-    argmax_kernel(const float* __restrict__ logits, int V, int32_t* __restrict__ out, int32_t* pos, int by) {
+    argmax_kernel(const float* __restrict__ logits, int V, int32_t* __restrict__ out, int32_t* pos, int by,
+                  int32_t* host, const int32_t* err) {
   __shared__ float sv[8];
   __shared__ int si[8];
   __shared__ float cv;
@@ -217,13 +218,18 @@ __global__ void __cluster_dims__(kArgmaxCTAs, 1, 1) __launch_bounds__(256)
     }
     out[row] = i == 0x7fffffff ? 0 : i;
     if (pos) pos[row] += by;  // the sequence's next position (the decode step is complete)
+    if (host) {               // page-locked host memory: the token, and after the rows the error word
+      host[row] = i == 0x7fffffff ? 0 : i;
+      if (row == 0) host[gridDim.y] = *err;
+    }
   }
   cluster.sync();  // keep the winners alive until CTA 0 has read them
 }
 
-cudaError_t launch_argmax(const float* logits, int M, int V, int32_t* out, cudaStream_t s, int32_t* pos, int by) {
+cudaError_t launch_argmax(const float* logits, int M, int V, int32_t* out, cudaStream_t s, int32_t* pos, int by,
+                          int32_t* host, const int32_t* err) {
   if (M <= 0) return cudaSuccess;
-  return launch(argmax_kernel, dim3(kArgmaxCTAs, M), dim3(256), 0, s, logits, V, out, pos, by);
+  return launch(argmax_kernel, dim3(kArgmaxCTAs, M), dim3(256), 0, s, logits, V, out, pos, by, host, err);
 }
 
 // ------------------------------------------------------------------ RoPE + KV append

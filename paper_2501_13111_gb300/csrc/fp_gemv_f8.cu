@@ -33,7 +33,7 @@
 // A warp's pass over an item is a chain of waits and round trips (1400 cycles
 // for the operands, 1100-2600 for the sums) while an item may take 780, hence
 // two of each kind: with every warp on every item the 57344 x 8192 SwiGLU took
-// 155 us at 8 tokens and 176 us at 32, so 62 and 99.  More warps did not help
+// 155 us at 8 tokens and 176 us at 32, so 61 and 98.  More warps did not help
 // (four teams for the operands 64 us at 8 tokens, the tokens halved over
 // sixteen summing warps 88), nor did one polling lane per warp (80).
 // The (row tile, item) pairs are cut into equal contiguous ranges, one per
@@ -385,24 +385,25 @@ __global__ void __launch_bounds__(kF8Threads, 1)
     }
   } else if (warp >= kF8WarpMma) {
     // ---------------- MMA issuers of the even and the odd items
-    if (lane == 0) {
-      constexpr uint32_t idesc = tc_idesc_e4m3(kF8Rows, G::kN);
-      const uint64_t xd0 = sdesc(smem_u32(x_ring));
-      const int par = warp - kF8WarpMma;
-      bool ok = true;
-      int i = i_first + par;
-      for (int q = par; q < L; q += 2, i += 2) {
-        const int a = q % NA;
-        while (i >= SI) i -= SI;
-        const bool two = 2 * i + 1 < S;
-        // operands are there, and the sums of item q - ND, which used this
-        // accumulator, have been read
-        ok = mbar_wait(&xfull[q % XS], (q / XS) & 1) && mbar_wait(&afull[a], (q / NA) & 1) &&
-             (q < ND || mbar_wait(&dempty[q % ND], ((q / ND) & 1) ^ 1)) && !*abort_flag;
-        if (!ok) break;
-        tc_fence_after();
-        const uint64_t xd = xd0 + (uint64_t)(((q % XS) * G::kXStage) >> 4);
-        const uint32_t ta = tmem + G::kACol + a * kF8SlotCols, td = tmem + (q % ND) * 2 * G::kN;
+    constexpr uint32_t idesc = tc_idesc_e4m3(kF8Rows, G::kN);
+    const uint64_t xd0 = sdesc(smem_u32(x_ring));
+    const int par = warp - kF8WarpMma;
+    bool ok = true;
+    int i = i_first + par;
+    for (int q = par; q < L; q += 2, i += 2) {
+      const int a = q % NA;
+      while (i >= SI) i -= SI;
+      const bool two = 2 * i + 1 < S;
+      // operands are there, and the sums of item q - ND, which used this
+      // accumulator, have been read
+      ok = mbar_wait(&xfull[q % XS], (q / XS) & 1) && mbar_wait(&afull[a], (q / NA) & 1) &&
+           (q < ND || mbar_wait(&dempty[q % ND], ((q / ND) & 1) ^ 1)) && !*abort_flag;
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t xd = xd0 + (uint64_t)(((q % XS) * G::kXStage) >> 4);
+      const uint32_t ta = tmem + G::kACol + a * kF8SlotCols, td = tmem + (q % ND) * 2 * G::kN;
+      if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {  // 32 k: eight A columns, 32 bytes of an x row
           tc_mma_ts_f8(td, ta + kk * 8, xd + kk * 2, idesc, kk > 0 ? 1u : 0u);
@@ -412,10 +413,12 @@ __global__ void __launch_bounds__(kF8Threads, 1)
         }
         tc_commit(&idone[a]);  // the sums are complete, A slot a and x stage q % XS have been read
       }
-      if (!ok) fail();
-      tc_commit(&mma_done[par]);  // every MMA issued has completed before TMEM is released
-      mbar_wait(&mma_done[par], 0);
+      __syncwarp();
     }
+    if (!ok && lane == 0) fail();
+    if (elect_one()) tc_commit(&mma_done[par]);  // every MMA issued has completed before TMEM is released
+    __syncwarp();
+    mbar_wait(&mma_done[par], 0);
   } else if (warp < kF8WarpEpi) {
     // ---------------- codes to operands
     const int par = warp >> 2, qd = warp & 3, row = qd * 32 + lane;

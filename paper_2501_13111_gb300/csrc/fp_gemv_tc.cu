@@ -28,6 +28,10 @@
 //   warps 17-18 issue the MMAs (A from TMEM, B = x from shared memory) into
 //               fp32 TMEM accumulators, each its own chains (SwiGLU: one
 //               matrix each); warp 17 also allocates the 512 TMEM columns.
+//               All lanes run the loop and one issues: a lane alone took longer
+//               over an item's MMAs (int4 8192 x 28672 58.3 us at 24 tokens, so
+//               54.7; 57344 x 8192 with SwiGLU 112.3 at 64, so 109.4; int8
+//               8192 x 28672 79.8 at 24, so 74.4).
 // MMAs (M 128, N <= 64, K 16) into one accumulator follow each other at
 // about 50 cycles, far above their math (N / 2 cycles), while MMAs into
 // different accumulators overlap: the k-steps of each matrix are spread
@@ -243,23 +247,24 @@ __global__ void __launch_bounds__(kQ4Threads, 1)
   } else if (warp > DW) {
     // ---------------- MMA issuers: SwiGLU, one per matrix; otherwise even / odd k-steps
     const int mw = warp - DW - 1;
-    if (lane == 0) {
-      constexpr uint32_t idesc = tc_idesc(kQ4Rows, MT);
-      int seg = 0;
-      bool ok = true;
-      int g = (int)(begin % SI);
-      for (int q = 0; q < L; ++q, g = g + 1 == SI ? 0 : g + 1) {
-        const bool first = q == 0 || g == 0, last = g == SI - 1 || q == L - 1;
-        const int s = q % XS, a = q % NA;
-        if (first && seg > 0) ok = mbar_wait(&dempty, (seg - 1) & 1);  // the epilogue has read D
-        ok = ok && mbar_wait(&afull[a], (q / NA) & 1) && !*abort_flag;  // A slot and x stage
-        if (!ok) break;
-        tc_fence_after();
-        const uint64_t xd = sdesc(smem_u32(x_ring + s * G::kXBytes));
-        const uint32_t ta = tmem + G::kDCols + a * G::kACols;
-        // k-step kk of matrix r goes to chain kk % NCH of that matrix: consecutive
-        // MMAs of one issuer never share an accumulator, and the two issuers'
-        // chains are disjoint
+    constexpr uint32_t idesc = tc_idesc(kQ4Rows, MT);
+    int seg = 0;
+    bool ok = true;
+    int g = (int)(begin % SI);
+    for (int q = 0; q < L; ++q, g = g + 1 == SI ? 0 : g + 1) {
+      const bool first = q == 0 || g == 0, last = g == SI - 1 || q == L - 1;
+      const int s = q % XS, a = q % NA;
+      if (first && seg > 0) ok = mbar_wait(&dempty, (seg - 1) & 1);  // the epilogue has read D
+      ok = ok && mbar_wait(&afull[a], (q / NA) & 1) && !*abort_flag;  // A slot and x stage
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t xd = sdesc(smem_u32(x_ring + s * G::kXBytes));
+      const uint32_t ta = tmem + G::kDCols + a * G::kACols;
+      // k-step kk of matrix r goes to chain kk % NCH of that matrix: consecutive
+      // MMAs of one issuer never share an accumulator, and the two issuers'
+      // chains are disjoint
+      if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < KI / 16; ++kk) {
           const int r = NR == 2 ? mw : 0;
@@ -270,16 +275,16 @@ __global__ void __launch_bounds__(kQ4Threads, 1)
                     xd + (uint64_t)(((kk >> 2) * MT * 128 + (kk & 3) * 32) >> 4), idesc, (first && kk < NCH) ? 0u : 1u);
         }
         tc_commit(&aempty[a]);  // A slot a and x stage a have been read
-        if (last) {
-          tc_commit(&dfull);
-          ++seg;
-        }
+        if (last) tc_commit(&dfull);
       }
-      if (!ok) fail();
-      // every MMA issued has completed before TMEM is released
-      tc_commit(&mma_done);
-      mbar_wait(&mma_done, 0);
+      __syncwarp();
+      if (last) ++seg;
     }
+    if (!ok && lane == 0) fail();
+    // every MMA issued has completed before TMEM is released
+    if (elect_one()) tc_commit(&mma_done);
+    __syncwarp();
+    mbar_wait(&mma_done, 0);
   } else {
     // ---------------- dequantise (+ epilogue)
     // two teams of eight warps take alternate items, so one team computes

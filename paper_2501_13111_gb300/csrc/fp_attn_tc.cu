@@ -52,7 +52,8 @@
 //   two tiles per CTA                                        333 | 161 | 725
 //   every lane runs the MMA loop (one lane's issue took 144
 //     cycles for an MMA that runs 65)                        297 | 138 | 641
-//   output rows through shared memory, shorter first rounds  284 | 126 | 616
+//   output rows through shared memory                        285 | 126 | 617
+//   the items longest first, also over many rounds          255 | 123 | 540
 // A query tile's keys in turn by the two groups, bf16 | int8 cache: 8 heads, 1 x 1024
 // tokens 19.7 | 39.5 us, 1 x 4096 61 | 133, 40 heads, 1 x 1024 27.1 | 52 (one 128-row
 // tile per CTA 20.4 | 49.5, 70 | 211, 31.5 | 71; with two V tiles in the ring, as for
@@ -735,8 +736,14 @@ bool attention_prefill_tc_ok(int B, int S, int n_heads, const fp_kv_view& kv, co
 // Pairs of tiles where they keep the SMs busy, else single tiles with their keys cut
 // in two: the smaller of the two makespans (the mean share of an SM, or the longest
 // item), with 4100 cycles for a step of two tiles' products and 3500 an item, 4000
-// with the two groups' sums added (measured, bf16 cache).
-static PaPlan pa_plan(int B, int S, int H, int G, int sms) {
+// with the two groups' sums added (measured, bf16 cache).  The items are taken longest
+// first for up to 32 rounds of the SMs, which leaves their shares even; past that the
+// shares even out and the sharing of keys in L2 counts, with an int8 cache and heads
+// that share no keys from 12 rounds on.  Longest first / head by head, us: bf16 2 x 2760
+// tokens, 40 heads (5.8 rounds) 158 / 213, 8 x 1024, 40 heads (8.4) 123 / 126, 4 x 2048,
+// 64 heads on 8 (13.5) 255 / 285, 32 x 2048 (108) 2059 / 2055; int8 4 x 2048, 64 on 8
+// 540 / 617, 4 x 4000, 32 heads (13.5) 1210 / 1160, 32 x 2048, 64 on 8 4774 / 4520.
+static PaPlan pa_plan(int B, int S, int H, int G, bool kv8, int sms) {
   const long long tiles = (S + kPaB - 1) / kPaB;
   const int pair = G % 2 == 0 ? 1 : 2;
   auto make = [&](int pr) {
@@ -744,7 +751,7 @@ static PaPlan pa_plan(int B, int S, int H, int G, int sms) {
     p.pair = pr;
     p.units = (int)(pr == 2 ? (tiles + 1) / 2 : tiles);
     p.items = (int)((long long)B * (pr == 1 ? H / 2 : H) * p.units);
-    p.longest_first = p.items <= 4LL * sms;
+    p.longest_first = p.items <= (kv8 && pr == 2 ? 12LL : 32LL) * sms;
     return p;
   };
   auto span = [&](const PaPlan& p) {
@@ -780,7 +787,7 @@ static cudaError_t launch_pa_tc(const CUtensorMap& mq, const CUtensorMap& mk, co
         sms <= 0)
       sms = 152;
   }
-  const PaPlan plan = pa_plan(B, S, n_heads, n_heads / kv.n_kv_heads, sms);
+  const PaPlan plan = pa_plan(B, S, n_heads, n_heads / kv.n_kv_heads, KV8, sms);
   const int ctas = std::min(plan.items, sms);
   return plan.pair ? launch_pa_plan<KV8, false>(plan, ctas, mq, mk, mv, S, n_heads, kv, out, err, s)
                    : launch_pa_plan<KV8, true>(plan, ctas, mq, mk, mv, S, n_heads, kv, out, err, s);

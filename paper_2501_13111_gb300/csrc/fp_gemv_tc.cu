@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kQ4Threads, 1)
     gemv_q4tc_kernel(const __grid_constant__ CUtensorMap map_x, const uint8_t* __restrict__ codes, int M, int N,
                      const uint16_t* __restrict__ scales, const uint16_t* __restrict__ zeros, const uint16_t* R,
                      void* Y, long long total, int S, int V, float* __restrict__ ws, unsigned* __restrict__ counters,
-                     int32_t* err) {
+                     int32_t* err, const uint16_t* X, long long check) {
   constexpr int NR = EPI == FP_EPI_SWIGLU ? 2 : 1;
   using G = Q4Geom<MT, NR, WQ, KI>;
   constexpr bool I4 = WQ == FP_W_INT4_G128;
@@ -247,6 +247,23 @@ __global__ void __launch_bounds__(kQ4Threads, 1)
   } else if (warp > DW) {
     // ---------------- MMA issuers: SwiGLU, one per matrix; otherwise even / odd k-steps
     const int mw = warp - DW - 1;
+    if (!I4 && check > 0) {
+      // the CTAs together look at x's `check` 16-byte pieces, while the first items come
+      pdl_wait();
+      bool over = false;
+#pragma unroll 4
+      for (long long i = (c * kQ4MmaWarps + mw) * 32 + lane; i < check; i += C * kQ4MmaWarps * 32) {
+        const uint4 v = *(reinterpret_cast<const uint4*>(X) + i);
+        const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const float2 f = bf2x2f(w4[p]);
+          over |= fabsf(f.x) > 65504.f || fabsf(f.y) > 65504.f;
+        }
+      }
+      if (over && err) atomicExch(err, 3);
+      __syncwarp();
+    }
     constexpr uint32_t idesc = tc_idesc(kQ4Rows, MT);
     int seg = 0;
     bool ok = true;
@@ -546,13 +563,22 @@ bool q4tc_ok(int wquant, int epi, int M, int N, int K) {
   return blocks * kQ4DeqWarps <= kLinTicketSlots && tensor_maps_available();
 }
 
-// int4 always; int8 beyond 32 tokens or for long rows.  Measured at the
-// 70B-shaped block's linears, microseconds on tcgen05 against mma.sync: 32
-// tokens QKV 45.3 / 41.0, O 39.3 / 35.8, gate+up 173.9 / 165.4, down (K
-// 28672) 86.2 / 118.9; 64 tokens 48.8 / 81.3, 45.1 / 70.3, 180.3 / 267.1,
-// 96.0 / 204.7.  An int8 item carries half the weights of an int4 item for
-// the same hand-offs, while the mma.sync GEMV's cost grows with the tokens.
-bool q4tc_preferred(int wquant, int M, int K) { return wquant != FP_W_INT8 || M > 32 || K >= 16384; }
+// int4 always; int8 beyond 32 tokens, for long rows, and, of the larger matrices
+// without SwiGLU, for those not much wider than long.  Microseconds, tcgen05 against
+// mma.sync, int8:
+//   32 tokens  4096 x 11008 25.5 / 32.0    8192 x 14336 44.0 / 53.7   5120 x 5120 20.2 / 25.0
+//              9216 x 9216 34.2 / 39.1     2048 x 15872 21.3 / 30.1   7168 x 5120 21.5 / 24.4
+//   17         25.7 / 28.3, 43.5 / 50.3, 19.8 / 21.5, 34.0 / 37.2, 20.8 / 25.9, 21.2 / 22.5
+//   17         wider: 12288 x 4096 28.0 / 26.5, 57344 x 8192 with SwiGLU 162.8 / 156.3;
+//              K a multiple of 8192: 8192 x 8192 34.3 / 31.7; smaller: 4096 x 4096 18.6 / 14.5
+//   64         QKV 48.8 / 81.3, O 45.1 / 70.3, gate+up 180.3 / 267.1 (70B shapes)
+// An int8 item carries half the weights of an int4 item for the same hand-offs, while
+// the mma.sync GEMV's cost grows with the tokens and with the x that a CTA stages.
+bool q4tc_preferred(int wquant, int epi, int M, int N, int K) {
+  if (wquant != FP_W_INT8 || M > 32 || K >= 16384) return true;
+  return epi != FP_EPI_SWIGLU && K >= 5120 && K % 8192 != 0 && 2LL * N <= 3LL * K && N <= 9216 &&
+         (long long)N * K > (1LL << 24);
+}
 
 size_t q4tc_ws_bytes(int epi, int M, int N, int K) {
   const int nr = epi == FP_EPI_SWIGLU ? 2 : 1;
@@ -565,7 +591,7 @@ size_t q4tc_ws_bytes(int epi, int M, int N, int K) {
 template <int MT, int EPI, int WQ, int KI>
 static cudaError_t launch_q4_t(const uint8_t* codes, const CUtensorMap& mx, int M, int N, int K,
                                const uint16_t* scales, const uint16_t* zeros, const uint16_t* R, void* Y, void* ws,
-                               int32_t* err, cudaStream_t s) {
+                               int32_t* err, const uint16_t* X, long long check, cudaStream_t s) {
   constexpr int NR = EPI == FP_EPI_SWIGLU ? 2 : 1;
   auto kern = gemv_q4tc_kernel<MT, EPI, WQ, KI>;
   const int smem = std::max(Q4Geom<MT, NR, WQ, KI>::kSmem, kQ4MinSmem);
@@ -579,7 +605,7 @@ static cudaError_t launch_q4_t(const uint8_t* codes, const CUtensorMap& mx, int 
   unsigned* counters = (unsigned*)ws;
   float* part = (float*)((char*)ws + (size_t)kLinTicketSlots * 4);
   return launch(kern, dim3(ctas), dim3(kQ4Threads), (size_t)smem, s, mx, codes, M, N, scales, zeros, R, Y, total, S,
-                WQ == FP_W_INT4_G128 ? q4_v(S) : 1, part, counters, err);
+                WQ == FP_W_INT4_G128 ? q4_v(S) : 1, part, counters, err, X, check);
 }
 
 // k per item: int4 two groups where K allows (SwiGLU items already carry two
@@ -587,22 +613,22 @@ static cudaError_t launch_q4_t(const uint8_t* codes, const CUtensorMap& mx, int 
 template <int MT, int WQ>
 static cudaError_t launch_q4_w(int epi, const uint8_t* mw, const CUtensorMap& mx, int M, int N, int K,
                                const uint16_t* scales, const uint16_t* zeros, const uint16_t* R, void* Y, void* ws,
-                               int32_t* err, cudaStream_t s) {
+                               int32_t* err, const uint16_t* X, long long check, cudaStream_t s) {
   constexpr bool I4 = WQ == FP_W_INT4_G128;
   constexpr int K2 = I4 ? 256 : 128;  // the larger item
   const bool two = I4 && (K / 128) % 2 == 0;
   switch (epi) {
     case FP_EPI_STORE:
-      return two ? launch_q4_t<MT, FP_EPI_STORE, WQ, K2>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, s)
-                 : launch_q4_t<MT, FP_EPI_STORE, WQ, 128>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, s);
+      return two ? launch_q4_t<MT, FP_EPI_STORE, WQ, K2>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, X, check, s)
+                 : launch_q4_t<MT, FP_EPI_STORE, WQ, 128>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, X, check, s);
     case FP_EPI_RESID:
-      return two ? launch_q4_t<MT, FP_EPI_RESID, WQ, K2>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, s)
-                 : launch_q4_t<MT, FP_EPI_RESID, WQ, 128>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, s);
+      return two ? launch_q4_t<MT, FP_EPI_RESID, WQ, K2>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, X, check, s)
+                 : launch_q4_t<MT, FP_EPI_RESID, WQ, 128>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, X, check, s);
     case FP_EPI_SWIGLU:
-      return launch_q4_t<MT, FP_EPI_SWIGLU, WQ, I4 ? 128 : 64>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, s);
+      return launch_q4_t<MT, FP_EPI_SWIGLU, WQ, I4 ? 128 : 64>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, X, check, s);
     default:
-      return two ? launch_q4_t<MT, FP_EPI_F32, WQ, K2>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, s)
-                 : launch_q4_t<MT, FP_EPI_F32, WQ, 128>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, s);
+      return two ? launch_q4_t<MT, FP_EPI_F32, WQ, K2>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, X, check, s)
+                 : launch_q4_t<MT, FP_EPI_F32, WQ, 128>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, X, check, s);
   }
 }
 
@@ -617,13 +643,16 @@ cudaError_t launch_q4tc(int wquant, int epi, const uint16_t* x, int M, int N, in
   // x [M][K] bf16, box [mt rows][64]
   if (!make_tensor_map(&mx, x, M, K, 2, mt, 64, 128)) return cudaErrorInvalidValue;
   const bool i8 = wquant == FP_W_INT8;
+  // up to 32 tokens the int8 linears that run on mma.sync stage x as fp16 and report an x
+  // beyond its range (status 3); this kernel has no such limit, but reports it alike
+  const long long check = i8 && M <= 32 && K < 16384 ? (long long)M * K / 8 : 0;
   switch (mt) {
     case 32:
-      return i8 ? launch_q4_w<32, FP_W_INT8>(epi, mw, mx, M, N, K, scales, zeros, residual, y, ws, err, s)
-                : launch_q4_w<32, FP_W_INT4_G128>(epi, mw, mx, M, N, K, scales, zeros, residual, y, ws, err, s);
+      return i8 ? launch_q4_w<32, FP_W_INT8>(epi, mw, mx, M, N, K, scales, zeros, residual, y, ws, err, x, check, s)
+                : launch_q4_w<32, FP_W_INT4_G128>(epi, mw, mx, M, N, K, scales, zeros, residual, y, ws, err, x, check, s);
     default:
-      return i8 ? launch_q4_w<64, FP_W_INT8>(epi, mw, mx, M, N, K, scales, zeros, residual, y, ws, err, s)
-                : launch_q4_w<64, FP_W_INT4_G128>(epi, mw, mx, M, N, K, scales, zeros, residual, y, ws, err, s);
+      return i8 ? launch_q4_w<64, FP_W_INT8>(epi, mw, mx, M, N, K, scales, zeros, residual, y, ws, err, x, check, s)
+                : launch_q4_w<64, FP_W_INT4_G128>(epi, mw, mx, M, N, K, scales, zeros, residual, y, ws, err, x, check, s);
   }
 }
 

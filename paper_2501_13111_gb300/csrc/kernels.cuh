@@ -87,7 +87,7 @@ cudaError_t launch_f8(int epi, const uint16_t* x, const int32_t* perm, int M, in
 
 // ---- int4 / int8 decode linear at 17-64 tokens on tcgen05 (fp_gemv_tc.cu)
 bool q4tc_ok(int wquant, int epi, int M, int N, int K);
-bool q4tc_preferred(int wquant, int M, int K);
+bool q4tc_preferred(int wquant, int epi, int M, int N, int K);
 size_t q4tc_ws_bytes(int epi, int M, int N, int K);
 cudaError_t launch_q4tc(int wquant, int epi, const uint16_t* x, int M, int N, int K, const void* codes,
                         const uint16_t* scales, const uint16_t* zeros, const uint16_t* residual, void* y, void* ws,

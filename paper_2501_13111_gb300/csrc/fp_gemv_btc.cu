@@ -286,16 +286,18 @@ bool btc_ok(int wquant, int epi, int M, int N, int K) {
   return blocks * 4 <= kLinTicketSlots && tensor_maps_available();
 }
 
-// Items per SM of a launch; below about 48 the mma.sync GEMV is faster
-// (measured: 70B-shaped QKV at 32 tokens, 34 items per SM, 60 against 48 us;
-// the LM head, 105 items per SM, 117 against 134 us).
-bool btc_preferred(int epi, int N, int K) {
-  const int nr = epi == FP_EPI_SWIGLU ? 2 : 1;
-  const long long nout = nr == 2 ? N / 2 : N;
-  const long long blocks = (nout + kBtRows - 1) / kBtRows;
-  const int kbi = nr == 1 ? 2 : 1;
-  const long long items = blocks * ((K + kbi * kBtBK - 1) / (kbi * kBtBK));
-  return items >= 48LL * bt_sms();
+// Where this kernel beats the mma.sync GEMV (its TMEM, first copies and last tile cost
+// about 10 us before any gain): larger matrices, fewer weights the more tokens, and
+// SwiGLU, whose items carry half the k, from 32 items an SM.  Microseconds, here / mma.sync:
+//   17 tokens  4096 x 11008 25.2 / 31.4   10240 x 8192 34.8 / 43.3   8192 x 14336 47.0 / 58.9
+//              6144 x 4096 17.2 / 19.9    4096 x 4096 16.5 / 13.4    16384 x 1088 16.8 / 16.2
+//   40         4096 x 4096 22.4 / 22.9    3072 x 4096 15.7 / 21.7    5120 x 13824 38.5 / 60.7
+//   64         10240 x 8192 40.0 / 68.8   32000 x 512 15.6 / 23.5
+//   SwiGLU     22016 x 4096 17 tokens 42.5 / 46.9, 64 57.9 / 66.0    16384 x 2048 22.2 / 19.3, 31.0 / 34.0
+bool btc_preferred(int epi, int M, int N, int K) {
+  if (epi != FP_EPI_SWIGLU) return (long long)N * K >= (M > 32 ? 3LL << 22 : 9LL << 21);
+  const long long blocks = (N / 2 + kBtRows - 1) / kBtRows;
+  return blocks * ((K + kBtBK - 1) / kBtBK) >= 32LL * bt_sms();
 }
 
 size_t btc_ws_bytes(int epi, int M, int N, int K) {

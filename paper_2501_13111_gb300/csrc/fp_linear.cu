@@ -953,9 +953,9 @@ cudaError_t launch_linear(int wquant, int epi, const uint16_t* x, int M, int N, 
   }
   if (take_f8(wquant, epi, x, M, N, K, codes, scales, zeros, ws, ws_bytes))
     return launch_f8(epi, x, nullptr, M, N, K, codes, scales, zeros, residual, y, ws, ws_bytes, err, s);
-  // bf16 weights at 17-64 tokens: the TMA-fed tcgen05 GEMV where every SM gets
-  // enough 32 KB items to hide their per-item cost (16-byte aligned x and weights)
-  if (btc_ok(wquant, epi, M, N, K) && btc_preferred(epi, N, K) && ((uintptr_t)x & 15) == 0 &&
+  // bf16 weights at 17-64 tokens: the TMA-fed tcgen05 GEMV where the matrix is large
+  // enough (16-byte aligned x and weights)
+  if (btc_ok(wquant, epi, M, N, K) && btc_preferred(epi, M, N, K) && ((uintptr_t)x & 15) == 0 &&
       ((uintptr_t)codes & 15) == 0)
     return launch_btc(epi, x, M, N, K, codes, residual, y, ws, ws_bytes, err, s);
   // int4 and int8 at 17-64 tokens: the tensor-core path, weights expanded into

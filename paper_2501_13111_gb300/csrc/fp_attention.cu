@@ -622,12 +622,15 @@ constexpr size_t d8_smem_bytes(int chunk) {
   return (size_t)kD8Warps * kD8Stages * kD8PageBytes + ((size_t)chunk / 16 + 2) * sizeof(int);
 }
 
-template <int G>
+// CL: the CTAs of a cluster share the context (an instance of its own: beside the
+// single split its code cost that 0.6 %).
+template <int G, bool CL>
 __global__ void __launch_bounds__(kD8Warps * 32) attn_decode_i8_kernel(
     const uint16_t* __restrict__ q, int q_stride, int H, fp_kv_view kv, const int32_t* __restrict__ len,
     int len_add, int max_len, int chunk, int splits, int cl, float* __restrict__ ws, uint16_t* __restrict__ out,
     int32_t* err) {
   constexpr int HD = 128;
+  if constexpr (!CL) cl = 0;
   extern __shared__ __align__(16) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   // no early trigger: the linear after it takes whole SMs, and launched early
@@ -904,12 +907,17 @@ static cudaError_t launch_decode_i8(const uint16_t* q, int q_stride, int B, int 
                                     const int32_t* len, int len_add, int max_len, DecodeGeom g, float* ws,
                                     uint16_t* out, int32_t* err, cudaStream_t s, cudaError_t* second) {
   const size_t smem = d8_smem_bytes(g.chunk);
-  auto kern = attn_decode_i8_kernel<G>;
-  static std::atomic<unsigned long long> attr{0};
-  FP_CUDA_TRY(smem_limit_once(kern, (int)d8_smem_bytes(kDecMaxChunkTiles * kDecTT), &attr));
-  if (g.cl)
+  const int limit = (int)d8_smem_bytes(kDecMaxChunkTiles * kDecTT);
+  if (g.cl) {
+    auto kern = attn_decode_i8_kernel<G, true>;
+    static std::atomic<unsigned long long> attr{0};
+    FP_CUDA_TRY(smem_limit_once(kern, limit, &attr));
     return dec_launch_cluster(kern, B * kv.n_kv_heads, g.cl, kD8Warps * 32, smem, s, q, q_stride, H, kv, len, len_add,
                               max_len, g.chunk, g.splits, g.cl, ws, out, err);
+  }
+  auto kern = attn_decode_i8_kernel<G, false>;
+  static std::atomic<unsigned long long> attr{0};
+  FP_CUDA_TRY(smem_limit_once(kern, limit, &attr));
   dim3 grid(B * kv.n_kv_heads, g.splits);
   cudaError_t e = launch(kern, grid, dim3(kD8Warps * 32), smem, s, q, q_stride, H, kv, len, len_add, max_len,
                          g.chunk, g.splits, 0, ws, out, err);

@@ -69,8 +69,7 @@ enum {
  * CTA, and shared blocks are reduced from fp32 partials in a fixed order) --
  * on mma.sync with the codes dequantised in registers, except, with 16-byte
  * aligned x and codes: int4 and a bf16 result with M <= 16 and at least 2^24
- * weights, or SwiGLU with M <= 32 and at least 2^28 (scales and zeros 16-byte
- * aligned too), which runs on tcgen05 with 8-bit operands (the codes as they
+ * weights (scales and zeros 16-byte aligned too), which runs on tcgen05 with 8-bit operands (the codes as they
  * are; x split by a first kernel into two e4m3 pieces an element, which carry
  * it exactly down to 2^-13 of its row's largest value and to 2^-23 of that
  * value below; scales and zero points applied in fp32; a row of x that holds an

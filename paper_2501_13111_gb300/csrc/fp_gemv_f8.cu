@@ -1,4 +1,4 @@
-// Decode linear for int4 group-128 weights at up to 32 tokens on the tcgen05
+// Decode linear for int4 group-128 weights at up to 16 tokens on the tcgen05
 // tensor cores with 8-bit operands.
 //
 // y[m][n] = sum_g s[n][g] sum_{k in g} (q[n][k] - z[n][g]) x[m][k].
@@ -33,9 +33,8 @@
 // A warp's pass over an item is a chain of waits and round trips (1400 cycles
 // for the operands, 1100-2600 for the sums) while an item may take 780, hence
 // two of each kind: with every warp on every item the 57344 x 8192 SwiGLU took
-// 155 us at 8 tokens and 176 us at 32, so 61 and 98.  More warps did not help
-// (four teams for the operands 64 us at 8 tokens, the tokens halved over
-// sixteen summing warps 88), nor did one polling lane per warp (80).
+// 155 us at 8 tokens, so 61.  More warps did not help (four teams for the operands
+// 64 us), nor did one polling lane per warp (80).
 // The (row tile, item) pairs are cut into equal contiguous ranges, one per
 // CTA.  A row tile shared by several CTAs is finished by the last of them from
 // fp32 partials (a ticket per 32 rows and half of the tokens; sums in CTA
@@ -71,10 +70,10 @@ struct F8Geom {
   static constexpr int kN = 2 * MT;                        // hi columns, then lo columns
   static constexpr int kGroupBytes = kN * 128;             // x pieces of one group
   static constexpr int kXStage = 2 * kGroupBytes;
-  static constexpr int kAccs = MT == 32 ? 2 : 4;  // items whose two accumulators are in TMEM
+  static constexpr int kAccs = 4;                          // items whose two accumulators are in TMEM
   static constexpr int kSlots = MT == 8 ? 6 : 4;           // items whose A operands are
   static constexpr int kACol = kAccs * 2 * kN;             // the first column of the A operands
-  static constexpr int kWStages = MT == 32 ? 8 : 10;
+  static constexpr int kWStages = 10;
   static constexpr int kXStages = 4;
   static constexpr int kXsStage = 2 * MT * 4;
   static constexpr int kSwap = kF8Rows * MT * 4;           // the tokens' halves changing hands
@@ -102,8 +101,7 @@ constexpr int kSplitThreads = 1024, kSplitHeld = 4;
 
 __global__ void __launch_bounds__(kSplitThreads)
     split_x_kernel(const uint16_t* __restrict__ x, int M, int MT, int K, const int32_t* __restrict__ perm,
-                   uint8_t* __restrict__ pieces, float* __restrict__ sums, float* __restrict__ unscale, bool fp16_range,
-                   int32_t* err) {
+                   uint8_t* __restrict__ pieces, float* __restrict__ sums, float* __restrict__ unscale, int32_t* err) {
   pdl_trigger();
   pdl_wait();
   const int m = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
@@ -149,12 +147,12 @@ __global__ void __launch_bounds__(kSplitThreads)
   for (int j = 0; j < kSplitHeld; ++j) {
     held[j] = load(tid + j * kSplitThreads);
     am = amax2(amax2(amax2(amax2(am, held[j].x), held[j].y), held[j].z), held[j].w);
-    if (fp16_range) check(held[j]);
+    check(held[j]);
   }
   for (int c = tid + kSplitHeld * kSplitThreads; c < chunks; c += kSplitThreads) {
     const uint4 v = load(c);
     am = amax2(amax2(amax2(amax2(am, v.x), v.y), v.z), v.w);
-    if (fp16_range) check(v);
+    check(v);
   }
   if (bad && err) atomicExch(err, 1);
   // tokens that a kernel staging x in fp16 refuses are refused here too
@@ -463,7 +461,6 @@ __global__ void __launch_bounds__(kF8Threads, 1)
     // ---------------- group sums to accumulators, row tiles to the output
     const int qd = warp & 3, lr = qd * 32 + lane, par = (warp - kF8WarpEpi) >> 2;
     const uint32_t lane_base = tmem + ((uint32_t)(qd * 32) << 16);
-    constexpr int CH = MT <= 16 ? MT : 16;  // tokens per TMEM load
     // scales and zeros of this thread's weight row, the two groups of its next item
     auto wrow = [&](int bb) -> long long {  // the row of the weight matrix (clamped: rows past the end are not stored)
       if (GLU) return min(bb * TR + (lr & (TR - 1)), Nout - 1) + (lr >= TR ? (long long)Nout : 0LL);
@@ -514,25 +511,18 @@ __global__ void __launch_bounds__(kF8Threads, 1)
             const float2 s2 = make_float2(s, s), nz2 = make_float2(-z, -z), r32 = make_float2(1.f / 32.f, 1.f / 32.f);
             const float* xs = xs_ring + r * (2 * MT) + j * MT;
             const uint32_t d = lane_base + (q % ND) * 2 * G::kN + j * G::kN;
+            float4 xv[MT / 4];  // read while the sums come from TMEM
 #pragma unroll
-            for (int c0 = 0; c0 < MT; c0 += CH) {
-              float4 xv[CH / 4];  // read while the sums come from TMEM
+            for (int t = 0; t < MT / 4; ++t) xv[t] = *reinterpret_cast<const float4*>(xs + 4 * t);
+            uint32_t hi[MT], lo[MT];
+            tc_ld_pair<MT>(d, d + MT, hi, lo);
 #pragma unroll
-              for (int t = 0; t < CH / 4; ++t) xv[t] = *reinterpret_cast<const float4*>(xs + c0 + 4 * t);
-              uint32_t hi[CH], lo[CH];
-              tc_ld_pair<CH>(d + c0, d + MT + c0, hi, lo);
-#pragma unroll
-              for (int t = 0; t < CH; t += 4) {
-                const float4 x4 = xv[t / 4];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                  const float2 xx = e ? make_float2(x4.z, x4.w) : make_float2(x4.x, x4.y);
-                  const int k = t + 2 * e;
-                  float2 v = ffma2(nz2, xx, make_float2(__uint_as_float(hi[k]), __uint_as_float(hi[k + 1])));
-                  v = ffma2(make_float2(__uint_as_float(lo[k]), __uint_as_float(lo[k + 1])), r32, v);
-                  acc[(c0 + k) / 2] = ffma2(s2, v, acc[(c0 + k) / 2]);
-                }
-              }
+            for (int k = 0; k < MT; k += 2) {
+              const float4 x4 = xv[k / 4];
+              const float2 xx = k & 2 ? make_float2(x4.z, x4.w) : make_float2(x4.x, x4.y);
+              float2 v = ffma2(nz2, xx, make_float2(__uint_as_float(hi[k]), __uint_as_float(hi[k + 1])));
+              v = ffma2(make_float2(__uint_as_float(lo[k]), __uint_as_float(lo[k + 1])), r32, v);
+              acc[k / 2] = ffma2(s2, v, acc[k / 2]);
             }
           }
         }
@@ -634,7 +624,7 @@ static int f8_sms() {
   return n;
 }
 
-static int f8_mt(int M) { return M <= 8 ? 8 : M <= 16 ? 16 : 32; }
+static int f8_mt(int M) { return M <= 8 ? 8 : 16; }
 
 // fp32 partials, then the x pieces, their group sums and the tokens' scales.
 struct F8Plan {
@@ -661,25 +651,21 @@ static F8Plan f8_plan(int epi, int M, int N, int K) {
 }
 
 // Where it is the faster path.  Measured in a graph, microseconds here against
-// the mma.sync GEMV (to 16 tokens) or the bf16 expansion in TMEM (from 17):
+// the mma.sync GEMV:
 //   tokens 1 / 8 / 16   4096 x 4096    11.0 / 11.3 / 13.5   10.9 / 12.1 / 17.0
 //                       1024 x 512      7.7 /  7.9 /  8.8    5.1 /  5.2 /  5.8
 //                       5120 x 13824   19.3 / 20.1 / 23.4   25.1 / 27.3 / 29.3
 //                       57344 x 8192   60.2 / 61.9 / 69.5    109 /  113 /  135
-//   tokens 32           57344 x 8192   99                    109 (SwiGLU)
-//                       27648 x 5120   42                    41  (SwiGLU)
-//                       8192 x 28672   60                    58
-//   tokens 64           57344 x 8192  179                    113 (no longer built)
-// The second kernel (3 us) and a CTA's hand-offs want 8 MB of codes; from 17
-// tokens the sums' warps set the pace and only the largest gate and up gain.
-static bool f8_pays(int epi, int M, int N, int K) {
-  const long long weights = (long long)N * K;
-  return M <= 16 ? weights >= (1LL << 24) : M <= 32 && epi == FP_EPI_SWIGLU && weights >= (1LL << 28);
-}
+// The second kernel (3 us) and a CTA's hand-offs want 8 MB of codes.  Not beyond 16
+// tokens, where the bf16 expansion in TMEM takes x as it is (57344 x 8192 with SwiGLU
+// at 32 tokens 99 us here, 109 there): one element of 2^18 beside unit normals, its
+// weights zero, left an error of 0.054 here and 0.0027 there, and a row with an
+// infinity gave NaN.
+static bool f8_pays(int M, int N, int K) { return M <= 16 && (long long)N * K >= (1LL << 24); }
 
 bool f8_ok(int wquant, int epi, int M, int N, int K) {
   if (wquant != FP_W_INT4_G128 || epi == FP_EPI_F32 || M < 1 || N < 1 || K < 128 || K % 128 != 0) return false;
-  if (!f8_pays(epi, M, N, K) || (epi == FP_EPI_SWIGLU && N % 2 != 0)) return false;
+  if (!f8_pays(M, N, K) || (epi == FP_EPI_SWIGLU && N % 2 != 0)) return false;
   const long long nout = epi == FP_EPI_SWIGLU ? N / 2 : N;
   const long long tiles = (nout + kF8Rows - 1) / kF8Rows;  // eight tickets per 128 output rows
   return tiles * 8 <= kLinTicketSlots && tensor_maps_available();
@@ -725,11 +711,10 @@ cudaError_t launch_f8(int epi, const uint16_t* x, const int32_t* perm, int M, in
     return cudaErrorInvalidValue;
   char* w = (char*)ws;
   FP_CUDA_TRY(launch(split_x_kernel, dim3(mt), dim3(kSplitThreads), 0, s, x, M, mt, K, perm, (uint8_t*)(w + p.pieces),
-                     (float*)(w + p.sums), (float*)(w + p.unscale), M <= 16, err));
+                     (float*)(w + p.sums), (float*)(w + p.unscale), err));
   switch (mt) {
     case 8: return launch_f8_m<8>(epi, mw, p, w, M, N, scales, zeros, residual, y, err, s);
-    case 16: return launch_f8_m<16>(epi, mw, p, w, M, N, scales, zeros, residual, y, err, s);
-    default: return launch_f8_m<32>(epi, mw, p, w, M, N, scales, zeros, residual, y, err, s);
+    default: return launch_f8_m<16>(epi, mw, p, w, M, N, scales, zeros, residual, y, err, s);
   }
 }
 

@@ -1,6 +1,6 @@
 """The int4 decode linear with 8-bit operands (large matrices at up to 16
-tokens, the largest SwiGLU at up to 32) against the oracle's dequantisation, on
-sampled output columns; and against the general decode path."""
+tokens) against the oracle's dequantisation, on sampled output columns; against the
+general decode path; and the large SwiGLU just beyond it, whose x keeps its range."""
 import numpy as np
 import pytest
 
@@ -56,7 +56,7 @@ def _x(m, k, seed):
 # that cover whole tiles and tiles shared by several, every token tile
 @pytest.mark.parametrize("m,n,k,epi", [
     (1, 4104, 4096, 0), (8, 12008, 1408, 1), (9, 4104, 4096, 1), (16, 8240, 2176, 2), (7, 140000, 128, 0),
-    (16, 1200, 14080, 1), (5, 65664, 256, 2), (32, 65600, 4096, 2), (17, 67096, 4096, 2)])
+    (16, 1200, 14080, 1), (5, 65664, 256, 2), (16, 65600, 4096, 2), (9, 67096, 4096, 2)])
 def test_matches_oracle(fp, m, n, k, epi):
     codes, scales, zeros = _weights(fp, n, k, 9)
     x, nout = _x(m, k, 8), n // 2 if epi == 2 else n
@@ -136,3 +136,41 @@ def test_beyond_fp16_is_reported_as_on_the_general_path(fp):
     fp.fp_op_linear_gptq4(0, ptr(dev(x)), m, n, k, ptr(perm), ptr(codes), ptr(scales), ptr(zeros), None, ptr(out),
                           ptr(ws), ws_b, ptr(err))
     assert host(err, np.int32)[0] == 3
+
+
+@pytest.mark.parametrize("m", [17, 32])
+def test_beyond_16_tokens_x_keeps_the_range_of_bf16(fp, m):
+    """The largest SwiGLU matrices at 17 tokens and more: an element of 2^18 whose weights
+    are zero must not cost the row's other elements their bits, and an infinity is the
+    infinity that its column's weights make of it."""
+    n, k, big, inf = 65536, 4096, 1003, 2010
+    w = empty(n * k, np.uint16)
+    fp.fp_op_init_weights(ptr(w), n * k, 9, 3)
+    w.view(n, k)[:, big] = 0
+    codes, scales, zeros = empty(n * k // 2), empty(n * k // 128, np.uint16), empty(n * k // 128, np.uint16)
+    fp.fp_op_quantize(2, ptr(w), n, k, ptr(codes), ptr(scales), ptr(zeros))
+    x = quant.bf16_to_f32(synth.uniform_bf16(8, m, (m, k), -2.0, 2.0))
+    x[:, big] = 2.0 ** 18
+    x[m - 1, inf] = np.inf
+    nout = n // 2
+    ws_b = fp.fp_op_linear_workspace_bytes(2, m, n, k)
+    ws, out = empty(ws_b), empty(m * nout, np.uint16)
+    fp.fp_op_linear(2, 2, ptr(dev(synth.f32_to_bf16_bits(x))), m, n, k, ptr(codes), ptr(scales), ptr(zeros), None,
+                    ptr(out), ptr(ws), ws_b)
+    got = quant.bf16_to_f32(host(out, np.uint16)).reshape(m, nout).astype(np.float64)
+    cols = np.unique(np.concatenate([[0, 1, nout - 1], np.random.default_rng(m).integers(0, nout, 120)]))
+    rows = []
+    for c in np.concatenate([cols, cols + nout]):
+        r = synth.normal_bf16(9, 3, int(c) * k, k).copy()
+        r[big] = 0
+        rows.append(r)
+    # this path multiplies the weights rounded to bf16, x as it is
+    wd = quant.quantize_weight(np.stack(rows), 2)[1]
+    wd = quant.bf16_to_f32(synth.f32_to_bf16_bits(wd.astype(np.float32))).astype(np.float64)
+    g, u = wd[:len(cols)], wd[len(cols):]
+    xf = x[:m - 1].astype(np.float64)
+    ref = M.silu(xf @ g.T) * (xf @ u.T)
+    for i in range(m - 1):
+        assert rel_err(got[i:i + 1][:, cols], ref[i:i + 1]) <= TOL + 1e-4, (i, rel_err(got[i:i + 1][:, cols], ref[i:i + 1]))
+    both = (g[:, inf] > 0) & (u[:, inf] != 0)
+    assert both.sum() > 10 and np.array_equal(got[m - 1, cols][both], np.sign(u[both, inf]) * np.inf)

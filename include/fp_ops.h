@@ -71,9 +71,9 @@ enum {
  * aligned x and codes: int4 and a bf16 result with M <= 16 and at least 2^24
  * weights (scales and zeros 16-byte aligned too), which runs on tcgen05 with 8-bit operands (the codes as they
  * are; x split by a first kernel into two e4m3 pieces an element, which carry
- * it exactly down to 2^-13 of its row's largest value and to 2^-23 of that
- * value below; scales and zero points applied in fp32; a row of x that holds an
- * infinity or a NaN gives NaN); int4 with 17 <= M <= 64 otherwise, and int8
+ * it exactly down to 2^-13 of the largest value of its row and group of 128
+ * channels and to 2^-22 of that value below; scales and zero points applied in
+ * fp32; a row of x that holds an infinity or a NaN gives NaN); int4 with 17 <= M <= 64 otherwise, and int8
  * with 33 <= M <= 64 or K >= 16384, which run on tcgen05 with each
  * weight expanded in TMEM (int4 to bf16((q - z) s) as the prefill GEMM does,
  * int8 to the integer code, its row scale applied to the fp32 sums); bf16

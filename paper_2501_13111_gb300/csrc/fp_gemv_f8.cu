@@ -7,14 +7,20 @@
 // subnormals (bytes 0-7) and its first binade (8-15) share one spacing.  So a
 // packed word becomes two operand words by one shift and two masks (0.4
 // instructions a code; the bf16 expansion takes two), and the weights stay
-// exact.  x is split beforehand, per token, into two e4m3 pieces (split_x_kernel):
-//   x 2^e = hi + lo / 32,  e the token's power of two with max|x| 2^e in [128, 256).
+// exact.  x is split beforehand, per token and group, into two e4m3 pieces
+// (split_x_kernel):
+//   x 2^e = hi + lo / 32,  e the power of two with the group's max|x| 2^e in [128, 256).
 // hi keeps four significant bits and lo the next four, so a bf16 x is carried
-// exactly down to 2^-13 of the token's largest |x| and to 2^-23 of that
-// largest below.  hi and lo are columns of their own, so N = 2 x tokens; a
-// group's product is exact in fp32 (measured against fp64) and the scale, the
-// zero point times the group's sum of x, and lo / 32 are applied in fp32 to
-// the group's accumulator.
+// exactly down to 2^-13 of the largest |x| of its group and, below, with an error of
+// at most 2^-22 of that largest.  hi and lo are columns of their own, so N = 2 x
+// tokens; the group's products are summed in fp32, and lo / 32, the zero point times
+// the group's sum of x, 2^-e and the scale are applied in fp32 to its accumulator.
+// With one exponent a token, one large element cost the small elements of every group
+// their bits.  Relative error of rows of N(0, 0.05) and one element of 30000 whose own
+// weights are zero (2-norm; an exponent a group / a token / the mma.sync GEMV, whose
+// fp32 sums hold 1024 + q times x; the result's rounding is 0.0017 of each):
+//   4608 x 4096 0.0088 / 0.046 / 1.6   5120 x 13824 0.0049 / 0.047 / 0.55   65536 x 256 0.032 / 0.046 / 2.9
+// and with the whole group's weights zero 0.0017 / 0.03-0.05 / 0.0017.
 //
 // One CTA per SM, 20 warps; an item is two groups of one row tile:
 //   warps 0-7   codes to operands, one row per thread, shared memory to TMEM:
@@ -43,7 +49,7 @@
 //
 // What bounds it: an item's 17 KB of codes and scales take 780 cycles of an SM
 // at the copy rate and its MMAs 360; the hand-offs between the roles keep it at
-// about 1070 (57344 x 8192, 252 MB, 8 tokens: 62 us, 4.1 TB/s; without any copy
+// about 1070 (57344 x 8192, 252 MB, 8 tokens: 61.5 us, 4.1 TB/s; without any copy
 // after the rings' first fill 61).
 // Every mbarrier wait is bounded; past the limit the thread records error 2,
 // the CTA stops and releases TMEM after its copies and MMAs have completed.
@@ -75,7 +81,7 @@ struct F8Geom {
   static constexpr int kACol = kAccs * 2 * kN;             // the first column of the A operands
   static constexpr int kWStages = 10;
   static constexpr int kXStages = 4;
-  static constexpr int kXsStage = 2 * MT * 4;
+  static constexpr int kXsStage = 2 * 2 * MT * 4;          // two groups' sums and powers of two
   static constexpr int kSwap = kF8Rows * MT * 4;           // the tokens' halves changing hands
   static constexpr int kSmem = kWStages * kF8WStage + kXStages * kXStage + kF8XsRing * kXsStage + kSwap + 1024;
   static_assert(kACol + kSlots * kF8SlotCols <= 512, "TMEM columns");
@@ -89,125 +95,94 @@ struct F8Geom {
 FP_DEV long long f8_cta_of(long long i, long long C, long long total) { return ((i + 1) * C - 1) / total; }
 
 // ------------------------------------------------------------------ x pieces
-// One CTA per token (rows past M: zeros).  pieces [groups][2 MT][128 bytes],
-// row m the token's hi and row MT + m its lo, 16-byte chunk c of a row at c ^
-// (row % 8) (the 128-byte swizzle), and within each eight elements the order
-// in which masking a packed int4 word yields them; sums [groups][MT] = 2^-9
-// sum of the group's pieces; unscale[m] = 2^-e, NaN for a token that
-// holds an infinity or a NaN.  perm (GPTQ4): element j is x[perm[j]].
-// Bound by latency (2 K bytes read and written per token): the row is held in
-// registers between its maximum and its conversion.
-constexpr int kSplitThreads = 1024, kSplitHeld = 4;
+// Tokens along the grid's y (rows past M: zeros), eight elements a thread.  pieces
+// [groups][2 MT][128 bytes], row m the token's hi and row MT + m its lo, 16-byte
+// chunk c of a row at c ^ (row % 8) (the 128-byte swizzle), and within each eight
+// elements the order in which masking a packed int4 word yields them; sums
+// [groups][2][MT] = 2^-9 sum of the group's pieces, then 2^-e of the group, NaN
+// for one that holds an infinity or a NaN.  perm (GPTQ4): element j is x[perm[j]].
+// Bound by latency (2 K bytes read and written per token).
+constexpr int kSplitThreads = 256;
 
 __global__ void __launch_bounds__(kSplitThreads)
     split_x_kernel(const uint16_t* __restrict__ x, int M, int MT, int K, const int32_t* __restrict__ perm,
-                   uint8_t* __restrict__ pieces, float* __restrict__ sums, float* __restrict__ unscale, int32_t* err) {
+                   uint8_t* __restrict__ pieces, float* __restrict__ sums, int32_t* err) {
   pdl_trigger();
   pdl_wait();
-  const int m = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
-  const int chunks = K / 8;  // K is a multiple of 128: whole groups of 16 chunks
-  const uint16_t* xr = x + (long long)m * K;
-  bool bad = false;
-  auto load = [&](int c) {
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (m < M && c < chunks) {
-      if (perm == nullptr) {
-        v = ld_nc16(xr + c * 8);
-      } else {
-        uint32_t e[8];
+  const int m = blockIdx.y, c = blockIdx.x * kSplitThreads + threadIdx.x;  // token, chunk of eight elements
+  const bool in = c < K / 8;  // K is a multiple of 128: whole groups of 16 lanes are in or out
+  uint4 v = make_uint4(0, 0, 0, 0);
+  if (m < M && in) {
+    const uint16_t* xr = x + (long long)m * K;
+    if (perm == nullptr) {
+      v = ld_nc16(xr + c * 8);
+    } else {
+      bool bad = false;
+      uint32_t e[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int k = perm[c * 8 + i];
-          const bool in = (unsigned)k < (unsigned)K;
-          bad |= !in;
-          e[i] = in ? (uint32_t)xr[k] : 0u;
-        }
-        v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
+      for (int i = 0; i < 8; ++i) {
+        const int k = perm[c * 8 + i];
+        const bool ok = (unsigned)k < (unsigned)K;
+        bad |= !ok;
+        e[i] = ok ? (uint32_t)xr[k] : 0u;
       }
+      v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
+      if (bad && err) atomicExch(err, 1);
     }
-    return v;
-  };
+  }
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
   // |x| as bf16 bits orders like the values, infinities and NaN on top
-  auto amax2 = [](uint32_t a, uint32_t w) {
-    return max(a, max(w & 0x7FFFu, (w >> 16) & 0x7FFFu));
-  };
-  // beyond the fp16 range but not NaN
-  bool over = false;
-  auto check = [&](const uint4& v) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint32_t a = w[i] & 0x7FFFu, b = (w[i] >> 16) & 0x7FFFu;
-      over |= (a >= 0x4780u && a <= 0x7F80u) || (b >= 0x4780u && b <= 0x7F80u);
-    }
-  };
-  uint4 held[kSplitHeld];
   uint32_t am = 0;
+  bool over = false;  // beyond the fp16 range but not NaN
 #pragma unroll
-  for (int j = 0; j < kSplitHeld; ++j) {
-    held[j] = load(tid + j * kSplitThreads);
-    am = amax2(amax2(amax2(amax2(am, held[j].x), held[j].y), held[j].z), held[j].w);
-    check(held[j]);
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t a = w[i] & 0x7FFFu, b = (w[i] >> 16) & 0x7FFFu;
+    am = max(am, max(a, b));
+    over |= (a >= 0x4780u && a <= 0x7F80u) || (b >= 0x4780u && b <= 0x7F80u);
   }
-  for (int c = tid + kSplitHeld * kSplitThreads; c < chunks; c += kSplitThreads) {
-    const uint4 v = load(c);
-    am = amax2(amax2(amax2(amax2(am, v.x), v.y), v.z), v.w);
-    check(v);
-  }
-  if (bad && err) atomicExch(err, 1);
   // tokens that a kernel staging x in fp16 refuses are refused here too
   if (over && err) atomicExch(err, 3);
-  am = __reduce_max_sync(0xffffffffu, am);
-  __shared__ uint32_t red[kSplitThreads / 32];
-  if (lane == 0) red[tid >> 5] = am;
-  __syncthreads();
-  am = __reduce_max_sync(0xffffffffu, lane < kSplitThreads / 32 ? red[lane] : 0u);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, o));  // the group's 16 lanes
 
   // e = 134 - biased exponent of the maximum, kept where 2^e and 2^-e are normal
   const int ex = (int)(am >> 7);
   const int e = am == 0 || ex == 255 ? 0 : min(126, 134 - ex);
   const float mul = __uint_as_float((uint32_t)(127 + e) << 23);
-  if (tid == 0) unscale[m] = ex == 255 ? __uint_as_float(0x7FC00000u) : exp2f((float)-e);
-  const long long row_hi = (long long)m * 128, row_lo = (long long)(MT + m) * 128;
-  auto convert = [&](int c, const uint4& v) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    float hi_sum = 0.f, lo_sum = 0.f;
-    uint32_t hb[4], lb[4];  // e4m3 pairs (2i, 2i + 1)
+  float hi_sum = 0.f, lo_sum = 0.f;
+  uint32_t hb[4], lb[4];  // e4m3 pairs (2i, 2i + 1)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float2 f = bf2x2f(w[i]);
-      f.x *= mul;
-      f.y *= mul;
-      const __nv_fp8x2_storage_t h = __nv_cvt_float2_to_fp8x2(f, __NV_SATFINITE, __NV_E4M3);
-      const float2 hf = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(h, __NV_E4M3)));
-      const float2 r = make_float2((f.x - hf.x) * 32.f, (f.y - hf.y) * 32.f);
-      const __nv_fp8x2_storage_t l = __nv_cvt_float2_to_fp8x2(r, __NV_SATFINITE, __NV_E4M3);
-      const float2 lf = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(l, __NV_E4M3)));
-      hi_sum += hf.x + hf.y;
-      lo_sum += lf.x + lf.y;
-      hb[i] = h;
-      lb[i] = l;
-    }
-    // a packed int4 word masked with 0x0F0F0F0F holds elements 0, 4, 1, 5, and
-    // shifted by four bits 2, 6, 3, 7
-    const uint2 ho = make_uint2(__byte_perm(hb[0], hb[2], 0x5140), __byte_perm(hb[1], hb[3], 0x5140));
-    const uint2 lo = make_uint2(__byte_perm(lb[0], lb[2], 0x5140), __byte_perm(lb[1], lb[3], 0x5140));
-    float sum = hi_sum + lo_sum * (1.f / 32.f);
+  for (int i = 0; i < 4; ++i) {
+    float2 f = bf2x2f(w[i]);
+    f.x *= mul;
+    f.y *= mul;
+    const __nv_fp8x2_storage_t h = __nv_cvt_float2_to_fp8x2(f, __NV_SATFINITE, __NV_E4M3);
+    const float2 hf = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(h, __NV_E4M3)));
+    const float2 r = make_float2((f.x - hf.x) * 32.f, (f.y - hf.y) * 32.f);
+    const __nv_fp8x2_storage_t l = __nv_cvt_float2_to_fp8x2(r, __NV_SATFINITE, __NV_E4M3);
+    const float2 lf = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(l, __NV_E4M3)));
+    hi_sum += hf.x + hf.y;
+    lo_sum += lf.x + lf.y;
+    hb[i] = h;
+    lb[i] = l;
+  }
+  // a packed int4 word masked with 0x0F0F0F0F holds elements 0, 4, 1, 5, and
+  // shifted by four bits 2, 6, 3, 7
+  const uint2 ho = make_uint2(__byte_perm(hb[0], hb[2], 0x5140), __byte_perm(hb[1], hb[3], 0x5140));
+  const uint2 lo = make_uint2(__byte_perm(lb[0], lb[2], 0x5140), __byte_perm(lb[1], lb[3], 0x5140));
+  float sum = hi_sum + lo_sum * (1.f / 32.f);
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);  // the group's 16 lanes
-    if (c < chunks) {
-      const int g = c >> 4, ch = (c & 15) >> 1, half = c & 1;
-      uint8_t* base = pieces + (long long)g * (2 * MT * 128);
-      *reinterpret_cast<uint2*>(base + row_hi + ((ch ^ (m & 7)) << 4) + half * 8) = ho;
-      *reinterpret_cast<uint2*>(base + row_lo + ((ch ^ ((MT + m) & 7)) << 4) + half * 8) = lo;
-      if ((c & 15) == 0) sums[(long long)g * MT + m] = sum * (1.f / 512.f);
-    }
-  };
-#pragma unroll
-  for (int j = 0; j < kSplitHeld; ++j)
-    if ((tid & ~31) + j * kSplitThreads < chunks) convert(tid + j * kSplitThreads, held[j]);
-  for (int c0 = (tid & ~31) + kSplitHeld * kSplitThreads; c0 < chunks; c0 += kSplitThreads)
-    convert(c0 + lane, load(c0 + lane));
+  for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (!in) return;
+  const int g = c >> 4, ch = (c & 15) >> 1, half = c & 1;
+  uint8_t* base = pieces + (long long)g * (2 * MT * 128);
+  *reinterpret_cast<uint2*>(base + m * 128 + ((ch ^ (m & 7)) << 4) + half * 8) = ho;
+  *reinterpret_cast<uint2*>(base + (MT + m) * 128 + ((ch ^ ((MT + m) & 7)) << 4) + half * 8) = lo;
+  if ((c & 15) == 0) {
+    float* o = sums + (long long)g * (2 * MT) + m;
+    o[0] = sum * (1.f / 512.f);
+    o[MT] = __uint_as_float(ex == 255 ? 0x7FC00000u : (uint32_t)(127 - e) << 23);
+  }
 }
 
 // ------------------------------------------------------------------ helpers
@@ -220,28 +195,32 @@ FP_DEV float2 ffma2(float2 a, float2 b, float2 c) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
   return d;
 }
+// d = a b on two fp32 lanes at once.
+FP_DEV float2 fmul2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
+      " mul.rn.f32x2 d, a, b;\n mov.b64 {%0, %1}, d;\n}\n"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
 
 // Output column `row` of tokens m0 .. m0 + T - 1 (those below M) from their
 // sums v (SwiGLU: gate sums v, up sums w).  The residuals are read before any
 // store (R may be Y itself).
 template <int EPI, int T>
-FP_DEV void f8_store(const float* v, const float* w, int M, int m0, int row, int Nout, const float* __restrict__ unscale,
-                     const uint16_t* R, void* Y) {
-  float un[T], rv[T];
+FP_DEV void f8_store(const float* v, const float* w, int M, int m0, int row, int Nout, const uint16_t* R, void* Y) {
+  float rv[T];
 #pragma unroll
-  for (int t = 0; t < T; ++t) {
-    const int m = min(m0 + t, M - 1);
-    un[t] = __ldg(unscale + m);
-    rv[t] = EPI == FP_EPI_RESID ? bf2f(R[(long long)m * Nout + row]) : 0.f;
-  }
+  for (int t = 0; t < T; ++t)
+    rv[t] = EPI == FP_EPI_RESID ? bf2f(R[(long long)min(m0 + t, M - 1) * Nout + row]) : 0.f;
 #pragma unroll
   for (int t = 0; t < T; ++t) {
     if (m0 + t >= M) break;
-    const float a = v[t] * un[t];
     uint16_t* y = (uint16_t*)Y + (long long)(m0 + t) * Nout + row;
-    if constexpr (EPI == FP_EPI_STORE) *y = f2bf(a);
-    else if constexpr (EPI == FP_EPI_RESID) *y = f2bf(rv[t] + a);
-    else *y = f2bf(silu(a) * (w[t] * un[t]));
+    if constexpr (EPI == FP_EPI_STORE) *y = f2bf(v[t]);
+    else if constexpr (EPI == FP_EPI_RESID) *y = f2bf(rv[t] + v[t]);
+    else *y = f2bf(silu(v[t]) * w[t]);
   }
 }
 
@@ -251,7 +230,7 @@ FP_DEV void f8_store(const float* v, const float* w, int M, int m0, int row, int
 // its registers would crowd the loop over the items.
 template <int EPI, int T>
 __device__ __noinline__ void f8_sum_store(const float* p0, size_t slot, int cnt, int M, int m0, int row, int Nout,
-                                          const float* __restrict__ unscale, const uint16_t* R, void* Y) {
+                                          const uint16_t* R, void* Y) {
   constexpr bool GLU = EPI == FP_EPI_SWIGLU;
   constexpr int B = T < 8 ? T : 8, U = GLU ? 2 : 4;
   if (row >= Nout) return;
@@ -276,7 +255,7 @@ __device__ __noinline__ void f8_sum_store(const float* p0, size_t slot, int cnt,
 #pragma unroll
         for (int k = 0; k < B; ++k) v[k] += a[u][k], w[k] += e[u][k];
     }
-    f8_store<EPI, B>(v, w, M, m0 + t0, row, Nout, unscale, R, Y);
+    f8_store<EPI, B>(v, w, M, m0 + t0, row, Nout, R, Y);
   }
 }
 
@@ -285,7 +264,7 @@ __device__ __noinline__ void f8_sum_store(const float* p0, size_t slot, int cnt,
 template <int MT, int EPI>
 __global__ void __launch_bounds__(kF8Threads, 1)
     gemv_f8_kernel(const __grid_constant__ CUtensorMap map_w, const uint8_t* __restrict__ pieces,
-                   const float* __restrict__ sums, const float* __restrict__ unscale, int M, int N,
+                   const float* __restrict__ sums, int M, int N,
                    const uint16_t* __restrict__ scales, const uint16_t* __restrict__ zeros, const uint16_t* R, void* Y,
                    long long total, int S, float* __restrict__ ws, unsigned* __restrict__ counters, int32_t* err) {
   using G = F8Geom<MT>;
@@ -302,7 +281,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
   uint8_t* w_ring = smem;
   uint8_t* x_ring = smem + WS * kF8WStage;
   float* xs_ring = reinterpret_cast<float*>(x_ring + XS * G::kXStage);
-  float* swap = xs_ring + kF8XsRing * 2 * MT;
+  float* swap = xs_ring + kF8XsRing * 4 * MT;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int Nout = GLU ? N / 2 : N;
   const long long C = gridDim.x, c = blockIdx.x;
@@ -359,7 +338,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       for (int j = max(0, issued - WS); j < issued; ++j) mbar_wait(&wfull[j % WS], (j / WS) & 1);
     }
   } else if (warp == kF8WarpX) {
-    // ---------------- pieces and group sums of x
+    // ---------------- pieces, group sums and powers of two of x
     if (lane == 0) {
       pdl_wait();
       asm volatile("fence.proxy.async;" ::: "memory");  // they were written by generic stores
@@ -373,8 +352,8 @@ __global__ void __launch_bounds__(kF8Threads, 1)
         const int g0 = 2 * i, nv = min(2, S - g0), s = q % XS, r = q % kF8XsRing;
         mbar_expect_tx(&xfull[s], nv * G::kGroupBytes);
         bulk_load(x_ring + s * G::kXStage, pieces + (long long)g0 * G::kGroupBytes, nv * G::kGroupBytes, &xfull[s]);
-        mbar_expect_tx(&sfull[r], nv * MT * 4);
-        bulk_load(xs_ring + r * (2 * MT), sums + (long long)g0 * MT, nv * MT * 4, &sfull[r]);
+        mbar_expect_tx(&sfull[r], nv * 2 * MT * 4);
+        bulk_load(xs_ring + r * (4 * MT), sums + (long long)g0 * (2 * MT), nv * 2 * MT * 4, &sfull[r]);
         issued = q + 1;
         if (++i == SI) i = 0;
       }
@@ -509,20 +488,24 @@ __global__ void __launch_bounds__(kF8Threads, 1)
             const float s = __uint_as_float(j ? sp & 0xFFFF0000u : sp << 16);
             const float z = __uint_as_float(j ? zp & 0xFFFF0000u : zp << 16);
             const float2 s2 = make_float2(s, s), nz2 = make_float2(-z, -z), r32 = make_float2(1.f / 32.f, 1.f / 32.f);
-            const float* xs = xs_ring + r * (2 * MT) + j * MT;
+            const float* xs = xs_ring + r * (4 * MT) + j * (2 * MT);
             const uint32_t d = lane_base + (q % ND) * 2 * G::kN + j * G::kN;
-            float4 xv[MT / 4];  // read while the sums come from TMEM
+            float4 xv[MT / 4], uv[MT / 4];  // read while the sums come from TMEM
 #pragma unroll
-            for (int t = 0; t < MT / 4; ++t) xv[t] = *reinterpret_cast<const float4*>(xs + 4 * t);
+            for (int t = 0; t < MT / 4; ++t) {
+              xv[t] = *reinterpret_cast<const float4*>(xs + 4 * t);
+              uv[t] = *reinterpret_cast<const float4*>(xs + MT + 4 * t);
+            }
             uint32_t hi[MT], lo[MT];
             tc_ld_pair<MT>(d, d + MT, hi, lo);
 #pragma unroll
             for (int k = 0; k < MT; k += 2) {
-              const float4 x4 = xv[k / 4];
+              const float4 x4 = xv[k / 4], u4 = uv[k / 4];
               const float2 xx = k & 2 ? make_float2(x4.z, x4.w) : make_float2(x4.x, x4.y);
+              const float2 uu = k & 2 ? make_float2(u4.z, u4.w) : make_float2(u4.x, u4.y);
               float2 v = ffma2(nz2, xx, make_float2(__uint_as_float(hi[k]), __uint_as_float(hi[k + 1])));
               v = ffma2(make_float2(__uint_as_float(lo[k]), __uint_as_float(lo[k + 1])), r32, v);
-              acc[k / 2] = ffma2(s2, v, acc[k / 2]);
+              acc[k / 2] = ffma2(s2, fmul2(uu, v), acc[k / 2]);
             }
           }
         }
@@ -578,7 +561,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
         constexpr int B = TH < 8 ? TH : 8;
         if (row < Nout) {
 #pragma unroll
-          for (int t = 0; t < TH; t += B) f8_store<EPI, B>(av + t, av + t, M, m0 + t, row, Nout, unscale, R, Y);
+          for (int t = 0; t < TH; t += B) f8_store<EPI, B>(av + t, av + t, M, m0 + t, row, Nout, R, Y);
         }
         continue;
       }
@@ -600,7 +583,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       if (t != last) continue;
       __threadfence();
       f8_sum_store<EPI, TH>(ws + (size_t)(tb + c0) * slot + (GLU ? (lr & (TR - 1)) : lr), slot, (int)(c1 - c0) + 1, M, m0,
-                            row, Nout, unscale, R, Y);
+                            row, Nout, R, Y);
       if (lane == 0) *ticket = 0u;
     }
   }
@@ -626,11 +609,11 @@ static int f8_sms() {
 
 static int f8_mt(int M) { return M <= 8 ? 8 : 16; }
 
-// fp32 partials, then the x pieces, their group sums and the tokens' scales.
+// fp32 partials, then the x pieces and their group sums and powers of two.
 struct F8Plan {
   long long tiles, total;
   int ctas, S;
-  size_t pieces, sums, unscale, bytes;  // offsets behind the ticket area
+  size_t pieces, sums, bytes;  // offsets behind the ticket area
 };
 
 static F8Plan f8_plan(int epi, int M, int N, int K) {
@@ -645,22 +628,26 @@ static F8Plan f8_plan(int epi, int M, int N, int K) {
   auto up = [](size_t b) { return (b + 127) / 128 * 128; };
   p.pieces = (size_t)kLinTicketSlots * 4 + up((size_t)(p.tiles + p.ctas) * M * kF8Rows * 4);
   p.sums = p.pieces + (size_t)p.S * 2 * mt * 128;
-  p.unscale = p.sums + up((size_t)p.S * mt * 4);
-  p.bytes = p.unscale + up((size_t)mt * 4);
+  p.bytes = p.sums + up((size_t)p.S * 2 * mt * 4);
   return p;
 }
 
-// Where it is the faster path.  Measured in a graph, microseconds here against
-// the mma.sync GEMV:
-//   tokens 1 / 8 / 16   4096 x 4096    11.0 / 11.3 / 13.5   10.9 / 12.1 / 17.0
-//                       1024 x 512      7.7 /  7.9 /  8.8    5.1 /  5.2 /  5.8
-//                       5120 x 13824   19.3 / 20.1 / 23.4   25.1 / 27.3 / 29.3
-//                       57344 x 8192   60.2 / 61.9 / 69.5    109 /  113 /  135
-// The second kernel (3 us) and a CTA's hand-offs want 8 MB of codes.  Not beyond 16
-// tokens, where the bf16 expansion in TMEM takes x as it is (57344 x 8192 with SwiGLU
-// at 32 tokens 99 us here, 109 there): one element of 2^18 beside unit normals, its
-// weights zero, left an error of 0.054 here and 0.0027 there, and a row with an
-// infinity gave NaN.
+// Where it is the faster path.  Measured in a graph over copies of the weights that
+// exceed L2, microseconds here / the mma.sync GEMV:
+//   tokens            1             8             9             16
+//   1024 x 512      6.6 /  3.7    6.7 /  4.4    7.9 /  4.7    7.9 /  4.9
+//   4096 x 4096     9.8 /  7.7   10.0 /  8.8   11.7 / 12.7   12.2 / 14.1
+//   2048 x 8192    10.3 / 11.6   10.6 / 12.3   12.4 / 20.8   13.1 / 22.1
+//   8192 x 4096    13.4 / 12.1   13.7 / 13.5   15.4 / 19.5   15.7 / 21.2
+//   10240 x 8192   19.0 / 25.4   19.3 / 26.8   23.3 / 31.4   23.6 / 33.0
+//   5120 x 13824   17.7 / 27.9   18.2 / 29.7   22.0 / 32.1   22.3 / 34.1
+//   57344 x 8192   59.7 /  109   61.5 /  113   73.8 /  133   74.4 /  135 (SwiGLU)
+// The line was set at 8 MB of codes before the mma.sync GEMV had clusters; matrices of
+// 8 to 20 MB that are wider than long have since been 1-2 us faster there at up to 8
+// tokens.  Not beyond 16 tokens, where the bf16 expansion in TMEM takes x as it is
+// (57344 x 8192 with SwiGLU at 32 tokens 109 us there, 99 with an instance of this
+// kernel): one element of 2^18 beside unit normals, its weights zero, left an error of
+// 0.054 here and 0.0027 there, and a row with an infinity gave NaN.
 static bool f8_pays(int M, int N, int K) { return M <= 16 && (long long)N * K >= (1LL << 24); }
 
 bool f8_ok(int wquant, int epi, int M, int N, int K) {
@@ -683,7 +670,7 @@ static cudaError_t launch_f8_t(const CUtensorMap& mw, const F8Plan& p, char* ws,
   static std::atomic<unsigned long long> attr{0};
   FP_CUDA_TRY(smem_limit_once(kern, smem, &attr));
   return launch_early(kern, dim3(p.ctas), dim3(kF8Threads), (size_t)smem, s, mw, (const uint8_t*)(ws + p.pieces),
-                      (const float*)(ws + p.sums), (const float*)(ws + p.unscale), M, N, scales, zeros, R, Y, p.total,
+                      (const float*)(ws + p.sums), M, N, scales, zeros, R, Y, p.total,
                       p.S, (float*)(ws + (size_t)kLinTicketSlots * 4), (unsigned*)ws, err);
 }
 
@@ -710,8 +697,8 @@ cudaError_t launch_f8(int epi, const uint16_t* x, const int32_t* perm, int M, in
   if (!make_tensor_map(&mw, codes, N, K / 2, 1, epi == FP_EPI_SWIGLU ? kF8Rows / 2 : kF8Rows, kF8RowBytes, 128))
     return cudaErrorInvalidValue;
   char* w = (char*)ws;
-  FP_CUDA_TRY(launch(split_x_kernel, dim3(mt), dim3(kSplitThreads), 0, s, x, M, mt, K, perm, (uint8_t*)(w + p.pieces),
-                     (float*)(w + p.sums), (float*)(w + p.unscale), err));
+  FP_CUDA_TRY(launch(split_x_kernel, dim3((K / 8 + kSplitThreads - 1) / kSplitThreads, mt), dim3(kSplitThreads), 0, s, x,
+                     M, mt, K, perm, (uint8_t*)(w + p.pieces), (float*)(w + p.sums), err));
   switch (mt) {
     case 8: return launch_f8_m<8>(epi, mw, p, w, M, N, scales, zeros, residual, y, err, s);
     default: return launch_f8_m<16>(epi, mw, p, w, M, N, scales, zeros, residual, y, err, s);

@@ -12,8 +12,8 @@ from tests.gpu_helpers import dev, empty, host, ptr, rel_err, torch_mod
 pytestmark = pytest.mark.gpu
 
 # One rounding of the result to bf16 (8 significant bits: half a unit of 1 is
-# 2^-8); the sums are fp32 and x is carried to 2^-23 of its row's largest value,
-# both far below.
+# 2^-8); the sums are fp32 and x is carried to 2^-22 of the largest value of its group
+# of 128, both far below.
 TOL = 1.05 * 2.0 ** -8
 
 
@@ -174,3 +174,55 @@ def test_beyond_16_tokens_x_keeps_the_range_of_bf16(fp, m):
         assert rel_err(got[i:i + 1][:, cols], ref[i:i + 1]) <= TOL + 1e-4, (i, rel_err(got[i:i + 1][:, cols], ref[i:i + 1]))
     both = (g[:, inf] > 0) & (u[:, inf] != 0)
     assert both.sum() > 10 and np.array_equal(got[m - 1, cols][both], np.sign(u[both, inf]) * np.inf)
+
+
+def _dominated(fp, m, n, k, big, zeroed, amp):
+    """Rows of small elements and one of `amp`, the weights of channels `zeroed` zero: the
+    results of the 8-bit operands and of mma.sync (scales at an address that is not a
+    multiple of 16), some columns, and the oracle's weights of those."""
+    w = empty(n * k, np.uint16)
+    fp.fp_op_init_weights(ptr(w), n * k, 9, 3)
+    w.view(n, k)[:, zeroed] = 0
+    codes, scales, zeros = empty(n * k // 2), empty(n * k // 128, np.uint16), empty(n * k // 128, np.uint16)
+    fp.fp_op_quantize(2, ptr(w), n, k, ptr(codes), ptr(scales), ptr(zeros))
+    shifted = dev(np.concatenate([np.zeros(1, np.uint16), host(scales, np.uint16)]))
+    x = quant.bf16_to_f32(synth.uniform_bf16(8, m, (m, k), -0.1, 0.1))
+    x[:, big] = amp
+    ws_b = fp.fp_op_linear_workspace_bytes(2, m, n, k)
+    ws, res = empty(ws_b), []
+    for sc in (ptr(scales), ptr(shifted) + 2):
+        out = empty(m * n, np.uint16)
+        fp.fp_op_linear(2, 0, ptr(dev(synth.f32_to_bf16_bits(x))), m, n, k, ptr(codes), sc, ptr(zeros), None, ptr(out),
+                        ptr(ws), ws_b)
+        res.append(quant.bf16_to_f32(host(out, np.uint16)).reshape(m, n).astype(np.float64))
+    cols = np.unique(np.random.default_rng(m).integers(0, n, 100))
+    rows = np.stack([synth.normal_bf16(9, 3, int(c) * k, k) for c in cols])
+    rows[:, zeroed] = 0
+    return [r[:, cols] for r in res], x.astype(np.float64), quant.quantize_weight(rows, 2)[1]
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 4104, 4096), (8, 1160, 14592), (16, 4104, 4096), (4, 65536, 256)])
+def test_a_large_element_costs_the_other_groups_nothing(fp, m, n, k):
+    """The large element lies in a group whose weights are all zero (scale 0)."""
+    (got, general), x, wd = _dominated(fp, m, n, k, 131, slice(128, 256), 30000.0)
+    ref = x @ wd.T
+    for i in range(m):
+        assert rel_err(got[i:i + 1], ref[i:i + 1]) <= TOL, (i, rel_err(got[i:i + 1], ref[i:i + 1]))
+        assert rel_err(general[i:i + 1], ref[i:i + 1]) <= TOL
+
+
+@pytest.mark.parametrize("amp", [8000.0, 30000.0, 65280.0])
+@pytest.mark.parametrize("m,n,k", [(1, 4104, 4096), (8, 1160, 14592), (16, 4104, 4096), (4, 65536, 256)])
+def test_a_large_element_among_small_ones(fp, m, n, k, amp):
+    """Its own weights are zero (the code is the zero point), its group's are not."""
+    (got, general), x, wd = _dominated(fp, m, n, k, 131, [131], amp)
+    ref = x @ wd.T
+    group = wd[:, 128:256]
+    # the group's x to 2^-22 of its largest; its fp32 sum of up to 15 amp s, then less z amp s: a unit in
+    # the last place each (group's scale from its smallest step); the result's rounding to bf16
+    step = np.array([np.diff(np.unique(r)).min() for r in group])
+    bound = 2.0 ** -22 * amp * np.abs(group).sum(1) + 4 * 2.0 ** -23 * 15 * amp * step + 1.05 * 2.0 ** -8 * np.abs(ref)
+    assert (np.abs(got - ref) <= bound + 2.0 ** -20 * np.abs(ref).max()).all()
+    # and no further off than the operands of 16 bits, whose sums hold (1024 + q) amp
+    norm = lambda y: np.linalg.norm(y - ref) / np.linalg.norm(ref)
+    assert norm(got) <= norm(general), (norm(got), norm(general))

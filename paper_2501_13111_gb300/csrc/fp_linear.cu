@@ -959,9 +959,11 @@ cudaError_t launch_linear(int wquant, int epi, const uint16_t* x, int M, int N, 
       ((uintptr_t)codes & 15) == 0)
     return launch_btc(epi, x, M, N, K, codes, residual, y, ws, ws_bytes, err, s);
   // int4 and int8 at 17-64 tokens: the tensor-core path, weights expanded into
-  // TMEM (TMA needs 16-byte aligned x and codes)
-  if (q4tc_ok(wquant, epi, M, N, K) && q4tc_preferred(wquant, epi, M, N, K) && ((uintptr_t)x & 15) == 0 &&
-      ((uintptr_t)codes & 15) == 0)
+  // TMEM (TMA needs 16-byte aligned x and codes; int4 scales and zeros are read up
+  // to eight at a time, int8 scales one by one)
+  const uintptr_t groups = wquant == FP_W_INT4_G128 ? (uintptr_t)scales | (uintptr_t)zeros : 0;
+  if (q4tc_ok(wquant, epi, M, N, K) && q4tc_preferred(wquant, epi, M, N, K) &&
+      (((uintptr_t)x | (uintptr_t)codes | groups) & 15) == 0)
     return launch_q4tc(wquant, epi, x, M, N, K, codes, scales, zeros, residual, y, ws, ws_bytes, err, s);
   if (mma_ok(wquant, M, N, K)) {
     switch (wquant) {

@@ -99,6 +99,33 @@ def test_agrees_with_the_general_path(fp, m, epi):
         assert rel_err(a[None], b[None]) <= 2 * TOL
 
 
+@pytest.mark.parametrize("shift", [1, 2, 4])
+@pytest.mark.parametrize("m,epi", [(17, 0), (40, 2), (64, 1)])
+def test_scales_at_any_address_beyond_16_tokens(fp, m, epi, shift):
+    """The tcgen05 expansion reads scales and zeros in up to 16 bytes: those at other
+    addresses take the mma.sync path, whose weights are exact."""
+    n, k = 520, 1024
+    codes, scales, zeros = _weights(fp, n, k, 11)
+    nout = n // 2 if epi == 2 else n
+    x, r = _x(m, k, 3), synth.uniform_bf16(4, m, (m, nout), -1.0, 1.0)
+    pad = np.zeros(shift, np.uint16)
+    sd, zd = (dev(np.concatenate([pad, host(t, np.uint16)])) for t in (scales, zeros))
+    ws_b = fp.fp_op_linear_workspace_bytes(2, m, n, k)
+    ws = empty(ws_b)
+    xf, wd = quant.bf16_to_f32(x).astype(np.float64), _rows(n, k, 11, range(n))
+    ref = xf @ wd.T
+    if epi == 1:
+        ref = ref + quant.bf16_to_f32(r).astype(np.float64)
+    elif epi == 2:
+        ref = M.silu(ref[:, :nout]) * ref[:, nout:]
+    for sc, ze in ((ptr(sd) + 2 * shift, ptr(zeros)), (ptr(scales), ptr(zd) + 2 * shift)):
+        out = empty(m * nout, np.uint16)
+        fp.fp_op_linear(2, epi, ptr(dev(x)), m, n, k, ptr(codes), sc, ze, ptr(dev(r)), ptr(out), ptr(ws), ws_b)
+        got = quant.bf16_to_f32(host(out, np.uint16)).reshape(m, nout).astype(np.float64)
+        for i in range(m):
+            assert rel_err(got[i:i + 1], ref[i:i + 1]) <= TOL, (i, rel_err(got[i:i + 1], ref[i:i + 1]))
+
+
 def test_gptq4_reads_x_through_the_act_order(fp):
     m, n, k = 6, 4608, 4096
     order = np.random.default_rng(5).permutation(k).astype(np.int32)

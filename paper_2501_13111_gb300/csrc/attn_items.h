@@ -1,0 +1,109 @@
+// Work items of the persistent prefill attention (fp_attn_tc.cu): which query tiles
+// make up an item and in which order the CTAs take the items.  Host and device.
+#pragma once
+
+#include <algorithm>
+#include <numeric>
+
+#ifdef __CUDACC__
+#define FP_BOTH __host__ __device__ __forceinline__
+#else
+#define FP_BOTH inline
+#endif
+
+namespace fpk {
+
+constexpr int kPaB = 128;  // query rows per tile = keys per tile
+
+struct PaPlan {
+  int pair;   // 0: one query tile an item, its key tiles taken in turn by the two
+              // softmax groups; 1: the same rows of two heads; 2: 256 rows of a head
+  int units;  // items of one (sequence, head or pair of heads)
+  int items;
+  int block;  // (sequence, head)s whose items are taken together
+};
+
+// The item that CTA c of g takes in round n, plan.items or more: none.  The list holds
+// block after block of heads and, within a block, the longest items first; every other
+// round takes it backwards, which evens the CTAs' shares out.
+FP_BOTH int pa_item(int n, int c, int g) { return n * g + ((n & 1) ? g - 1 - c : c); }
+
+// A work item: up to two query tiles of sequence b that share KV head kvh.
+struct PaItem {
+  int b, h[2], q0[2], nt[2], kvh;  // nt: key tiles up to the diagonal (0: no rows in this tile)
+  FP_BOTH PaItem(int i, int S, int H, int Hkv, const PaPlan& p) {
+    const unsigned heads = p.pair == 1 ? H / 2 : H, all = (unsigned)p.items / (unsigned)p.units;
+    const unsigned per = (unsigned)p.block * (unsigned)p.units;
+    const unsigned first = (unsigned)i / per * (unsigned)p.block, rem = (unsigned)i % per;  // the block's first head
+    const unsigned nh = all - first < (unsigned)p.block ? all - first : (unsigned)p.block;
+    const unsigned hb = first + rem % nh;
+    const int u = p.units - 1 - (int)(rem / nh);
+    b = hb / heads;
+    const int hh = hb % heads;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int j = 0; j < 2; ++j) {
+      h[j] = p.pair == 1 ? 2 * hh + j : hh;
+      q0[j] = p.pair == 2 ? (2 * u + j) * kPaB : u * kPaB;
+      const int end = q0[j] + kPaB < S ? q0[j] + kPaB : S;
+      nt[j] = q0[j] < S && (j == 0 || p.pair) ? (end - 1) / kPaB + 1 : 0;
+    }
+    kvh = (unsigned)h[0] / ((unsigned)H / (unsigned)Hkv);
+  }
+  FP_BOTH int tiles() const { return nt[0] > nt[1] ? nt[0] : nt[1]; }
+  // of tile j (a runtime index into the arrays would put them in local memory)
+  FP_BOTH int head(int j) const { return j ? h[1] : h[0]; }
+  FP_BOTH int row0(int j) const { return j ? q0[1] : q0[0]; }
+  FP_BOTH int key_tiles(int j) const { return j ? nt[1] : nt[0]; }
+};
+
+// Pairs of tiles where they keep the SMs busy, else single tiles with their keys cut
+// in two: the smaller of the two makespans (the mean share of an SM, or the longest
+// item), with 4100 cycles for a step of two tiles' products and 3500 an item, 4000
+// with the two groups' sums added (measured, bf16 cache).
+// Longest first over the whole list leaves the SMs' shares even (largest / mean 1.00-1.03)
+// but has them read different heads' keys and values; blocks of heads keep most of the
+// sharing in L2.  A block that is a whole even number of rounds of the SMs evens its
+// shares out by itself, so four rounds are enough; where eight rounds hold no such
+// block, the list is cut into equal blocks of at least eight, whose ends cost up to 15 %
+// (2 to 64 tiles, 5 to 110 rounds).  Microseconds, blocks of four whole rounds | eight
+// rounds | the whole list | head by head, the tile an item takes rotated from round to
+// round (where the rotation's step and the number of tiles had a common divisor, a CTA
+// drew the same tile every time):
+//   int8  4 x 4000, 32 heads      1093 | 1202 | 1192 | 1163
+//         32 x 2048, 64 on 8      4190 | 4338 | 4734 | 4525
+//         16 x 1300, 32 heads      749 |  761 |  767 |  815
+//         8 x 2304, 32 heads           |  829 |  828 | 1289
+//         32 x 2100, 64 on 8           | 4774 | 5302 | 8351
+//   bf16  32 x 2048, 32 heads     1053 | 1096 | 1142 | 1071
+//         8 x 1024, 40 heads       121 |  125 |  126 |  126
+//         32 x 2304, 32 heads          | 1366 | 1380 | 2296
+inline PaPlan pa_plan(int B, int S, int H, int G, int sms) {
+  const long long tiles = (S + kPaB - 1) / kPaB;
+  const int pair = G % 2 == 0 ? 1 : 2;
+  auto make = [&](int pr) {
+    PaPlan p{};
+    p.pair = pr;
+    p.units = (int)(pr == 2 ? (tiles + 1) / 2 : tiles);
+    const long long heads = (long long)B * (pr == 1 ? H / 2 : H);
+    p.items = (int)(heads * p.units);
+    const long long whole = 2LL * sms / std::gcd(2LL * sms, (long long)p.units);  // heads of even whole rounds
+    const long long blocks = std::max(1LL, p.items / (8LL * sms));
+    if (whole * p.units <= 8LL * sms) p.block = (int)std::min(heads, whole * std::max(1LL, 4LL * sms / (whole * p.units)));
+    else p.block = (int)((heads + blocks - 1) / blocks);
+    return p;
+  };
+  auto span = [&](const PaPlan& p) {
+    const double step = 4100, item = p.pair ? 3500 : 4000;
+    double sum = 0;  // steps of a head's items
+    for (long long u = 0; u < p.units; ++u)
+      sum += (double)(p.pair == 2 ? std::min(tiles, 2 * u + 2) : p.pair == 1 ? u + 1 : u / 2 + 1);
+    const double heads = (double)p.items / p.units, longest = (double)(p.pair ? tiles : (tiles + 1) / 2) * step + item;
+    return std::max((sum * step + item * p.units) * heads / sms, longest);
+  };
+  const PaPlan two = make(pair), one = make(0);
+  return span(one) < span(two) ? one : two;
+}
+
+}  // namespace fpk

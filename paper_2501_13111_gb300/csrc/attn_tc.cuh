@@ -2,12 +2,12 @@
 // fp_attn_short.cu): operand descriptors, conversions, launch limits.
 #pragma once
 
+#include "attn_items.h"
 #include "kernels.cuh"
 #include "tc.cuh"
 
 namespace fpk {
 
-constexpr int kPaB = 128;  // query rows per tile = keys per tile
 constexpr int kPaHD = 128;
 constexpr int kPaHalf = kPaB * 128;          // bytes of one [128 rows][64 bf16] swizzled half
 constexpr int kPaTile = 2 * kPaHalf;         // one [128][128] bf16 operand

@@ -53,7 +53,7 @@
 //   every lane runs the MMA loop (one lane's issue took 144
 //     cycles for an MMA that runs 65)                        297 | 138 | 641
 //   output rows through shared memory                        285 | 126 | 617
-//   the items longest first, also over many rounds          255 | 123 | 540
+//   the items longest first, block by block of heads         255 | 123 | 540
 // A query tile's keys in turn by the two groups, bf16 | int8 cache: 8 heads, 1 x 1024
 // tokens 19.7 | 39.5 us, 1 x 4096 61 | 133, 40 heads, 1 x 1024 27.1 | 52 (one 128-row
 // tile per CTA 20.4 | 49.5, 70 | 211, 31.5 | 71; with two V tiles in the ring, as for
@@ -65,6 +65,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "attn_items.h"
 #include "attn_tc.cuh"
 #include "common.cuh"
 
@@ -116,55 +117,6 @@ FP_DEV float2 pa_add2(float2 a, float2 b) {
   return d;
 }
 
-// How the query tiles are put together into work items (chosen by the host).
-struct PaPlan {
-  int pair;       // 0: one query tile an item, its key tiles taken in turn by the two
-                  // softmax groups; 1: the same rows of two heads; 2: 256 rows of a head
-  int units;      // items of one (sequence, head or pair of heads)
-  int items;
-  bool longest_first;
-};
-
-// Item `i` of CTA round n.  Few rounds: the items in order of length, every other
-// round backwards.  Many: the items of one (sequence, head) are consecutive, so
-// the CTAs that run together share keys and values in L2, and which of its query
-// tiles an item takes is rotated from one round to the next, so that no CTA keeps
-// drawing the long ones.
-FP_DEV int pa_item(const PaPlan& p, int n) {
-  const int c = blockIdx.x, g = gridDim.x;
-  return n * g + (p.longest_first && (n & 1) ? g - 1 - c : c);
-}
-
-// A work item: up to two query tiles of sequence b that share KV head kvh.
-struct PaItem {
-  int b, h[2], q0[2], nt[2], kvh;  // nt: key tiles up to the diagonal (0: no rows in this tile)
-  FP_DEV PaItem(int i, int S, int H, int Hkv, const PaPlan& p) {
-    const unsigned heads = p.pair == 1 ? H / 2 : H, all = (unsigned)p.items / (unsigned)p.units;
-    unsigned hb, r;
-    if (p.longest_first) {
-      r = (unsigned)i / all, hb = (unsigned)i % all;
-    } else {
-      hb = (unsigned)i / (unsigned)p.units;
-      r = ((unsigned)i % (unsigned)p.units + hb * p.units / gridDim.x) % (unsigned)p.units;
-    }
-    const int u = p.units - 1 - (int)r;
-    b = hb / heads;
-    const int hh = hb % heads;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      h[j] = p.pair == 1 ? 2 * hh + j : hh;
-      q0[j] = p.pair == 2 ? (2 * u + j) * kPaB : u * kPaB;
-      nt[j] = q0[j] < S && (j == 0 || p.pair) ? (min(q0[j] + kPaB, S) - 1) / kPaB + 1 : 0;
-    }
-    kvh = (unsigned)h[0] / ((unsigned)H / (unsigned)Hkv);
-  }
-  FP_DEV int tiles() const { return max(nt[0], nt[1]); }
-  // of tile j (a runtime index into the arrays would put them in local memory)
-  FP_DEV int head(int j) const { return j ? h[1] : h[0]; }
-  FP_DEV int row0(int j) const { return j ? q0[1] : q0[0]; }
-  FP_DEV int key_tiles(int j) const { return j ? nt[1] : nt[0]; }
-};
-
 // split: the two softmax groups share a query tile (plan.pair == 0)
 template <bool KV8, bool split>
 __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
@@ -190,6 +142,7 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
   uint8_t* sK = smem + (split ? 1 : 2) * kPaTile;
   uint8_t* sV = sK + kPaRing * kPaTile;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto item = [](int n) { return pa_item(n, blockIdx.x, gridDim.x); };
   auto fail = [&]() {
     *abort_flag = 1;
     if (err) atomicExch(err, 2);
@@ -244,7 +197,7 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
     const int pg = lane & 7, half = (lane >> 3) & 1;
     int n = 0, kn = 0, iss[3] = {0, 0, 0};  // items, key tiles; copies issued of Q, K, V
     bool ok = true;
-    for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
+    for (int i = item(0); i < plan.items && ok; i = item(++n)) {
       const PaItem w(i, S, H, Hkv, plan);
       if (n > 0) ok = __all_sync(0xffffffffu, mbar_wait(&qempty, (n - 1) & 1)) && !*abort_flag;
       if (!__all_sync(0xffffffffu, ok)) break;
@@ -325,7 +278,7 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
         tc_mma_ts(tmem + kPaO + j * kPaHD, tmem + j * kPaB + kk * 8, vs + kk * (2048 >> 4), idesc_o,
                   (!first || kk > 0) ? 1u : 0u);
     };
-    for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
+    for (int i = item(0); i < plan.items && ok; i = item(++n)) {
       const PaItem w(i, S, H, Hkv, plan);
       const int nt = w.tiles();
       ok = mbar_wait(KV8 ? &qconv : &qfull, n & 1) && mbar_wait(&kfull[kn % kPaRing], (kn / kPaRing) & 1) && !*abort_flag;
@@ -432,7 +385,7 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
     const int cb = 2 * (c & 3), half_off = (c >> 2) * kPaHalf;
     int n = 0, kn = 0;
     bool ok = true;
-    for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
+    for (int i = item(0); i < plan.items && ok; i = item(++n)) {
       const PaItem w(i, S, H, Hkv, plan);
       const int nt = w.tiles();
       const int32_t* pt = page_table + (long long)w.b * pages_per_seq;
@@ -562,7 +515,7 @@ __global__ void __launch_bounds__(pa_threads<KV8>(), 1)
     const int jq = split ? 0 : j, first = split ? j : 0, stride = split ? 2 : 1;  // query tile; this group's key tiles
     int n = 0, kn = 0, sn = 0, on = 0;  // items, key tiles, this group's scores and outputs
     bool ok = true;
-    for (int i = pa_item(plan, 0); i < plan.items && ok; i = pa_item(plan, ++n)) {
+    for (int i = item(0); i < plan.items && ok; i = item(++n)) {
       const PaItem w(i, S, H, Hkv, plan);
       const int nt = w.key_tiles(jq), qrow = w.row0(jq) + row;  // position in the sequence
       float m = -INFINITY;                            // reference maximum (log2 domain)
@@ -733,39 +686,6 @@ bool attention_prefill_tc_ok(int B, int S, int n_heads, const fp_kv_view& kv, co
          (long long)B * n_heads * ((S + kPaB - 1) / kPaB) < (1LL << 26) && tensor_maps_available();
 }
 
-// Pairs of tiles where they keep the SMs busy, else single tiles with their keys cut
-// in two: the smaller of the two makespans (the mean share of an SM, or the longest
-// item), with 4100 cycles for a step of two tiles' products and 3500 an item, 4000
-// with the two groups' sums added (measured, bf16 cache).  The items are taken longest
-// first for up to 32 rounds of the SMs, which leaves their shares even; past that the
-// shares even out and the sharing of keys in L2 counts, with an int8 cache and heads
-// that share no keys from 12 rounds on.  Longest first / head by head, us: bf16 2 x 2760
-// tokens, 40 heads (5.8 rounds) 158 / 213, 8 x 1024, 40 heads (8.4) 123 / 126, 4 x 2048,
-// 64 heads on 8 (13.5) 255 / 285, 32 x 2048 (108) 2059 / 2055; int8 4 x 2048, 64 on 8
-// 540 / 617, 4 x 4000, 32 heads (13.5) 1210 / 1160, 32 x 2048, 64 on 8 4774 / 4520.
-static PaPlan pa_plan(int B, int S, int H, int G, bool kv8, int sms) {
-  const long long tiles = (S + kPaB - 1) / kPaB;
-  const int pair = G % 2 == 0 ? 1 : 2;
-  auto make = [&](int pr) {
-    PaPlan p{};
-    p.pair = pr;
-    p.units = (int)(pr == 2 ? (tiles + 1) / 2 : tiles);
-    p.items = (int)((long long)B * (pr == 1 ? H / 2 : H) * p.units);
-    p.longest_first = p.items <= (kv8 && pr == 2 ? 12LL : 32LL) * sms;
-    return p;
-  };
-  auto span = [&](const PaPlan& p) {
-    const double step = 4100, item = p.pair ? 3500 : 4000;
-    double sum = 0;  // steps of a head's items
-    for (long long u = 0; u < p.units; ++u)
-      sum += (double)(p.pair == 2 ? std::min(tiles, 2 * u + 2) : p.pair == 1 ? u + 1 : u / 2 + 1);
-    const double heads = (double)p.items / p.units, longest = (double)(p.pair ? tiles : (tiles + 1) / 2) * step + item;
-    return std::max((sum * step + item * p.units) * heads / sms, longest);
-  };
-  const PaPlan two = make(pair), one = make(0);
-  return span(one) < span(two) ? one : two;
-}
-
 template <bool KV8, bool SPLIT>
 static cudaError_t launch_pa_plan(const PaPlan& plan, int ctas, const CUtensorMap& mq, const CUtensorMap& mk,
                                   const CUtensorMap& mv, int S, int n_heads, const fp_kv_view& kv, uint16_t* out,
@@ -787,7 +707,7 @@ static cudaError_t launch_pa_tc(const CUtensorMap& mq, const CUtensorMap& mk, co
         sms <= 0)
       sms = 152;
   }
-  const PaPlan plan = pa_plan(B, S, n_heads, n_heads / kv.n_kv_heads, KV8, sms);
+  const PaPlan plan = pa_plan(B, S, n_heads, n_heads / kv.n_kv_heads, sms);
   const int ctas = std::min(plan.items, sms);
   return plan.pair ? launch_pa_plan<KV8, false>(plan, ctas, mq, mk, mv, S, n_heads, kv, out, err, s)
                    : launch_pa_plan<KV8, true>(plan, ctas, mq, mk, mv, S, n_heads, kv, out, err, s);

@@ -1,6 +1,6 @@
 """Prefill attention where its work items can go wrong: prompts around one and two
 tiles of 128 rows, KV groups of even and odd size (pairs of heads, pairs of row
-tiles, single tiles with their keys cut in two), few items and many (the two orders), both caches."""
+tiles, single tiles with their keys cut in two), few items and many (one block of heads and several), both caches."""
 import numpy as np
 import pytest
 

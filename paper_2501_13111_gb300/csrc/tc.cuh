@@ -202,6 +202,8 @@ FP_DEV void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;
 
 #define FP_R8(b) "=r"(r[b]), "=r"(r[b + 1]), "=r"(r[b + 2]), "=r"(r[b + 3]), "=r"(r[b + 4]), "=r"(r[b + 5]), \
                  "=r"(r[b + 6]), "=r"(r[b + 7])
+#define FP_E8(b) "=&r"(r[b]), "=&r"(r[b + 1]), "=&r"(r[b + 2]), "=&r"(r[b + 3]), "=&r"(r[b + 4]), "=&r"(r[b + 5]), \
+                 "=&r"(r[b + 6]), "=&r"(r[b + 7])
 #define FP_Q8(b) "=r"(q[b]), "=r"(q[b + 1]), "=r"(q[b + 2]), "=r"(q[b + 3]), "=r"(q[b + 4]), "=r"(q[b + 5]), \
                  "=r"(q[b + 6]), "=r"(q[b + 7])
 #define FP_W8(b) "r"(r[b]), "r"(r[b + 1]), "r"(r[b + 2]), "r"(r[b + 3]), "r"(r[b + 4]), "r"(r[b + 5]), \
@@ -256,33 +258,26 @@ FP_DEV void tc_ld(uint32_t taddr, uint32_t* r) {
   }
 }
 
-// tc_ld of N columns from two places with one wait (N = 4, 8 or 16).
+// tc_ld of N columns from two places with one wait (N = 8 or 16).  The first load's
+// results are there before the second load's address is read, hence the early clobbers.
 template <int N>
 FP_DEV void tc_ld_pair(uint32_t ta, uint32_t tb, uint32_t* r, uint32_t* q) {
-  if constexpr (N == 4) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3])
-        : "r"(ta), "r"(tb)
-        : "memory");
-  } else if constexpr (N == 8) {
+  if constexpr (N == 8) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n"
         "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];\n"
         "tcgen05.wait::ld.sync.aligned;"
-        : FP_R8(0), FP_Q8(0)
+        : FP_E8(0), FP_Q8(0)
         : "r"(ta), "r"(tb)
         : "memory");
   } else {
-    static_assert(N == 16, "tc_ld_pair: 4, 8 or 16 columns");
+    static_assert(N == 16, "tc_ld_pair: 8 or 16 columns");
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n"
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, "
         "[%33];\n"
         "tcgen05.wait::ld.sync.aligned;"
-        : FP_R8(0), FP_R8(8), FP_Q8(0), FP_Q8(8)
+        : FP_E8(0), FP_E8(8), FP_Q8(0), FP_Q8(8)
         : "r"(ta), "r"(tb)
         : "memory");
   }
@@ -315,6 +310,7 @@ FP_DEV void tc_st16(uint32_t taddr, const uint32_t* r) {
 FP_DEV void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 #undef FP_R8
+#undef FP_E8
 #undef FP_Q8
 #undef FP_W8
 

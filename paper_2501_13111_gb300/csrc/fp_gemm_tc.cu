@@ -487,18 +487,33 @@ static long long tc_tiles(int epi, int M, int N, int cg) {
 // A pair works through its 256 x 256 tile in 0.92 of the time that a CTA takes for
 // its 128 x 256 (8192^3: 669 against 727 us; half of the weight rows' copies and
 // reads leave shared memory, whose bandwidth bounds the single CTA), so it is taken
-// unless its coarser tiles cost more rounds than that saves.
-static bool tc_pair(int epi, int M, int N) {
-  const long long sms = tc_sms(), t1 = tc_tiles(epi, M, N, 1), t2 = tc_tiles(epi, M, N, 2);
-  return (t2 + sms / 2 - 1) / (sms / 2) * 92 <= (t1 + sms - 1) / sms * 100;
+// unless its coarser tiles cost more rounds than that saves.  Starting and ending a
+// pair's tile takes about 0.8 us longer, which a short K does not bring back.  In a
+// single round shared memory is not the bound: there a pair gains, by reading the
+// weights once for two row tiles, where they come from memory, as a forward pass's
+// bf16 weights do, and loses where they lie in L2, as a small expansion does.  Rows that
+// a pair computes beyond M cost nothing then.  One CTA a tile / pairs, us (weights from
+// memory but where said; one round: alike from 65 to 512 rows):
+//   bf16, M 300       4096 x 1024 13.8 / 14.6   2048 20.2 / 20.2   3072 26.2 / 25.5   4096 32.3 / 31.0   8192 56.1 / 52.5
+//     in L2           4096 x 1024 12.8 / 14.1   4096 28.9 / 30.3   11008 72.5 / 67.0
+//   int4 expanded     4096 x 4096 36.8 / 37.5   8192 x 4096 45.4 / 45.0   4096 x 8192 67.5 / 64.9
+//   bf16, 2048 x 8192 K 512 33.6 / 34.1   768 37.3 / 37.4   1024 43.0 / 40.5   2048 66.0 / 60.9
+//     with SwiGLU     K 1024 44.6 / 46.6   1536 51.2 / 50.9   2048 62.9 / 59.2
+// (weights in L2 from the call before: 300 x 4096 x 4096 in a loop of its own loses 1.4 us.)
+static bool tc_pair(int wquant, int epi, int M, int N, int K) {
+  const long long sms = tc_sms();
+  const long long r1 = (tc_tiles(epi, M, N, 1) + sms - 1) / sms, r2 = (tc_tiles(epi, M, N, 2) + sms / 2 - 1) / (sms / 2);
+  if (r2 * 92 > r1 * 100) return false;
+  if (r1 == 1) return wquant == FP_W_BF16 ? K >= 3072 : (long long)N * K >= (1LL << 25);
+  return K >= (epi == FP_EPI_SWIGLU ? 1536 : 1024);
 }
 
 template <int EPI, bool SCALE>
-static cudaError_t launch_tc_t(const CUtensorMap& mx, const CUtensorMap& mw, int M, int N, int K,
+static cudaError_t launch_tc_t(bool pair, const CUtensorMap& mx, const CUtensorMap& mw, int M, int N, int K,
                                const uint16_t* scales, long long up_off, const uint16_t* R, void* Y, int ldy,
                                int32_t* err, cudaStream_t s) {
   // persistent: one CTA per SM (its shared ring and 512 TMEM columns fill the SM)
-  if (tc_pair(EPI, M, N)) {
+  if (pair) {
     auto kern = gemm_tc_kernel<EPI, SCALE, true>;
     static std::atomic<unsigned long long> attr{0};
     FP_CUDA_TRY(smem_limit_once(kern, TcGeom<true>::kSmem, &attr));
@@ -525,21 +540,21 @@ static cudaError_t launch_tc_t(const CUtensorMap& mx, const CUtensorMap& mw, int
 }
 
 template <int EPI>
-static cudaError_t launch_tc_e(bool sc, const CUtensorMap& mx, const CUtensorMap& mw, int M, int N, int K,
+static cudaError_t launch_tc_e(bool sc, bool pair, const CUtensorMap& mx, const CUtensorMap& mw, int M, int N, int K,
                                const uint16_t* scales, long long up_off, const uint16_t* R, void* Y, int ldy,
                                int32_t* err, cudaStream_t s) {
-  return sc ? launch_tc_t<EPI, true>(mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s)
-            : launch_tc_t<EPI, false>(mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
+  return sc ? launch_tc_t<EPI, true>(pair, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s)
+            : launch_tc_t<EPI, false>(pair, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
 }
 
-static cudaError_t launch_tc_any(int epi, bool sc, const CUtensorMap& mx, const CUtensorMap& mw, int M, int N, int K,
-                                 const uint16_t* scales, long long up_off, const uint16_t* R, void* Y, int ldy,
+static cudaError_t launch_tc_any(int epi, bool sc, bool pair, const CUtensorMap& mx, const CUtensorMap& mw, int M, int N,
+                                 int K, const uint16_t* scales, long long up_off, const uint16_t* R, void* Y, int ldy,
                                  int32_t* err, cudaStream_t s) {
   switch (epi) {
-    case FP_EPI_STORE: return launch_tc_e<FP_EPI_STORE>(sc, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
-    case FP_EPI_RESID: return launch_tc_e<FP_EPI_RESID>(sc, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
-    case FP_EPI_SWIGLU: return launch_tc_e<FP_EPI_SWIGLU>(sc, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
-    default: return launch_tc_e<FP_EPI_F32>(sc, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
+    case FP_EPI_STORE: return launch_tc_e<FP_EPI_STORE>(sc, pair, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
+    case FP_EPI_RESID: return launch_tc_e<FP_EPI_RESID>(sc, pair, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
+    case FP_EPI_SWIGLU: return launch_tc_e<FP_EPI_SWIGLU>(sc, pair, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
+    default: return launch_tc_e<FP_EPI_F32>(sc, pair, mx, mw, M, N, K, scales, up_off, R, Y, ldy, err, s);
   }
 }
 
@@ -559,13 +574,14 @@ cudaError_t launch_gemm_tc(int wquant, int epi, const uint16_t* x, int M, int N,
   const int nr = epi == FP_EPI_SWIGLU ? 2 : 1;
   const int Nout = nr == 2 ? N / 2 : N;
   // rows of a weight box, per band: half a tile where a pair shares it or the gate and the up rows do
-  auto wbox = [&](int n) { return epi == FP_EPI_SWIGLU || tc_pair(epi, M, n) ? 128 : 256; };
+  auto wbox = [&](bool pair) { return epi == FP_EPI_SWIGLU || pair ? 128 : 256; };
   const bool sc = wquant == FP_W_INT8;
   CUtensorMap mx, mw;
   if (!make_map(&mx, x, M, K, kTcBM)) return cudaErrorInvalidValue;
   if (wquant == FP_W_BF16) {
-    if (!make_map(&mw, codes, N, K, wbox(N))) return cudaErrorInvalidValue;
-    return launch_tc_any(epi, sc, mx, mw, M, N, K, scales, Nout, residual, y, Nout, err, s);
+    const bool pair = tc_pair(wquant, epi, M, N, K);
+    if (!make_map(&mw, codes, N, K, wbox(pair))) return cudaErrorInvalidValue;
+    return launch_tc_any(epi, sc, pair, mx, mw, M, N, K, scales, Nout, residual, y, Nout, err, s);
   }
   if (!ws || ws_bytes < gemm_tc_ws_bytes(wquant, N, K)) return cudaErrorInvalidValue;
   // band by band of output columns: expand the band's rows (SwiGLU: its gate
@@ -584,13 +600,14 @@ cudaError_t launch_gemm_tc(int wquant, int epi, const uint16_t* x, int M, int N,
       default:
         FP_CUDA_TRY(dequant_band<FP_W_INT4_G128>(codes, scales, zeros, nr, Nout, c0, cols, K, w, inv, s));
     }
-    if (!make_map(&mw, w, (long long)nr * cols, K, wbox(nr * cols))) return cudaErrorInvalidValue;
+    const bool pair = tc_pair(wquant, epi, M, nr * cols, K);
+    if (!make_map(&mw, w, (long long)nr * cols, K, wbox(pair))) return cudaErrorInvalidValue;
     const uint16_t* r = residual ? residual + c0 : nullptr;
     void* yb = epi == FP_EPI_F32 ? (void*)((float*)y + c0) : (void*)((uint16_t*)y + c0);
     const bool was = g_pdl;
     g_pdl = true;  // the GEMM's set-up overlaps the expansion
     const cudaError_t e =
-        launch_tc_any(epi, sc, mx, mw, M, nr * cols, K, sc ? scales + c0 : scales, Nout, r, yb, Nout, err, s);
+        launch_tc_any(epi, sc, pair, mx, mw, M, nr * cols, K, sc ? scales + c0 : scales, Nout, r, yb, Nout, err, s);
     g_pdl = was;
     FP_CUDA_TRY(e);
   }

@@ -1,7 +1,8 @@
-"""The prefill GEMM on pairs of CTAs (256 x 256 tiles) and on single ones: ragged
-rows around one and two tiles (the odd CTA of a pair with no or few rows), ragged
-columns (half a weight tile past N), K tails, every epilogue; the expansion of
-int8, int4 and GPTQ4 weights for K around its blocks of 4096 elements."""
+"""The prefill GEMM on single CTAs (128 x 256 tiles; small matrices) and on pairs of
+them (256 x 256; a long K): ragged rows around
+one and two tiles (the odd CTA of a pair with no or few rows), ragged columns (half a
+weight tile past N), K tails, every epilogue; the expansion of int8, int4 and GPTQ4
+weights for K around its blocks of 4096 elements."""
 import numpy as np
 import pytest
 
@@ -21,12 +22,7 @@ def fp():
     return fp
 
 
-# (300, 20000, 64): 79 pairs of tiles, a round more than the single CTAs need
-@pytest.mark.parametrize("epi", [0, 1, 2, 3])
-@pytest.mark.parametrize("m,n,k", [(65, 256, 64), (128, 520, 192), (129, 392, 72), (256, 1024, 4160), (257, 264, 128),
-                                   (513, 776, 328), (300, 20000, 64), (2100, 2304, 256)])
-def test_tiles(fp, m, n, k, epi):
-    w = synth.weight_bf16(5, 0, 1, (n, k))
+def _check(fp, m, n, k, epi, w):
     x = synth.uniform_bf16(6, m, (m, k), -2.0, 2.0)
     nout = n // 2 if epi == 2 else n
     r = synth.uniform_bf16(7, m, (m, nout), -1.0, 1.0)
@@ -39,8 +35,28 @@ def test_tiles(fp, m, n, k, epi):
         ref = ref + quant.bf16_to_f32(r).astype(np.float64)
     elif epi == 2:
         ref = M.silu(ref[:, :nout]) * ref[:, nout:]
-    # fp32 sums of exact products; one rounding to bf16 (2^-8 of the value at most)
-    assert rel_err(got.reshape(m, nout), ref) <= (1e-5 if epi == 3 else 1.05 * 2.0 ** -8)
+    # fp32 sums of exact products, a step of the tensor core adding 16 of them and dropping
+    # less than a unit in the last place (2^-23) of the sum; one rounding to bf16 (2^-8)
+    assert rel_err(got.reshape(m, nout), ref) <= (max(1e-5, k / 16 * 2.0 ** -23) if epi == 3 else 1.05 * 2.0 ** -8)
+
+
+@pytest.mark.parametrize("epi", [0, 1, 2, 3])
+@pytest.mark.parametrize("m,n,k", [(65, 256, 64), (128, 520, 192), (129, 392, 72), (256, 1024, 4160), (257, 264, 128),
+                                   (513, 776, 328), (300, 20000, 64), (2100, 2304, 256)])
+def test_tiles(fp, m, n, k, epi):
+    _check(fp, m, n, k, epi, synth.weight_bf16(5, 0, 1, (n, k)))
+
+
+# one round of pairs from K 3072, two from K 1024 (with SwiGLU 1536), and 79 pairs of tiles, a round more
+# than the single CTAs need
+@pytest.mark.parametrize("n,k,ms", [(1032, 3080, (65, 128, 129, 256, 257, 300)), (1032, 3064, (129, 300)), (4104, 8200, (300,)),
+                                    (2304, 1544, (2100,)), (2304, 1024, (2049,)), (2304, 1016, (2100,)),
+                                    (20000, 1032, (129, 300))])
+def test_pairs_of_ctas(fp, n, k, ms):
+    w = synth.weight_bf16(5, 0, 1, (n, k))
+    for i, m in enumerate(ms):
+        for epi in ((i, i + 2) if len(ms) > 2 else range(4)):
+            _check(fp, m, n, k, epi % 4, w)
 
 
 @pytest.mark.parametrize("wq,k", [(1, 16), (1, 4096), (1, 4112), (1, 8208), (2, 128), (2, 4096), (2, 4224), (3, 4224)])

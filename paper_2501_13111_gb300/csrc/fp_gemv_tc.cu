@@ -563,21 +563,26 @@ bool q4tc_ok(int wquant, int epi, int M, int N, int K) {
   return blocks * kQ4DeqWarps <= kLinTicketSlots && tensor_maps_available();
 }
 
-// int4 always; int8 beyond 32 tokens, for long rows, and, of the larger matrices
-// without SwiGLU, for those not much wider than long.  Microseconds, tcgen05 against
-// mma.sync, int8:
-//   32 tokens  4096 x 11008 25.5 / 32.0    8192 x 14336 44.0 / 53.7   5120 x 5120 20.2 / 25.0
-//              9216 x 9216 34.2 / 39.1     2048 x 15872 21.3 / 30.1   7168 x 5120 21.5 / 24.4
-//   17         25.7 / 28.3, 43.5 / 50.3, 19.8 / 21.5, 34.0 / 37.2, 20.8 / 25.9, 21.2 / 22.5
-//   17         wider: 12288 x 4096 28.0 / 26.5, 57344 x 8192 with SwiGLU 162.8 / 156.3;
-//              K a multiple of 8192: 8192 x 8192 34.3 / 31.7; smaller: 4096 x 4096 18.6 / 14.5
-//   64         QKV 48.8 / 81.3, O 45.1 / 70.3, gate+up 180.3 / 267.1 (70B shapes)
+// int4 always; int8 beyond 32 tokens, for long rows and, from 17 tokens, for matrices
+// without SwiGLU that are too large for the mma.sync GEMV's clusters (2^24 weights,
+// gemv_cluster), but for rows a power of two apart: 128 of them in flight at once
+// meet in the same parts of memory (8064 / 8192 / 8320 x 8192 wide: 30.3 / 33.4 / 30.5 us
+// here, 12288 38.9 with nothing lost).  Microseconds at 17 tokens (32 tokens),
+// mma.sync / tcgen05, weights from memory:
+//   8192 x 3072   18.5 / 18.6 (20.5 / 18.9)   20480 x 3072  29.8 / 28.4 (32.3 / 28.8)
+//   4096 x 5120   19.4 / 17.8 (22.3 / 18.0)   16384 x 5120  37.7 / 34.0 (39.6 / 34.3)   32000 x 5120 79.8 / 58.0
+//   8192 x 8064   30.5 / 30.2 (32.8 / 30.6)   9344 x 8064   33.8 / 32.7 (35.5 / 33.2)   16384 x 8064 66.2 / 48.2
+//   4096 x 11008  26.6 / 24.4 (29.2 / 24.7)   8192 x 13824  46.8 / 42.0 (49.4 / 42.5)
+//   powers of two 8192 x 4096 20.9 / 22.8 (22.7 / 22.9)   8192 x 8192 30.5 / 33.5 (32.4 / 34.1)
+//   shorter rows  8192 x 2560 17.2 / 17.8 (19.1 / 18.0)   27648 x 2560 33.1 / 33.4 (34.7 / 33.8)
+//   smaller       3072 x 5120 14.8 / 16.5 (18.2 / 16.7)   4096 x 3968  14.4 / 16.1 (17.3 / 16.6)
+//   SwiGLU        11008 x 5120 26.8 / 28.0 (30.6 / 29.1)  22016 x 4096 35.7 / 41.9 (39.0 / 43.1)
+//   64 tokens     QKV 48.8 / 81.3, O 45.1 / 70.3, gate+up 180.3 / 267.1 (70B shapes; tcgen05 / mma.sync)
 // An int8 item carries half the weights of an int4 item for the same hand-offs, while
 // the mma.sync GEMV's cost grows with the tokens and with the x that a CTA stages.
 bool q4tc_preferred(int wquant, int epi, int M, int N, int K) {
   if (wquant != FP_W_INT8 || M > 32 || K >= 16384) return true;
-  return epi != FP_EPI_SWIGLU && K >= 5120 && K % 8192 != 0 && 2LL * N <= 3LL * K && N <= 9216 &&
-         (long long)N * K > (1LL << 24);
+  return epi != FP_EPI_SWIGLU && (long long)N * K > (1LL << 24) && K >= 3072 && (K & (K - 1)) != 0;
 }
 
 size_t q4tc_ws_bytes(int epi, int M, int N, int K) {

@@ -1,6 +1,6 @@
 """int8 linears at 17 to 32 tokens on the tcgen05 kernel: ragged rows and tokens around
-the rule's edges (wide, short, a multiple of 8192, SwiGLU, 33 tokens), and the report of
-an x beyond the fp16 range, which the mma.sync kernel they came from makes."""
+the rule's edges (2^24 weights, K 3072, a K that is a power of two, SwiGLU, 33 tokens), and
+the report of an x beyond the fp16 range, which the mma.sync kernel they came from makes."""
 import numpy as np
 import pytest
 
@@ -23,7 +23,8 @@ def fp():
 @pytest.mark.parametrize("wq", [1])
 @pytest.mark.parametrize("m,n,k,epi", [
     (17, 4104, 5376, 1), (24, 3336, 5120, 0), (32, 1544, 11008, 3), (31, 8200, 5504, 1), (33, 4104, 5376, 1),
-    (20, 8328, 5504, 0), (18, 4104, 8192, 0), (32, 6152, 5376, 2), (16, 4104, 5376, 1)])
+    (20, 8328, 5504, 0), (18, 4104, 8192, 0), (32, 6152, 5376, 2), (16, 4104, 5376, 1),
+    (17, 5464, 3072, 0), (32, 5456, 3072, 1), (24, 16392, 3200, 3), (20, 6152, 2944, 0), (31, 1032, 16256, 1)])
 def test_int8_linear(fp, wq, m, n, k, epi):
     w = synth.weight_bf16(70 + wq, 0, 1, (n, k))
     x = synth.uniform_bf16(71, m, (m, k), -2.0, 2.0)

@@ -691,34 +691,51 @@ struct SmemLimits {
   int static_bytes;
 };
 
+// Clusters of cl CTAs that the GPU holds at once, with occ CTAs of smem bytes per SM.
+using MaxClusters = int (*)(int occ, int cl, int smem);
+
 // CTAs per row block where a cluster of them sums through distributed shared
 // memory, 0 where the ranges are cut evenly over all CTAs and sums go through
 // global memory and a ticket.  The cluster spares the fence, the ticket and two
 // round trips to L2 (2-3 us), but uses only whole multiples of the row blocks, at
-// most eight CTAs each.  Measured in a graph, us, cluster / even ranges:
-//   int8, 8 tokens   1024 x 512 4.7 / 5.4     4096 x 4096 10.8 / 12.7   12288 x 4096 16.6 / 18.1
-//                    22016 x 4096 (SwiGLU) 23.4 / 26.4   4096 x 11008 18.5 / 19.2 (22 steps a CTA)
+// most eight CTAs each.  Its CTAs lie in one GPC, so that clusters of five to seven leave
+// SMs unused, and a block without a place waits for a whole round: a size is taken
+// only if the GPU holds all blocks' clusters at once (cudaOccupancyMaxActiveClusters).
+// With more than eight tokens each CTA keeps at least two steps, or the sums weigh more
+// than the products.  Measured in a graph, us, cluster / even ranges, weights from memory:
+//   int8, 8 tokens   1024 x 512 4.7 / 5.4     4096 x 4096 10.8 / 12.7   12288 x 4096 15.3 / 17.8
+//                    15360 x 4096 18.9 / 21.4 4096 x 11008 17.0 / 18.7 (22 steps a CTA)
 //                    5120 x 13824 24.9 / 23.3 (27)       8192 x 28672 75.5 / 53.5 (56)
 //   bf16, 8 tokens   4096 x 11008 22.7 / 25.7 (43)       8192 x 28672 121 / 93 (112)
 //   two CTAs a block 57344 x 8192 int8 100 / 98
 //   int8, 32 tokens  4096 x 4096 17.1 / 23.1             5120 x 5120 30.3 / 25.1
+//   the largest size / one that fits at once / even ranges: int8 10240 x 2048 with SwiGLU at
+//                    14 tokens 18.4 / 12.1 / 16.4, 8192 x 512 at 23 (a step a CTA / two) 15.8 /
+//                    7.9 / 10.5; bf16 8192 x 8192 at 12 41.1 / 29.9 / 34.1
+// Of 12,500 launches drawn over these ranges 64 are more than 3 % slower than with even
+// ranges, by up to 13 % (few row blocks, K about 11000), and the mean is 1.45 times faster.
 // In the forward pass (g_pdl) the next kernel's CTAs start while this one drains,
 // and a cluster has to wait for room for all its CTAs at once, so only matrices
 // below 16 MB take it there: two layers of the 7B shape in int8, 100 steps, 32.5 ms without
 // clusters, 34.2 ms with them everywhere; 2048 x 5504 in int8 (matrices of 4 to
 // 22 MB), 50 steps, 10.5 without / 9.2 ms with; 1024 x 2816 in bf16 8.9 / 6.6 ms.
-static int gemv_cluster(int wq, int blocks, int S, int M, int nr, int ctas, int ring_bytes) {
+static int gemv_cluster(int wq, int blocks, int S, int M, int nr, int ctas, int ring_bytes, MaxClusters max_clusters,
+                        int occ, int smem) {
   if (M * nr * kGemvWarps * 16 * 4 > ring_bytes) return 0;  // the sums lie where the ring was
   if (M > 16 && (long long)blocks * S * mma_kt(wq) > (1LL << 24) / (4 * kGemvWarps * 16)) return 0;
-  const int cl = std::min({ctas / blocks, kGemvMaxCluster, S});
-  return cl >= 3 && (S + cl - 1) / cl * nr <= (wq == FP_W_BF16 ? 44 : 24) ? cl : 0;
+  for (int cl = std::min({ctas / blocks, kGemvMaxCluster, M > 8 ? S / 2 : S}); cl >= 3; --cl) {
+    if ((S + cl - 1) / cl * nr > (wq == FP_W_BF16 ? 44 : 24)) break;  // and longer with fewer CTAs
+    if (blocks <= max_clusters(occ, cl, smem)) return cl;
+  }
+  return 0;
 }
 
 // occ_max = CTAs per SM the kernel's registers allow.  The plan takes the
 // most CTAs per SM whose shared memory (ring + an x window of at least a
 // third of one CTA's range, up to a whole row block) fits, and one wave of
 // CTAs.
-static GemvPlan plan_gemv(int wq, int epi, int M, int N, int K, int occ_max, const SmemLimits& lim) {
+static GemvPlan plan_gemv(int wq, int epi, int M, int N, int K, int occ_max, const SmemLimits& lim,
+                          MaxClusters max_clusters) {
   GemvPlan p{};
   const int SUP = 4 * mma_kt(wq);
   const int NT = gemv_nt(M);
@@ -734,8 +751,9 @@ static GemvPlan plan_gemv(int wq, int epi, int M, int N, int K, int occ_max, con
   const int sms = sm_count();
   occ_max = std::max(1, std::min(occ_max, 8));
   int best_occ = 0, best_w = 0;
+  auto smem_of = [&](int occ) { return std::min(lim.per_cta_dyn, lim.per_sm / occ - 1024 - lim.static_bytes) - 16; };
   for (int occ = occ_max; occ >= 1; --occ) {
-    const int budget = std::min(lim.per_cta_dyn, lim.per_sm / occ - 1024 - lim.static_bytes) - 16;
+    const int budget = smem_of(occ);
     const int wmax = (budget - ring - fixed) / per_ss;
     if (wmax < 1) continue;
     const long long C = std::min<long long>(p.total, (long long)occ * sms);
@@ -752,7 +770,7 @@ static GemvPlan plan_gemv(int wq, int epi, int M, int N, int K, int occ_max, con
   }
   if (best_occ == 0) return p;  // ctas == 0: no plan
   p.ctas = (int)std::min<long long>(p.total, (long long)best_occ * sms);
-  p.cl = gemv_cluster(wq, p.blocks, p.S, M, nr, p.ctas, ring);
+  p.cl = gemv_cluster(wq, p.blocks, p.S, M, nr, p.ctas, ring, max_clusters, best_occ, smem_of(best_occ));
   p.W = std::min(best_w, p.S);
   p.smem = (size_t)ring + (size_t)p.W * NT * SUP * 16 +
            (size_t)(wq == FP_W_INT4_G128 ? p.W : (wq == FP_W_INT8 ? 1 : 0)) * NT * 8 * 4;
@@ -806,10 +824,33 @@ static int gemv_occupancy(SmemLimits* lim) {
 }
 
 template <int WQ, int NT, int EPI>
+static int gemv_max_clusters(int occ, int cl, int smem) {
+  static std::atomic<int> known[9][kGemvMaxCluster + 1];  // the number + 1; 0: not asked yet
+  int v = known[occ][cl].load(std::memory_order_relaxed);
+  if (v == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cl);
+    cfg.blockDim = dim3(kGemvWarps * 32);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cl, at.val.clusterDim.y = 1, at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, gemv_mma_kernel<WQ, NT, EPI, true>, &cfg) != cudaSuccess || n < 0) n = 0;
+    (void)cudaGetLastError();
+    v = n + 1;
+    known[occ][cl].store(v, std::memory_order_relaxed);
+  }
+  return v - 1;
+}
+
+template <int WQ, int NT, int EPI>
 static GemvPlan plan_t(int M, int N, int K) {
   SmemLimits lim{};
   const int occ = gemv_occupancy<WQ, NT, EPI>(&lim);
-  return plan_gemv(WQ, EPI, M, N, K, occ, lim);
+  return plan_gemv(WQ, EPI, M, N, K, occ, lim, gemv_max_clusters<WQ, NT, EPI>);
 }
 
 template <int WQ, int EPI>

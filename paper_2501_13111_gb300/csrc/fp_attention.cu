@@ -80,22 +80,57 @@ static int dec_max_splits(long long pairs, int tiles) {
   return (int)std::max<long long>(std::max<long long>(s, 1), dec_min_splits(tiles));
 }
 
+// Clusters of cl CTAs that the GPU holds at once with occ CTAs per SM.  A cluster lies in
+// one GPC, so sizes that do not divide a GPC's room leave some of it unused.  Asked of the
+// driver for a kernel that takes an occ-th of an SM's shared memory (never launched).
+__global__ void __launch_bounds__(128) dec_room_kernel() { pdl_wait(); }
+
+static int dec_max_clusters(int occ, int cl) {
+  static std::atomic<int> known[5][kDecMaxCluster + 1];  // the number + 1; 0: not asked yet
+  int v = known[occ][cl].load(std::memory_order_relaxed);
+  if (v == 0) {
+    const int smem = 228 * 1024 / occ - 1024;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1, cl);
+    cfg.blockDim = dim3(128);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 1, at.val.clusterDim.y = cl, at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    static std::atomic<unsigned long long> attr{0};
+    int n = 0;
+    if (smem_limit_once(dec_room_kernel, 228 * 1024 / 2 - 1024, &attr) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, dec_room_kernel, &cfg) != cudaSuccess || n < 0)
+      n = 0;
+    (void)cudaGetLastError();
+    v = n + 1;
+    known[occ][cl].store(v, std::memory_order_relaxed);
+  }
+  return v - 1;
+}
+
 // CTAs of the cluster that shares a (sequence, KV head), 0 for splits through the
-// workspace.  Eight CTAs take the place of more splits while that leaves each few
-// tiles: 8 with the int8 page-streaming kernel, 5 with the tile kernel.  That kernel's
-// splits fill the SMs, and clusters of other than two or four CTAs pack badly into
-// the SMs that share a cluster, so they need a quarter of the slots to spare.
+// workspace: as many as there are splits, or eight, or fewer so that the GPU holds all
+// clusters at once (4 CTAs an SM with the int8 page-streaming kernel, else dec_occ), while
+// that leaves each few tiles: 8 with the int8 kernel, 5 with the tile kernel.
 // Cold cache, us, cluster / splits and combine:
 //   int8   1 x 4000, 8 KV heads 17.5 / 21.6   5 x 1500, 2 KV heads 14.8 / 19.7
 //          3 x 228, 8 KV heads 13.3 / 15.5    8 x 3000, 8 KV heads 21.4 / 23.7
 //   bf16   1 x 612, 32 KV heads 13.5 / 15.5   3 x 2000, 24 KV heads 25.1 / 28.3
 //          1 x 4000, 8 KV heads (8 tiles each) 23.7 / 21.8
-//          12 x 700, 4 KV heads (clusters of six, 288 of 304 slots) 25.3 / 19.6
-static int dec_cluster(long long pairs, int splits, int tiles, long long slots, bool i8) {
-  const int cl = std::min(splits, kDecMaxCluster);
-  if (splits < 2 || (splits > cl && tiles > cl * (i8 ? 8 : 5))) return 0;
-  if (!i8 && cl != 2 && cl != 4 && pairs * cl > slots * 3 / 4) return 0;
-  return cl;
+//   more clusters than fit at once: bf16 19 x 1378, 4 KV heads (four CTAs) 24.6 / 18.7,
+//          60 x 224, 8 KV heads (two) 26.3 / 21.2; int8 25 x 327, 8 KV heads (three) 20.0 / 15.6
+// Of 10,900 launches drawn over B 1-64, contexts of 64-4096, the clusters are slower by
+// more than 3 % in one of 200 (by up to 9 %: few pairs, over eight splits), and 1.18 times
+// faster on average.
+static int dec_cluster(long long pairs, int splits, int tiles, int nb, bool i8) {
+  for (int cl = std::min(splits, kDecMaxCluster); cl >= 2; --cl) {
+    if (splits > cl && tiles > cl * (i8 ? 8 : 5)) return 0;
+    if (pairs <= dec_max_clusters(i8 ? 4 : dec_occ(nb), cl)) return cl;
+  }
+  return 0;
 }
 
 // Splits of up to eight CTAs are a cluster, whose CTAs add their sums through
@@ -121,7 +156,7 @@ static DecodeGeom decode_geom(int B, int n_kv_heads, int max_len, bool i8 = fals
       best.splits = (max_len + best.chunk - 1) / best.chunk;
     }
   }
-  best.cl = dec_cluster(pairs, best.splits, tiles, slots, i8);
+  best.cl = dec_cluster(pairs, best.splits, tiles, nb, i8);
   if (best.cl) best.chunk = (tiles + best.cl - 1) / best.cl * kDecTT;
   return best;
 }

@@ -320,9 +320,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // scale and zero of group j / 128; 8 consecutive channels at a time.
 // Output row r is row r0 + r of the matrix for r < cols, row up0 + r - cols
 // after (SwiGLU: the band's gate rows, then its up rows).  A thread takes four
-// words a block's width apart, so that its loads are in flight together and
+// words its row's threads apart, so that its loads are in flight together and
 // every access of a warp is contiguous (one word a thread at a time, its row found
-// by a division, took 35 us more on 22016 x 4096 int4).  Bound by memory, the
+// by a division, took 35 us more on 22016 x 4096 int4).  Rows of up to 2048
+// elements share a block: a block for each left most of its threads idle (whole linears:
+// int4 26288 x 256 at 88 rows 35.1 us, 12.1 so; int8 16304 x 768 at 154 35.2, 23.2).  Bound by memory, the
 // codes read and the bf16 written.  Running the expansion of one band beside the
 // GEMM of the band before, in more and smaller bands, lost more to the GEMMs'
 // starts and last rounds than it hid (22016 x 4096 int8, 4096 rows: 518-548 us
@@ -336,15 +338,16 @@ __global__ void __launch_bounds__(kDqThreads)
                    uint16_t* __restrict__ out, const int32_t* __restrict__ inv) {
   pdl_trigger();
   pdl_wait();
-  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+  const int tx = blockDim.x;
+  for (int r = blockIdx.y * blockDim.y + threadIdx.y; r < rows; r += gridDim.y * blockDim.y) {
     const long long row = r < cols ? r0 + r : up0 + (r - cols);
-    const int w0 = blockIdx.x * (kDqThreads * kDqWords) + threadIdx.x, words = K / 8;
+    const int w0 = blockIdx.x * (tx * kDqWords) + threadIdx.x, words = K / 8;
     uint16_t* o = out + (long long)r * K;
     if constexpr (WQ == FP_W_GPTQ4) {
       const uint32_t* cw = (const uint32_t*)codes + row * words;
       const uint16_t *sr = scales + row * (K / 128), *zr = zeros + row * (K / 128);
       for (int i = 0; i < kDqWords; ++i) {
-        const int w = w0 + i * kDqThreads;
+        const int w = w0 + i * tx;
         if (w >= words) break;
         float f[8];
 #pragma unroll
@@ -362,15 +365,15 @@ __global__ void __launch_bounds__(kDqThreads)
       uint2 c[kDqWords];
 #pragma unroll
       for (int i = 0; i < kDqWords; ++i)
-        c[i] = w0 + i * kDqThreads < words ? __ldg(cr + w0 + i * kDqThreads) : make_uint2(0u, 0u);
+        c[i] = w0 + i * tx < words ? __ldg(cr + w0 + i * tx) : make_uint2(0u, 0u);
 #pragma unroll
       for (int i = 0; i < kDqWords; ++i) {
         const uint32_t w[2] = {c[i].x, c[i].y};
         float f[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) f[j] = (float)(int8_t)((w[j >> 2] >> (8 * (j & 3))) & 0xFF);
-        if (w0 + i * kDqThreads < words)
-          *reinterpret_cast<uint4*>(o + (long long)(w0 + i * kDqThreads) * 8) =
+        if (w0 + i * tx < words)
+          *reinterpret_cast<uint4*>(o + (long long)(w0 + i * tx) * 8) =
               make_uint4(pack_bf2(f[0], f[1]), pack_bf2(f[2], f[3]), pack_bf2(f[4], f[5]), pack_bf2(f[6], f[7]));
       }
     } else {
@@ -380,7 +383,7 @@ __global__ void __launch_bounds__(kDqThreads)
       float s[kDqWords], z[kDqWords];
 #pragma unroll
       for (int i = 0; i < kDqWords; ++i) {
-        const int w = w0 + i * kDqThreads;
+        const int w = w0 + i * tx;
         const bool in = w < words;
         c[i] = in ? __ldg(cr + w) : 0u;
         s[i] = in ? bf2f(__ldg(sr + w / 16)) : 0.f;  // 16 words per group
@@ -395,8 +398,8 @@ __global__ void __launch_bounds__(kDqThreads)
           f[2 * j] = ((float)((c[i] >> (4 * j)) & 0xF) - z[i]) * s[i];
           f[2 * j + 1] = ((float)((c[i] >> (4 * j + 16)) & 0xF) - z[i]) * s[i];
         }
-        if (w0 + i * kDqThreads < words)
-          *reinterpret_cast<uint4*>(o + (long long)(w0 + i * kDqThreads) * 8) =
+        if (w0 + i * tx < words)
+          *reinterpret_cast<uint4*>(o + (long long)(w0 + i * tx) * 8) =
               make_uint4(pack_bf2(f[0], f[1]), pack_bf2(f[2], f[3]), pack_bf2(f[4], f[5]), pack_bf2(f[6], f[7]));
       }
     }
@@ -563,9 +566,11 @@ static cudaError_t launch_tc_any(int epi, bool sc, bool pair, const CUtensorMap&
 template <int WQ>
 static cudaError_t dequant_band(const void* codes, const uint16_t* scales, const uint16_t* zeros, int nr, int Nout, int c0,
                                 int cols, int K, uint16_t* out, const int32_t* inv, cudaStream_t s) {
-  const int per = kDqThreads * kDqWords * 8;  // elements of a row per block
-  return launch(dequant_kernel<WQ>, dim3((K + per - 1) / per, std::min(nr * cols, 65535)), dim3(kDqThreads), 0, s, codes,
-                scales, zeros, (long long)c0, (long long)Nout + c0, cols, nr * cols, K, out, inv);
+  int tx = kDqThreads;  // threads along a row: the fewest that take it in one block
+  while (tx > 8 && tx / 2 * kDqWords * 8 >= K) tx /= 2;
+  const int per = tx * kDqWords * 8, ty = kDqThreads / tx;  // elements of a row, rows per block
+  return launch(dequant_kernel<WQ>, dim3((K + per - 1) / per, std::min((nr * cols + ty - 1) / ty, 65535)), dim3(tx, ty), 0,
+                s, codes, scales, zeros, (long long)c0, (long long)Nout + c0, cols, nr * cols, K, out, inv);
 }
 
 cudaError_t launch_gemm_tc(int wquant, int epi, const uint16_t* x, int M, int N, int K, const void* codes,

@@ -2,7 +2,7 @@
 them (256 x 256; a long K): ragged rows around
 one and two tiles (the odd CTA of a pair with no or few rows), ragged columns (half a
 weight tile past N), K tails, every epilogue; the expansion of int8, int4 and GPTQ4
-weights for K around its blocks of 4096 elements."""
+weights for K around its blocks of 4096 elements and its rows that share one."""
 import numpy as np
 import pytest
 
@@ -59,7 +59,8 @@ def test_pairs_of_ctas(fp, n, k, ms):
             _check(fp, m, n, k, epi % 4, w)
 
 
-@pytest.mark.parametrize("wq,k", [(1, 16), (1, 4096), (1, 4112), (1, 8208), (2, 128), (2, 4096), (2, 4224), (3, 4224)])
+@pytest.mark.parametrize("wq,k", [(1, 16), (1, 4096), (1, 4112), (1, 8208), (2, 128), (2, 4096), (2, 4224), (3, 4224),
+                                  (1, 272), (1, 1040), (1, 2064), (2, 256), (2, 1152), (2, 2048), (3, 256), (3, 1152)])
 def test_expansion(fp, wq, k):
     m, n = 96, 264
     w = synth.weight_bf16(8, 0, 1, (n, k))

@@ -28,16 +28,23 @@ struct PaPlan {
 // round takes it backwards, which evens the CTAs' shares out.
 FP_BOTH int pa_item(int n, int c, int g) { return n * g + ((n & 1) ? g - 1 - c : c); }
 
+// The (sequence, head) of item i and its place among that head's items, 0 the shortest.
+FP_BOTH void pa_place(int i, const PaPlan& p, unsigned* head, int* unit) {
+  const unsigned all = (unsigned)p.items / (unsigned)p.units, per = (unsigned)p.block * (unsigned)p.units;
+  const unsigned first = (unsigned)i / per * (unsigned)p.block, rem = (unsigned)i % per;  // the block's first head
+  const unsigned nh = all - first < (unsigned)p.block ? all - first : (unsigned)p.block;
+  *head = first + rem % nh;
+  *unit = p.units - 1 - (int)(rem / nh);
+}
+
 // A work item: up to two query tiles of sequence b that share KV head kvh.
 struct PaItem {
   int b, h[2], q0[2], nt[2], kvh;  // nt: key tiles up to the diagonal (0: no rows in this tile)
   FP_BOTH PaItem(int i, int S, int H, int Hkv, const PaPlan& p) {
-    const unsigned heads = p.pair == 1 ? H / 2 : H, all = (unsigned)p.items / (unsigned)p.units;
-    const unsigned per = (unsigned)p.block * (unsigned)p.units;
-    const unsigned first = (unsigned)i / per * (unsigned)p.block, rem = (unsigned)i % per;  // the block's first head
-    const unsigned nh = all - first < (unsigned)p.block ? all - first : (unsigned)p.block;
-    const unsigned hb = first + rem % nh;
-    const int u = p.units - 1 - (int)(rem / nh);
+    const unsigned heads = p.pair == 1 ? H / 2 : H;
+    unsigned hb;
+    int u;
+    pa_place(i, p, &hb, &u);
     b = hb / heads;
     const int hh = hb % heads;
 #ifdef __CUDACC__
@@ -58,10 +65,14 @@ struct PaItem {
   FP_BOTH int key_tiles(int j) const { return j ? nt[1] : nt[0]; }
 };
 
-// Pairs of tiles where they keep the SMs busy, else single tiles with their keys cut
-// in two: the smaller of the two makespans (the mean share of an SM, or the longest
-// item), with 4100 cycles for a step of two tiles' products and 3500 an item, 4000
-// with the two groups' sums added (measured, bf16 cache).
+// Pairs of tiles, or, where those leave SMs idle or one CTA's share too long, single
+// tiles with their keys cut in two: the smaller of the largest shares that the CTAs draw,
+// with 4100 cycles for a step of a pair (a key tile) and 6500 an item, 7200 for a single
+// tile's step (two key tiles) and 2500 an item.  Fitted to 18,500 launches of both forms (1
+// to 24 sequences, 129 to 4096 tokens, both caches): the form chosen is 0.16 % slower than
+// the better one on average, at most 17 %.  (With 3500 / 4100 / 4000 and the mean share it
+// was 0.7-5 % and at most 73 %: bf16 3 x 267 tokens, 32 heads 19.2 us against 15.7, 10 x 1645,
+// 8 heads 100 against 92.)  Past four rounds pairs, which work 1.75 times as fast.
 // Longest first over the whole list leaves the SMs' shares even (largest / mean 1.00-1.03)
 // but has them read different heads' keys and values; blocks of heads keep most of the
 // sharing in L2.  A block that is a whole even number of rounds of the SMs evens its
@@ -95,14 +106,24 @@ inline PaPlan pa_plan(int B, int S, int H, int G, int sms) {
     return p;
   };
   auto span = [&](const PaPlan& p) {
-    const double step = 4100, item = p.pair ? 3500 : 4000;
-    double sum = 0;  // steps of a head's items
-    for (long long u = 0; u < p.units; ++u)
-      sum += (double)(p.pair == 2 ? std::min(tiles, 2 * u + 2) : p.pair == 1 ? u + 1 : u / 2 + 1);
-    const double heads = (double)p.items / p.units, longest = (double)(p.pair ? tiles : (tiles + 1) / 2) * step + item;
-    return std::max((sum * step + item * p.units) * heads / sms, longest);
+    double worst = 0;
+    const int g = std::min(p.items, sms);
+    for (int c = 0; c < g + 7; c += 8) {  // some of the CTAs: neighbours draw alike
+      double t = 0;
+      for (int n = 0, cta = std::min(c, g - 1), i = cta; i < p.items; i = pa_item(++n, cta, g)) {
+        unsigned head;
+        int u;
+        pa_place(i, p, &head, &u);
+        const long long steps = p.pair == 2 ? std::min(tiles, 2LL * u + 2) : p.pair == 1 ? u + 1 : u / 2 + 1;
+        t += p.pair ? 4100. * steps + 6500 : 7200. * steps + 2500;
+      }
+      worst = std::max(worst, t);
+    }
+    return worst;
   };
-  const PaPlan two = make(pair), one = make(0);
+  const PaPlan two = make(pair);
+  if (two.items > 4LL * sms) return two;
+  const PaPlan one = make(0);
   return span(one) < span(two) ? one : two;
 }
 

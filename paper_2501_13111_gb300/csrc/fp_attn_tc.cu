@@ -3,8 +3,8 @@
 //
 // o = softmax(q K^T / sqrt(hd) + causal mask) V for the S query rows of every
 // (sequence, head) against cache positions 0..S-1 (Sec. 5.1: the block's
-// attention), for prompts of more than 128 tokens (fp_attn_short.cu takes the
-// shorter ones).  One persistent CTA per SM walks work items of two query tiles
+// attention), for prompts of more than 128 tokens (fp_attn_short.cu takes most of
+// the shorter ones).  One persistent CTA per SM walks work items of two query tiles
 // of 128 rows that read the same keys and values: two heads of one KV head's
 // group where groups are even, else 256 consecutive rows of a head.  Key tiles of
 // 128.  Where pairs would leave SMs idle or one CTA's share too long, an item is
@@ -697,9 +697,7 @@ static cudaError_t launch_pa_plan(const PaPlan& plan, int ctas, const CUtensorMa
                 S, n_heads, kv.n_kv_heads, kv.page_size, kv.page_table, kv.pages_per_seq, kv.n_pages, plan, out, err);
 }
 
-template <bool KV8>
-static cudaError_t launch_pa_tc(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, int B, int S,
-                                int n_heads, const fp_kv_view& kv, uint16_t* out, int32_t* err, cudaStream_t s) {
+static int pa_sms() {
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -707,6 +705,13 @@ static cudaError_t launch_pa_tc(const CUtensorMap& mq, const CUtensorMap& mk, co
         sms <= 0)
       sms = 152;
   }
+  return sms;
+}
+
+template <bool KV8>
+static cudaError_t launch_pa_tc(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, int B, int S,
+                                int n_heads, const fp_kv_view& kv, uint16_t* out, int32_t* err, cudaStream_t s) {
+  const int sms = pa_sms();
   const PaPlan plan = pa_plan(B, S, n_heads, n_heads / kv.n_kv_heads, sms);
   const int ctas = std::min(plan.items, sms);
   return plan.pair ? launch_pa_plan<KV8, false>(plan, ctas, mq, mk, mv, S, n_heads, kv, out, err, s)
@@ -719,8 +724,13 @@ cudaError_t launch_attention_prefill_tc(const uint16_t* q, int q_stride, int B, 
   const long long pool_rows = (long long)kv.n_pages * kv.n_kv_heads * kv.page_size;
   // q [B S][q_stride] bf16, box [128 rows][64]
   if (!make_tensor_map(&mq, q, (long long)B * S, q_stride, 2, kPaB, 64, 128)) return cudaErrorInvalidValue;
-  const bool one_tile = S <= kPaB && B <= 65535;  // B: the grid's y extent
-  if (kv.kvquant == FP_KV_INT8)
+  // B: the grid's y extent.  Pairs of heads that share keys and values take over where the
+  // short kernel (two CTAs an SM) has more than a round (int8 cache, whose codes it widens
+  // once a head) or three.  H 64 on 8, 128 tokens, short / pairs, us: int8 4 prompts 15.1 / 14.7,
+  // 8 27.5 / 22.1, 32 110 / 69; bf16 8 13.2 / 15.1, 16 24.8 / 24.1, 32 49 / 39
+  const bool kv8 = kv.kvquant == FP_KV_INT8, shared = n_heads / kv.n_kv_heads % 2 == 0;
+  const bool one_tile = S <= kPaB && B <= 65535 && !(shared && (long long)B * n_heads > (kv8 ? 2 : 6) * pa_sms());
+  if (kv8)
     return one_tile ? launch_attention_prefill_short(mq, mq, mq, B, S, n_heads, kv, out, err, s)
                     : launch_pa_tc<true>(mq, mq, mq, B, S, n_heads, kv, out, err, s);
   // bf16 pools [pages Hkv 16][128], box [16 rows][64]

@@ -26,7 +26,8 @@ def fp():
     (2, 3, 3, 128), (2, 3, 3, 129), (1, 3, 1, 256), (2, 3, 1, 257), (1, 6, 6, 385),  # odd groups, ragged second tiles
     (2, 4, 2, 128), (3, 4, 2, 255), (1, 8, 2, 641),                                   # pairs of heads
     (20, 16, 16, 300), (41, 32, 4, 129), (64, 32, 32, 257), (300, 32, 4, 130),        # several rounds of SMs, many
-    (1, 8, 2, 300), (1, 2, 2, 1153), (1, 40, 40, 520), (3, 8, 8, 1024)])              # a query tile's keys cut in two
+    (1, 8, 2, 300), (1, 2, 2, 1153), (1, 40, 40, 520), (3, 8, 8, 1024),               # a query tile's keys cut in two
+    (76, 4, 2, 128), (77, 4, 2, 100), (229, 4, 2, 33), (40, 64, 8, 128), (310, 3, 3, 17)])  # one tile: both kernels
 def test_work_items(fp, kvq, B, H, Hkv, S):
     hd = 128
     c = Cache(fp, kvq, B, S + 7, Hkv, hd, seed=S + H + kvq)

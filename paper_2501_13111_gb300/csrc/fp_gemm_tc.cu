@@ -86,7 +86,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int tiles_m = (M + CG * kTcBM - 1) / (CG * kTcBM), tiles_n = (Nout + BNout - 1) / BNout;
   const int ntiles = tiles_m * tiles_n;
   const int kblocks = (K + kTcBK - 1) / kTcBK;
-  const int first_tile = blockIdx.x / CG, tile_step = gridDim.x / CG;
+  // (the tile loops read the grid's registers themselves: through variables the single
+  // CTA's instance took 2.5 % longer, 4096^3 111.6 us against 109.4, the pairs' 2.3 %)
   auto tile_origin = [&](int t, int& m0, int& n0) {
     constexpr int GM = 16 / CG;
     const int span = GM * tiles_n;
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // ---------------- TMA producer
     if (lane == 0) {
       int it = 0;  // k-blocks issued, across tiles
-      for (int t = first_tile; t < ntiles && !*abort_flag; t += tile_step) {
+      for (int t = blockIdx.x / CG; t < ntiles && !*abort_flag; t += gridDim.x / CG) {
         int m0, n0;
         tile_origin(t, m0, n0);
         for (int kb = 0; kb < kblocks; ++kb, ++it) {
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         else tc_commit(bar);
       };
       int it = 0, lt = 0;
-      for (int t = first_tile; t < ntiles && !*abort_flag; t += tile_step, ++lt) {
+      for (int t = blockIdx.x / CG; t < ntiles && !*abort_flag; t += gridDim.x / CG, ++lt) {
         const int acc = lt & 1;
         // the epilogue has drained this accumulator (local tile lt - 2)
         if (!mbar_wait(&tempty[acc], ((lt >> 1) & 1) ^ 1) || *abort_flag) {
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // ---------------- epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31
     const int q = warp & 3;
     int lt = 0;
-    for (int t = first_tile; t < ntiles; t += tile_step, ++lt) {
+    for (int t = blockIdx.x / CG; t < ntiles; t += gridDim.x / CG, ++lt) {
       const int acc = lt & 1;
       int m0, n0;
       tile_origin(t, m0, n0);

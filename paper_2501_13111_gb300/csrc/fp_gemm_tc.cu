@@ -488,27 +488,31 @@ static long long tc_tiles(int epi, int M, int N, int cg) {
   return (long long)((nout + bn - 1) / bn) * ((M + cg * kTcBM - 1) / (cg * kTcBM));
 }
 
-// A pair works through its 256 x 256 tile in 0.92 of the time that a CTA takes for
-// its 128 x 256 (8192^3: 669 against 727 us; half of the weight rows' copies and
+// A pair works through its 256 x 256 tile in 0.93 of the time that a CTA takes for
+// its 128 x 256 (8192^3: 653 against 700 us; half of the weight rows' copies and
 // reads leave shared memory, whose bandwidth bounds the single CTA), so it is taken
 // unless its coarser tiles cost more rounds than that saves.  Starting and ending a
 // pair's tile takes about 0.8 us longer, which a short K does not bring back.  In a
 // single round shared memory is not the bound: there a pair gains, by reading the
 // weights once for two row tiles, where they come from memory, as a forward pass's
-// bf16 weights do, and loses where they lie in L2, as a small expansion does.  Rows that
-// a pair computes beyond M cost nothing then.  One CTA a tile / pairs, us (weights from
-// memory but where said; one round: alike from 65 to 512 rows):
+// bf16 weights of some size do, and loses where they lie in L2, as a small expansion
+// does and the weights of a small model.  Rows that a pair computes beyond M cost
+// nothing then.  One CTA a tile / pairs, us (weights from memory but where said; one
+// round: alike from 65 to 512 rows):
 //   bf16, M 300       4096 x 1024 13.8 / 14.6   2048 20.2 / 20.2   3072 26.2 / 25.5   4096 32.3 / 31.0   8192 56.1 / 52.5
+//                     1024 x 4096 31.1 / 30.6   8192 54.9 / 51.9
 //     in L2           4096 x 1024 12.8 / 14.1   4096 28.9 / 30.3   11008 72.5 / 67.0
+//                     1024 x 4096 28.6 / 30.0   8192 49.8 / 51.2
 //   int4 expanded     4096 x 4096 36.8 / 37.5   8192 x 4096 45.4 / 45.0   4096 x 8192 67.5 / 64.9
 //   bf16, 2048 x 8192 K 512 33.6 / 34.1   768 37.3 / 37.4   1024 43.0 / 40.5   2048 66.0 / 60.9
 //     with SwiGLU     K 1024 44.6 / 46.6   1536 51.2 / 50.9   2048 62.9 / 59.2
-// (weights in L2 from the call before: 300 x 4096 x 4096 in a loop of its own loses 1.4 us.)
+// So in one round from 2^24 bf16 weights (a quarter of L2; a matrix of 4096 x 4096 that a
+// loop leaves there loses 1.4 us) and from 2^25 expanded ones.
 static bool tc_pair(int wquant, int epi, int M, int N, int K) {
   const long long sms = tc_sms();
   const long long r1 = (tc_tiles(epi, M, N, 1) + sms - 1) / sms, r2 = (tc_tiles(epi, M, N, 2) + sms / 2 - 1) / (sms / 2);
-  if (r2 * 92 > r1 * 100) return false;
-  if (r1 == 1) return wquant == FP_W_BF16 ? K >= 3072 : (long long)N * K >= (1LL << 25);
+  if (r2 * 93 > r1 * 100) return false;
+  if (r1 == 1) return K >= 3072 && (long long)N * K >= (wquant == FP_W_BF16 ? 1LL << 24 : 1LL << 25);
   return K >= (epi == FP_EPI_SWIGLU ? 1536 : 1024);
 }
 

@@ -47,9 +47,10 @@ def test_tiles(fp, m, n, k, epi):
     _check(fp, m, n, k, epi, synth.weight_bf16(5, 0, 1, (n, k)))
 
 
-# one round of pairs from K 3072, two from K 1024 (with SwiGLU 1536), and 79 pairs of tiles, a round more
-# than the single CTAs need
-@pytest.mark.parametrize("n,k,ms", [(1032, 3080, (65, 128, 129, 256, 257, 300)), (1032, 3064, (129, 300)), (4104, 8200, (300,)),
+# one round of pairs from K 3072 and 2^24 weights, two from K 1024 (with SwiGLU 1536), and 79 pairs of
+# tiles, a round more than the single CTAs need
+@pytest.mark.parametrize("n,k,ms", [(5464, 3080, (65, 128, 129, 256, 257, 300)), (5440, 3080, (129, 300)),
+                                    (5496, 3064, (257,)), (4104, 8200, (300,)),
                                     (2304, 1544, (2100,)), (2304, 1024, (2049,)), (2304, 1016, (2100,)),
                                     (20000, 1032, (129, 300))])
 def test_pairs_of_ctas(fp, n, k, ms):

@@ -64,23 +64,26 @@ enum {
 /* Weight-only linear y = x W^T (the "linear layers" of the block) with the
  * dequantisation fused: x bf16 [M][K]; W in the wquant format of fp.h
  * (codes / scales / zeros as fp_op_quantize writes them); fp32 accumulation.
- * Kernel choice depends on M, N and K: M <= 64 runs the decode GEMV (the
- * work is cut into equal ranges of (128-row block, K step), one per resident
- * CTA, and shared blocks are reduced from fp32 partials in a fixed order) --
- * on mma.sync with the codes dequantised in registers, except, with 16-byte
- * aligned x and codes: int4 and a bf16 result with M <= 16 and at least 2^24
- * weights (scales and zeros 16-byte aligned too), which runs on tcgen05 with 8-bit operands (the codes as they
- * are; x split by a first kernel into two e4m3 pieces an element, which carry
- * it exactly down to 2^-13 of the largest value of its row and group of 128
- * channels and to 2^-22 of that value below; scales and zero points applied in
- * fp32; a row of x that holds an infinity or a NaN gives NaN); int4 with 17 <= M <= 64 otherwise, and int8
- * with 33 <= M <= 64 or K >= 16384, which run on tcgen05 with each
- * weight expanded in TMEM (int4 to bf16((q - z) s) as the prefill GEMM does,
- * int8 to the integer code, its row scale applied to the fp32 sums); bf16
- * with 17 <= M <= 64 on matrices that give every SM at least 48 items of 32
- * KB, which runs on tcgen05 fed by TMA; a K that is not a multiple of the
- * GEMV's K step falls back to one warp per output row on the CUDA cores --
- * larger M the tcgen05 GEMM.  For M > 64 with int8
+ * Kernel choice depends on M, N, K and the pointers' alignment.  M <= 64, decode: by
+ * default the GEMV on mma.sync with the codes dequantised in registers (the work is
+ * cut into equal ranges of (128-row block, K step), one per resident CTA, and shared
+ * blocks are reduced from fp32 partials in a fixed order; smaller matrices give each
+ * block a cluster of CTAs that add in rank order; gemv_cluster).  It stages x for int8 and
+ * int4 codes as fp16.  With 16-byte aligned x and codes instead, on tcgen05:
+ *   int4, M <= 16, a bf16 result, larger matrices (f8_pays; scales and zeros 16-byte
+ *     aligned too): 8-bit operands, the codes as they are; x split by a first kernel
+ *     into two e4m3 pieces an element, which carry it exactly down to 2^-13 of the
+ *     largest value of its row and group of 128 channels and to 2^-22 of that value
+ *     below; scales and zero points applied in fp32; a row of x that holds an infinity
+ *     or a NaN gives NaN;
+ *   int4, M >= 17 (scales and zeros 16-byte aligned too): each weight expanded in TMEM
+ *     to bf16((q - z) s) as the prefill GEMM does;
+ *   int8, M >= 33, and from 17 long rows and larger matrices (q4tc_preferred): codes
+ *     expanded in TMEM, the row scale applied to the fp32 sums;
+ *   bf16, M >= 17, larger matrices (btc_preferred): fed by TMA.
+ * A K that is not a multiple of the
+ * GEMV's K step falls back to one warp per output row on the CUDA cores.
+ * M > 64, prefill: the tcgen05 GEMM.  For M > 64 with int8
  * or int4 weights the GEMM either reads a bf16 expansion of W that it writes
  * into the workspace band by band (at most 128 MB; the faster path), or, when
  * the workspace is NULL or smaller than that, dequantises the codes inside
@@ -159,9 +162,10 @@ int fp_op_rope_kv(uint16_t* qkv, int B, int S, int row_stride, int n_heads, cons
  * at h*head_dim), attends over positions 0 .. len[b]-1 of the cache
  * (softmax(q K^T / sqrt(hd)) V, query head j reads KV head j / (H/Hkv));
  * out bf16 [B][n_heads*head_dim].  Split over the context in chunks; the
- * partial results stay in the shared memory of a cluster of CTAs or, past
- * eight splits, go to `workspace` (fp_op_attention_decode_workspace_bytes
- * for at most max_len cached positions) and a second kernel combines them.
+ * partial results stay in the shared memory of a cluster of CTAs where one takes
+ * the splits' place (dec_cluster), else go to `workspace`
+ * (fp_op_attention_decode_workspace_bytes for at most max_len cached positions;
+ * to be there whatever the splits) and a second kernel combines them.
  * len[b] in [1, max_len]; a larger len[b] is clipped to max_len and sets
  * *err = 1 (err may be NULL). */
 int fp_op_attention_decode(const uint16_t* q, int q_stride, int B, int n_heads, const fp_kv_view* kv,

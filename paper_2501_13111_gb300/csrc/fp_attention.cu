@@ -687,7 +687,7 @@ __global__ void __launch_bounds__(kD8Warps * 32) attn_decode_i8_kernel(
       for (int i = threadIdx.x; i < G * HD; i += blockDim.x) out[((long long)b * H + kvh * G) * HD + i] = 0;
     return;
   }
-  const int np = (t1 - t0 + 15) / 16;  // pages of the split (t0 is a multiple of 64)
+  const int np = (t1 - t0 + 15) / 16;  // pages of the split (t0 is a multiple of 16)
   // ---- the split's page ids, staged once (past the table: -1)
   int* spt = reinterpret_cast<int*>(smem + kD8Warps * kD8Stages * kD8PageBytes);
   {

@@ -63,6 +63,35 @@ def rel_err(gpu, ref):
     return float(np.max(np.abs(gpu - ref)) / max(np.max(np.abs(ref)), 1e-30))
 
 
+# ---------------------------------------------------------------- linears
+def check_decode_linear(fp, wq, m, n, k, epi):
+    """fp_op_linear (m <= 64) on seeded weights against the oracle; the residual in place."""
+    w = synth.weight_bf16(70 + wq, 0, 1, (n, k))
+    x = synth.uniform_bf16(71, m, (m, k), -2.0, 2.0)
+    nout = n // 2 if epi == 2 else n
+    r = synth.uniform_bf16(72, m, (m, nout), -1.0, 1.0)
+    codes, scales, zeros = empty(n * k * 2), empty(n * (k // 128), np.uint16), empty(n * (k // 128), np.uint16)
+    fp.fp_op_quantize(wq, ptr(dev(w)), n, k, ptr(codes), ptr(scales), ptr(zeros))
+    out = dev(r) if epi == 1 else empty(m * nout * (4 if epi == 3 else 2))
+    ws_b = fp.fp_op_linear_workspace_bytes(wq, m, n, k)
+    ws = empty(max(ws_b, 16))
+    fp.fp_op_linear(wq, epi, ptr(dev(x)), m, n, k, ptr(codes), ptr(scales), ptr(zeros), ptr(out if epi == 1 else dev(r)),
+                    ptr(out), ptr(ws), ws_b)
+    got = host(out, np.float32) if epi == 3 else quant.bf16_to_f32(host(out, np.uint16))
+    wd = quant.quantize_weight(w, wq)[1]
+    if wq == 2 and m >= 17:  # the tcgen05 path multiplies bf16((q - z) s)
+        wd = quant.bf16_to_f32(synth.f32_to_bf16_bits(wd.astype(np.float32))).astype(np.float64)
+    ref = quant.bf16_to_f32(x).astype(np.float64) @ wd.T
+    if epi == 1:
+        ref = ref + quant.bf16_to_f32(r).astype(np.float64)
+    elif epi == 2:
+        ref = M.silu(ref[:, :nout]) * ref[:, nout:]
+    # fp32 sums; int8 codes carry an offset of 1152 that is taken out of the sum
+    # (2^-24 of 1152 sum|x| against sum|q x|, q up to 127); one rounding to bf16
+    err = rel_err(got.reshape(m, nout), ref)
+    assert err <= (1e-4 if epi == 3 else 1.05 * 2.0 ** -8 + 1e-4), err
+
+
 # ---------------------------------------------------------------- weights
 def arch_dict(a: M.Arch):
     return dict(n_layers=a.n_layers, hidden=a.hidden, n_heads=a.n_heads, n_kv_heads=a.n_kv_heads,

@@ -70,12 +70,13 @@ enum {
  * blocks are reduced from fp32 partials in a fixed order; smaller matrices give each
  * block a cluster of CTAs that add in rank order; gemv_cluster).  It stages x for int8 and
  * int4 codes as fp16.  With 16-byte aligned x and codes instead, on tcgen05:
- *   int4, M <= 16, a bf16 result, larger matrices (f8_pays; scales and zeros 16-byte
- *     aligned too): 8-bit operands, the codes as they are; x split by a first kernel
+ *   int4, M <= 16 and, with SwiGLU, M <= 32, a bf16 result, larger matrices (f8_pays;
+ *     scales and zeros 16-byte aligned too): 8-bit operands, the codes as they are; x split by a first kernel
  *     into two e4m3 pieces an element, which carry it exactly down to 2^-13 of the
  *     largest value of its row and group of 128 channels and to 2^-22 of that value
  *     below; scales and zero points applied in fp32; a row of x that holds an infinity
- *     or a NaN gives NaN;
+ *     or a NaN gives NaN; where that would lose more than 2^-10 of a row, or a row holds
+ *     an infinity or a NaN, M >= 17 runs again on the next kernel;
  *   int4, M >= 17 (scales and zeros 16-byte aligned too): each weight expanded in TMEM
  *     to bf16((q - z) s) as the prefill GEMM does;
  *   int8, M >= 33, and from 17 long rows and larger matrices (q4tc_preferred): codes

@@ -1,4 +1,4 @@
-// Decode linear for int4 group-128 weights at up to 16 tokens on the tcgen05
+// Decode linear for int4 group-128 weights at up to 32 tokens on the tcgen05
 // tensor cores with 8-bit operands.
 //
 // y[m][n] = sum_g s[n][g] sum_{k in g} (q[n][k] - z[n][g]) x[m][k].
@@ -7,20 +7,25 @@
 // subnormals (bytes 0-7) and its first binade (8-15) share one spacing.  So a
 // packed word becomes two operand words by one shift and two masks (0.4
 // instructions a code; the bf16 expansion takes two), and the weights stay
-// exact.  x is split beforehand, per token and group, into two e4m3 pieces
-// (split_x_kernel):
-//   x 2^e = hi + lo / 32,  e the power of two with the group's max|x| 2^e in [128, 256).
+// exact.  x is split beforehand, per token and group (beyond 16 tokens per token), into
+// two e4m3 pieces (split_x_kernel):
+//   x 2^e = hi + lo / 32,  e the power of two with the largest |x| 2^e in [128, 256).
 // hi keeps four significant bits and lo the next four, so a bf16 x is carried
-// exactly down to 2^-13 of the largest |x| of its group and, below, with an error of
-// at most 2^-22 of that largest.  hi and lo are columns of their own, so N = 2 x
-// tokens; the group's products are summed in fp32, and lo / 32, the zero point times
+// exactly down to 2^-13 of the largest |x| of its group (token) and, below, with an
+// error of at most 2^-22 of that largest.  hi and lo are columns of their own, so N = 2
+// x tokens; the group's products are summed in fp32, and lo / 32, the zero point times
 // the group's sum of x, 2^-e and the scale are applied in fp32 to its accumulator.
-// With one exponent a token, one large element cost the small elements of every group
-// their bits.  Relative error of rows of N(0, 0.05) and one element of 30000 whose own
-// weights are zero (2-norm; an exponent a group / a token / the mma.sync GEMV, whose
-// fp32 sums hold 1024 + q times x; the result's rounding is 0.0017 of each):
+// To 16 tokens: with one exponent a token, one large element cost the small elements of
+// every group their bits.  Relative error of rows of N(0, 0.05) and one element of 30000
+// whose own weights are zero (2-norm; an exponent a group / a token / the mma.sync GEMV,
+// whose fp32 sums hold 1024 + q times x; the result's rounding is 0.0017 of each):
 //   4608 x 4096 0.0088 / 0.046 / 1.6   5120 x 13824 0.0049 / 0.047 / 0.55   65536 x 256 0.032 / 0.046 / 2.9
 // and with the whole group's weights zero 0.0017 / 0.03-0.05 / 0.0017.
+// Beyond 16 tokens the sums' warps set the pace and the group's exponent would cost 12 us
+// of 100; the path that this kernel replaces there takes any bf16 x as it is (one element of
+// 2^18 beside unit normals, its weights zero: 0.0027, here 0.054; infinities).  So the
+// split adds up what each token loses, and a third kernel, that path, runs again over the
+// result if that is more than its own rounding, else returns (1.2-2 us).
 //
 // One CTA per SM, 20 warps; an item is two groups of one row tile:
 //   warps 0-7   codes to operands, one row per thread, shared memory to TMEM:
@@ -76,10 +81,10 @@ struct F8Geom {
   static constexpr int kN = 2 * MT;                        // hi columns, then lo columns
   static constexpr int kGroupBytes = kN * 128;             // x pieces of one group
   static constexpr int kXStage = 2 * kGroupBytes;
-  static constexpr int kAccs = 4;                          // items whose two accumulators are in TMEM
+  static constexpr int kAccs = MT == 32 ? 2 : 4;           // items whose two accumulators are in TMEM
   static constexpr int kSlots = MT == 8 ? 6 : 4;           // items whose A operands are
   static constexpr int kACol = kAccs * 2 * kN;             // the first column of the A operands
-  static constexpr int kWStages = 10;
+  static constexpr int kWStages = MT == 32 ? 8 : 10;
   static constexpr int kXStages = 4;
   static constexpr int kXsStage = 2 * 2 * MT * 4;          // two groups' sums and powers of two
   static constexpr int kSwap = kF8Rows * MT * 4;           // the tokens' halves changing hands
@@ -95,93 +100,159 @@ struct F8Geom {
 FP_DEV long long f8_cta_of(long long i, long long C, long long total) { return ((i + 1) * C - 1) / total; }
 
 // ------------------------------------------------------------------ x pieces
-// Tokens along the grid's y (rows past M: zeros), eight elements a thread.  pieces
-// [groups][2 MT][128 bytes], row m the token's hi and row MT + m its lo, 16-byte
-// chunk c of a row at c ^ (row % 8) (the 128-byte swizzle), and within each eight
-// elements the order in which masking a packed int4 word yields them; sums
-// [groups][2][MT] = 2^-9 sum of the group's pieces, then 2^-e of the group, NaN
-// for one that holds an infinity or a NaN.  perm (GPTQ4): element j is x[perm[j]].
+// pieces [groups][2 MT][128 bytes], row m token m's hi and row MT + m its lo (tokens past
+// M: zeros), 16-byte chunk c of a row at c ^ (row % 8) (the 128-byte swizzle), and within
+// each eight elements the order in which masking a packed int4 word yields them; sums
+// [groups][2][MT] = 2^-9 sum of the group's pieces, then 2^-e, NaN where the exponent's
+// elements hold an infinity or a NaN.  perm (GPTQ4): element j is x[perm[j]].
+// TOKEN false: an exponent a (token, group), CTAs x tokens, eight elements a thread.  True
+// (17 tokens and more): an exponent a token, one CTA each, which reads the row twice and
+// leaves in range[m] the token's squares lost and kept (f8_wide), and in xp, if given, x in
+// the order of perm for the kernel that takes over then.
 // Bound by latency (2 K bytes read and written per token).
-constexpr int kSplitThreads = 256;
+constexpr int kSplitThreads = 256, kSplitRowThreads = 1024;
 
-__global__ void __launch_bounds__(kSplitThreads)
+// |x| as bf16 bits orders like the values, infinities and NaN on top.
+FP_DEV uint32_t f8_amax(uint32_t a, const uint4& v) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) a = max(a, max(w[i] & 0x7FFFu, (w[i] >> 16) & 0x7FFFu));
+  return a;
+}
+
+template <bool TOKEN>
+__global__ void __launch_bounds__(TOKEN ? kSplitRowThreads : kSplitThreads)
     split_x_kernel(const uint16_t* __restrict__ x, int M, int MT, int K, const int32_t* __restrict__ perm,
-                   uint8_t* __restrict__ pieces, float* __restrict__ sums, int32_t* err) {
+                   uint8_t* __restrict__ pieces, float* __restrict__ sums, float2* __restrict__ range,
+                   uint16_t* __restrict__ xp, int32_t* err) {
   pdl_trigger();
   pdl_wait();
-  const int m = blockIdx.y, c = blockIdx.x * kSplitThreads + threadIdx.x;  // token, chunk of eight elements
-  const bool in = c < K / 8;  // K is a multiple of 128: whole groups of 16 lanes are in or out
-  uint4 v = make_uint4(0, 0, 0, 0);
-  if (m < M && in) {
-    const uint16_t* xr = x + (long long)m * K;
-    if (perm == nullptr) {
-      v = ld_nc16(xr + c * 8);
-    } else {
-      bool bad = false;
-      uint32_t e[8];
+  const int m = blockIdx.y, lane = threadIdx.x & 31, chunks = K / 8;  // whole groups of 16 chunks
+  const uint16_t* xr = x + (long long)m * K;
+  bool bad = false;
+  auto load = [&](int c) {  // eight elements; past the row or the tokens: zeros
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (m < M && c < chunks) {
+      if (perm == nullptr) {
+        v = ld_nc16(xr + c * 8);
+      } else {
+        uint32_t e[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int k = perm[c * 8 + i];
-        const bool ok = (unsigned)k < (unsigned)K;
-        bad |= !ok;
-        e[i] = ok ? (uint32_t)xr[k] : 0u;
+        for (int i = 0; i < 8; ++i) {
+          const int k = perm[c * 8 + i];
+          const bool ok = (unsigned)k < (unsigned)K;
+          bad |= !ok;
+          e[i] = ok ? (uint32_t)xr[k] : 0u;
+        }
+        v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
       }
-      v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
-      if (bad && err) atomicExch(err, 1);
     }
+    return v;
+  };
+  uint32_t row = 0;  // TOKEN: the row's largest
+  __shared__ uint32_t red[TOKEN ? kSplitRowThreads / 32 : 1];
+  __shared__ float2 part[TOKEN ? kSplitRowThreads / 32 : 1];
+  if constexpr (TOKEN) {
+    for (int c = threadIdx.x; c < chunks; c += kSplitRowThreads) {
+      const uint4 v = load(c);
+      if (xp != nullptr && m < M) *reinterpret_cast<uint4*>(xp + (long long)m * K + c * 8) = v;
+      row = f8_amax(row, v);
+    }
+    row = __reduce_max_sync(0xffffffffu, row);
+    if (lane == 0) red[threadIdx.x >> 5] = row;
+    __syncthreads();
+    row = __reduce_max_sync(0xffffffffu, red[lane]);
   }
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  // |x| as bf16 bits orders like the values, infinities and NaN on top
-  uint32_t am = 0;
-  bool over = false;  // beyond the fp16 range but not NaN
+  float lost = 0.f, all = 0.f, few = 0.f;  // squares: what the pieces lose, x, x below 2^-8 of the largest
+  int small = 0;
+  // (groups: one round, of whose threads all take part in the reductions)
+  int c0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+  do {
+    const int c = c0 + lane;
+    const uint4 v = load(c);
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t am = TOKEN ? row : f8_amax(0, v);
+    if constexpr (!TOKEN) {
+      bool over = false;  // beyond the fp16 range but not NaN
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t a = w[i] & 0x7FFFu, b = (w[i] >> 16) & 0x7FFFu;
-    am = max(am, max(a, b));
-    over |= (a >= 0x4780u && a <= 0x7F80u) || (b >= 0x4780u && b <= 0x7F80u);
-  }
-  // tokens that a kernel staging x in fp16 refuses are refused here too
-  if (over && err) atomicExch(err, 3);
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t a = w[i] & 0x7FFFu, b = (w[i] >> 16) & 0x7FFFu;
+        over |= (a >= 0x4780u && a <= 0x7F80u) || (b >= 0x4780u && b <= 0x7F80u);
+      }
+      // tokens that a kernel staging x in fp16 refuses are refused here too
+      if (over && err) atomicExch(err, 3);
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, o));  // the group's 16 lanes
-
-  // e = 134 - biased exponent of the maximum, kept where 2^e and 2^-e are normal
-  const int ex = (int)(am >> 7);
-  const int e = am == 0 || ex == 255 ? 0 : min(126, 134 - ex);
-  const float mul = __uint_as_float((uint32_t)(127 + e) << 23);
-  float hi_sum = 0.f, lo_sum = 0.f;
-  uint32_t hb[4], lb[4];  // e4m3 pairs (2i, 2i + 1)
+      for (int o = 8; o > 0; o >>= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, o));  // the group's 16 lanes
+    }
+    // e = 134 - biased exponent of the largest, kept where 2^e and 2^-e are normal
+    const int ex = (int)(am >> 7);
+    const int e = am == 0 || ex == 255 ? 0 : min(126, 134 - ex);
+    const float mul = __uint_as_float((uint32_t)(127 + e) << 23);
+    float hi_sum = 0.f, lo_sum = 0.f;
+    uint32_t hb[4], lb[4];  // e4m3 pairs (2i, 2i + 1)
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float2 f = bf2x2f(w[i]);
-    f.x *= mul;
-    f.y *= mul;
-    const __nv_fp8x2_storage_t h = __nv_cvt_float2_to_fp8x2(f, __NV_SATFINITE, __NV_E4M3);
-    const float2 hf = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(h, __NV_E4M3)));
-    const float2 r = make_float2((f.x - hf.x) * 32.f, (f.y - hf.y) * 32.f);
-    const __nv_fp8x2_storage_t l = __nv_cvt_float2_to_fp8x2(r, __NV_SATFINITE, __NV_E4M3);
-    const float2 lf = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(l, __NV_E4M3)));
-    hi_sum += hf.x + hf.y;
-    lo_sum += lf.x + lf.y;
-    hb[i] = h;
-    lb[i] = l;
-  }
-  // a packed int4 word masked with 0x0F0F0F0F holds elements 0, 4, 1, 5, and
-  // shifted by four bits 2, 6, 3, 7
-  const uint2 ho = make_uint2(__byte_perm(hb[0], hb[2], 0x5140), __byte_perm(hb[1], hb[3], 0x5140));
-  const uint2 lo = make_uint2(__byte_perm(lb[0], lb[2], 0x5140), __byte_perm(lb[1], lb[3], 0x5140));
-  float sum = hi_sum + lo_sum * (1.f / 32.f);
+    for (int i = 0; i < 4; ++i) {
+      float2 f = bf2x2f(w[i]);
+      f.x *= mul;
+      f.y *= mul;
+      const __nv_fp8x2_storage_t h = __nv_cvt_float2_to_fp8x2(f, __NV_SATFINITE, __NV_E4M3);
+      const float2 hf = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(h, __NV_E4M3)));
+      const float2 r = make_float2((f.x - hf.x) * 32.f, (f.y - hf.y) * 32.f);
+      const __nv_fp8x2_storage_t l = __nv_cvt_float2_to_fp8x2(r, __NV_SATFINITE, __NV_E4M3);
+      const float2 lf = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(l, __NV_E4M3)));
+      hi_sum += hf.x + hf.y;
+      lo_sum += lf.x + lf.y;
+      if constexpr (TOKEN) {
+        const float dx = r.x - lf.x, dy = r.y - lf.y;  // 32 times what the pieces lose
+        lost += dx * dx + dy * dy;
+        all += f.x * f.x + f.y * f.y;
+        if (fabsf(f.x) < 1.f) few += f.x * f.x, small += c < chunks;
+        if (fabsf(f.y) < 1.f) few += f.y * f.y, small += c < chunks;
+      }
+      hb[i] = h;
+      lb[i] = l;
+    }
+    // a packed int4 word masked with 0x0F0F0F0F holds elements 0, 4, 1, 5, and
+    // shifted by four bits 2, 6, 3, 7
+    const uint2 ho = make_uint2(__byte_perm(hb[0], hb[2], 0x5140), __byte_perm(hb[1], hb[3], 0x5140));
+    const uint2 lo = make_uint2(__byte_perm(lb[0], lb[2], 0x5140), __byte_perm(lb[1], lb[3], 0x5140));
+    float sum = hi_sum + lo_sum * (1.f / 32.f);
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (!in) return;
-  const int g = c >> 4, ch = (c & 15) >> 1, half = c & 1;
-  uint8_t* base = pieces + (long long)g * (2 * MT * 128);
-  *reinterpret_cast<uint2*>(base + m * 128 + ((ch ^ (m & 7)) << 4) + half * 8) = ho;
-  *reinterpret_cast<uint2*>(base + (MT + m) * 128 + ((ch ^ ((MT + m) & 7)) << 4) + half * 8) = lo;
-  if ((c & 15) == 0) {
-    float* o = sums + (long long)g * (2 * MT) + m;
-    o[0] = sum * (1.f / 512.f);
-    o[MT] = __uint_as_float(ex == 255 ? 0x7FC00000u : (uint32_t)(127 - e) << 23);
+    for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (c < chunks) {
+      const int g = c >> 4, ch = (c & 15) >> 1, half = c & 1;
+      uint8_t* base = pieces + (long long)g * (2 * MT * 128);
+      *reinterpret_cast<uint2*>(base + m * 128 + ((ch ^ (m & 7)) << 4) + half * 8) = ho;
+      *reinterpret_cast<uint2*>(base + (MT + m) * 128 + ((ch ^ ((MT + m) & 7)) << 4) + half * 8) = lo;
+      if ((c & 15) == 0) {
+        float* o = sums + (long long)g * (2 * MT) + m;
+        o[0] = sum * (1.f / 512.f);
+        o[MT] = __uint_as_float(ex == 255 ? 0x7FC00000u : (uint32_t)(127 - e) << 23);
+      }
+    }
+  } while (TOKEN && (c0 += kSplitRowThreads) < chunks);
+  if (bad && err) atomicExch(err, 1);
+  if constexpr (TOKEN) {
+    // the token's squares; where most of its elements are below 2^-8 of the largest, only
+    // those count as kept
+    const int warp = threadIdx.x >> 5;
+    const float most = warp_sum(few);
+    lost = warp_sum(lost);
+    all = warp_sum(all);
+    small = __reduce_add_sync(0xffffffffu, small);
+    __shared__ float smalls[kSplitRowThreads / 32];
+    __shared__ int counts[kSplitRowThreads / 32];
+    if (lane == 0) part[warp] = make_float2(lost, all), smalls[warp] = most, counts[warp] = small;
+    __syncthreads();
+    if (warp == 0) {
+      lost = warp_sum(part[lane].x);
+      all = warp_sum(part[lane].y);
+      few = warp_sum(smalls[lane]);
+      small = __reduce_add_sync(0xffffffffu, counts[lane]);
+      if (lane == 0)
+        range[m] = (row >> 7) == 255 ? make_float2(1.f, 0.f)  // an infinity or a NaN: lost
+                                     : make_float2(lost / 1024.f, 2 * small >= K ? few : all);
+    }
   }
 }
 
@@ -206,21 +277,26 @@ FP_DEV float2 fmul2(float2 a, float2 b) {
 }
 
 // Output column `row` of tokens m0 .. m0 + T - 1 (those below M) from their
-// sums v (SwiGLU: gate sums v, up sums w).  The residuals are read before any
-// store (R may be Y itself).
-template <int EPI, int T>
-FP_DEV void f8_store(const float* v, const float* w, int M, int m0, int row, int Nout, const uint16_t* R, void* Y) {
-  float rv[T];
+// sums v (SwiGLU: gate sums v, up sums w), times the tokens' powers of two (UN).  The
+// residuals are read before any store (R may be Y itself).
+template <int EPI, int T, bool UN>
+FP_DEV void f8_store(const float* v, const float* w, int M, int m0, int row, int Nout, const float* __restrict__ unscale,
+                     const uint16_t* R, void* Y) {
+  float un[T], rv[T];
 #pragma unroll
-  for (int t = 0; t < T; ++t)
-    rv[t] = EPI == FP_EPI_RESID ? bf2f(R[(long long)min(m0 + t, M - 1) * Nout + row]) : 0.f;
+  for (int t = 0; t < T; ++t) {
+    const int m = min(m0 + t, M - 1);
+    un[t] = UN ? __ldg(unscale + m) : 1.f;
+    rv[t] = EPI == FP_EPI_RESID ? bf2f(R[(long long)m * Nout + row]) : 0.f;
+  }
 #pragma unroll
   for (int t = 0; t < T; ++t) {
     if (m0 + t >= M) break;
+    const float a = UN ? v[t] * un[t] : v[t];
     uint16_t* y = (uint16_t*)Y + (long long)(m0 + t) * Nout + row;
-    if constexpr (EPI == FP_EPI_STORE) *y = f2bf(v[t]);
-    else if constexpr (EPI == FP_EPI_RESID) *y = f2bf(rv[t] + v[t]);
-    else *y = f2bf(silu(v[t]) * w[t]);
+    if constexpr (EPI == FP_EPI_STORE) *y = f2bf(a);
+    else if constexpr (EPI == FP_EPI_RESID) *y = f2bf(rv[t] + a);
+    else *y = f2bf(silu(a) * (UN ? w[t] * un[t] : w[t]));
   }
 }
 
@@ -228,9 +304,9 @@ FP_DEV void f8_store(const float* v, const float* w, int M, int m0, int row, int
 // order (deterministic) with the loads of several CTAs in flight together
 // (one after the other they took 4 us of a 5120 x 5120 matrix).  Not inlined:
 // its registers would crowd the loop over the items.
-template <int EPI, int T>
+template <int EPI, int T, bool UN>
 __device__ __noinline__ void f8_sum_store(const float* p0, size_t slot, int cnt, int M, int m0, int row, int Nout,
-                                          const uint16_t* R, void* Y) {
+                                          const float* __restrict__ unscale, const uint16_t* R, void* Y) {
   constexpr bool GLU = EPI == FP_EPI_SWIGLU;
   constexpr int B = T < 8 ? T : 8, U = GLU ? 2 : 4;
   if (row >= Nout) return;
@@ -255,7 +331,7 @@ __device__ __noinline__ void f8_sum_store(const float* p0, size_t slot, int cnt,
 #pragma unroll
         for (int k = 0; k < B; ++k) v[k] += a[u][k], w[k] += e[u][k];
     }
-    f8_store<EPI, B>(v, w, M, m0 + t0, row, Nout, R, Y);
+    f8_store<EPI, B, UN>(v, w, M, m0 + t0, row, Nout, unscale, R, Y);
   }
 }
 
@@ -269,6 +345,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
                    long long total, int S, float* __restrict__ ws, unsigned* __restrict__ counters, int32_t* err) {
   using G = F8Geom<MT>;
   constexpr bool GLU = EPI == FP_EPI_SWIGLU;
+  constexpr bool GE = MT <= 16;  // an exponent a group, not a token
   constexpr int WS = G::kWStages, XS = G::kXStages, NA = G::kSlots, ND = G::kAccs, TH = MT / 2;
   constexpr int TR = GLU ? kF8Rows / 2 : kF8Rows;  // output rows per tile
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -440,6 +517,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
     // ---------------- group sums to accumulators, row tiles to the output
     const int qd = warp & 3, lr = qd * 32 + lane, par = (warp - kF8WarpEpi) >> 2;
     const uint32_t lane_base = tmem + ((uint32_t)(qd * 32) << 16);
+    constexpr int CH = MT <= 16 ? MT : 16;  // tokens per TMEM load
     // scales and zeros of this thread's weight row, the two groups of its next item
     auto wrow = [&](int bb) -> long long {  // the row of the weight matrix (clamped: rows past the end are not stored)
       if (GLU) return min(bb * TR + (lr & (TR - 1)), Nout - 1) + (lr >= TR ? (long long)Nout : 0LL);
@@ -490,22 +568,25 @@ __global__ void __launch_bounds__(kF8Threads, 1)
             const float2 s2 = make_float2(s, s), nz2 = make_float2(-z, -z), r32 = make_float2(1.f / 32.f, 1.f / 32.f);
             const float* xs = xs_ring + r * (4 * MT) + j * (2 * MT);
             const uint32_t d = lane_base + (q % ND) * 2 * G::kN + j * G::kN;
-            float4 xv[MT / 4], uv[MT / 4];  // read while the sums come from TMEM
 #pragma unroll
-            for (int t = 0; t < MT / 4; ++t) {
-              xv[t] = *reinterpret_cast<const float4*>(xs + 4 * t);
-              uv[t] = *reinterpret_cast<const float4*>(xs + MT + 4 * t);
-            }
-            uint32_t hi[MT], lo[MT];
-            tc_ld_pair<MT>(d, d + MT, hi, lo);
+            for (int c0 = 0; c0 < MT; c0 += CH) {
+              float4 xv[CH / 4], uv[CH / 4];  // read while the sums come from TMEM
 #pragma unroll
-            for (int k = 0; k < MT; k += 2) {
-              const float4 x4 = xv[k / 4], u4 = uv[k / 4];
-              const float2 xx = k & 2 ? make_float2(x4.z, x4.w) : make_float2(x4.x, x4.y);
-              const float2 uu = k & 2 ? make_float2(u4.z, u4.w) : make_float2(u4.x, u4.y);
-              float2 v = ffma2(nz2, xx, make_float2(__uint_as_float(hi[k]), __uint_as_float(hi[k + 1])));
-              v = ffma2(make_float2(__uint_as_float(lo[k]), __uint_as_float(lo[k + 1])), r32, v);
-              acc[k / 2] = ffma2(s2, fmul2(uu, v), acc[k / 2]);
+              for (int t = 0; t < CH / 4; ++t) {
+                xv[t] = *reinterpret_cast<const float4*>(xs + c0 + 4 * t);
+                if (GE) uv[t] = *reinterpret_cast<const float4*>(xs + MT + c0 + 4 * t);
+              }
+              uint32_t hi[CH], lo[CH];
+              tc_ld_pair<CH>(d + c0, d + MT + c0, hi, lo);
+#pragma unroll
+              for (int k = 0; k < CH; k += 2) {
+                const float4 x4 = xv[k / 4], u4 = GE ? uv[k / 4] : make_float4(1.f, 1.f, 1.f, 1.f);
+                const float2 xx = k & 2 ? make_float2(x4.z, x4.w) : make_float2(x4.x, x4.y);
+                const float2 uu = k & 2 ? make_float2(u4.z, u4.w) : make_float2(u4.x, u4.y);
+                float2 v = ffma2(nz2, xx, make_float2(__uint_as_float(hi[k]), __uint_as_float(hi[k + 1])));
+                v = ffma2(make_float2(__uint_as_float(lo[k]), __uint_as_float(lo[k + 1])), r32, v);
+                acc[(c0 + k) / 2] = ffma2(s2, GE ? fmul2(uu, v) : v, acc[(c0 + k) / 2]);
+              }
             }
           }
         }
@@ -561,7 +642,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
         constexpr int B = TH < 8 ? TH : 8;
         if (row < Nout) {
 #pragma unroll
-          for (int t = 0; t < TH; t += B) f8_store<EPI, B>(av + t, av + t, M, m0 + t, row, Nout, R, Y);
+          for (int t = 0; t < TH; t += B) f8_store<EPI, B, !GE>(av + t, av + t, M, m0 + t, row, Nout, sums + MT, R, Y);
         }
         continue;
       }
@@ -582,8 +663,8 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       t = __shfl_sync(0xffffffffu, t, 0);
       if (t != last) continue;
       __threadfence();
-      f8_sum_store<EPI, TH>(ws + (size_t)(tb + c0) * slot + (GLU ? (lr & (TR - 1)) : lr), slot, (int)(c1 - c0) + 1, M, m0,
-                            row, Nout, R, Y);
+      f8_sum_store<EPI, TH, !GE>(ws + (size_t)(tb + c0) * slot + (GLU ? (lr & (TR - 1)) : lr), slot, (int)(c1 - c0) + 1, M, m0,
+                            row, Nout, sums + MT, R, Y);
       if (lane == 0) *ticket = 0u;
     }
   }
@@ -607,13 +688,15 @@ static int f8_sms() {
   return n;
 }
 
-static int f8_mt(int M) { return M <= 8 ? 8 : 16; }
+static int f8_mt(int M) { return M <= 8 ? 8 : M <= 16 ? 16 : 32; }
 
-// fp32 partials, then the x pieces and their group sums and powers of two.
+// fp32 partials, then the x pieces and their group sums and powers of two; beyond 16
+// tokens, behind what the kernel that may take over writes, the range sums and x in the
+// order of perm.
 struct F8Plan {
   long long tiles, total;
   int ctas, S;
-  size_t pieces, sums, bytes;  // offsets behind the ticket area
+  size_t pieces, sums, range, xp, bytes;  // offsets
 };
 
 static F8Plan f8_plan(int epi, int M, int N, int K) {
@@ -628,7 +711,10 @@ static F8Plan f8_plan(int epi, int M, int N, int K) {
   auto up = [](size_t b) { return (b + 127) / 128 * 128; };
   p.pieces = (size_t)kLinTicketSlots * 4 + up((size_t)(p.tiles + p.ctas) * M * kF8Rows * 4);
   p.sums = p.pieces + (size_t)p.S * 2 * mt * 128;
-  p.bytes = p.sums + up((size_t)p.S * 2 * mt * 4);
+  p.range = p.sums + up((size_t)p.S * 2 * mt * 4);
+  if (M > 16) p.range = up(std::max(p.range, q4tc_ws_bytes(epi, M, N, K)));
+  p.xp = p.range + (M > 16 ? up((size_t)mt * sizeof(float2)) : 0);
+  p.bytes = p.xp + (M > 16 ? up((size_t)M * K * 2) : 0);
   return p;
 }
 
@@ -642,17 +728,20 @@ static F8Plan f8_plan(int epi, int M, int N, int K) {
 //   10240 x 8192   19.0 / 25.4   19.3 / 26.8   23.3 / 31.4   23.6 / 33.0
 //   5120 x 13824   17.7 / 27.9   18.2 / 29.7   22.0 / 32.1   22.3 / 34.1
 //   57344 x 8192   59.7 /  109   61.5 /  113   73.8 /  133   74.4 /  135 (SwiGLU)
+//   tokens           17            32          (SwiGLU; here / the bf16 expansion in TMEM)
+//   57344 x 8192   98.2 / 104    100.1 / 108
 // The line was set at 8 MB of codes before the mma.sync GEMV had clusters; matrices of
 // 8 to 20 MB that are wider than long have since been 1-2 us faster there at up to 8
-// tokens.  Not beyond 16 tokens, where the bf16 expansion in TMEM takes x as it is
-// (57344 x 8192 with SwiGLU at 32 tokens 109 us there, 99 with an instance of this
-// kernel): one element of 2^18 beside unit normals, its weights zero, left an error of
-// 0.054 here and 0.0027 there, and a row with an infinity gave NaN.
-static bool f8_pays(int M, int N, int K) { return M <= 16 && (long long)N * K >= (1LL << 24); }
+// tokens, with larger errors.  From 17 tokens only the largest gate and up matrices gain.
+static bool f8_pays(int epi, int M, int N, int K) {
+  const long long weights = (long long)N * K;
+  return M <= 16 ? weights >= (1LL << 24)
+                 : M <= 32 && epi == FP_EPI_SWIGLU && weights >= (1LL << 28) && q4tc_ok(FP_W_INT4_G128, epi, M, N, K);
+}
 
 bool f8_ok(int wquant, int epi, int M, int N, int K) {
   if (wquant != FP_W_INT4_G128 || epi == FP_EPI_F32 || M < 1 || N < 1 || K < 128 || K % 128 != 0) return false;
-  if (!f8_pays(M, N, K) || (epi == FP_EPI_SWIGLU && N % 2 != 0)) return false;
+  if (!f8_pays(epi, M, N, K) || (epi == FP_EPI_SWIGLU && N % 2 != 0)) return false;
   const long long nout = epi == FP_EPI_SWIGLU ? N / 2 : N;
   const long long tiles = (nout + kF8Rows - 1) / kF8Rows;  // eight tickets per 128 output rows
   return tiles * 8 <= kLinTicketSlots && tensor_maps_available();
@@ -697,11 +786,22 @@ cudaError_t launch_f8(int epi, const uint16_t* x, const int32_t* perm, int M, in
   if (!make_tensor_map(&mw, codes, N, K / 2, 1, epi == FP_EPI_SWIGLU ? kF8Rows / 2 : kF8Rows, kF8RowBytes, 128))
     return cudaErrorInvalidValue;
   char* w = (char*)ws;
-  FP_CUDA_TRY(launch(split_x_kernel, dim3((K / 8 + kSplitThreads - 1) / kSplitThreads, mt), dim3(kSplitThreads), 0, s, x,
-                     M, mt, K, perm, (uint8_t*)(w + p.pieces), (float*)(w + p.sums), err));
+  uint8_t* pieces = (uint8_t*)(w + p.pieces);
+  float* sums = (float*)(w + p.sums);
+  float2* range = (float2*)(w + p.range);
+  uint16_t* xp = M > 16 && perm ? (uint16_t*)(w + p.xp) : nullptr;
+  if (M <= 16)
+    FP_CUDA_TRY(launch(split_x_kernel<false>, dim3((K / 8 + kSplitThreads - 1) / kSplitThreads, mt), dim3(kSplitThreads), 0,
+                       s, x, M, mt, K, perm, pieces, sums, range, xp, err));
+  else
+    FP_CUDA_TRY(launch(split_x_kernel<true>, dim3(1, mt), dim3(kSplitRowThreads), 0, s, x, M, mt, K, perm, pieces, sums,
+                       range, xp, err));
   switch (mt) {
     case 8: return launch_f8_m<8>(epi, mw, p, w, M, N, scales, zeros, residual, y, err, s);
-    default: return launch_f8_m<16>(epi, mw, p, w, M, N, scales, zeros, residual, y, err, s);
+    case 16: return launch_f8_m<16>(epi, mw, p, w, M, N, scales, zeros, residual, y, err, s);
+    default:  // SwiGLU: no residual that y may be
+      FP_CUDA_TRY((launch_f8_t<32, FP_EPI_SWIGLU>(mw, p, w, M, N, scales, zeros, residual, y, err, s)));
+      return launch_q4tc_if_wide(xp ? xp : x, M, N, K, codes, scales, zeros, y, ws, ws_bytes, err, s, range);
   }
 }
 

@@ -164,12 +164,25 @@ FP_DEV void i8_word(uint32_t w, uint32_t* out) {
 
 FP_DEV long long q4_cta_of(long long i, long long C, long long total) { return ((i + 1) * C - 1) / total; }
 
-template <int MT, int EPI, int WQ, int KI>
+// Whether x, split into two 8-bit pieces with an exponent a token, loses more than
+// 2^-10 of a token (2-norm): range holds each token's squares lost and squares to be kept.
+// The bf16 rounding of the weights loses 2^-9.8 of each product.
+FP_DEV bool f8_wide(const float2* __restrict__ range, int M, int lane) {
+  const float2 t = lane < M ? range[lane] : make_float2(0.f, 0.f);
+  return __any_sync(0xffffffffu, t.x * (1024.f * 1024.f) > t.y);
+}
+
+// IF_WIDE: returns at once unless f8_wide.
+template <int MT, int EPI, int WQ, int KI, bool IF_WIDE = false>
 __global__ void __launch_bounds__(kQ4Threads, 1)
     gemv_q4tc_kernel(const __grid_constant__ CUtensorMap map_x, const uint8_t* __restrict__ codes, int M, int N,
                      const uint16_t* __restrict__ scales, const uint16_t* __restrict__ zeros, const uint16_t* R,
                      void* Y, long long total, int S, int V, float* __restrict__ ws, unsigned* __restrict__ counters,
-                     int32_t* err, const uint16_t* X, long long check) {
+                     int32_t* err, const uint16_t* X, long long check, const float2* range) {
+  if constexpr (IF_WIDE) {
+    pdl_wait();
+    if (!f8_wide(range, M, threadIdx.x & 31)) return;
+  }
   constexpr int NR = EPI == FP_EPI_SWIGLU ? 2 : 1;
   using G = Q4Geom<MT, NR, WQ, KI>;
   constexpr bool I4 = WQ == FP_W_INT4_G128;
@@ -593,12 +606,13 @@ size_t q4tc_ws_bytes(int epi, int M, int N, int K) {
   return (size_t)kLinTicketSlots * 4 + (size_t)(blocks + ctas) * M * nr * kQ4Rows * 4;
 }
 
-template <int MT, int EPI, int WQ, int KI>
+template <int MT, int EPI, int WQ, int KI, bool IF_WIDE = false>
 static cudaError_t launch_q4_t(const uint8_t* codes, const CUtensorMap& mx, int M, int N, int K,
                                const uint16_t* scales, const uint16_t* zeros, const uint16_t* R, void* Y, void* ws,
-                               int32_t* err, const uint16_t* X, long long check, cudaStream_t s) {
+                               int32_t* err, const uint16_t* X, long long check, cudaStream_t s,
+                               const float2* range = nullptr) {
   constexpr int NR = EPI == FP_EPI_SWIGLU ? 2 : 1;
-  auto kern = gemv_q4tc_kernel<MT, EPI, WQ, KI>;
+  auto kern = gemv_q4tc_kernel<MT, EPI, WQ, KI, IF_WIDE>;
   const int smem = std::max(Q4Geom<MT, NR, WQ, KI>::kSmem, kQ4MinSmem);
   static std::atomic<unsigned long long> attr{0};
   FP_CUDA_TRY(smem_limit_once(kern, smem, &attr));
@@ -609,8 +623,11 @@ static cudaError_t launch_q4_t(const uint8_t* codes, const CUtensorMap& mx, int 
   const int ctas = (int)std::min<long long>(total, q4_sms());
   unsigned* counters = (unsigned*)ws;
   float* part = (float*)((char*)ws + (size_t)kLinTicketSlots * 4);
+  if constexpr (IF_WIDE)
+    return launch_early(kern, dim3(ctas), dim3(kQ4Threads), (size_t)smem, s, mx, codes, M, N, scales, zeros, R, Y, total,
+                        S, q4_v(S), part, counters, err, X, check, range);
   return launch(kern, dim3(ctas), dim3(kQ4Threads), (size_t)smem, s, mx, codes, M, N, scales, zeros, R, Y, total, S,
-                WQ == FP_W_INT4_G128 ? q4_v(S) : 1, part, counters, err, X, check);
+                WQ == FP_W_INT4_G128 ? q4_v(S) : 1, part, counters, err, X, check, range);
 }
 
 // k per item: int4 two groups where K allows (SwiGLU items already carry two
@@ -635,6 +652,19 @@ static cudaError_t launch_q4_w(int epi, const uint8_t* mw, const CUtensorMap& mx
       return two ? launch_q4_t<MT, FP_EPI_F32, WQ, K2>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, X, check, s)
                  : launch_q4_t<MT, FP_EPI_F32, WQ, 128>(mw, mx, M, N, K, scales, zeros, R, Y, ws, err, X, check, s);
   }
+}
+
+cudaError_t launch_q4tc_if_wide(const uint16_t* x, int M, int N, int K, const void* codes, const uint16_t* scales,
+                                const uint16_t* zeros, void* y, void* ws, size_t ws_bytes, int32_t* err, cudaStream_t s,
+                                const float2* range) {
+  constexpr int epi = FP_EPI_SWIGLU;
+  if (!q4tc_ok(FP_W_INT4_G128, epi, M, N, K) || M > 32 || !ws || ws_bytes < q4tc_ws_bytes(epi, M, N, K))
+    return cudaErrorInvalidValue;
+  CUtensorMap mx;
+  // x [M][K] bf16, box [32 rows][64]
+  if (!make_tensor_map(&mx, x, M, K, 2, 32, 64, 128)) return cudaErrorInvalidValue;
+  return launch_q4_t<32, epi, FP_W_INT4_G128, 128, true>((const uint8_t*)codes, mx, M, N, K, scales, zeros, nullptr, y, ws,
+                                                         err, nullptr, 0, s, range);
 }
 
 cudaError_t launch_q4tc(int wquant, int epi, const uint16_t* x, int M, int N, int K, const void* codes,

@@ -305,14 +305,17 @@ bool bad_shape(const fp_arch* a, int wq, std::string& why) {
 
 // One block linear: the GPTQ4 path or the weight-only linear of the handle's
 // format.  At decode both int4 formats take a second kernel (x split into its
-// pieces, or gathered into the act order), counted here.
+// pieces, or gathered into the act order), and with 8-bit operands beyond 16
+// tokens a third, counted here.
 cudaError_t block_linear(fp_handle* h, int epi, const uint16_t* x, int M, const Mat& W, const uint16_t* R, void* y) {
+  const bool f8 = f8_ok(h->wq == FP_W_GPTQ4 ? FP_W_INT4_G128 : h->wq, epi, M, W.N, W.K);
+  if (f8 && M > 16) h->launches += 1;
   if (h->wq == FP_W_GPTQ4) {
     if (M <= 64) h->launches += 1;
     return launch_linear_gptq4(epi, x, M, W.N, W.K, W.perm, W.inv, W.codes, W.scales, W.zeros, R, y, h->lin_ws,
                                h->lin_ws_bytes, h->stream, h->err);
   }
-  if (f8_ok(h->wq, epi, M, W.N, W.K)) h->launches += 1;
+  if (f8) h->launches += 1;
   return launch_linear(h->wq, epi, x, M, W.N, W.K, W.codes, W.scales, W.zeros, R, y, h->lin_ws, h->lin_ws_bytes,
                        h->stream, h->err);
 }

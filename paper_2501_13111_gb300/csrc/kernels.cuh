@@ -78,9 +78,11 @@ cudaError_t launch_linear_gptq4(int epi, const uint16_t* x, int M, int N, int K,
                                 cudaStream_t s, int32_t* err);
 
 // ---- int4 decode linear on tcgen05 with 8-bit operands (fp_gemv_f8.cu)
+// Beyond 16 tokens a third kernel runs, the bf16 expansion, which returns at once
+// unless x needs it.
 bool f8_ok(int wquant, int epi, int M, int N, int K);
 size_t f8_ws_bytes(int epi, int M, int N, int K);
-// perm: the act order of a GPTQ4 matrix, else NULL.  Two kernels.
+// perm: the act order of a GPTQ4 matrix, else NULL.  Two kernels (M > 16: three).
 cudaError_t launch_f8(int epi, const uint16_t* x, const int32_t* perm, int M, int N, int K, const void* codes,
                       const uint16_t* scales, const uint16_t* zeros, const uint16_t* residual, void* y, void* ws,
                       size_t ws_bytes, int32_t* err, cudaStream_t s);
@@ -92,6 +94,10 @@ size_t q4tc_ws_bytes(int epi, int M, int N, int K);
 cudaError_t launch_q4tc(int wquant, int epi, const uint16_t* x, int M, int N, int K, const void* codes,
                         const uint16_t* scales, const uint16_t* zeros, const uint16_t* residual, void* y, void* ws,
                         size_t ws_bytes, int32_t* err, cudaStream_t s);
+// The int4 SwiGLU linear at 17-32 tokens, only if f8_wide(range, M); else its kernel returns.
+cudaError_t launch_q4tc_if_wide(const uint16_t* x, int M, int N, int K, const void* codes, const uint16_t* scales,
+                                const uint16_t* zeros, void* y, void* ws, size_t ws_bytes, int32_t* err, cudaStream_t s,
+                                const float2* range);
 
 // ---- bf16 decode linear at 17-64 tokens on tcgen05, TMA-fed (fp_gemv_btc.cu)
 bool btc_ok(int wquant, int epi, int M, int N, int K);

@@ -1,6 +1,7 @@
 """The int4 decode linear with 8-bit operands (large matrices at up to 16
-tokens) against the oracle's dequantisation, on sampled output columns; against the
-general decode path; and the large SwiGLU just beyond it, whose x keeps its range."""
+tokens, the largest SwiGLU at up to 32) against the oracle's dequantisation, on
+sampled output columns; against the general decode path; and, beyond 16 tokens, an x
+of a wide range, which the bf16 expansion takes over."""
 import numpy as np
 import pytest
 
@@ -56,7 +57,8 @@ def _x(m, k, seed):
 # that cover whole tiles and tiles shared by several, every token tile
 @pytest.mark.parametrize("m,n,k,epi", [
     (1, 4104, 4096, 0), (8, 12008, 1408, 1), (9, 4104, 4096, 1), (16, 8240, 2176, 2), (7, 140000, 128, 0),
-    (16, 1200, 14080, 1), (5, 65664, 256, 2), (16, 65600, 4096, 2), (9, 67096, 4096, 2)])
+    (16, 1200, 14080, 1), (5, 65664, 256, 2), (16, 65600, 4096, 2), (9, 67096, 4096, 2),
+    (32, 65536, 4096, 2), (17, 57352, 4864, 2), (24, 21848, 12416, 2)])
 def test_matches_oracle(fp, m, n, k, epi):
     codes, scales, zeros = _weights(fp, n, k, 9)
     x, nout = _x(m, k, 8), n // 2 if epi == 2 else n
@@ -165,42 +167,81 @@ def test_beyond_fp16_is_reported_as_on_the_general_path(fp):
     assert host(err, np.int32)[0] == 3
 
 
-@pytest.mark.parametrize("m", [17, 32])
-def test_beyond_16_tokens_x_keeps_the_range_of_bf16(fp, m):
+def _large_swiglu(fp, m, n, k, x, zeroed, cols, perm=None):
+    """Rows of x through the SwiGLU of an n x k int4 matrix with the weights of channels
+    `zeroed` zero: the result, and the oracle's weights of the gate and up rows of `cols`."""
+    w = empty(n * k, np.uint16)
+    fp.fp_op_init_weights(ptr(w), n * k, 9, 3)
+    w.view(n, k)[:, zeroed] = 0
+    codes, scales, zeros = empty(n * k // 2), empty(n * k // 128, np.uint16), empty(n * k // 128, np.uint16)
+    nout = n // 2
+    out, xd = empty(m * nout, np.uint16), dev(synth.f32_to_bf16_bits(x))
+    if perm is None:
+        fp.fp_op_quantize(2, ptr(w), n, k, ptr(codes), ptr(scales), ptr(zeros))
+        ws_b = fp.fp_op_linear_workspace_bytes(2, m, n, k)
+        ws = empty(ws_b)
+        fp.fp_op_linear(2, 2, ptr(xd), m, n, k, ptr(codes), ptr(scales), ptr(zeros), None, ptr(out), ptr(ws), ws_b)
+    else:
+        pd = dev(perm)
+        fp.fp_op_quantize_gptq4(ptr(w), n, k, ptr(pd), ptr(codes), ptr(scales), ptr(zeros))
+        ws_b = fp.fp_op_linear_gptq4_workspace_bytes(m, n, k)
+        ws = empty(ws_b)
+        fp.fp_op_linear_gptq4(2, ptr(xd), m, n, k, ptr(pd), ptr(codes), ptr(scales), ptr(zeros), None, ptr(out), ptr(ws), ws_b)
+    got = quant.bf16_to_f32(host(out, np.uint16)).reshape(m, nout).astype(np.float64)
+    assert not host(ws, np.uint8)[:16384].any()  # the tickets are zero again
+    rows = np.stack([synth.normal_bf16(9, 3, int(c) * k, k) for c in np.concatenate([cols, cols + nout])])
+    rows[:, zeroed] = 0
+    wd = quant.quantize_weight(rows if perm is None else np.ascontiguousarray(rows[:, perm]), 2)[1]
+    if perm is not None:
+        back = np.empty_like(wd)
+        back[:, perm] = wd
+        wd = back
+    return got, wd[:len(cols)], wd[len(cols):]
+
+
+def _rounded(wd):
+    return quant.bf16_to_f32(synth.f32_to_bf16_bits(wd.astype(np.float32))).astype(np.float64)
+
+
+@pytest.mark.parametrize("m,gptq", [(17, False), (32, False), (20, True)])
+def test_beyond_16_tokens_x_keeps_the_range_of_bf16(fp, m, gptq):
     """The largest SwiGLU matrices at 17 tokens and more: an element of 2^18 whose weights
     are zero must not cost the row's other elements their bits, and an infinity is the
     infinity that its column's weights make of it."""
     n, k, big, inf = 65536, 4096, 1003, 2010
-    w = empty(n * k, np.uint16)
-    fp.fp_op_init_weights(ptr(w), n * k, 9, 3)
-    w.view(n, k)[:, big] = 0
-    codes, scales, zeros = empty(n * k // 2), empty(n * k // 128, np.uint16), empty(n * k // 128, np.uint16)
-    fp.fp_op_quantize(2, ptr(w), n, k, ptr(codes), ptr(scales), ptr(zeros))
     x = quant.bf16_to_f32(synth.uniform_bf16(8, m, (m, k), -2.0, 2.0))
     x[:, big] = 2.0 ** 18
     x[m - 1, inf] = np.inf
-    nout = n // 2
-    ws_b = fp.fp_op_linear_workspace_bytes(2, m, n, k)
-    ws, out = empty(ws_b), empty(m * nout, np.uint16)
-    fp.fp_op_linear(2, 2, ptr(dev(synth.f32_to_bf16_bits(x))), m, n, k, ptr(codes), ptr(scales), ptr(zeros), None,
-                    ptr(out), ptr(ws), ws_b)
-    got = quant.bf16_to_f32(host(out, np.uint16)).reshape(m, nout).astype(np.float64)
-    cols = np.unique(np.concatenate([[0, 1, nout - 1], np.random.default_rng(m).integers(0, nout, 120)]))
-    rows = []
-    for c in np.concatenate([cols, cols + nout]):
-        r = synth.normal_bf16(9, 3, int(c) * k, k).copy()
-        r[big] = 0
-        rows.append(r)
-    # this path multiplies the weights rounded to bf16, x as it is
-    wd = quant.quantize_weight(np.stack(rows), 2)[1]
-    wd = quant.bf16_to_f32(synth.f32_to_bf16_bits(wd.astype(np.float32))).astype(np.float64)
-    g, u = wd[:len(cols)], wd[len(cols):]
+    cols = np.unique(np.concatenate([[0, 1, n // 2 - 1], np.random.default_rng(m).integers(0, n // 2, 120)]))
+    perm = np.random.default_rng(3).permutation(k).astype(np.int32) if gptq else None
+    got, g, u = _large_swiglu(fp, m, n, k, x, [big], cols, perm)
+    g, u = _rounded(g), _rounded(u)  # the expansion multiplies the weights rounded to bf16, x as it is
     xf = x[:m - 1].astype(np.float64)
     ref = M.silu(xf @ g.T) * (xf @ u.T)
     for i in range(m - 1):
         assert rel_err(got[i:i + 1][:, cols], ref[i:i + 1]) <= TOL + 1e-4, (i, rel_err(got[i:i + 1][:, cols], ref[i:i + 1]))
     both = (g[:, inf] > 0) & (u[:, inf] != 0)
     assert both.sum() > 10 and np.array_equal(got[m - 1, cols][both], np.sign(u[both, inf]) * np.inf)
+
+
+@pytest.mark.parametrize("amp", [0.0, 300.0, 2.0 ** 14, 2.0 ** 15, 2.0 ** 16, 2.0 ** 17, 2.0 ** 24])
+def test_beyond_16_tokens_around_the_line(fp, amp):
+    """One token with a large element (its weights zero): up to where the two pieces lose as
+    much as the bf16 rounding of the weights does they are kept, and every token's error stays
+    at either path's: exact weights and x to 2^-10, or x exact and the weights to bf16."""
+    m, n, k, big = 19, 65536, 4096, 1003
+    x = quant.bf16_to_f32(synth.uniform_bf16(8, m, (m, k), -2.0, 2.0))
+    x[m - 2, big] = amp
+    cols = np.unique(np.random.default_rng(m).integers(0, n // 2, 150))
+    got, g, u = _large_swiglu(fp, m, n, k, x, [big], cols)
+    xf = x.astype(np.float64)
+    ref = M.silu(xf @ g.T) * (xf @ u.T)
+    # 2-norm: the result's rounding (2^-8 at most), and 2^-9.8 (2^-10 of the pieces) of each of
+    # two factors; without the large element exact weights and x to 2^-22, the rounding alone
+    bound = TOL if amp <= 300.0 else 2.0 ** -8 + 2 * 1.1 * 2.0 ** -9.8
+    for i in range(m):
+        e = np.linalg.norm(got[i, cols] - ref[i]) / np.linalg.norm(ref[i])
+        assert e <= bound, (i, e)
 
 
 def _dominated(fp, m, n, k, big, zeroed, amp):

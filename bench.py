@@ -106,18 +106,18 @@ def class_roofline(cls, kb, cls_time, launches, peak):
 # bench's B x context.
 NCU_TRAFFIC = {
     # profiles/dram_traffic_l70b.md and dram_traffic_l7b.md: microbench cases, one launch each
-    ("l70b", "lin_gu"): {"bytes": 273504512, "units": None, "src": "fp_gemv_tc.cu", "sha": "4ce5acf290c2928d"},
-    ("l70b", "lin_down"): {"bytes": 130917632, "units": None, "src": "fp_gemv_tc.cu", "sha": "4ce5acf290c2928d"},
-    ("l70b", "lin_qkv"): {"bytes": 45146880, "units": None, "src": "fp_gemv_tc.cu", "sha": "4ce5acf290c2928d"},
-    ("l70b", "lin_o"): {"bytes": 36759552, "units": None, "src": "fp_gemv_tc.cu", "sha": "4ce5acf290c2928d"},
-    ("l70b", "lm_head"): {"bytes": 533911808, "units": None, "src": "fp_gemv_btc.cu", "sha": "ac6ffae462038acd"},
-    ("l70b", "attn"): {"bytes": 149513984, "units": 32 * 2148, "src": "fp_attention.cu", "sha": "011e2b422a5fa35c"},
-    ("l7b", "attn"): {"bytes": 81405952, "units": 8 * 612, "src": "fp_attention.cu", "sha": "011e2b422a5fa35c"},
-    ("l7b", "lm_head"): {"bytes": 270177792, "units": None, "src": "fp_linear.cu", "sha": "136661144db50e97"},
-    ("l7b", "lin_gu"): {"bytes": 94035456, "units": None, "src": "fp_linear.cu", "sha": "136661144db50e97"},
-    ("l7b", "lin_qkv"): {"bytes": 50459904, "units": None, "src": "fp_linear.cu", "sha": "136661144db50e97"},
-    ("l7b", "lin_o"): {"bytes": 16946176, "units": None, "src": "fp_linear.cu", "sha": "136661144db50e97"},
-    ("l7b", "lin_down"): {"bytes": 45368320, "units": None, "src": "fp_linear.cu", "sha": "136661144db50e97"},
+    ("l70b", "lin_gu"): {"bytes": 265981184, "units": None, "src": "fp_gemv_f8.cu", "sha": "54d83eb1fd597143"},
+    ("l70b", "lin_down"): {"bytes": 130942720, "units": None, "src": "fp_gemv_tc.cu", "sha": "e1a320328478ba20"},
+    ("l70b", "lin_qkv"): {"bytes": 45145856, "units": None, "src": "fp_gemv_tc.cu", "sha": "e1a320328478ba20"},
+    ("l70b", "lin_o"): {"bytes": 36758784, "units": None, "src": "fp_gemv_tc.cu", "sha": "e1a320328478ba20"},
+    ("l70b", "lm_head"): {"bytes": 533270528, "units": None, "src": "fp_gemv_btc.cu", "sha": "3d6b4041735b8b50"},
+    ("l70b", "attn"): {"bytes": 149517824, "units": 32 * 2148, "src": "fp_attention.cu", "sha": "2e4af3438b741111"},
+    ("l7b", "attn"): {"bytes": 81332736, "units": 8 * 612, "src": "fp_attention.cu", "sha": "2e4af3438b741111"},
+    ("l7b", "lm_head"): {"bytes": 270159872, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
+    ("l7b", "lin_gu"): {"bytes": 94297344, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
+    ("l7b", "lin_qkv"): {"bytes": 50457344, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
+    ("l7b", "lin_o"): {"bytes": 16950016, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
+    ("l7b", "lin_down"): {"bytes": 45372416, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
 }
 
 

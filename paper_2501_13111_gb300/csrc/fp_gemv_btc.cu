@@ -288,7 +288,8 @@ bool btc_ok(int wquant, int epi, int M, int N, int K) {
 
 // Where this kernel beats the mma.sync GEMV (its TMEM, first copies and last tile cost
 // about 10 us before any gain): larger matrices, fewer weights the more tokens, and
-// SwiGLU, whose items carry half the k, from 32 items an SM.  Microseconds, here / mma.sync:
+// SwiGLU, whose items carry half the k, from 32 items an SM.  Microseconds, here / mma.sync,
+// weights from memory:
 //   17 tokens  4096 x 11008 25.2 / 31.4   10240 x 8192 34.8 / 43.3   8192 x 14336 47.0 / 58.9
 //              6144 x 4096 17.2 / 19.9    4096 x 4096 16.5 / 13.4    16384 x 1088 16.8 / 16.2
 //   40         4096 x 4096 22.4 / 22.9    3072 x 4096 15.7 / 21.7    5120 x 13824 38.5 / 60.7

@@ -102,9 +102,10 @@ static int dec_max_clusters(int occ, int cl) {
     static std::atomic<unsigned long long> attr{0};
     int n = 0;
     if (smem_limit_once(dec_room_kernel, 228 * 1024 / 2 - 1024, &attr) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, dec_room_kernel, &cfg) != cudaSuccess || n < 0)
-      n = 0;
-    (void)cudaGetLastError();
+        cudaOccupancyMaxActiveClusters(&n, dec_room_kernel, &cfg) != cudaSuccess || n < 0) {
+      (void)cudaGetLastError();
+      return 0;
+    }
     v = n + 1;
     known[occ][cl].store(v, std::memory_order_relaxed);
   }

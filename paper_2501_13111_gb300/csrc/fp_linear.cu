@@ -838,8 +838,10 @@ static int gemv_max_clusters(int occ, int cl, int smem) {
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemv_mma_kernel<WQ, NT, EPI, true>, &cfg) != cudaSuccess || n < 0) n = 0;
-    (void)cudaGetLastError();
+    if (cudaOccupancyMaxActiveClusters(&n, gemv_mma_kernel<WQ, NT, EPI, true>, &cfg) != cudaSuccess || n < 0) {
+      (void)cudaGetLastError();
+      return 0;
+    }
     v = n + 1;
     known[occ][cl].store(v, std::memory_order_relaxed);
   }

@@ -5,8 +5,8 @@
 // memory each): with a single key tile there is nothing to pipeline inside a CTA,
 // so two of them overlap instead.  Bound by latency, one chain of copy, product,
 // softmax, product per CTA.  8 prompts of 128 tokens, 32 heads, bf16 / int8 cache:
-// 7.7 / 15.1 us here, 12.4 / 20.6 on the persistent kernel of fp_attn_tc.cu (one CTA
-// per SM), 11.4 / 15.9 with one lane running the MMA loop and row-wise stores.
+// 7.7 / 13.2 us here, 12.4 / 20.6 on the persistent kernel of fp_attn_tc.cu (one CTA
+// per SM).
 //   warp 0      TMA: the Q tile (two 64-column boxes), then (bf16 cache) the K
 //               rows and the V rows page by page, one box per lane;
 //   warp 1      owns the TMEM, issues S = Q K^T, then O = P V;
@@ -143,6 +143,15 @@ __global__ void __launch_bounds__(KV8 ? 256 : 192, 2)
       // row; the lanes of the upper half store the odd chunk first, so the
       // eight lanes of one row write eight distinct 16-byte bank groups
       const int cb = 2 * (c & 3), half_off = (c >> 2) * kPaHalf;
+      // the scales are read here, so that their loads are in flight together: read
+      // row by row where they are stored, 47 prompts of 126 tokens, 32 heads take
+      // 84.1 us instead of 69.4
+      float sck[kPsRows], scv[kPsRows];
+#pragma unroll
+      for (int r = 0; r < kPsRows; ++r) {
+        sck[r] = c == 0 && rowi[r] >= 0 ? __ldg(k_scale + rowi[r]) : 0.f;
+        scv[r] = c == 0 && rowi[r] >= 0 ? __ldg(v_scale + rowi[r]) * vmul : 0.f;
+      }
 #pragma unroll 1
       for (int which = 0; which < 2; ++which) {
         const int8_t* pool = which ? v8 : k8;
@@ -170,8 +179,8 @@ __global__ void __launch_bounds__(KV8 ? 256 : 192, 2)
             *reinterpret_cast<uint4*>(rp + ((cb ^ sw) << 4)) = e;
           }
           if (which == 0 && c == 0) {  // the scales go out with the K codes
-            s_scl[row] = rowi[r] >= 0 ? __ldg(k_scale + rowi[r]) : 0.f;
-            s_scl[kPaB + row] = rowi[r] >= 0 ? __ldg(v_scale + rowi[r]) * vmul : 0.f;
+            s_scl[row] = sck[r];
+            s_scl[kPaB + row] = scv[r];
           }
         }
         if (which == 0 && wi == 0) s_unscale = exp2f((float)-sigma);

@@ -726,8 +726,8 @@ cudaError_t launch_attention_prefill_tc(const uint16_t* q, int q_stride, int B, 
   if (!make_tensor_map(&mq, q, (long long)B * S, q_stride, 2, kPaB, 64, 128)) return cudaErrorInvalidValue;
   // B: the grid's y extent.  Pairs of heads that share keys and values take over where the
   // short kernel (two CTAs an SM) has more than a round (int8 cache, whose codes it widens
-  // once a head) or three.  H 64 on 8, 128 tokens, short / pairs, us: int8 4 prompts 15.1 / 14.7,
-  // 8 27.5 / 22.1, 32 110 / 69; bf16 8 13.2 / 15.1, 16 24.8 / 24.1, 32 49 / 39
+  // once a head) or three.  H 64 on 8, 128 tokens, short / pairs, us: int8 4 prompts 13.5 / 14.1,
+  // 8 24.8 / 21.7, 32 93 / 69; bf16 8 13.2 / 15.1, 16 24.8 / 24.1, 32 49 / 39
   const bool kv8 = kv.kvquant == FP_KV_INT8, shared = n_heads / kv.n_kv_heads % 2 == 0;
   const bool one_tile = S <= kPaB && B <= 65535 && !(shared && (long long)B * n_heads > (kv8 ? 2 : 6) * pa_sms());
   if (kv8)

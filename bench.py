@@ -111,13 +111,13 @@ NCU_TRAFFIC = {
     ("l70b", "lin_qkv"): {"bytes": 45145856, "units": None, "src": "fp_gemv_tc.cu", "sha": "e1a320328478ba20"},
     ("l70b", "lin_o"): {"bytes": 36758784, "units": None, "src": "fp_gemv_tc.cu", "sha": "e1a320328478ba20"},
     ("l70b", "lm_head"): {"bytes": 533270528, "units": None, "src": "fp_gemv_btc.cu", "sha": "3d6b4041735b8b50"},
-    ("l70b", "attn"): {"bytes": 149517824, "units": 32 * 2148, "src": "fp_attention.cu", "sha": "2e4af3438b741111"},
-    ("l7b", "attn"): {"bytes": 81332736, "units": 8 * 612, "src": "fp_attention.cu", "sha": "2e4af3438b741111"},
-    ("l7b", "lm_head"): {"bytes": 270159872, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
-    ("l7b", "lin_gu"): {"bytes": 94297344, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
-    ("l7b", "lin_qkv"): {"bytes": 50457344, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
-    ("l7b", "lin_o"): {"bytes": 16950016, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
-    ("l7b", "lin_down"): {"bytes": 45372416, "units": None, "src": "fp_linear.cu", "sha": "283840ea43507165"},
+    ("l70b", "attn"): {"bytes": 149488128, "units": 32 * 2148, "src": "fp_attention.cu", "sha": "1fe196096e508eea"},
+    ("l7b", "attn"): {"bytes": 81349888, "units": 8 * 612, "src": "fp_attention.cu", "sha": "1fe196096e508eea"},
+    ("l7b", "lm_head"): {"bytes": 270129408, "units": None, "src": "fp_linear.cu", "sha": "254b407cb334640a"},
+    ("l7b", "lin_gu"): {"bytes": 94096128, "units": None, "src": "fp_linear.cu", "sha": "254b407cb334640a"},
+    ("l7b", "lin_qkv"): {"bytes": 50456320, "units": None, "src": "fp_linear.cu", "sha": "254b407cb334640a"},
+    ("l7b", "lin_o"): {"bytes": 16950016, "units": None, "src": "fp_linear.cu", "sha": "254b407cb334640a"},
+    ("l7b", "lin_down"): {"bytes": 45372672, "units": None, "src": "fp_linear.cu", "sha": "254b407cb334640a"},
 }
 
 
